@@ -1,9 +1,9 @@
 """``torch.autograd`` front end of the library: ``blossom_attention(q, k, v, gate_logits, ...)``.
 
-Plumbing only: it allocates the outputs and the workspace with PyTorch, calls
-``blossom_attn_fwd`` / ``blossom_attn_bwd`` through the C ABI on the current stream and hands the
-gradients back to autograd.  Every step of the method runs in the CUDA library; there is no
-PyTorch fallback.  The selection is not differentiated (top-k is piecewise constant).
+Plumbing only, and native (``csrc/front.cpp``, built into ``_front.so``): it allocates the outputs
+and the workspace with PyTorch, calls ``blossom_attn_fwd`` / ``blossom_attn_bwd`` through the C ABI
+on the current stream and hands the gradients back to autograd.  Every step of the method runs in
+the CUDA library; there is no PyTorch fallback.  The selection is not differentiated (top-k is piecewise constant).
 """
 from __future__ import annotations
 
@@ -61,61 +61,23 @@ def check_arguments(q, k, v, gate_logits, seq_lens, require_cuda=True, gate_mode
     return seq_lens
 
 
-class _BlossomAttention(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, q, k, v, gate_logits, seq_lens, block_size, top_k, window, sm_scale,
-                stis_mode, stis_block, cmp_block, cmp_stride, per_query=0, phi_logits=None,
-                gate_mode=0, causal=1, rope_theta=0.0):
-        seq_lens = check_arguments(q, k, v, gate_logits, seq_lens, gate_mode=gate_mode)
-        B, H, L, D = q.shape
-        Hkv = k.shape[1]
-        # The library addresses every q-shaped buffer with q's strides and every k-shaped one with
-        # k's: views that are not dense (a slice of a packed projection) are copied first.
-        if not (_dense(q) and q.stride(3) == 1):
-            q = q.contiguous()
-        if not (_dense(k) and k.stride(3) == 1 and k.stride() == v.stride()):
-            k, v = k.contiguous(), v.contiguous()
-        if Hkv == H and k.stride() != q.stride():
-            k, v = _like(q).copy_(k), _like(q).copy_(v)
-        params = binding.make_params(B, H, L, D, block_size, top_k, window, _DT[q.dtype],
-                                     sm_scale=sm_scale, strides=q.stride()[:3], stis_mode=stis_mode,
-                                     stis_block=stis_block, cmp_block=cmp_block, cmp_stride=cmp_stride,
-                                     kv_heads=Hkv, kv_strides=k.stride()[:3], select_mode=int(per_query),
-                                     phi_logits=phi_logits, gate_mode=int(gate_mode), causal=int(causal),
-                                     rope_theta=float(rope_theta))
-        nbytes = binding.blossom_workspace_bytes(params)
-        if nbytes == 0:
-            raise binding.BlossomError(binding.BLOSSOM_ERR_UNSUPPORTED, "blossom_workspace_bytes")
-        dev = q.device
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=dev)
-        gate = gate_logits.detach().to(torch.float32).contiguous()
-        M = -(-L // block_size)
-        idx = torch.empty((B, Hkv, L if per_query else M, top_k), dtype=torch.int32, device=dev)
-        out, out_lt, out_st = _like(q), _like(q), _like(q)
-        lse = torch.empty((2, B, H, L), dtype=torch.float32, device=dev)
-        binding.blossom_attn_fwd(params, q, k, v, gate, seq_lens, idx, 0, out, out_lt, out_st, lse,
-                                 workspace)
-        ctx.params, ctx.workspace, ctx.seq_lens = params, workspace, seq_lens
-        ctx.phi_logits = phi_logits  # the params hold its address: keep it alive until the backward
-        ctx.gate_dtype = gate_logits.dtype
-        ctx.save_for_backward(q, k, v, gate, idx, out_lt, out_st, lse)
-        ctx.mark_non_differentiable(idx)
-        return out, idx
+_native = None
 
-    @staticmethod
-    def backward(ctx, dout, _didx):
-        q, k, v, gate, idx, out_lt, out_st, lse = ctx.saved_tensors
-        if dout.stride() != q.stride() or dout.dtype != q.dtype:  # the library wants q's layout
-            dout = _like(q).copy_(dout)
-        dq, dk, dv = _like(q), _like(k), _like(k)
-        dgate = torch.empty(tuple(gate.shape), dtype=torch.float32, device=q.device)
-        # the workspace is this call's own and its last user was the training forward above (or an
-        # earlier backward, which leaves the lists alone): the backward may reuse that call's tile lists
-        params = binding.blossom_params.from_buffer_copy(ctx.params)
-        params.reuse_tile_lists = 1
-        binding.blossom_attn_bwd(params, q, k, v, gate, ctx.seq_lens, idx, out_lt, out_st, lse,
-                                 dout, dq, dk, dv, dgate, ctx.workspace)
-        return (dq, dk, dv, dgate.to(ctx.gate_dtype)) + (None,) * 14
+
+def _front():
+    """The native front end (``csrc/front.cpp``), loaded on first use: it validates, allocates the
+    outputs and one scratch buffer, calls ``blossom_attn_fwd`` and puts a C++ node into the autograd
+    graph that calls ``blossom_attn_bwd``."""
+    global _native
+    if _native is None:
+        binding.load()  # the same instance of the library, and its own message if it is missing
+        try:
+            from . import _front as m
+        except ImportError as e:
+            raise RuntimeError("_front.so is missing or stale: build it with "
+                               "`python -m paper_2512_13368_b200.build`") from e
+        _native = m.attention
+    return _native
 
 
 def blossom_attention(q, k, v, gate_logits, block_size, top_k, window, seq_lens=None, sm_scale=0.0,
@@ -155,9 +117,11 @@ def blossom_attention(q, k, v, gate_logits, block_size, top_k, window, seq_lens=
         phi_logits = phi_logits.detach().contiguous()
     if short_term not in ("window", "power-law"):
         raise ValueError("short_term must be 'window' or 'power-law'")
-    out, idx = _BlossomAttention.apply(q, k, v, gate_logits, seq_lens, int(block_size), int(top_k),
-                                       int(window), float(sm_scale),
-                                       1 if short_term == "power-law" else 0, int(mask_block),
-                                       int(cmp_block), int(cmp_stride), int(bool(select_per_query)), phi_logits,
-                                       int(bool(input_dependent_gate)), int(bool(causal)), float(rope_theta))
-    return (out, idx) if return_indices else out
+    res = (_native or _front())(
+        q, k, v, gate_logits, seq_lens, phi_logits, block_size, top_k, window, sm_scale,
+        1 if short_term == "power-law" else 0, mask_block, cmp_block, cmp_stride, 1 if select_per_query else 0,
+        1 if input_dependent_gate else 0, 1 if causal else 0, rope_theta)
+    if res is None:  # not what the library can be handed: say why
+        check_arguments(q, k, v, gate_logits, seq_lens, gate_mode=int(bool(input_dependent_gate)))
+        raise ValueError("blossom_attention: unusable arguments")
+    return res if return_indices else res[0]

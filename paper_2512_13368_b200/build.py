@@ -1,7 +1,8 @@
-"""Builds the CUDA library in-tree: ``paper_2512_13368_b200/libblossom.so`` (sm_100a only).
+"""Builds the CUDA library in-tree, ``paper_2512_13368_b200/libblossom.so`` (sm_100a only), and the
+native half of the autograd front end, ``_front.so``.
 
 Run as ``python -m paper_2512_13368_b200.build`` or call ``build()``; nvcc cross-compiles
-without a GPU.  The shared object is loaded with ctypes (see ``binding.py``).
+without a GPU.  The library is loaded with ctypes (see ``binding.py``); the front end links it.
 """
 from __future__ import annotations
 
@@ -13,6 +14,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libblossom.so")
+FRONT_SRC = os.path.join(CSRC, "front.cpp")
+FRONT = os.path.join(HERE, "_front.so")  # native half of autograd.py (links libblossom.so and PyTorch)
 OBJ = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = [
@@ -32,6 +35,20 @@ def _stale(target, deps):
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def front_command(out):
+    """g++ command of the autograd front end: a CPython module against PyTorch's headers and libraries."""
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    inc = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], "/usr/local/cuda/include"]
+    libs = [a for d in cpp_extension.library_paths() for a in ("-L" + d,)]
+    return ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-w",
+             "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)]
+            + [a for d in inc for a in ("-isystem", d)] + [FRONT_SRC, "-o", out] + libs
+            + ["-L" + HERE, "-l:libblossom.so", "-Wl,-rpath,$ORIGIN", "-ltorch_python", "-ltorch", "-ltorch_cpu",
+               "-ltorch_cuda", "-lc10", "-lc10_cuda"])
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -65,8 +82,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     if force or procs or _stale(LIB, objs):
         tmp = LIB + ".tmp.%d" % os.getpid()
-        subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ["-cudart", "static"])
+        subprocess.check_call([nvcc, "-shared", "-Xlinker", "-soname=libblossom.so", "-o", tmp] + objs + ["-cudart", "static"])
         os.replace(tmp, LIB)
+    if force or _stale(FRONT, [FRONT_SRC, headers[-1]]):
+        tmp = FRONT + ".tmp.%d" % os.getpid()
+        subprocess.check_call(front_command(tmp))
+        os.replace(tmp, FRONT)
     return LIB
 
 

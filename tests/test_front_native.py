@@ -1,0 +1,54 @@
+"""The native half of the autograd front end: calls without a gradient, partial gradients, repeated
+backwards, and what it refuses."""
+import pytest
+
+from paper_2512_13368_b200 import build
+
+
+def test_host_tensors_are_refused_with_the_reason():
+    import torch
+    build.build()
+    from paper_2512_13368_b200.autograd import blossom_attention
+    q = torch.zeros(1, 2, 32, 32)
+    with pytest.raises(ValueError):
+        blossom_attention(q, q, q, torch.zeros(2, 2), 16, 2, 8)
+    with pytest.raises(TypeError):
+        blossom_attention(q.double(), q.double(), q.double(), torch.zeros(2, 2), 16, 2, 8)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,L,lens", [("bf16", 33, None), ("bf16", 300, "int64"), ("fp32", 70, "int32")])
+def test_calls_without_a_gradient_and_partial_gradients(dtype, L, lens):
+    import torch
+    from paper_2512_13368_b200.autograd import blossom_attention
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda")  # noqa: E731
+    q, k, v = (mk(3, 2, L, 32).to(dt).requires_grad_(True) for _ in range(3))
+    gate, dout = mk(2, 2).requires_grad_(True), mk(3, 2, L, 32).to(dt)
+    n = None if lens is None else torch.tensor([L, 1, L // 2], dtype=getattr(torch, lens), device="cuda")
+    call = lambda *a: blossom_attention(*a, 16, 3, 9, seq_lens=n, return_indices=True)  # noqa: E731
+    out, idx = call(q, k, v, gate)
+    assert out.requires_grad and not idx.requires_grad
+    full = torch.autograd.grad(out, (q, k, v, gate), dout, retain_graph=True)
+    again = torch.autograd.grad(out, (q, k, v, gate), dout)
+    assert all(torch.equal(a, b) for a, b in zip(full, again))
+    with pytest.raises(RuntimeError):   # the graph has been released
+        torch.autograd.grad(out, (q,), dout)
+    with torch.no_grad():
+        out2, idx2 = call(q, k, v, gate)
+    assert not out2.requires_grad and torch.equal(out, out2) and torch.equal(idx, idx2)
+    d = [t.detach() for t in (q, k, v, gate)]
+    for i in range(4):                  # only one input wants a gradient
+        a = list(d)
+        a[i] = d[i].clone().requires_grad_(True)
+        o, _ = call(*a)
+        (gi,) = torch.autograd.grad(o, (a[i],), dout)
+        assert torch.equal(o, out) and torch.equal(gi, full[i])
+    half = d[3].to(torch.bfloat16).requires_grad_(True)   # a gate stored in another type gets its gradient in it
+    (gh,) = torch.autograd.grad(call(d[0], d[1], d[2], half)[0], (half,), dout)
+    assert gh.dtype == torch.bfloat16
+    with pytest.raises(ValueError):
+        blossom_attention(d[0], d[1], d[2], mk(3, 2), 16, 3, 9)
+    with pytest.raises(RuntimeError):   # BlossomError: the library does not take top_k = 0
+        blossom_attention(*d, 16, 0, 9)
