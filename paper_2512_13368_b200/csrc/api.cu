@@ -223,10 +223,14 @@ static bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintp
 // selection clears both sets (a new step begins), a backward only its own, so a wait that ran out
 // in the forward is still on record after the backward that follows it on the same workspace.
 static int check_workspace(const Shape &s, void *ws, size_t bytes, cudaStream_t st, Workspace *out,
-                           bool backward = false) {
+                           bool backward = false, bool short_path = false) {
   if (!ws || misaligned(ws, 256)) return BLOSSOM_ERR_WORKSPACE;
   *out = carve_workspace(s, ws);
   if (bytes < out->bytes) return BLOSSOM_ERR_WORKSPACE;
+  // (the short-history forward clears the words itself, and with them what its backward counts in)
+  if (short_path && (!backward || s.reuse_lists)) return BLOSSOM_OK;
+  if (short_path)
+    return cudaMemsetAsync(out->status_bwd, 0, (sh::kCounterWord - 3) * 4, st) == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
   if (cudaMemsetAsync(backward ? out->status_bwd : out->status, 0, backward ? 16 : 32, st) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
   return BLOSSOM_OK;
@@ -291,11 +295,15 @@ int blossom_attn_fwd(const blossom_params *params, const void *q, const void *k,
       misaligned(gate_logits, 4) || misaligned(block_idx, 4) || misaligned(seq_lens, 4))
     return BLOSSOM_ERR_INVALID_ARG;
   Workspace ws;
-  rc = check_workspace(s, workspace, workspace_bytes, (cudaStream_t)stream, &ws);
-  if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  const bool short_path = !force_simt() && sh::fwd_short_supported(s, params->dtype, out_lt != nullptr);
+  rc = check_workspace(s, workspace, workspace_bytes, st, &ws, false, short_path);
+  if (rc) return rc;
   rc = rotate_inputs(s, params->dtype, ws, &q, &k, st);
   if (rc) return rc;
+  if (short_path)
+    return sh::launch_fwd_short(s, q, k, v, gate_logits, seq_lens, block_idx, idx_is_input, out, out_lt, out_st, lse, ws,
+                                st);
   if (!idx_is_input) {
     rc = launch_select(s, params->dtype, q, k, seq_lens, block_idx, ws, st);
     if (rc) return rc;
@@ -329,12 +337,17 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
       misaligned(gate_logits, 4) || misaligned(block_idx, 4) || misaligned(seq_lens, 4))
     return BLOSSOM_ERR_INVALID_ARG;
   Workspace ws;
-  rc = check_workspace(s, workspace, workspace_bytes, (cudaStream_t)stream, &ws, true);
-  if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  const bool short_path = !force_simt() && sh::bwd_short_supported(s, params->dtype);
+  rc = check_workspace(s, workspace, workspace_bytes, st, &ws, true, short_path);
+  if (rc) return rc;
   rc = rotate_inputs(s, params->dtype, ws, &q, &k, st, s.reuse_lists != 0);
   if (rc) return rc;
-  if (!force_simt() && tc::fwd_tc_supported(s, params->dtype)) {
+  if (!force_simt() && sh::fwd_short_supported(s, params->dtype, true)) s.reuse_lists = 0;  // (that forward builds no lists)
+  if (short_path) {
+    rc = sh::launch_bwd_short(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout, dq, dk, dv, dgate,
+                              ws, st);
+  } else if (!force_simt() && tc::fwd_tc_supported(s, params->dtype)) {
     if (s.gate_mode) {
       rc = tc::launch_bwd_tc_gate(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout,
                                   dq, dk, dv, dgate, ws, st);
@@ -444,7 +457,7 @@ int blossom_profile_stop(int32_t *kernel_ids, float *ms, int capacity) {
 const char *blossom_kernel_name(int id) {
   static const char *names[K_COUNT] = {
       "summary", "score_select", "fwd_simt", "bwd_dq_simt", "bwd_dkdv_simt", "gate_grad",
-      "fwd_tc", "bwd_dq_tc", "bwd_dkdv_tc", "score_fast", "bwd_prep", "tc_meta", "rope"};
+      "fwd_tc", "bwd_dq_tc", "bwd_dkdv_tc", "score_fast", "bwd_prep", "tc_meta", "rope", "bwd_short"};
   return (id >= 0 && id < K_COUNT) ? names[id] : "unknown";
 }
 

@@ -73,7 +73,8 @@ extern unsigned long long g_launches;  // host-side launch counter
 // Kernel identifiers reported by the optional per-launch event profile.
 enum KernelId {
   K_SUMMARY = 0, K_SCORE_SELECT, K_FWD_SIMT, K_BWD_DQ_SIMT, K_BWD_DKDV_SIMT, K_GATE_GRAD,
-  K_FWD_TC, K_BWD_DQ_TC, K_BWD_DKDV_TC, K_SCORE_FAST, K_BWD_PREP, K_TC_META, K_ROPE, K_COUNT
+  K_FWD_TC, K_BWD_DQ_TC, K_BWD_DKDV_TC, K_SCORE_FAST, K_BWD_PREP, K_TC_META, K_ROPE, K_BWD_SHORT,
+  K_COUNT
 };
 void prof_mark(int id, int phase, cudaStream_t st);  // no-op unless a profile is running
 
@@ -225,6 +226,21 @@ int launch_fwd_tc(const Shape &s, const void *q, const void *k, const void *v, c
                   const int32_t *seq_lens, const int32_t *idx, void *out, void *out_lt, void *out_st,
                   float *lse, const Workspace &ws, cudaStream_t st);
 }  // namespace tc
+
+namespace sh {
+// Short histories (bf16): one kernel per direction.  The choices depend on the shape (and on whether the
+// forward saves for a backward) alone, so a backward knows what the forward before it ran.
+bool fwd_short_supported(const Shape &s, int dtype, bool training);
+bool bwd_short_supported(const Shape &s, int dtype);
+int launch_fwd_short(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
+                     const int32_t *seq_lens, int32_t *idx, int idx_is_input, void *out, void *out_lt, void *out_st,
+                     float *lse, const Workspace &ws, cudaStream_t st);
+int launch_bwd_short(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
+                     const int32_t *seq_lens, const int32_t *idx, const void *out_lt, const void *out_st,
+                     const float *lse, const void *dout, void *dq, void *dk, void *dv, float *dgate,
+                     const Workspace &ws, cudaStream_t st);
+constexpr int kCounterWord = 16;  // word of the status area: CTAs of the short backward that have finished
+}  // namespace sh
 
 // BLOSSOM_FORCE_SIMT=1 in the environment routes every call to the fp32 CUDA-core kernels.
 bool force_simt();

@@ -24,7 +24,7 @@
 // With left padding a block is live exactly when it reaches past the padding, so liveness is a
 // comparison of indices (cmin, jmin below); the counts of valid keys are kept for callers that
 // want them.
-#include "common.cuh"
+#include "select_geom.cuh"
 
 #include <cooperative_groups.h>
 
@@ -33,36 +33,6 @@ namespace blossom {
 namespace cg = cooperative_groups;
 
 namespace {
-
-// Geometry of the scored blocks.
-struct SelGeom {
-  int n;       // scored blocks per (batch, key/value head): Mc, or M in the plain mode
-  int l, s;    // their length and stride in positions
-  int rs, rl;  // Bk / s and l / s, the two sums of Eq. 11 (1, 1 in the plain mode)
-  int plain;
-};
-
-SelGeom sel_geom(const Shape &sh) {
-  SelGeom g;
-  if (sh.cmp_l > 0) {
-    g.n = sh.Mc; g.l = sh.cmp_l; g.s = sh.cmp_s; g.rs = sh.Bk / sh.cmp_s; g.rl = sh.cmp_l / sh.cmp_s;
-    g.plain = 0;
-  } else {
-    g.n = sh.M; g.l = sh.Bk; g.s = sh.Bk; g.rs = 1; g.rl = 1; g.plain = 1;
-  }
-  return g;
-}
-
-// scored blocks 0 .. nc - 1 end before query block b starts
-__device__ __forceinline__ int n_candidates(const Shape &sh, const SelGeom &g, int b) {
-  if (g.plain) return b;
-  const int start = b * sh.Bk;
-  return start >= g.l ? min(g.n, (start - g.l) / g.s + 1) : 0;
-}
-// the first scored block that holds a valid key (pad0 = number of padded positions)
-__device__ __forceinline__ int first_live_scored(const SelGeom &g, int pad0) {
-  return pad0 < g.l ? 0 : (pad0 - g.l) / g.s + 1;
-}
 
 // Eight consecutive elements as loaded (16 bytes of bf16, 32 of fp32), unpacked to floats on use.
 template <typename T>

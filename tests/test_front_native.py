@@ -37,7 +37,8 @@ def test_calls_without_a_gradient_and_partial_gradients(dtype, L, lens):
         torch.autograd.grad(out, (q,), dout)
     with torch.no_grad():
         out2, idx2 = call(q, k, v, gate)
-    assert not out2.requires_grad and torch.equal(out, out2) and torch.equal(idx, idx2)
+    assert not out2.requires_grad and torch.equal(idx, idx2)   # (other kernels may serve it: not the same bits)
+    assert torch.allclose(out.float(), out2.float(), rtol=1e-2, atol=1e-2 if dtype == "bf16" else 1e-5)
     d = [t.detach() for t in (q, k, v, gate)]
     for i in range(4):                  # only one input wants a gradient
         a = list(d)
