@@ -88,7 +88,7 @@ Workspace carve_workspace(const Shape &s, void *base) {
   w.klive = reinterpret_cast<int32_t *>(take(units * s.M * sizeof(int32_t)));
   w.kmean32 = reinterpret_cast<float *>(take(units * s.M * s.D * sizeof(float)));
   w.knorm = reinterpret_cast<float *>(take(units * s.M * sizeof(float)));
-  w.sel_list = reinterpret_cast<int32_t *>(take(units * s.M * sizeof(int32_t)));
+  w.sel_list = reinterpret_cast<int32_t *>(take((size_t)s.B * (s.pq ? (size_t)s.Hkv * s.L : (size_t)s.H * s.M) * sizeof(int32_t)));
   w.sel_count = reinterpret_cast<int32_t *>(take(256));
   w.delta = reinterpret_cast<float *>(take(2 * units * s.L * sizeof(float)));
   w.dalpha = reinterpret_cast<double *>(take(units * s.M * sizeof(double)));

@@ -42,7 +42,8 @@ struct Workspace {
   int32_t *klive;    // [B][H][M]     number of valid keys in the block
   float *kmean32;    // [B][H][M][D]  the means rounded to fp32 (single-precision scoring stage)
   float *knorm;      // [B][H][M]     upper bound of the Euclidean norm of each fp32 mean
-  int32_t *sel_list; // [B][H][M]     query blocks whose choice the fp32 stage could not certify
+  int32_t *sel_list; // [B][H][M]     query blocks (per position: [B][Hkv][L] positions) whose choice the
+                     //               fp32 stage could not certify
   int32_t *sel_count;// [1]           length of that list
   float *delta;      // [2][B][H][L]  rowsum(G_branch o O_branch) for the backward
   double *dalpha;    // [B][H][M]     per query block partial of d alpha

@@ -24,7 +24,7 @@
 // With left padding a block is live exactly when it reaches past the padding, so liveness is a
 // comparison of indices (cmin, jmin below); the counts of valid keys are kept for callers that
 // want them.
-#include "select_geom.cuh"
+#include "select_rows.cuh"
 
 #include <cooperative_groups.h>
 
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kFastThreads, 3) score_fast_kernel(
   }
 }
 
-// ---- stage 2: the same scores in double precision ------------------------------------------
+// ---- stage 2: the same scores in double precision (more than 128 scored blocks) --------------
 // One CTA of 256 threads per query block of the work list (every query block when worklist ==
 // nullptr).  64 query rows at a time (the block's queries of the group's heads, head-major)
 // against 64 candidate means at a time: thread (row tid / 4, part tid % 4) forms the 16 logits of
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kFastThreads, 3) score_fast_kernel(
 // is the order a single CTA adds them in.  The work of a query block is otherwise serial, and the
 // work list is short (a few per cent of the query blocks), so without the split the kernel's time
 // is that of one CTA walking G * Bk rows.
-template <typename T, int D, int NZ>  // NZ: chunks of 64 candidates whose logits a thread may keep in registers
+template <typename T, int D>
 __global__ void __launch_bounds__(256, 2) score_exact_kernel(
     Shape sh, SelGeom g, const T *__restrict__ q, const double *__restrict__ mean,
     const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx, const int32_t *__restrict__ worklist,
@@ -713,36 +713,16 @@ __global__ void __launch_bounds__(256, 2) score_exact_kernel(
           __syncthreads();
           if (tid < nb) Sc[c0 + tid] += (csum[tid] + csum[64 + tid]) + (csum[128 + tid] + csum[192 + tid]);
         };
-        double mx = -INFINITY, den = 0.0;
-        if (ch_hi - ch_lo <= NZ) {
-          // the logits of all (one or two) chunks stay in registers
-          double za[16], zb[NZ > 1 ? 16 : 1];
-          uint32_t ona = 0u, onb = 0u;
-          const bool two = NZ > 1 && ch_hi - ch_lo == 2;
-          logits(ch_lo, za, ona);
-          fold(za, ona, mx, den);
-          if constexpr (NZ > 1) {
-            if (two) {
-              logits(ch_lo + 1, zb, onb);
-              fold(zb, onb, mx, den);
-            }
-          }
-          columns(ch_lo, za, ona, mx, den);
-          if constexpr (NZ > 1) {
-            if (two) columns(ch_lo + 1, zb, onb, mx, den);
-          }
-        } else {
-          // more: one pass for the maxima and normalisers, a second one for the probabilities
-          double z[16];
-          uint32_t on;
-          for (int ch = ch_lo; ch < ch_hi; ++ch) {
-            logits(ch, z, on);
-            fold(z, on, mx, den);
-          }
-          for (int ch = ch_lo; ch < ch_hi; ++ch) {
-            logits(ch, z, on);
-            columns(ch, z, on, mx, den);
-          }
+        // one pass for the maxima and normalisers, a second one for the probabilities
+        double mx = -INFINITY, den = 0.0, z[16];
+        uint32_t on;
+        for (int ch = ch_lo; ch < ch_hi; ++ch) {
+          logits(ch, z, on);
+          fold(z, on, mx, den);
+        }
+        for (int ch = ch_lo; ch < ch_hi; ++ch) {
+          logits(ch, z, on);
+          columns(ch, z, on, mx, den);
         }
       }
     }
@@ -783,220 +763,286 @@ __global__ void __launch_bounds__(256, 2) score_exact_kernel(
   }
 }
 
+// The same for up to 128 scored blocks, 16 rows per CTA: a query block's rows go to the CTAs of a cluster
+// (CTA r takes the 16-row groups r, r + cluster size, ...), whose column sums CTA 0 adds in rank order.
+// The list is short (a few per cent of the query blocks, often a single wave of CTAs), so its time is the
+// latency of one query block: with 64 rows per CTA, a serial chain of 1024 multiply-adds and 16
+// exponentials per thread, it was 21 - 35 us whatever the size.  Here a warp has four rows; a lane forms
+// the logits of one of them against every eighth candidate, two at a time, out of shared memory (16-byte
+// loads, the pitch spreads eight candidates over the banks).
+template <typename T, int D>
+__global__ void __launch_bounds__(128) score_exact16_kernel(
+    Shape sh, SelGeom g, const T *__restrict__ q, const double *__restrict__ mean,
+    const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx, const int32_t *__restrict__ worklist,
+    const int32_t *__restrict__ work_count) {
+  grid_chain_enter();
+  constexpr int PD = D + 2;
+  extern __shared__ __align__(16) double dsm[];
+  __shared__ double bound_d[2];
+  const int M = sh.M, Bk = sh.Bk, nz = (g.n + 1) | 1;
+  double *kd = dsm;                  // [n + 1][PD] candidate means
+  double *qd = kd + (g.n + 1) * PD;  // [16][PD] query rows
+  double *zd = qd + 16 * PD;         // [16][nz] logits, exponentials
+  double *part = zd + 16 * nz;       // [4 warps][128] column sums
+  double *Sc = part + 4 * 128;       // [128] of this CTA
+  double *S = Sc + 128;              // [M] scores of the selection blocks
+  uint8_t *taken = reinterpret_cast<uint8_t *>(S + M);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int r = lane & 3, pt = lane >> 2;
+  const int total = worklist ? *work_count : M * sh.B * sh.Hkv;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int nrank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  // (every CTA of a cluster walks the same query blocks, so the cluster barriers below match up)
+  for (int wi = blockIdx.x / nrank; wi < total; wi += gridDim.x / nrank) {
+    const int row_id = worklist ? worklist[wi] : wi;
+    const int b = row_id % M, u = row_id / M, n = u / sh.Hkv, hk = u % sh.Hkv;
+    int len = seq_lens ? seq_lens[n] : sh.L;
+    len = min(max(len, 0), sh.L);
+    const int pad0 = sh.L - len;
+    const int qlo = max(b * Bk, pad0), qhi = min((b + 1) * Bk, sh.L);
+    int32_t *row = idx + ((int64_t)u * M + b) * sh.topk;
+    __syncthreads();   // shared memory is reused from the previous query block
+    if (qlo >= qhi) {  // the query block holds only padding
+      if (rank == 0)
+        for (int i = tid; i < sh.topk; i += 128) row[i] = -1;
+      continue;
+    }
+    const int cmin = first_live_scored(g, pad0), jmin = pad0 / Bk;
+    // without the causal mask (plain selection only) every other live block is a candidate
+    const int hi = sh.causal ? b : M, own = sh.causal ? 0 : 1;
+    const int nc = sh.causal ? n_candidates(sh, g, b) : g.n, ncol = nc - cmin, skip = own ? b - cmin : -1;
+    const int nsel = max(0, hi - jmin - own), want = min(sh.topk - 1, nsel);
+    const bool score = nsel > want && want > 0 && ncol - own > 0;
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;  // column sums of candidates lane, lane + 32, ...
+    if (score) {
+      const double2 *kb = reinterpret_cast<const double2 *>(mean + ((int64_t)u * g.n + cmin) * D);
+      for (int i = tid; i < ncol * (D / 2); i += 128)
+        *reinterpret_cast<double2 *>(kd + (i / (D / 2)) * PD + (i % (D / 2)) * 2) = kb[i];
+      const int nq = qhi - qlo, nrows = nq * sh.G;  // rows: head x / nq of the group, query qlo + x % nq
+      for (int r0 = 16 * rank; r0 < nrows; r0 += 16 * nrank) {
+        __syncthreads();
+        for (int i = tid; i < 16 * (D / 4); i += 128) {
+          const int lr = i / (D / 4), c = (i % (D / 4)) * 4, x = r0 + lr;
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (x < nrows) v = ld4(q + row_offset(sh, n, hk * sh.G + x / nq, qlo + x % nq) + c);
+          double2 *d = reinterpret_cast<double2 *>(qd + lr * PD + c);
+          d[0] = make_double2((double)v.x, (double)v.y);
+          d[1] = make_double2((double)v.z, (double)v.w);
+        }
+        __syncthreads();
+        const int lr = 4 * warp + r;
+        const double2 *qr = reinterpret_cast<const double2 *>(qd + lr * PD);
+        double *z = zd + lr * nz;
+        double mx = -INFINITY, den = 0.0;
+        for (int c = pt; c < ncol; c += 16) {
+          const int c1 = c + 8 < ncol ? c + 8 : c;
+          const double2 *k0 = reinterpret_cast<const double2 *>(kd + c * PD), *k1 = reinterpret_cast<const double2 *>(kd + c1 * PD);
+          double x0 = 0.0, y0 = 0.0, x1 = 0.0, y1 = 0.0;
+#pragma unroll 8
+          for (int e = 0; e < D / 2; ++e) {
+            const double2 qv = qr[e], a = k0[e], bb = k1[e];
+            x0 = fma(qv.x, a.x, x0);
+            y0 = fma(qv.y, a.y, y0);
+            x1 = fma(qv.x, bb.x, x1);
+            y1 = fma(qv.y, bb.y, y1);
+          }
+          const double z0 = c == skip ? -INFINITY : sh.scale_d * (x0 + y0);
+          const double z1 = c1 == skip ? -INFINITY : sh.scale_d * (x1 + y1);
+          z[c] = z0;
+          if (c1 != c) z[c1] = z1;
+          mx = fmax(mx, fmax(z0, z1));
+        }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        for (int c = pt; c < ncol; c += 8) {
+          const double e = exp(z[c] - mx);  // exp(-inf) = 0
+          z[c] = e;
+          den += e;
+        }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+        const double inv = r0 + lr < nrows ? 1.0 / den : 0.0;
+        __syncwarp();
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const double iv = __shfl_sync(0xffffffffu, inv, x);
+          const double *zx = zd + (4 * warp + x) * nz;
+          if (lane < ncol) s0 = fma(zx[lane], iv, s0);
+          if (lane + 32 < ncol) s1 = fma(zx[lane + 32], iv, s1);
+          if (lane + 64 < ncol) s2 = fma(zx[lane + 64], iv, s2);
+          if (lane + 96 < ncol) s3 = fma(zx[lane + 96], iv, s3);
+        }
+      }
+      part[warp * 128 + lane] = s0;
+      part[warp * 128 + lane + 32] = s1;
+      part[warp * 128 + lane + 64] = s2;
+      part[warp * 128 + lane + 96] = s3;
+      __syncthreads();
+      Sc[tid] = (part[tid] + part[128 + tid]) + (part[256 + tid] + part[384 + tid]);
+    }
+    if (nrank > 1) {
+      cluster.sync();  // every CTA's column sums are complete
+      if (rank == 0 && score && tid < ncol) {
+        double a = Sc[tid];
+        for (int x = 1; x < nrank; ++x) a += cluster.map_shared_rank(Sc, x)[tid];
+        Sc[tid] = a;
+      }
+      cluster.sync();  // the other CTAs' sums have been read: they may go on (or exit)
+      if (rank != 0) continue;
+    }
+    __syncthreads();
+    if (score) {
+      for (int j = jmin + tid; j < hi; j += 128) {  // Eq. 11
+        double acc = 0.0;
+        for (int m = 0; m < g.rs; ++m)
+          for (int e = 0; e < g.rl; ++e) {
+            const int i = g.rs * j - m - e;
+            if (i >= cmin && i < nc) acc += Sc[i - cmin];
+          }
+        S[j] = own && j == b ? -INFINITY : acc;  // the own block is not ranked: it is kept anyway
+      }
+      __syncthreads();
+      for (int j = jmin + tid; j < hi; j += 128) {  // Eq. 13 by rank
+        const double sj = S[j];
+        int rk = 0;
+#pragma unroll 4
+        for (int i = jmin; i < hi; ++i) {
+          const double si = S[i];
+          rk += (si > sj || (si == sj && i < j)) ? 1 : 0;
+        }
+        taken[j] = rk < want ? 1 : 0;
+      }
+    } else {
+      for (int j = jmin + tid; j < hi; j += 128)
+        taken[j] = nsel > want && want > 0 ? (j - jmin < want ? 1 : 0) : (want > 0 ? 1 : 0);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      if (sh.causal) {
+        emit_row(row, taken, jmin, b, sh.topk, lane);
+      } else {  // the own block takes its place in the ascending row
+        if (lane == 0) taken[b] = 1;
+        __syncwarp();
+        emit_flags(row, taken, jmin, hi, sh.topk, lane);
+      }
+    }
+  }
+}
+
 // ---- selection per query position (Eq. 13 as printed), double precision -------------------
-// One warp per (batch, key/value head, position t): the softmax of Eq. 10 over the live blocks
-// before t's block for every head of the group, the probabilities summed over the heads (Eq. 12),
-// the top_k - 1 largest kept together with t's own block, ties to the lower index.  block_idx is
-// [B][Hkv][L][top_k].  Lanes stride over the candidate blocks; the means come from global memory
-// (they are shared by the neighbouring positions and stay in L2).
+// One warp per (batch, key/value head, position t) of the work list (every position when worklist ==
+// nullptr): the softmax of Eq. 10 over the live scored blocks that end before t's block for every head
+// of the group, the probabilities summed over the heads (Eq. 12), Eq. 11, the top_k - 1 largest kept
+// together with t's own block, ties to the lower index.  block_idx is [B][Hkv][L][top_k].  Lanes stride
+// over the candidates; the means come from global memory (they are shared by the neighbouring
+// positions and stay in L2).
 template <typename T, int D>
 __global__ void __launch_bounds__(256) score_per_query_kernel(
-    Shape sh, const T *__restrict__ q, const double *__restrict__ mean,
-    const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx) {
+    Shape sh, SelGeom g, const T *__restrict__ q, const double *__restrict__ mean,
+    const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx, const int32_t *__restrict__ worklist,
+    const int32_t *__restrict__ work_count) {
   grid_chain_enter();
   extern __shared__ double dsm[];
   __shared__ double bound_d[8][2];
   const int M = sh.M, Bk = sh.Bk;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double *P = dsm + (size_t)warp * (2 * M + D);  // [M] summed probabilities of this warp's position
-  double *Z = P + M;                             // [M] logits of the current head
-  double *qrow = Z + M;                          // [D]
-  uint8_t *taken = reinterpret_cast<uint8_t *>(dsm + (size_t)8 * (2 * M + D)) + (size_t)warp * M;
-  const int64_t pos = (int64_t)blockIdx.x * 8 + warp;
-  if (pos >= (int64_t)sh.B * sh.Hkv * sh.L) return;
-  const int t = (int)(pos % sh.L), u = (int)(pos / sh.L), n = u / sh.Hkv, hk = u % sh.Hkv;
-  int len = seq_lens ? seq_lens[n] : sh.L;
-  len = min(max(len, 0), sh.L);
-  const int pad0 = sh.L - len;
-  int32_t *row = idx + pos * sh.topk;
-  if (t < pad0) {
-    for (int i = lane; i < sh.topk; i += 32) row[i] = -1;
-    return;
-  }
-  const int b = t / Bk, jmin = pad0 / Bk;  // live blocks before the own one: jmin .. b - 1
-  const int nsel = max(0, b - jmin), want = min(sh.topk - 1, nsel);
-  if (nsel > want && want > 0) {
-    for (int j = jmin + lane; j < b; j += 32) P[j] = 0.0;
-    const double *kbase = mean + (int64_t)u * M * D;
-    for (int hg = 0; hg < sh.G; ++hg) {
-      __syncwarp();
-      const T *qp = q + row_offset(sh, n, hk * sh.G + hg, t);
-      for (int c = lane; c < D; c += 32) qrow[c] = (double)ld1(qp + c);
-      __syncwarp();
-      double mx = -INFINITY;
-      for (int j = jmin + lane; j < b; j += 32) {
-        const double *kj = kbase + (int64_t)j * D;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-#pragma unroll 4
-        for (int c = 0; c < D; c += 4) {
-          a0 = fma(qrow[c], kj[c], a0);
-          a1 = fma(qrow[c + 1], kj[c + 1], a1);
-          a2 = fma(qrow[c + 2], kj[c + 2], a2);
-          a3 = fma(qrow[c + 3], kj[c + 3], a3);
-        }
-        const double z = sh.scale_d * ((a0 + a1) + (a2 + a3));
-        Z[j] = z;
-        mx = fmax(mx, z);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      double den = 0.0;
-      for (int j = jmin + lane; j < b; j += 32) {
-        const double e = exp(Z[j] - mx);
-        Z[j] = e;
-        den += e;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
-      for (int j = jmin + lane; j < b; j += 32) P[j] += Z[j] / den;  // heads in ascending order
-    }
-    __syncwarp();
-    rank_select<double>(P, jmin, b, want, taken, bound_d[warp], lane);
-  } else {
-    for (int j = jmin + lane; j < b; j += 32) taken[j] = want > 0 ? 1 : 0;
-  }
-  __syncwarp();
-  emit_row(row, taken, jmin, b, sh.topk, lane);
-}
-
-// The same selection, tiled: one CTA of 256 threads per 64 consecutive positions of a (batch,
-// key/value head), for up to 64 NZ scored blocks (the selection blocks themselves, or overlapping
-// compression blocks whose probabilities Eq. 11 maps onto the selection blocks, row by row).  The 64 query rows of one head at a time and
-// 64 candidate means at a time sit in shared memory as doubles; thread (row tid / 4, part tid % 4)
-// forms the 16 logits of candidates part + 4 k per chunk (sixteen independent accumulation
-// chains) and keeps the logits of all chunks in registers; the row's softmax takes 4 lanes; the
-// probabilities are added, head after head, into a [64 rows][64 NZ] table in shared memory, from
-// which one warp per row ranks and emits.  The means are read once per tile and head instead of
-// once per position and head.
-template <typename T, int D, int NZ>
-__global__ void __launch_bounds__(256, NZ == 1 ? 2 : 1) score_per_query_tile_kernel(
-    Shape sh, SelGeom g, const T *__restrict__ q, const double *__restrict__ mean,
-    const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx) {
-  grid_chain_enter();
-  constexpr int PD = D + 1, MP = 64 * NZ;
-  extern __shared__ double dsm[];
-  __shared__ double bound_d[8][2];
-  double *qd = dsm;                // [64][PD] query rows of the current head
-  double *kd = qd + 64 * PD;       // [64][PD] a chunk of candidate means
-  double *P = kd + 64 * PD;        // [64][MP] probabilities summed over the group's heads
-  double *Smap = P + 64 * MP;      // [8 warps][MP] a row's scores of the selection blocks (Eq. 11; overlapping mode)
-  uint8_t *taken_all = reinterpret_cast<uint8_t *>(Smap + (g.plain ? 0 : 8 * MP));  // [8 warps][MP]
-  const int M = sh.M, Bk = sh.Bk;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rt = tid >> 2, part = tid & 3;
-  const int ntile = (sh.L + 63) / 64;
-  const int u = (int)(blockIdx.x / ntile), tile = (int)(blockIdx.x % ntile), n = u / sh.Hkv, hk = u % sh.Hkv;
-  int len = seq_lens ? seq_lens[n] : sh.L;
-  len = min(max(len, 0), sh.L);
-  const int pad0 = sh.L - len;
-  const int t0 = tile * 64, t_last = min(t0 + 63, sh.L - 1);
-  const int jmin = pad0 / Bk;                    // selectable selection blocks: j >= jmin
-  const int cmin = first_live_scored(g, pad0);   // live scored blocks: c >= cmin
-  // candidates of the tile's rows: scored blocks cmin .. nc - 1 (row t: those that end before block t / Bk)
-  const int nc = n_candidates(sh, g, t_last / Bk);
-  const int t = t0 + rt;
-  const bool row_on = t >= pad0 && t < sh.L;
-  const int nc_row = row_on ? n_candidates(sh, g, t / Bk) : 0;
-
-  if (t_last >= pad0 && nc > cmin) {
-    for (int i = tid; i < 64 * MP; i += 256) P[i] = 0.0;
-    const int ch_lo = cmin / 64, ch_hi = (nc + 63) / 64;  // at most NZ chunks apart (host-checked: blocks <= 64 NZ)
-    const double *kbase = mean + (int64_t)u * g.n * D;
-    for (int hg = 0; hg < sh.G; ++hg) {
-      __syncthreads();  // the previous head's rows are no longer read
-      for (int i = tid; i < 64 * (D / 4); i += 256) {
-        const int lr = i / (D / 4), c = (i % (D / 4)) * 4, tt = t0 + lr;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tt >= pad0 && tt < sh.L) v = ld4(q + row_offset(sh, n, hk * sh.G + hg, tt) + c);
-        double *d = qd + lr * PD + c;
-        d[0] = (double)v.x; d[1] = (double)v.y; d[2] = (double)v.z; d[3] = (double)v.w;
-      }
-      const double *qr = qd + rt * PD;
-      double z[NZ][16];
-      uint32_t on[NZ];
-      double mx = -INFINITY;
-#pragma unroll
-      for (int ci = 0; ci < NZ; ++ci) {
-        on[ci] = 0u;
-        const int ch = ch_lo + ci;
-        if (ch < ch_hi) {  // (block-uniform)
-          const int c0 = ch * 64, nb = min(64, nc - c0);
-          __syncthreads();  // previous users of kd are done (and qd is complete)
-          for (int i = tid; i < 64 * (D / 2); i += 256) {
-            const int lj = i / (D / 2), c = (i % (D / 2)) * 2;
-            double2 v = make_double2(0.0, 0.0);
-            if (lj < nb && c0 + lj >= cmin) v = *reinterpret_cast<const double2 *>(kbase + (int64_t)(c0 + lj) * D + c);
-            kd[lj * PD + c] = v.x;
-            kd[lj * PD + c + 1] = v.y;
-          }
-          __syncthreads();
-#pragma unroll
-          for (int k = 0; k < 16; ++k) z[ci][k] = 0.0;
-#pragma unroll 2
-          for (int c = 0; c < D; ++c) {
-            const double qv = qr[c];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) z[ci][k] = fma(qv, kd[(part + 4 * k) * PD + c], z[ci][k]);
-          }
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            z[ci][k] *= sh.scale_d;
-            const int c = c0 + part + 4 * k;
-            if (row_on && c >= cmin && c < nc_row) {
-              on[ci] |= 1u << k;
-              mx = fmax(mx, z[ci][k]);
-            }
-          }
-        }
-      }
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      double den = 0.0;
-#pragma unroll
-      for (int ci = 0; ci < NZ; ++ci)
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if ((on[ci] >> k) & 1u) {
-            z[ci][k] = exp(z[ci][k] - mx);
-            den += z[ci][k];
-          }
-      den += __shfl_xor_sync(0xffffffffu, den, 1);
-      den += __shfl_xor_sync(0xffffffffu, den, 2);
-#pragma unroll
-      for (int ci = 0; ci < NZ; ++ci)
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if ((on[ci] >> k) & 1u) P[rt * MP + (ch_lo + ci) * 64 - ch_lo * 64 + part + 4 * k] += z[ci][k] / den;  // heads in ascending order
-    }
-  }
-  __syncthreads();
-  // one warp per row: Eq. 11 and Eq. 13 from the row's summed probabilities (table column =
-  // scored block - 64 ch_lo)
-  const int col0 = (cmin / 64) * 64;
-  uint8_t *taken = taken_all + warp * MP;
-  double *Srow = Smap + warp * MP;
-  for (int lr = warp; lr < 64; lr += 8) {
-    const int tt = t0 + lr;
-    if (tt >= sh.L) break;
-    int32_t *row = idx + ((int64_t)u * sh.L + tt) * sh.topk;
-    if (tt < pad0) {
+  const int per_warp = (5 * g.n + (g.plain ? 0 : M) + 4 * D + 1) / 2 * 2;
+  double *qrow = dsm + (size_t)warp * per_warp;  // [4][D] the current heads' rows
+  double *P = qrow + 4 * D;                      // [n] summed probabilities of this warp's position
+  double *Z = P + g.n;                           // [4][n] logits of the current heads
+  double *Smap = Z + 4 * g.n;                    // [M] scores of the selection blocks (overlapping mode)
+  uint8_t *taken = reinterpret_cast<uint8_t *>(dsm + (size_t)8 * per_warp) + (size_t)warp * M;
+  const int64_t total = worklist ? *work_count : (int64_t)sh.B * sh.Hkv * sh.L;
+  for (int64_t wi = (int64_t)blockIdx.x * 8 + warp; wi < total; wi += (int64_t)gridDim.x * 8) {
+    const int64_t pos = worklist ? worklist[wi] : wi;
+    const int t = (int)(pos % sh.L), u = (int)(pos / sh.L), n = u / sh.Hkv, hk = u % sh.Hkv;
+    int len = seq_lens ? seq_lens[n] : sh.L;
+    len = min(max(len, 0), sh.L);
+    const int pad0 = sh.L - len;
+    int32_t *row = idx + pos * sh.topk;
+    __syncwarp();  // the warp's arrays are reused from its previous position
+    if (t < pad0) {
       for (int i = lane; i < sh.topk; i += 32) row[i] = -1;
       continue;
     }
-    const int b = tt / Bk, nsel = max(0, b - jmin), want = min(sh.topk - 1, nsel);
-    __syncwarp();
-    if (nsel > want && want > 0) {
-      if (g.plain) {
-        rank_select<double>(P + lr * MP - col0, jmin, b, want, taken, bound_d[warp], lane);
-      } else if (n_candidates(sh, g, b) > cmin) {
-        map_scores<double>(g, P + lr * MP - col0, cmin, n_candidates(sh, g, b), jmin, b, Srow, lane);
+    const int b = t / Bk, jmin = pad0 / Bk;  // live blocks before the own one: jmin .. b - 1
+    const int cmin = first_live_scored(g, pad0), nc = n_candidates(sh, g, b);
+    const int nsel = max(0, b - jmin), want = min(sh.topk - 1, nsel);
+    if (nsel > want && want > 0 && nc > cmin) {
+      for (int j = cmin + lane; j < nc; j += 32) P[j] = 0.0;
+      const double *kbase = mean + (int64_t)u * g.n * D;
+      // Up to four heads of the group at a time, so that a candidate's mean is read (a lane per candidate,
+      // eight 16-byte loads in flight) once for all of them.
+      for (int h0 = 0; h0 < sh.G; h0 += 4) {
+        const int nh = min(4, sh.G - h0);
         __syncwarp();
-        rank_select<double>(Srow, jmin, b, want, taken, bound_d[warp], lane);
-      } else {  // no compression block lies in the past yet: all scores are zero, the lowest blocks win the ties
-        for (int j = jmin + lane; j < b; j += 32) taken[j] = j - jmin < want ? 1 : 0;
+        for (int c = lane; c < 4 * D; c += 32) {
+          const int h = c / D;
+          qrow[c] = h < nh ? (double)ld1(q + row_offset(sh, n, hk * sh.G + h0 + h, t) + c % D) : 0.0;
+        }
+        __syncwarp();
+        double mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, den[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int j = cmin + lane; j < nc; j += 32) {
+          const double2 *kj = reinterpret_cast<const double2 *>(kbase + (int64_t)j * D);
+          double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+          for (int c = 0; c < D / 2; c += 8) {
+            double2 kv[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) kv[e] = kj[c + e];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                const double2 qv = *reinterpret_cast<const double2 *>(qrow + h * D + 2 * (c + e));
+                a[h] = fma(qv.x, kv[e].x, a[h]);
+                a[h] = fma(qv.y, kv[e].y, a[h]);
+              }
+          }
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const double z = sh.scale_d * a[h];
+            Z[h * g.n + j] = z;
+            mx[h] = fmax(mx[h], z);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) mx[h] = fmax(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], o));
+        }
+        for (int j = cmin + lane; j < nc; j += 32)
+          for (int h = 0; h < nh; ++h) {
+            const double e = exp(Z[h * g.n + j] - (h == 0 ? mx[0] : h == 1 ? mx[1] : h == 2 ? mx[2] : mx[3]));
+            Z[h * g.n + j] = e;
+            if (h == 0) den[0] += e;
+            else if (h == 1) den[1] += e;
+            else if (h == 2) den[2] += e;
+            else den[3] += e;
+          }
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) den[h] += __shfl_xor_sync(0xffffffffu, den[h], o);
+        }
+        for (int j = cmin + lane; j < nc; j += 32) {  // heads in ascending order
+          double a = P[j];
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            if (h < nh) a += Z[h * g.n + j] / den[h];
+          P[j] = a;
+        }
       }
-    } else {
-      for (int j = jmin + lane; j < b; j += 32) taken[j] = want > 0 ? 1 : 0;
+      __syncwarp();
+      const double *S = P;
+      if (!g.plain) {
+        map_scores<double>(g, P, cmin, nc, jmin, b, Smap, lane);
+        __syncwarp();
+        S = Smap;
+      }
+      rank_select<double>(S, jmin, b, want, taken, bound_d[warp], lane);
+    } else {  // everything, or (no candidate lies in the past yet: all scores are zero) the lowest blocks
+      for (int j = jmin + lane; j < b; j += 32) taken[j] = j - jmin < want ? 1 : 0;
     }
     __syncwarp();
     emit_row(row, taken, jmin, b, sh.topk, lane);
@@ -1038,34 +1084,39 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   } else if (cudaMemsetAsync(w.count, 0, sizeof(int32_t), st) != cudaSuccess) {
     return BLOSSOM_ERR_CUDA;
   }
+  // First stage: single precision with a bound; what it cannot certify goes on the work list.
+  RowsGeom rg;
+  size_t rsm = 0;
+  const bool rows = g.n > 0 && rows_geom(sh, g, &rg, &rsm);
+  const int dtype = sizeof(T) == 2 ? BLOSSOM_DTYPE_BF16 : BLOSSOM_DTYPE_FP32;
   if (sh.pq) {  // one selection per query position: block_idx is [B][Hkv][L][top_k]
-    if (g.n <= 128 && sh.M <= 128) {  // the tiled kernel keeps the logits of up to two chunks of 64 blocks in registers
-      const int nz = (g.n <= 64 && sh.M <= 64) ? 1 : 2;
-      const size_t tsm = ((size_t)2 * 64 * (D + 1) + (size_t)64 * 64 * nz + (g.plain ? 0 : (size_t)8 * 64 * nz)) * sizeof(double) +
-                         (size_t)8 * 64 * nz + 16;
-      auto kern = nz == 1 ? score_per_query_tile_kernel<T, D, 1> : score_per_query_tile_kernel<T, D, 2>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm) != cudaSuccess)
-        return BLOSSOM_ERR_CUDA;
-      LaunchScope ls(K_SCORE_SELECT, st);
-      launch_chained(kern, dim3((unsigned)(units * ((sh.L + 63) / 64))), dim3(256), tsm, st, sh, g, q,
-                     (const double *)w.mean, seq_lens, idx);
-      return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
+    if (!rows && !g.plain && g.n > 128) return BLOSSOM_ERR_UNSUPPORTED;  // (see make_shape)
+    const bool listed = rows && !exact_select_only();
+    if (listed) {
+      rg.exact = 0;
+      if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, seq_lens, idx, w.list, w.count, st))
+        return rc;
     }
-    if (!g.plain) return BLOSSOM_ERR_UNSUPPORTED;  // (more than 128 blocks: the per-warp kernel scores selection blocks only)
-    const size_t psm = (size_t)8 * (2 * sh.M + D) * sizeof(double) + (size_t)8 * sh.M + 16;
-    if (psm > 48 * 1024 && cudaFuncSetAttribute(score_per_query_kernel<T, D>,
+    const size_t psm = (size_t)8 * ((5 * g.n + (g.plain ? 0 : sh.M) + 4 * D + 1) / 2 * 2) * sizeof(double) + (size_t)8 * sh.M + 16;
+    if (psm > 40 * 1024 && cudaFuncSetAttribute(score_per_query_kernel<T, D>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm) != cudaSuccess)
       return BLOSSOM_ERR_CUDA;
     LaunchScope ls(K_SCORE_SELECT, st);
-    launch_chained(score_per_query_kernel<T, D>, dim3((unsigned)((units * sh.L + 7) / 8)), dim3(256), psm, st, sh, q,
-                   (const double *)w.mean, seq_lens, idx);
+    const int64_t ctas = (units * sh.L + 7) / 8;
+    launch_chained(score_per_query_kernel<T, D>, dim3((unsigned)(listed && ctas > 592 ? 592 : ctas)), dim3(256), psm, st, sh,
+                   g, q, (const double *)w.mean, seq_lens, idx, (const int32_t *)(listed ? w.list : nullptr),
+                   (const int32_t *)w.count);
     return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
   }
   int sc_pitch = 0, sc_len = 0;
   const size_t fsm = fast_smem_bytes(sh, g, D, &sc_pitch);
-  // (without the causal mask the candidates are not a prefix of the blocks: double precision only)
-  const bool exact_only = exact_select_only() || fsm == 0 || !sh.causal;
-  if (!exact_only) {
+  // (the tiled kernel for more than 128 blocks takes candidates that are a prefix of the blocks only)
+  const bool use_rows = rows && sh.Bk >= 16;  // (it sums the columns in groups of 16 rows)
+  const bool exact_only = exact_select_only() || (!use_rows && (fsm == 0 || !sh.causal));
+  if (!exact_only && use_rows) {
+    rg.exact = 0;
+    if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, seq_lens, idx, w.list, w.count, st)) return rc;
+  } else if (!exact_only) {
     if (fsm > 48 * 1024 && cudaFuncSetAttribute(score_fast_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)fsm) != cudaSuccess)
       return BLOSSOM_ERR_CUDA;
@@ -1074,38 +1125,55 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
     launch_chained(score_fast_kernel<T, D>, dim3(ntiles * (unsigned)units), dim3(kFastThreads), fsm, st, sh, g, q,
                    (const float *)w.mean32, (const float *)w.norm, seq_lens, idx, w.list, w.count, sc_pitch);
   }
+  // double precision: every query block (exact_only) or the work list of the kernel above, in clusters
+  // of as many CTAs (up to 8) as a query block's rows fill
+  const int32_t *list = exact_only ? nullptr : w.list;
+  const int64_t nblocks = units * sh.M;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // chained behind the kernel before it
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained_launches() ? 2 : 1;
+  auto plan = [&](int rows_per_cta, int max_ctas) {
+    const int chunks = (sh.G * sh.Bk + rows_per_cta - 1) / rows_per_cta;
+    const unsigned cl = chunks >= 8 ? 8u : chunks >= 4 ? 4u : chunks >= 2 ? 2u : 1u;
+    attr[0].val.clusterDim.x = cl;
+    const int64_t max_clusters = max_ctas / cl;
+    cfg.gridDim = dim3((unsigned)(nblocks < max_clusters ? nblocks : max_clusters) * cl);
+  };
+  LaunchScope ls(K_SCORE_SELECT, st);
+  if (g.n <= 128 && sh.M <= 128) {
+    auto exact = score_exact16_kernel<T, D>;
+    const size_t esm = ((size_t)(g.n + 1 + 16) * (D + 2) + (size_t)16 * ((g.n + 1) | 1) + 4 * 128 + 128 + sh.M) * sizeof(double) +
+                       (size_t)sh.M + 16;
+    if (esm > 40 * 1024 &&
+        cudaFuncSetAttribute(exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm) != cudaSuccess)
+      return BLOSSOM_ERR_CUDA;
+    plan(16, 1184);
+    cfg.blockDim = dim3(128);
+    cfg.dynamicSmemBytes = esm;
+    if (cudaLaunchKernelEx(&cfg, exact, sh, g, q, (const double *)w.mean, seq_lens, idx, list, (const int32_t *)w.count) !=
+        cudaSuccess)
+      return BLOSSOM_ERR_CUDA;
+    return BLOSSOM_OK;
+  }
   const size_t esm = exact_smem_bytes(sh, g, D, &sc_len);
-  auto exact = g.n > 64 ? score_exact_kernel<T, D, 2> : score_exact_kernel<T, D, 1>;
+  auto exact = score_exact_kernel<T, D>;
   if (esm > 48 * 1024 &&
       cudaFuncSetAttribute(exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
-  {
-    // double precision: every query block (exact_only) or the work list of the kernel above
-    LaunchScope ls(K_SCORE_SELECT, st);
-    const int64_t rows = units * sh.M;
-    const int chunks = (sh.G * sh.Bk + 63) / 64;  // 64-row chunks of a query block
-    const unsigned cl = chunks >= 8 ? 8u : chunks >= 4 ? 4u : chunks >= 2 ? 2u : 1u;
-    const int64_t max_clusters = 592 / cl;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(rows < max_clusters ? rows : max_clusters) * cl);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = esm;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cl;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // chained behind the kernel before it
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = chained_launches() ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, exact, sh, g, q, (const double *)w.mean, seq_lens, idx,
-                           (const int32_t *)(exact_only ? nullptr : w.list), (const int32_t *)w.count,
-                           sc_len) != cudaSuccess)
-      return BLOSSOM_ERR_CUDA;
-  }
-  return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
+  plan(64, 592);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = esm;
+  if (cudaLaunchKernelEx(&cfg, exact, sh, g, q, (const double *)w.mean, seq_lens, idx, list, (const int32_t *)w.count,
+                         sc_len) != cudaSuccess)
+    return BLOSSOM_ERR_CUDA;
+  return BLOSSOM_OK;
 }
 
 int launch_select_buffers(const Shape &s, int dtype, const void *q, const void *k, const int32_t *seq_lens,
