@@ -3,8 +3,8 @@
 // Which 64-key tiles a 128-row query tile has to visit (the blocks its query blocks selected,
 // Eq. 13, and the tiles its window reaches, Eq. 15), in which order, and which of its warps a tile
 // concerns, depends only on the block indices and the sequence lengths.  Building that inside the
-// attention kernels cost every CTA several thousand cycles before its first product; here one warp
-// per attention CTA builds the image of the bookkeeping the attention kernel wants in shared
+// attention kernels cost every CTA several thousand cycles before its first product; here a warp
+// (or four, see the kernel) per attention CTA builds the image of the bookkeeping the attention kernel wants in shared
 // memory, and the attention kernel fetches it with one bulk copy while its first tiles load.
 //
 // Query-major image (forward and dQ kernel), see meta_layout():
@@ -33,10 +33,13 @@ namespace blossom {
 namespace tc {
 namespace {
 
-constexpr int kMetaWarps = 4;  // images per CTA, one warp each
+constexpr int kMetaWarps = 4;  // warps per CTA
 
-// One warp builds one image: no block-wide barrier anywhere, so the (latency-bound) images of a
-// whole launch are in flight at once.
+// NW warps build one image.  One: no block-wide barrier anywhere, so the images of a large launch are in
+// flight at once and the issue slots are what counts.  Four: an image's loops are a chain of loads and
+// atomics that one warp takes 8 - 40 us for (the selection per position has 128 index rows to go through),
+// so a launch of few images is shorter with the loops split.  The compactions stay with the first warp.
+template <int NW>
 __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const int32_t *__restrict__ seq_lens,
                                                                   const int32_t *__restrict__ idx,
                                                                   uint8_t *__restrict__ qmeta,
@@ -45,14 +48,20 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                                                                   int branches, int with_fwd,
                                                                   uint32_t *__restrict__ inv_bits) {
   grid_chain_enter();
+  constexpr int NT = 32 * NW;  // threads per image
+  auto sync = [] {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+  };
   extern __shared__ __align__(16) uint8_t meta_all[];
   const MetaLayout ml = meta_layout(nT, s.pq);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int image = image0 + (int)blockIdx.x * kMetaWarps + warp;  // this launch builds [image0, image_end)
+  const int lane = threadIdx.x & 31, tid = threadIdx.x % NT, sub = threadIdx.x / NT;
+  const bool scans = tid < 32;  // the warp that compacts
+  const int image = image0 + (int)blockIdx.x * (kMetaWarps / NW) + sub;  // this launch builds [image0, image_end)
   if (image >= image_end) return;
   const int Lw = (s.L + 31) >> 5;  // words per key block of the bit table
   const int slice = ml.bytes + ((3 * nT + 15) / 16) * 16;  // the image and a scratch list behind it
-  uint8_t *meta = meta_all + (size_t)warp * slice;
+  uint8_t *meta = meta_all + (size_t)sub * slice;
   const int nST = (s.L + 127) >> 7;
   const bool key_major = image >= n_query_ctas;
   const int cta = key_major ? image - n_query_ctas : image;
@@ -78,8 +87,8 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   const int G = 128 / s.Bk, nb = 64 / s.Bk;
   const int bk_shift = __ffs(s.Bk) - 1;  // Bk is a power of two
 
-  for (int i = lane; i < ml.bytes / 4; i += 32) selw[i] = 0u;  // the whole image
-  __syncwarp();
+  for (int i = tid; i < ml.bytes / 4; i += NT) selw[i] = 0u;  // the whole image
+  sync();
 
   if (!key_major) {
     const int st = pack ? nT - 1 - cta % nT : nST - 1 - cta % nST;  // the attention kernels take long rows first
@@ -93,7 +102,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       uint32_t *roww = reinterpret_cast<uint32_t *>(meta + ml.rows);
       // the bit table is per key/value head: the group's first query head (or pair of heads) fills it
       const bool fills = inv_bits && (pack ? (2 * (u % (s.H / 2))) % s.G == 0 : (u % s.H) % s.G == 0);
-      for (int i = lane; i < 128 * s.topk; i += 32) {
+      for (int i = tid; i < 128 * s.topk; i += NT) {
         const int r = i / s.topk, slot = i % s.topk, t = pack ? row0 + (r & 63) : row0 + r;
         if (t < s.L) {
           const int blk = idx[((int64_t)uk * s.L + t) * s.topk + slot];
@@ -107,7 +116,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         }
       }
     } else {
-    for (int i = lane; i < G * s.topk; i += 32) {  // the selections of the CTA's query blocks
+    for (int i = tid; i < G * s.topk; i += NT) {  // the selections of the CTA's query blocks
       const int g = i / s.topk, slot = i % s.topk, qb = pack ? st * nb + g % nb : st * G + g;
       if (qb < s.M) {
         const int blk = idx[((int64_t)uk * s.M + qb) * s.topk + slot];
@@ -118,9 +127,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       }
     }
     }
-    __syncwarp();
-    int nv = 0;
-    {  // the tiles any row of the CTA needs, ascending
+    sync();
+    if (scans) {  // the tiles any row of the CTA needs, ascending
+      int nv = 0;
       const int jt_max = (s.causal ? row_last : s.L - 1) >> 6;
       for (int base = 0; base <= jt_max; base += 32) {
         const int jt = base + lane;
@@ -138,11 +147,13 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         }
         nv += __popc(bal);
       }
+      if (lane == 0) counts[0] = nv;
     }
-    __syncwarp();
+    sync();
+    const int nv = counts[0];
     const int gh = G / 2;
-    if (lane == 0) counts[0] = nv;
-    if (with_fwd) {  // ---- the forward's items and their classes ----
+    if (with_fwd) {
+    if (scans) {  // ---- the forward's items and their classes ----
     // Long-term items: the tiles both 64-row halves of the CTA need, then alternately a tile only
     // rows 0..63 need and a tile only rows 64..127 need.  A softmax warp may run ahead of the
     // slowest one, so with alternating items both pairs of warps have work at once.
@@ -189,16 +200,17 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       count += __popc(bal);
     }
     if (lane == 0) {
-      counts[0] = nv;
       counts[1] = nl;
       counts[2] = count - nl;
     }
-    __syncwarp();
+    }
+    sync();
+    const int nl = counts[1], count = nl + counts[2];
     // Class of every (item, softmax warp): 0 = no row of the warp needs the tile, 1 = every row
     // sees all 64 keys, 2 = mixed (the warp builds per-lane column masks).
     const bool uni = s.Bk >= 32;  // a warp's 32 rows share one query block
     const uint32_t allbits = (1u << (64 / s.Bk)) - 1u;
-    for (int e = lane; e < count * 4; e += 32) {
+    for (int e = tid; e < count * 4; e += NT) {
       const int it = e >> 2, w = e & 3;
       const int jt = items[it], p0 = jt * 64, t_lo = quarter_row0(w);
       const bool some = (p0 <= t_lo + 31 || !s.causal) && p0 + 63 >= pad0 && t_lo + 31 >= pad0 && t_lo < s.L;
@@ -219,12 +231,12 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       icls[e] = (uint8_t)cls;
     }
     }  // the forward's part
-    __syncwarp();
+    sync();
     // The dQ kernel walks `list` itself (a tile serves both branches there).  Same idea as above:
     // tiles both 64-row halves need first, then alternately a tile only rows 0..63 need and one
     // only rows 64..127 need, so that the two halves' warps work on neighbouring tiles at once.
     // (Backward call only; the forward reads `items`.)
-    if (kmeta) {
+    if (kmeta && scans) {
       uint16_t *tlist = reinterpret_cast<uint16_t *>(meta + ml.bytes);
       uint8_t *tflags = meta + ml.bytes + 2 * nT;
       int nA = 0, nB = 0, nC = 0;
@@ -274,13 +286,13 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         lflags[j] = tflags[j];
       }
     }
-    __syncwarp();
+    sync();
     // dQ kernel: class of every (listed tile, half tile of 32 keys, compute warp).  Warp w works
     // on rows 32 (w % 4) ... and keys 16 (w / 4) ... of the half tile.  Bit 0 / bit 1: every row of
     // the warp sees all 16 keys through the long-term / short-term branch and no row sees only a
     // part of them; 8: mixed, the warp builds per-lane column masks.  (A forward-only call has no
     // use for them.)
-    for (int e = lane; e < (kmeta ? nv * 16 : 0); e += 32) {
+    for (int e = tid; e < (kmeta ? nv * 16 : 0); e += NT) {
       const int it = e >> 4, hh = (e >> 3) & 1, w = e & 7, qtr = w & 3, c = w >> 2;
       const int jt = list[it], f = lflags[it];
       const int k_lo = jt * 64 + 32 * hh + 16 * c, k_hi = k_lo + 15, t_lo = quarter_row0(qtr), t_hi = t_lo + 31;
@@ -312,7 +324,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       // of a block holds positions 32 w ...; a position before the block never selected it)
       uint32_t *invw = reinterpret_cast<uint32_t *>(meta + ml.rows);
       const int qb0 = kt * G, w_lo = key0 >> 5;
-      for (int i = lane; i < G * (Lw - w_lo); i += 32) {
+      for (int i = tid; i < G * (Lw - w_lo); i += NT) {
         const int g = i / (Lw - w_lo), w = w_lo + i % (Lw - w_lo);
         if (qb0 + g >= s.M) continue;
         const uint32_t bits = inv_bits[((int64_t)uk * s.M + qb0 + g) * Lw + w];
@@ -330,16 +342,16 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       // (without the causal mask every query block may have selected them: the rows start at block 0)
       const int qb0 = kt * G, qb_first = s.causal ? qb0 : 0, total = (s.M - qb_first) * s.topk;
       const int32_t *rows = idx + ((int64_t)uk * s.M + qb_first) * s.topk;
-      for (int base = 0; base < total; base += 256) {
+      for (int base = 0; base < total; base += 8 * NT) {
         int blk[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int i = base + e * 32 + lane;
+          const int i = base + e * NT + tid;
           blk[e] = i < total ? rows[i] : -1;
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int i = base + e * 32 + lane, qb = qb_first + i / s.topk;
+          const int i = base + e * NT + tid, qb = qb_first + i / s.topk;
           if (blk[e] >= qb0 && blk[e] < qb0 + G && (blk[e] <= qb || !s.causal)) {
             const int a = (blk[e] - qb0) * nT + qb / nb;
             atomicOr(&selw[a >> 2], (1u << (qb % nb)) << ((a & 3) * 8));
@@ -347,8 +359,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         }
       }
     }
-    __syncwarp();
+    sync();
     const int qt_min = s.causal ? key0 >> 6 : 0, qt_max = (s.L - 1) >> 6;
+    if (scans) {
     int count = 0;
     for (int base = qt_min; base <= qt_max; base += 32) {
       const int qt = base + lane;
@@ -367,12 +380,14 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       count += __popc(bal);
     }
     if (lane == 0) counts[0] = count;
-    __syncwarp();
+    }
+    sync();
+    const int count = counts[0];
     // dK/dV kernel: class of every (listed tile, half tile of 32 queries, compute warp).  Warp w
     // works on key rows 32 (w % 4) ... of the CTA and on query columns 16 (w / 4) ... of the half
     // tile.  Same code as for the dQ kernel: bit 0 / bit 1 = every key row of the warp is seen in
     // full by all 16 queries through the long-term / short-term branch and none in part; 8 = mixed.
-    for (int e = lane; e < count * 16; e += 32) {
+    for (int e = tid; e < count * 16; e += NT) {
       const int it = e >> 4, hh = (e >> 3) & 1, w = e & 7, qtr = w & 3, hf = w >> 2;
       const int qt = list[it], f = lflags[it], c_lo = 32 * hh + 16 * hf;
       const int p_lo = key0 + 32 * qtr, p_hi = p_lo + 31, t_lo = qt * 64 + c_lo, t_hi = t_lo + 15;
@@ -397,10 +412,10 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       jcls[e] = (uint8_t)((cL == 2 || cS == 2) ? 8 : (cL | (cS << 1)));
     }
   }
-  __syncwarp();
+  sync();
   uint4 *dst = reinterpret_cast<uint4 *>((key_major ? kmeta : qmeta) + (size_t)cta * ml.bytes);
   const uint4 *src = reinterpret_cast<const uint4 *>(meta);
-  for (int i = lane; i < ml.bytes / 16; i += 32) dst[i] = src[i];
+  for (int i = tid; i < ml.bytes / 16; i += NT) dst[i] = src[i];
 }
 
 }  // namespace
@@ -410,15 +425,20 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   if (with_fwd < 0) with_fwd = kmeta == nullptr;
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
-  const size_t smem = (size_t)kMetaWarps * (meta_bytes(nT, s.pq) + ((3 * nT + 15) / 16) * 16);
+  // Four warps per image while its loops are long (a selection per position: 46 -> 28 us for 960 images at
+  // L 1500) or the images do not fill the SMs (18 -> 10 us for 256 images at L 4096); at 4096 images of L 1024
+  // four warps took 26 us and one 17.
+  const bool wide = n_images <= 148 * (s.pq ? 48 : 8);
+  const int per_cta = wide ? 1 : kMetaWarps;
+  const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((3 * nT + 15) / 16) * 16);
+  auto kern = wide ? tc_meta_kernel<kMetaWarps> : tc_meta_kernel<1>;
   if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(tc_meta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
   auto launch = [&](int image0, int image_end, uint32_t *inv_bits) {
     LaunchScope ls(K_TC_META, st);
-    launch_chained(tc_meta_kernel, dim3((unsigned)((image_end - image0 + kMetaWarps - 1) / kMetaWarps)),
-                   dim3(kMetaWarps * 32), smem, st, s, seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches,
-                   with_fwd, inv_bits);
+    launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,
+                   seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits);
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it

@@ -160,6 +160,8 @@ __device__ __forceinline__ bool st_visible(const Shape &s, int t, int p) {
   const int bd = abs(t / s.stis_blk - p / s.stis_blk);
   return (bd >= 1 && (bd & (bd - 1)) == 0) || p >= s.L - s.stis_blk;
 }
+// (the division by a block of 1, the paper's, is left out: the tile lists ask this for every tile)
+__device__ __forceinline__ int stis_block_of(const Shape &s, int t) { return s.stis_blk == 1 ? t : t / s.stis_blk; }
 // May some query in [t0, t1] see some key in [p0, p1] (p0 <= t1 under the causal mask) through the short-term branch?
 // Exact for the window; for the power-law mask a superset (any power of two inside the range of
 // block distances counts), which only costs a visit: st_visible decides every pair.
@@ -169,15 +171,15 @@ __device__ __forceinline__ bool st_ranges_touch(const Shape &s, int t0, int t1, 
     if (s.stis_mode == 0) return false;
     if (p1 >= s.L - s.stis_blk) return true;
     // is a power of two among the block distances of keys before the queries, or of keys after?
-    const int bq0 = t0 / s.stis_blk, bq1 = t1 / s.stis_blk, bk0 = p0 / s.stis_blk, bk1 = p1 / s.stis_blk;
+    const int bq0 = stis_block_of(s, t0), bq1 = stis_block_of(s, t1), bk0 = stis_block_of(s, p0), bk1 = stis_block_of(s, p1);
     const int lmax = bq1 - bk0, lmin = max(1, bq0 - bk1), rmax = bk1 - bq0, rmin = max(1, bk0 - bq1);
     return (lmax >= lmin && (1 << (31 - __clz(lmax))) >= lmin) || (rmax >= rmin && (1 << (31 - __clz(rmax))) >= rmin);
   }
   if (t0 - p1 < s.window) return true;
   if (s.stis_mode == 0) return false;
   if (p1 >= s.L - s.stis_blk) return true;
-  const int dmax = t1 / s.stis_blk - p0 / s.stis_blk;
-  const int dmin = max(1, t0 / s.stis_blk - p1 / s.stis_blk);
+  const int dmax = stis_block_of(s, t1) - stis_block_of(s, p0);
+  const int dmin = max(1, stis_block_of(s, t0) - stis_block_of(s, p1));
   return dmax >= dmin && (1 << (31 - __clz(dmax))) >= dmin;  // largest power of two <= dmax
 }
 
