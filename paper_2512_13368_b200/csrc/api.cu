@@ -353,8 +353,7 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
                                   dq, dk, dv, dgate, ws, st);
     } else {
       rc = tc::launch_bwd_tc(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout, dq,
-                             dk, dv, ws, st);
-      if (!rc) rc = launch_gate_grad(s, gate_logits, ws, dgate, st);
+                             dk, dv, dgate, ws, st);
     }
   } else {
     rc = launch_bwd_simt(s, params->dtype, q, k, v, gate_logits, seq_lens, block_idx, out_lt,

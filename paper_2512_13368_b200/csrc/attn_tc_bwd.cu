@@ -41,8 +41,11 @@
 // Every wait is bounded (tc_common.cuh).
 #include "tc_common.cuh"
 
+#include <cooperative_groups.h>
+
 namespace blossom {
 namespace tc {
+namespace cg = cooperative_groups;
 namespace {
 
 // warps 0..7 compute; 8 loader, 9 first-stage issuer, 10 second-stage issuer, 11 spare
@@ -169,7 +172,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     const uint8_t *__restrict__ qmeta, const __grid_constant__ CUtensorMap tmdq,
     const float4 *__restrict__ qstats, double *__restrict__ dalpha_part, int32_t *__restrict__ status,
     int nT) {
-  grid_chain_enter();
+  grid_wait();
+  grid_release();  // (the dK/dV kernel depends on nothing of this one)
   using C = Cfg<D>;
   constexpr int STAGES = kDqStages;
   constexpr int OC = D / 2;  // accumulator columns per thread
@@ -528,14 +532,40 @@ __device__ __forceinline__ void dkdv_tile(const float (&sv)[16], const float (&d
   }
 }
 
+// d alpha partials -> dgate[H][2], by one CTA, head after head: thread i adds the entries i, i + 384, ... in
+// ascending order, then a fixed shuffle tree and the warps in order.  (As a kernel of its own it was
+// another 8 us of launch and latency.)
+__device__ __forceinline__ void reduce_gate(const Shape &s, const float *gate, const double *part, float *dgate) {
+  __shared__ double red[2][kKvThreads / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, total = s.B * s.M;
+  for (int h = 0; h < s.H; ++h) {
+    double a = 0.0;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < total; i += kKvThreads) a += __ldcg(part + ((int64_t)(i / s.M) * s.H + h) * s.M + i % s.M);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) red[h & 1][warp] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double x = 0.0;
+      for (int w = 0; w < kKvThreads / 32; ++w) x += red[h & 1][w];
+      const double al = 1.0 / (1.0 + exp(-((double)gate[h * 2 + 0] - (double)gate[h * 2 + 1])));
+      const double g0 = al * (1.0 - al) * x;
+      dgate[h * 2 + 0] = (float)g0;
+      dgate[h * 2 + 1] = (float)(-g0);
+    }
+  }
+}
+
 template <int D, bool PLAIN>
 __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
     const int32_t *__restrict__ seq_lens, const uint8_t *__restrict__ kmeta,
     const float4 *__restrict__ qstats, const __grid_constant__ CUtensorMap tmdk,
-    const __grid_constant__ CUtensorMap tmdv, int32_t *__restrict__ status, int nT) {
-  grid_chain_enter();
+    const __grid_constant__ CUtensorMap tmdv, int32_t *__restrict__ status, int nT, int hs,
+    __nv_bfloat16 *__restrict__ dk, __nv_bfloat16 *__restrict__ dv, const float *__restrict__ gate,
+    const double *__restrict__ dalpha_part, float *__restrict__ dgate) {
   using C = Cfg<D>;
   constexpr int STAGES = kKvStages;
   constexpr int OC = D / 2;
@@ -547,12 +577,22 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   __shared__ int abort_flag;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  grid_release();
   const int nKT = (s.L + 127) >> 7;
   // A CTA owns 128 keys of one (batch, key/value head) and collects from every query head of the
   // group.  Early keys have the most visitors, so the grid runs tile-major: every unit's first
   // tile, then every unit's second, ... and the light tiles fill the tail.
+  // With clusters (hs CTAs) the heads of the group are split over a cluster's CTAs, rank r taking the
+  // r-th G / hs of them, and the CTAs add their sums at the end.
   const int nU = s.B * s.Hkv;
-  const int kt = (int)(blockIdx.x / nU), uk = (int)(blockIdx.x % nU), n = uk / s.Hkv, hk = uk % s.Hkv;
+  const int rank = (int)blockIdx.x % hs;
+  int blk = (int)blockIdx.x / hs;
+  if (dgate && --blk < 0) {  // one more CTA (or cluster), the first (as the last it would be the tail): the gate gradient
+    grid_wait();             // the dQ kernel's partial sums
+    if (rank == 0) reduce_gate(s, gate, dalpha_part, dgate);
+    return;
+  }
+  const int kt = blk / nU, uk = blk % nU, n = uk / s.Hkv, hk = uk % s.Hkv, Gs = s.G / hs, h_first = hk * s.G + rank * Gs;
   int len = seq_lens ? seq_lens[n] : s.L;
   len = min(max(len, 0), s.L);
   const int pad0 = s.L - len;
@@ -616,7 +656,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   // The tile list is the same for every query head of the group (one selection per group): the
   // kernel walks it once per head, item x = (head x / nlist, tile list[x % nlist]).
   const int nlist = *reinterpret_cast<const int *>(meta + ml.counts);
-  const int nvis = nlist * s.G;
+  const int nvis = nlist * Gs;
   const uint32_t tmem_base = tmem_slot;
   // half tile x uses buffer x % 2 at column 64 (x % 2): S^T in its first 32 columns, dP^T behind
   const uint32_t tmem_dv = tmem_base + 128, tmem_dk = tmem_base + 192;
@@ -626,7 +666,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     setmaxnreg_dec<kProducerRegs>();
     if (warp == kComputeWarps && nvis > 0) {
       // ---- loader: K, V once; Q, dO tiles and their row records up to STAGES ahead ----
-      int lj = 0, h = hk * s.G;
+      int lj = 0, h = h_first;
       for (int j = 0; j < nvis; ++j) {
         const int sj = j % STAGES;
         if (j >= STAGES) mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 214);
@@ -775,9 +815,19 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
       tmem_ld<OC>(tmem_dk + lane_off + half * OC, okk);
       tmem_wait_ld();
     }
-    {
+    const bool live = nvis > 0 && row_valid;
+    if (hs > 1) {
+      // this CTA's sums in fp32, in the (now free) Q/dO stages: [dV, dK][128 rows][D + 4]
+      float *acc = reinterpret_cast<float *>(qg_tiles) + r * (D + 4) + half * OC;
+#pragma unroll
+      for (int c = 0; c < OC; c += 4) {
+        *reinterpret_cast<float4 *>(acc + c) =
+            live ? make_float4(ov[c], ov[c + 1], ov[c + 2], ov[c + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4 *>(acc + 128 * (D + 4) + c) =
+            live ? make_float4(okk[c], okk[c + 1], okk[c + 2], okk[c + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    } else {
       // staged in the (now free) Q/dO stages, then two whole-line bulk stores clipped at L
-      const bool live = nvis > 0 && row_valid;
       uint8_t *sv_t = qg_tiles, *sk_t = qg_tiles + C::kBigBytes;
 #pragma unroll
       for (int ch = 0; ch < OC / 8; ++ch) {
@@ -800,8 +850,38 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
       }
     }
   }
+  if (hs > 1) {
+    // every CTA of the cluster adds its share of the rows over the cluster, in rank order
+    static_assert(2 * 128 * (D + 4) * 4 <= STAGES * kStageBytes, "the fp32 sums fit in the stages");
+    cg::cluster_group cluster = cg::this_cluster();
+    __syncwarp();
+    cluster.sync();
+    if (warp < kComputeWarps) {
+      const int rows = 128 / hs;
+      float *own = reinterpret_cast<float *>(qg_tiles);
+      for (int i = tid; i < 2 * rows * (D / 8); i += kComputeWarps * 32) {
+        const int ch = i % (D / 8), lr = (i / (D / 8)) % rows, which = i / (rows * (D / 8));
+        const int rr = rank * rows + lr, p = key0 + rr;
+        if (p >= s.L) continue;
+        float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int k = 0; k < hs; ++k) {
+          const float4 *o = reinterpret_cast<const float4 *>(cluster.map_shared_rank(own, k) +
+                                                             (which * 128 + rr) * (D + 4) + ch * 8);
+          const float4 a = o[0], b = o[1];
+          x[0] += a.x; x[1] += a.y; x[2] += a.z; x[3] += a.w; x[4] += b.x; x[5] += b.y; x[6] += b.z; x[7] += b.w;
+        }
+        const float f = which ? s.scale : 1.f;
+        *reinterpret_cast<uint4 *>((which ? dk : dv) + row_offset_kv(s, n, hk, p) + ch * 8) =
+            make_uint4(pack_bf16(x[0] * f, x[1] * f), pack_bf16(x[2] * f, x[3] * f), pack_bf16(x[4] * f, x[5] * f),
+                       pack_bf16(x[6] * f, x[7] * f));
+      }
+    }
+    __syncwarp();
+    cluster.sync();  // nobody leaves while its sums are being read
+  }
   if (nvis == 0 && tid == 0) mbar_wait(b_res, 0, &abort_flag, 222);  // no load may outlive the CTA
   finish(warp, tmem_base, kBwdTmemCols, &abort_flag, status);
+  if (tid == 0) grid_wait();  // (see grid_wait: by now the dQ kernel has mostly completed)
 }
 
 }  // namespace
@@ -810,7 +890,7 @@ template <int D>
 int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                     const int32_t *seq_lens, const int32_t *idx, const void *out_lt,
                     const void *out_st, const float *lse, const void *dout, void *dq, void *dk,
-                    void *dv, const Workspace &ws, cudaStream_t st, int branches, const float4 *records) {
+                    void *dv, float *dgate, const Workspace &ws, cudaStream_t st, int branches, const float4 *records) {
   typedef __nv_bfloat16 bf;
   using C = Cfg<D>;
   CUtensorMap q128, k64, v64, g128, q64, k128, v128, g64, tdq, tdk, tdv;
@@ -853,20 +933,32 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   }
   {
     LaunchScope ls(K_BWD_DKDV_TC, st);
-    const unsigned grid_k = (unsigned)nST * (unsigned)(s.B * s.Hkv);
-    launch_chained(kern_kv, dim3(grid_k), dim3(kKvThreads), smem_kv, st, q64, k128, v128, g64, s, seq_lens,
-                   (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT);
+    // Grouped heads: a CTA walks its tile list once per head, so with few CTAs the one with the first keys
+    // is the kernel's time (170 us at B 8, 8 heads on 2, L 1500, 192 CTAs): the heads are split over clusters
+    // while two waves of CTAs are not full.
+    const unsigned ctas = (unsigned)nST * (unsigned)(s.B * s.Hkv);
+    unsigned hs = 1;
+    while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < 592) hs *= 2;
+    const dim3 grid_k((ctas + (dgate ? 1 : 0)) * hs);
+    if (hs > 1)
+      launch_chained_cluster(kern_kv, grid_k, dim3(kKvThreads), smem_kv, hs, st, q64, k128, v128, g64, s, seq_lens,
+                             (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, (int)hs, (bf *)dk, (bf *)dv, gate,
+                             (const double *)ws.dalpha, dgate);
+    else
+      launch_chained(kern_kv, grid_k, dim3(kKvThreads), smem_kv, st, q64, k128, v128, g64, s, seq_lens,
+                     (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, 1, (bf *)dk, (bf *)dv, gate,
+                     (const double *)ws.dalpha, dgate);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
 template int launch_bwd_tc_t<32>(const Shape &, const void *, const void *, const void *, const float *,
                                  const int32_t *, const int32_t *, const void *, const void *,
-                                 const float *, const void *, void *, void *, void *, const Workspace &,
+                                 const float *, const void *, void *, void *, void *, float *, const Workspace &,
                                  cudaStream_t, int, const float4 *);
 template int launch_bwd_tc_t<64>(const Shape &, const void *, const void *, const void *, const float *,
                                  const int32_t *, const int32_t *, const void *, const void *,
-                                 const float *, const void *, void *, void *, void *, const Workspace &,
+                                 const float *, const void *, void *, void *, void *, float *, const Workspace &,
                                  cudaStream_t, int, const float4 *);
 
 }  // namespace tc

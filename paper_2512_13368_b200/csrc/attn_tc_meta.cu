@@ -426,7 +426,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
   // Four warps per image while its loops are long (a selection per position: 46 -> 28 us for 960 images at
-  // L 1500) or the images do not fill the SMs (18 -> 10 us for 256 images at L 4096); at 4096 images of L 1024
+  // L 1500) or the images do not fill the SMs (11 -> 10 us for 256 images at L 4096); at 4096 images of L 1024
   // four warps took 26 us and one 17.
   const bool wide = n_images <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;

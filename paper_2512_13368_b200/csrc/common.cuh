@@ -100,6 +100,12 @@ __device__ __forceinline__ void grid_chain_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// The two halves, for a pair of kernels that do not depend on each other: the first waits and only then
+// lets the second start (what precedes the first is then complete for the second too, which does not
+// wait at its start); the second waits before its CTAs exit, so that whoever waits for the second has
+// waited for the first as well.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 bool chained_launches();  // blossom_debug_switch(2, ...) / BLOSSOM_SERIAL_LAUNCH
 
 template <typename... KArgs, typename... Args>
@@ -115,6 +121,27 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained_launches() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// The same in thread-block clusters of `cluster` CTAs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster,
+                                          cudaStream_t st, Args &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained_launches() ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
@@ -212,10 +239,10 @@ size_t tc_inv_bits_bytes(const Shape &s);  // (selection per position) bytes of 
 // branches: bit 0 long-term, bit 1 short-term branch: the tile lists hold only the tiles those
 // branches need.  records: null = computed from out_lt, out_st, lse, dout and the per-head gate by
 // the pre-pass; otherwise the caller's per-row records (layout of Workspace::qstats) are used as
-// they are.
+// they are.  dgate: null = the gate gradient is not wanted.
 int launch_bwd_tc(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                   const int32_t *seq_lens, const int32_t *idx, const void *out_lt, const void *out_st,
-                  const float *lse, const void *dout, void *dq, void *dk, void *dv,
+                  const float *lse, const void *dout, void *dq, void *dk, void *dv, float *dgate,
                   const Workspace &ws, cudaStream_t st, int branches = 3, const float4 *records = nullptr);
 // the same two calls with the input-dependent gate (gate = F_o's parameters [H][2 D + 1])
 int launch_fwd_tc_gate(const Shape &s, const void *q, const void *k, const void *v, const float *gate,

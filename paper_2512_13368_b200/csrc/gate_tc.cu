@@ -272,11 +272,11 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
                                                  ws.qstats2, ws.dgate_part, Lpad);
     if (cudaGetLastError() != cudaSuccess) return BLOSSOM_ERR_CUDA;
   }
-  int rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, ws, st, 1,
+  int rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, nullptr, ws, st, 1,
                          ws.qstats);
   if (rc) return rc;
   rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_gst, ws.gate_dq, ws.gate_dk,
-                     ws.gate_dv, ws, st, 2, ws.qstats2);
+                     ws.gate_dv, nullptr, ws, st, 2, ws.qstats2);
   if (rc) return rc;
   if ((rc = add_into(s, false, dq, ws.gate_dq, st))) return rc;
   if ((rc = add_into(s, true, dk, ws.gate_dk, st))) return rc;

@@ -514,7 +514,7 @@ template <int D>
 int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                     const int32_t *seq_lens, const int32_t *idx, const void *out_lt,
                     const void *out_st, const float *lse, const void *dout, void *dq, void *dk,
-                    void *dv, const Workspace &ws, cudaStream_t st, int branches, const float4 *records);
+                    void *dv, float *dgate, const Workspace &ws, cudaStream_t st, int branches, const float4 *records);
 
 }  // namespace tc
 }  // namespace blossom

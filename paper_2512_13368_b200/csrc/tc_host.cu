@@ -102,12 +102,12 @@ int launch_fwd_tc(const Shape &s, const void *q, const void *k, const void *v, c
 
 int launch_bwd_tc(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                   const int32_t *seq_lens, const int32_t *idx, const void *out_lt, const void *out_st,
-                  const float *lse, const void *dout, void *dq, void *dk, void *dv,
+                  const float *lse, const void *dout, void *dq, void *dk, void *dv, float *dgate,
                   const Workspace &ws, cudaStream_t st, int branches, const float4 *records) {
   if (s.D == 32)
-    return launch_bwd_tc_t<32>(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, dout, dq, dk, dv, ws, st,
+    return launch_bwd_tc_t<32>(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, dout, dq, dk, dv, dgate, ws, st,
                                branches, records);
-  return launch_bwd_tc_t<64>(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, dout, dq, dk, dv, ws, st,
+  return launch_bwd_tc_t<64>(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, dout, dq, dk, dv, dgate, ws, st,
                              branches, records);
 }
 
