@@ -101,6 +101,7 @@ Workspace carve_workspace(const Shape &s, void *base) {
     // rotated copies of q and k span what the originals span (same strides)
     const size_t qspan = (size_t)((s.B - 1) * s.sb + (s.H - 1) * s.sh + (int64_t)(s.L - 1) * s.sl + s.D);
     const size_t kspan = (size_t)((s.B - 1) * s.ksb + (s.Hkv - 1) * s.ksh + (int64_t)(s.L - 1) * s.ksl + s.D);
+    w.rope_table = take(s.rope_theta > 0 ? (size_t)s.L * (s.D / 2) * 16 : 0);
     w.q_rot = take(s.rope_theta > 0 ? qspan * s.esz : 0);
     w.k_rot = take(s.rope_theta > 0 ? kspan * s.esz : 0);
   }
@@ -206,10 +207,7 @@ static int rotate_inputs(const Shape &s, int dtype, const Workspace &ws, const v
                          cudaStream_t st, bool reuse = false) {
   if (s.rope_theta <= 0) return BLOSSOM_OK;
   if (!reuse) {
-    int rc = launch_rope(s, dtype, false, +1, *q, ws.q_rot, st);
-    if (rc) return rc;
-    rc = launch_rope(s, dtype, true, +1, *k, ws.k_rot, st);
-    if (rc) return rc;
+    if (int rc = launch_rope(s, dtype, +1, *q, ws.q_rot, *k, ws.k_rot, ws.rope_table, false, st)) return rc;
   }
   *q = ws.q_rot;
   *k = ws.k_rot;
@@ -218,22 +216,18 @@ static int rotate_inputs(const Shape &s, int dtype, const Workspace &ws, const v
 
 static bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) != 0; }
 
-// Validates the workspace and clears status words on the stream (a memset, not a kernel).  The
-// forward (and the selection) report in words 0..3, the backward in words 4..7.  A forward or a
-// selection clears both sets (a new step begins), a backward only its own, so a wait that ran out
-// in the forward is still on record after the backward that follows it on the same workspace.
-static int check_workspace(const Shape &s, void *ws, size_t bytes, cudaStream_t st, Workspace *out,
-                           bool backward = false, bool short_path = false) {
+// The forward (and the selection) report in status words 0..3, the backward in words 4..7.  A forward or
+// a selection clears both sets (a new step begins), a backward only its own, so a wait that ran out in
+// the forward is still on record after the backward that follows it on the same workspace.  A kernel of
+// the call that starts before any that can report clears them where there is one; a memset on the stream
+// otherwise (it is a few microseconds of a short call, and it keeps the kernels around it from chaining).
+static int check_workspace(const Shape &s, void *ws, size_t bytes, Workspace *out) {
   if (!ws || misaligned(ws, 256)) return BLOSSOM_ERR_WORKSPACE;
   *out = carve_workspace(s, ws);
-  if (bytes < out->bytes) return BLOSSOM_ERR_WORKSPACE;
-  // (the short-history forward clears the words itself, and with them what its backward counts in)
-  if (short_path && (!backward || s.reuse_lists)) return BLOSSOM_OK;
-  if (short_path)
-    return cudaMemsetAsync(out->status_bwd, 0, (sh::kCounterWord - 3) * 4, st) == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
-  if (cudaMemsetAsync(backward ? out->status_bwd : out->status, 0, backward ? 16 : 32, st) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
-  return BLOSSOM_OK;
+  return bytes < out->bytes ? BLOSSOM_ERR_WORKSPACE : BLOSSOM_OK;
+}
+static int clear_words(int32_t *p, int n, cudaStream_t st) {
+  return cudaMemsetAsync(p, 0, (size_t)n * sizeof(int32_t), st) == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
 }  // namespace blossom
@@ -259,11 +253,11 @@ int blossom_select_blocks(const blossom_params *params, const void *q, const voi
   if (misaligned(q, 16) || misaligned(k, 16) || misaligned(block_idx, 4) || misaligned(seq_lens, 4))
     return BLOSSOM_ERR_INVALID_ARG;
   Workspace ws;
-  rc = check_workspace(s, workspace, workspace_bytes, (cudaStream_t)stream, &ws);
+  rc = check_workspace(s, workspace, workspace_bytes, &ws);
   if (rc) return rc;
   rc = rotate_inputs(s, params->dtype, ws, &q, &k, (cudaStream_t)stream);
   if (rc) return rc;
-  return launch_select(s, params->dtype, q, k, seq_lens, block_idx, ws, (cudaStream_t)stream);
+  return launch_select(s, params->dtype, q, k, seq_lens, block_idx, ws, (cudaStream_t)stream);  // (clears the words)
 }
 
 int blossom_select_blocks_static(const blossom_params *params, const void *q, const void *k,
@@ -297,7 +291,9 @@ int blossom_attn_fwd(const blossom_params *params, const void *q, const void *k,
   Workspace ws;
   cudaStream_t st = (cudaStream_t)stream;
   const bool short_path = !force_simt() && sh::fwd_short_supported(s, params->dtype, out_lt != nullptr);
-  rc = check_workspace(s, workspace, workspace_bytes, st, &ws, false, short_path);
+  rc = check_workspace(s, workspace, workspace_bytes, &ws);
+  // (the short-history kernel and the first kernel of the selection clear the words themselves)
+  if (!rc && !short_path && idx_is_input) rc = clear_words(ws.status, 8, st);
   if (rc) return rc;
   rc = rotate_inputs(s, params->dtype, ws, &q, &k, st);
   if (rc) return rc;
@@ -339,7 +335,12 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
   Workspace ws;
   cudaStream_t st = (cudaStream_t)stream;
   const bool short_path = !force_simt() && sh::bwd_short_supported(s, params->dtype);
-  rc = check_workspace(s, workspace, workspace_bytes, st, &ws, true, short_path);
+  const bool tc_path = !force_simt() && tc::fwd_tc_supported(s, params->dtype);
+  rc = check_workspace(s, workspace, workspace_bytes, &ws);
+  // (the tensor-core pre-pass clears the words itself; after a short-history forward they and the word that
+  // its backward counts in are zero)
+  if (!rc && short_path && !s.reuse_lists) rc = clear_words(ws.status_bwd, sh::kCounterWord - 3, st);
+  if (!rc && !short_path && !tc_path) rc = clear_words(ws.status_bwd, 4, st);
   if (rc) return rc;
   rc = rotate_inputs(s, params->dtype, ws, &q, &k, st, s.reuse_lists != 0);
   if (rc) return rc;
@@ -347,7 +348,7 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
   if (short_path) {
     rc = sh::launch_bwd_short(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout, dq, dk, dv, dgate,
                               ws, st);
-  } else if (!force_simt() && tc::fwd_tc_supported(s, params->dtype)) {
+  } else if (tc_path) {
     if (s.gate_mode) {
       rc = tc::launch_bwd_tc_gate(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout,
                                   dq, dk, dv, dgate, ws, st);
@@ -361,9 +362,8 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
   }
   if (rc || s.rope_theta <= 0) return rc;
   // dq, dk hold the gradients of the rotated tensors: turn them back (the transpose), in place
-  rc = launch_rope(s, params->dtype, false, -1, dq, dq, st);
-  if (rc) return rc;
-  return launch_rope(s, params->dtype, true, -1, dk, dk, st);
+  // (the table is there: this call, or the forward whose copies it reuses, has filled it)
+  return launch_rope(s, params->dtype, -1, dq, dq, dk, dk, ws.rope_table, true, st);
 }
 
 int blossom_device_status(const void *workspace, blossom_stream_t stream, int32_t *host_out) {

@@ -571,6 +571,7 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(Shape s, const float *__
 // adds the entries i, i + 32, ... in ascending order, then a fixed shuffle tree joins the lanes.
 __global__ void __launch_bounds__(256) gate_param_grad_kernel(Shape s, const double *__restrict__ part,
                                                               float *__restrict__ dgate) {
+  grid_chain_enter();
   const int GW = 2 * s.D + 1;
   const int w = (int)blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w >= s.H * GW) return;
@@ -649,7 +650,8 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
 int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st) {
   {
     LaunchScope ls(K_GATE_GRAD, st);
-    gate_param_grad_kernel<<<(unsigned)((s.H * (2 * s.D + 1) + 7) / 8), 256, 0, st>>>(s, ws.dgate_part, dgate);
+    launch_chained(gate_param_grad_kernel, dim3((unsigned)((s.H * (2 * s.D + 1) + 7) / 8)), dim3(256), 0, st, s,
+                   (const double *)ws.dgate_part, dgate);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

@@ -72,8 +72,10 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(Shape s, const float *__r
                                                        const __nv_bfloat16 *__restrict__ out_st,
                                                        const float *__restrict__ lse,
                                                        const __nv_bfloat16 *__restrict__ dout,
-                                                       float4 *__restrict__ qstats, int Lpad) {
+                                                       float4 *__restrict__ qstats, int Lpad,
+                                                       int32_t *__restrict__ status) {
   grid_chain_enter();
+  if (blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;  // the backward's status words
   constexpr int LPR = D / 8;         // lanes per row
   constexpr int RPB = 256 / LPR;     // rows per block
   const int blocks_per_unit = (Lpad + RPB - 1) / RPB;
@@ -923,7 +925,7 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     const int Lpad = nT * 64, rpb = 256 / (D / 8);
     const unsigned gp = (unsigned)(s.B * s.H) * (unsigned)((Lpad + rpb - 1) / rpb);
     launch_chained(bwd_prep_kernel<D>, dim3(gp), dim3(256), 0, st, s, gate, seq_lens, (const bf *)out_lt,
-                   (const bf *)out_st, lse, (const bf *)dout, ws.qstats, Lpad);
+                   (const bf *)out_st, lse, (const bf *)dout, ws.qstats, Lpad, ws.status_bwd);
   }
   {
     LaunchScope ls(K_BWD_DQ_TC, st);

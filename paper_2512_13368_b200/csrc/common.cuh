@@ -53,6 +53,7 @@ struct Workspace {
   int32_t *clive;    // [B][H][Mc]     their numbers of valid keys
   float *cmean32;    // [B][H][Mc][D]  the means rounded to fp32
   float *cnorm;      // [B][H][Mc]     upper bounds of the norms of the fp32 means
+  void *rope_table;     // [L][D / 2] (cos, sin) in double precision (rope_theta > 0)
   void *q_rot, *k_rot;  // rotated copies of q and k (rope_theta > 0), laid out with the originals' strides
   float *gate_ac;    // [2][B][H][L]  input-dependent gate: alpha_t and c_t of every row (backward)
   double *dgate_part;// [B][H][M][2 D + 1]  per query block partial of the gradient of F_o's parameters
@@ -211,6 +212,7 @@ __device__ __forceinline__ bool st_ranges_touch(const Shape &s, int t0, int t1, 
 }
 
 // launchers (one translation unit each)
+// (its first kernel clears the status words of the workspace)
 int launch_select(const Shape &s, int dtype, const void *q, const void *k, const int32_t *seq_lens,
                   int32_t *idx, const Workspace &ws, cudaStream_t st);
 int launch_fwd_simt(const Shape &s, int dtype, const void *q, const void *k, const void *v,
@@ -229,7 +231,8 @@ int launch_gate_grad(const Shape &s, const float *gate, const Workspace &ws, flo
                      cudaStream_t st);
 // input-dependent gate: fixed-order reduction of ws.dgate_part into dgate [H][2 D + 1]
 int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st);
-int launch_rope(const Shape &s, int dtype, bool kv, int dir, const void *src, void *dst, cudaStream_t st);
+int launch_rope(const Shape &s, int dtype, int dir, const void *qs, void *qd, const void *ks, void *kd, void *table,
+                bool have_table, cudaStream_t st);
 
 namespace tc {
 int launch_wait_selftest(int32_t *status, cudaStream_t st);

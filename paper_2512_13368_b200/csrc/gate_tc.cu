@@ -62,6 +62,7 @@ template <int D>
 __global__ void __launch_bounds__(256) gate_mix_kernel(Shape s, const float *__restrict__ gate,
                                                        const bf *__restrict__ out_lt, const bf *__restrict__ out_st,
                                                        bf *__restrict__ out) {
+  grid_chain_enter();
   constexpr int LPR = D / 8, RPB = 256 / LPR;
   const int blocks_per_unit = (s.L + RPB - 1) / RPB;
   const int u = blockIdx.x / blocks_per_unit, n = u / s.H, h = u % s.H;
@@ -103,7 +104,10 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
                                                         const float *__restrict__ lse, const bf *__restrict__ dout,
                                                         bf *__restrict__ g_lt, bf *__restrict__ g_st,
                                                         float4 *__restrict__ rec_lt, float4 *__restrict__ rec_st,
-                                                        double *__restrict__ dgate_part, int Lpad) {
+                                                        double *__restrict__ dgate_part, int Lpad,
+                                                        int32_t *__restrict__ status) {
+  grid_chain_enter();
+  if (blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;  // the backward's status words
   constexpr int LPR = D / 8, RPB = 256 / LPR, GW = 2 * D + 1;
   __shared__ double red[RPB][GW];
   const int u = blockIdx.x / s.M, qb = blockIdx.x % s.M, n = u / s.H, h = u % s.H;
@@ -208,33 +212,31 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
   }
 }
 
-// ---- dst += src over a q-shaped (or k-shaped) bf16 tensor, one rounding --------------------------
-__global__ void __launch_bounds__(256) grad_add_kernel(int B, int heads, int L, int D, int64_t sb, int64_t sh,
-                                                       int64_t sl, bf *__restrict__ dst, const bf *__restrict__ src) {
+// ---- dst += src over the three gradients, one rounding --------------------------------------------
+struct AddTensor {
+  bf *dst;
+  const bf *src;
+  int heads;
+  int64_t sb, sh, sl;
+};
+__global__ void __launch_bounds__(256) grad_add_kernel(int B, int L, int D, AddTensor x, AddTensor y, AddTensor z) {
+  grid_chain_enter();
   const int cpr = D / 8;
-  const int64_t total = (int64_t)B * heads * L * cpr;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t per = (int64_t)B * L * cpr, nx = per * x.heads, ny = per * y.heads, total = nx + 2 * ny;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const AddTensor &w = i < nx ? x : i < nx + ny ? y : z;
+    const int64_t e = i < nx ? i : i < nx + ny ? i - nx : i - nx - ny;
     const int ch = (int)(e % cpr);
     const int64_t row = e / cpr;
-    const int t = (int)(row % L), h = (int)((row / L) % heads), n = (int)(row / ((int64_t)L * heads));
-    const int64_t off = (int64_t)n * sb + (int64_t)h * sh + (int64_t)t * sl + ch * 8;
+    const int t = (int)(row % L), h = (int)((row / L) % w.heads), n = (int)(row / ((int64_t)L * w.heads));
+    const int64_t off = (int64_t)n * w.sb + (int64_t)h * w.sh + (int64_t)t * w.sl + ch * 8;
     float a[8], b[8];
-    unpack8(*reinterpret_cast<const uint4 *>(dst + off), a);
-    unpack8(*reinterpret_cast<const uint4 *>(src + off), b);
+    unpack8(*reinterpret_cast<const uint4 *>(w.dst + off), a);
+    unpack8(*reinterpret_cast<const uint4 *>(w.src + off), b);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] += b[i];
-    *reinterpret_cast<uint4 *>(dst + off) = pack8(a);
+    for (int j = 0; j < 8; ++j) a[j] += b[j];
+    *reinterpret_cast<uint4 *>(w.dst + off) = pack8(a);
   }
-}
-
-int add_into(const Shape &s, bool kv, void *dst, const void *src, cudaStream_t st) {
-  const int heads = kv ? s.Hkv : s.H;
-  const int64_t total = (int64_t)s.B * heads * s.L * (s.D / 8);
-  const unsigned grid = (unsigned)((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16);
-  LaunchScope ls(K_GATE_GRAD, st);
-  grad_add_kernel<<<grid, 256, 0, st>>>(s.B, heads, s.L, s.D, kv ? s.ksb : s.sb, kv ? s.ksh : s.sh,
-                                        kv ? s.ksl : s.sl, (bf *)dst, (const bf *)src);
-  return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
 }  // namespace
@@ -249,8 +251,8 @@ int launch_fwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
   const int rpb = 256 / (s.D / 8);
   const unsigned grid = (unsigned)(s.B * s.H) * (unsigned)((s.L + rpb - 1) / rpb);
   LaunchScope ls(K_GATE_GRAD, st);
-  if (s.D == 32) gate_mix_kernel<32><<<grid, 256, 0, st>>>(s, gate, (const bf *)olt, (const bf *)ost, (bf *)out);
-  else gate_mix_kernel<64><<<grid, 256, 0, st>>>(s, gate, (const bf *)olt, (const bf *)ost, (bf *)out);
+  launch_chained(s.D == 32 ? gate_mix_kernel<32> : gate_mix_kernel<64>, dim3(grid), dim3(256), 0, st, s, gate,
+                 (const bf *)olt, (const bf *)ost, (bf *)out);
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
@@ -262,14 +264,9 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
   {
     LaunchScope ls(K_BWD_PREP, st);
     const unsigned grid = (unsigned)(s.B * s.H) * (unsigned)s.M;
-    if (s.D == 32)
-      gate_prep_kernel<32><<<grid, 256, 0, st>>>(s, gate, seq_lens, (const bf *)out_lt, (const bf *)out_st, lse,
-                                                 (const bf *)dout, (bf *)ws.gate_glt, (bf *)ws.gate_gst, ws.qstats,
-                                                 ws.qstats2, ws.dgate_part, Lpad);
-    else
-      gate_prep_kernel<64><<<grid, 256, 0, st>>>(s, gate, seq_lens, (const bf *)out_lt, (const bf *)out_st, lse,
-                                                 (const bf *)dout, (bf *)ws.gate_glt, (bf *)ws.gate_gst, ws.qstats,
-                                                 ws.qstats2, ws.dgate_part, Lpad);
+    launch_chained(s.D == 32 ? gate_prep_kernel<32> : gate_prep_kernel<64>, dim3(grid), dim3(256), 0, st, s, gate, seq_lens,
+                   (const bf *)out_lt, (const bf *)out_st, lse, (const bf *)dout, (bf *)ws.gate_glt, (bf *)ws.gate_gst,
+                   ws.qstats, ws.qstats2, ws.dgate_part, Lpad, ws.status_bwd);
     if (cudaGetLastError() != cudaSuccess) return BLOSSOM_ERR_CUDA;
   }
   int rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, nullptr, ws, st, 1,
@@ -278,9 +275,15 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
   rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_gst, ws.gate_dq, ws.gate_dk,
                      ws.gate_dv, nullptr, ws, st, 2, ws.qstats2);
   if (rc) return rc;
-  if ((rc = add_into(s, false, dq, ws.gate_dq, st))) return rc;
-  if ((rc = add_into(s, true, dk, ws.gate_dk, st))) return rc;
-  if ((rc = add_into(s, true, dv, ws.gate_dv, st))) return rc;
+  {
+    const AddTensor x = {(bf *)dq, (const bf *)ws.gate_dq, s.H, s.sb, s.sh, s.sl};
+    const AddTensor y = {(bf *)dk, (const bf *)ws.gate_dk, s.Hkv, s.ksb, s.ksh, s.ksl};
+    const AddTensor z = {(bf *)dv, (const bf *)ws.gate_dv, s.Hkv, s.ksb, s.ksh, s.ksl};
+    const int64_t ctas = ((int64_t)s.B * (s.H + 2 * s.Hkv) * s.L * (s.D / 8) + 255) / 256;
+    LaunchScope ls(K_GATE_GRAD, st);
+    launch_chained(grad_add_kernel, dim3((unsigned)(ctas < 148 * 16 ? ctas : 148 * 16)), dim3(256), 0, st, s.B, s.L, s.D, x, y,
+                   z);
+  }
   return launch_gate_param_grad(s, ws, dgate, st);
 }
 

@@ -12,84 +12,124 @@
 namespace blossom {
 namespace {
 
-__device__ __forceinline__ void store_pair(float *p, double a, double b) {
-  *reinterpret_cast<float2 *>(p) = make_float2((float)a, (float)b);
-}
-__device__ __forceinline__ void store_pair(__nv_bfloat16 *p, double a, double b) {
-  __nv_bfloat162 h;
-  h.x = __double2bfloat16(a);
-  h.y = __double2bfloat16(b);
-  *reinterpret_cast<__nv_bfloat162 *>(p) = h;
-}
-__device__ __forceinline__ double2 load_pair(const float *p) {
-  const float2 v = *reinterpret_cast<const float2 *>(p);
-  return make_double2((double)v.x, (double)v.y);
-}
-__device__ __forceinline__ double2 load_pair(const __nv_bfloat16 *p) {
-  const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(p);
-  return make_double2((double)__bfloat162float(v.x), (double)__bfloat162float(v.y));
+// Eight consecutive elements (four pairs), rotated in double precision, rounded once.
+template <typename T>
+struct Vec8;
+template <>
+struct Vec8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float *p) {
+    a = reinterpret_cast<const float4 *>(p)[0];
+    b = reinterpret_cast<const float4 *>(p)[1];
+  }
+  __device__ __forceinline__ static void turn(float &x, float &y, double2 cs) {
+    const double u = x, v = y;
+    x = (float)(u * cs.x - v * cs.y);
+    y = (float)(u * cs.y + v * cs.x);
+  }
+  __device__ __forceinline__ void rotate_store(const double2 (&cs)[4], float *p) {
+    turn(a.x, a.y, cs[0]); turn(a.z, a.w, cs[1]); turn(b.x, b.y, cs[2]); turn(b.z, b.w, cs[3]);
+    reinterpret_cast<float4 *>(p)[0] = a;
+    reinterpret_cast<float4 *>(p)[1] = b;
+  }
+};
+template <>
+struct Vec8<__nv_bfloat16> {
+  uint4 r;
+  __device__ __forceinline__ void load(const __nv_bfloat16 *p) { r = *reinterpret_cast<const uint4 *>(p); }
+  __device__ __forceinline__ static uint32_t turn(uint32_t w, double2 cs) {
+    const double u = __uint_as_float(w << 16), v = __uint_as_float(w & 0xffff0000u);
+    __nv_bfloat162 h;
+    h.x = __double2bfloat16(u * cs.x - v * cs.y);
+    h.y = __double2bfloat16(u * cs.y + v * cs.x);
+    return *reinterpret_cast<uint32_t *>(&h);
+  }
+  __device__ __forceinline__ void rotate_store(const double2 (&cs)[4], __nv_bfloat16 *p) {
+    *reinterpret_cast<uint4 *>(p) = make_uint4(turn(r.x, cs[0]), turn(r.y, cs[1]), turn(r.z, cs[2]), turn(r.w, cs[3]));
+  }
+};
+
+// cos and sin of every (position, pair), once per call: [L][D / 2].
+__global__ void __launch_bounds__(128) rope_table_kernel(int L, int D, double theta, double2 *__restrict__ table) {
+  grid_chain_enter();
+  const int half = D / 2;
+  const int e = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (e >= L * half) return;
+  const int i = e % half, t = e / half;
+  double sn, cs;
+  sincos((double)t * pow(theta, -2.0 * (double)i / (double)D), &sn, &cs);
+  table[e] = make_double2(cs, sn);
 }
 
-// One thread per (position t, pair i) and slice of the (batch, head) rows: the angle, its sine and
-// cosine are evaluated once and applied to that pair of every row of the slice, so the
-// double-precision transcendental work is shared by all rows that sit at the same position.  A
-// warp's 32 pairs are 32 consecutive pairs of one row: whole 128-byte (bf16) lines.  heads /
-// strides describe the tensor ([B][heads][L][D]); dir = +1 rotates by the position's angle, -1 by
-// its negative (the transpose).  src may equal dst.
+// One or two tensors ([B][heads][L][D] with strides) rotated by the table's angles (dir = +1) or their
+// negatives (-1).  A thread owns four consecutive pairs of a position and walks a slice of the (batch,
+// head) rows of both tensors with them, four rows in flight: the table is read once per slice.  Double
+// precision per pair and one rounding; what bounds it then is memory (q and k of B 16, H 4, L 900, D 64:
+// 15 MB in and as much out).  Evaluating the angles in every slice of the rows instead took 16 us a tensor
+// at that size (900 x 32 angles, eleven times), four launches a training step.
+struct RopeTensor {
+  const void *src;  // may equal dst
+  void *dst;
+  int rows, heads;  // rows = B * heads
+  int64_t sb, sh, sl;
+};
 template <typename T>
-__global__ void __launch_bounds__(256) rope_kernel(int B, int heads, int L, int D, int64_t sb, int64_t sh,
-                                                   int64_t sl, double theta, int dir, const T *__restrict__ src,
-                                                   T *__restrict__ dst) {
-  const int half = D / 2;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)L * half) return;
-  const int i = (int)(e % half), t = (int)(e / half);
-  const double ang = (double)t * pow(theta, -2.0 * (double)i / (double)D) * (double)dir;
-  double sn, cs;
-  sincos(ang, &sn, &cs);
-  const int rows = B * heads;
-  const int64_t base = (int64_t)t * sl + 2 * i;
-  for (int r0 = (int)blockIdx.y * 4; r0 < rows; r0 += (int)gridDim.y * 4) {
-    double2 x[4];
-    int64_t off[4];
+__global__ void __launch_bounds__(256) rope_kernel(int L, int D, int dir, const double2 *__restrict__ table, RopeTensor x,
+                                                   RopeTensor y) {
+  grid_chain_enter();
+  const int quads = D / 8;
+  const int e = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (e >= L * quads) return;
+  const int t = e / quads, c = (e % quads) * 8;
+  double2 cs[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {  // four rows in flight
+  for (int j = 0; j < 4; ++j) {
+    cs[j] = table[t * (D / 2) + c / 2 + j];
+    if (dir < 0) cs[j].y = -cs[j].y;
+  }
+  const int rows = x.rows + y.rows;
+  for (int r0 = (int)blockIdx.y * 4; r0 < rows; r0 += (int)gridDim.y * 4) {
+    Vec8<T> v[4];
+    T *out[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
       const int r = r0 + j;
-      off[j] = base + (int64_t)(r / heads) * sb + (int64_t)(r % heads) * sh;
-      if (r < rows) x[j] = load_pair(src + off[j]);
+      if (r < rows) {
+        const RopeTensor &z = r < x.rows ? x : y;
+        const int k = r < x.rows ? r : r - x.rows;
+        const int64_t off = (int64_t)(k / z.heads) * z.sb + (int64_t)(k % z.heads) * z.sh + (int64_t)t * z.sl + c;
+        v[j].load(static_cast<const T *>(z.src) + off);
+        out[j] = static_cast<T *>(z.dst) + off;
+      }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (r0 + j < rows) store_pair(dst + off[j], x[j].x * cs - x[j].y * sn, x[j].x * sn + x[j].y * cs);
+      if (r0 + j < rows) v[j].rotate_store(cs, out[j]);
   }
-}
-
-template <typename T>
-int launch_rope_t(int B, int heads, int L, int D, int64_t sb, int64_t sh, int64_t sl, double theta, int dir,
-                  const T *src, T *dst, cudaStream_t st) {
-  const int64_t per_row = (int64_t)L * (D / 2);
-  const unsigned gx = (unsigned)((per_row + 255) / 256);
-  // enough slices of the rows to fill the GPU about eight CTAs deep, each of at least four rows
-  const int64_t want = (148 * 8 + gx - 1) / gx, most = ((int64_t)B * heads + 3) / 4;
-  int64_t gy = want < 1 ? 1 : (want > most ? most : want);
-  if (gy > 65535) gy = 65535;
-  {
-    LaunchScope ls(K_ROPE, st);
-    rope_kernel<T><<<dim3(gx, (unsigned)gy), 256, 0, st>>>(B, heads, L, D, sb, sh, sl, theta, dir, src, dst);
-  }
-  return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
 }  // namespace
 
-// kv = false: a q-shaped tensor (query heads, q strides); true: a k-shaped one.
-int launch_rope(const Shape &s, int dtype, bool kv, int dir, const void *src, void *dst, cudaStream_t st) {
-  const int heads = kv ? s.Hkv : s.H;
-  const int64_t sb = kv ? s.ksb : s.sb, sh = kv ? s.ksh : s.sh, sl = kv ? s.ksl : s.sl;
-  if (dtype == BLOSSOM_DTYPE_FP32)
-    return launch_rope_t<float>(s.B, heads, s.L, s.D, sb, sh, sl, s.rope_theta, dir, (const float *)src, (float *)dst, st);
-  return launch_rope_t<__nv_bfloat16>(s.B, heads, s.L, s.D, sb, sh, sl, s.rope_theta, dir,
-                                      (const __nv_bfloat16 *)src, (__nv_bfloat16 *)dst, st);
+// Rotates q-shaped `qs` into `qd` and k-shaped `ks` into `kd` (dir = +1) or back (-1).  table: [L][D / 2]
+// double2 in the workspace, filled first unless `have_table`.
+int launch_rope(const Shape &s, int dtype, int dir, const void *qs, void *qd, const void *ks, void *kd, void *table,
+                bool have_table, cudaStream_t st) {
+  double2 *tab = static_cast<double2 *>(table);
+  if (!have_table) {
+    LaunchScope ls(K_ROPE, st);
+    launch_chained(rope_table_kernel, dim3((unsigned)((s.L * (s.D / 2) + 127) / 128)), dim3(128), 0, st, s.L, s.D,
+                   s.rope_theta, tab);
+  }
+  const RopeTensor x = {qs, qd, s.B * s.H, s.H, s.sb, s.sh, s.sl}, y = {ks, kd, s.B * s.Hkv, s.Hkv, s.ksb, s.ksh, s.ksl};
+  const unsigned gx = (unsigned)((s.L * (s.D / 8) + 255) / 256);
+  // enough slices of the rows to fill the GPU about eight CTAs deep, each of at least four rows
+  const int64_t want = (148 * 8 + gx - 1) / gx, most = ((int64_t)x.rows + y.rows + 3) / 4;
+  int64_t gy = want < 1 ? 1 : (want > most ? most : want);
+  if (gy > 65535) gy = 65535;
+  LaunchScope ls(K_ROPE, st);
+  auto kern = dtype == BLOSSOM_DTYPE_FP32 ? rope_kernel<float> : rope_kernel<__nv_bfloat16>;
+  launch_chained(kern, dim3(gx, (unsigned)gy), dim3(256), 0, st, s.L, s.D, dir, (const double2 *)tab, x, y);
+  return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }
 
 }  // namespace blossom

@@ -76,8 +76,10 @@ __global__ void __launch_bounds__(256, PHI ? 2 : 4) summary_kernel(Shape sh, Sel
                                                          int32_t *__restrict__ live,
                                                          float *__restrict__ mean32,
                                                          float *__restrict__ norm,
-                                                         int32_t *__restrict__ sel_count) {
+                                                         int32_t *__restrict__ sel_count,
+                                                         int32_t *__restrict__ status) {
   grid_chain_enter();
+  if (status && blockIdx.x == 0 && threadIdx.x < 8) status[threadIdx.x] = 0;  // a new step's status words
   constexpr int LPR = D / 8;     // lanes per row
   constexpr int RPI = 32 / LPR;  // rows per warp iteration
   constexpr int NF = sizeof(T) == 2 ? 8 : 2;  // rows in flight per lane
@@ -1055,6 +1057,7 @@ struct SelBuffers {
   int32_t *live;
   float *mean32, *norm;
   int32_t *list, *count;
+  int32_t *status;  // the workspace's status words, to be cleared, or null
 };
 
 // Dynamic shared memory of the two scoring kernels; 0 = the single-precision stage does not take
@@ -1079,9 +1082,11 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   if (g.n > 0) {
     LaunchScope ls(K_SUMMARY, st);
     auto summary = sh.phi ? summary_kernel<T, D, true> : summary_kernel<T, D, false>;
-    summary<<<(unsigned)((units * g.n + 7) / 8), 256, 0, st>>>(sh, g, k, seq_lens, w.mean, w.live, w.mean32, w.norm,
-                                                               w.count);
-  } else if (cudaMemsetAsync(w.count, 0, sizeof(int32_t), st) != cudaSuccess) {
+    if (launch_chained(summary, dim3((unsigned)((units * g.n + 7) / 8)), dim3(256), 0, st, sh, g, k, seq_lens, w.mean, w.live,
+                       w.mean32, w.norm, w.count, w.status) != cudaSuccess)
+      return BLOSSOM_ERR_CUDA;
+  } else if (cudaMemsetAsync(w.count, 0, sizeof(int32_t), st) != cudaSuccess ||
+             (w.status && cudaMemsetAsync(w.status, 0, 8 * sizeof(int32_t), st) != cudaSuccess)) {
     return BLOSSOM_ERR_CUDA;
   }
   // First stage: single precision with a bound; what it cannot certify goes on the work list.
@@ -1197,6 +1202,7 @@ int launch_select(const Shape &s, int dtype, const void *q, const void *k, const
   } else {
     w.mean = ws.kmean; w.live = ws.klive; w.mean32 = ws.kmean32; w.norm = ws.knorm;
   }
+  w.status = ws.status;
   w.list = ws.sel_list;
   w.count = ws.sel_count;
   return launch_select_buffers(s, dtype, q, k, seq_lens, idx, w, st);
@@ -1240,6 +1246,7 @@ int launch_select_static(const Shape &s, int dtype, const void *q, const void *k
   }
   unsigned char *base = static_cast<unsigned char *>(g_scratch_addr[dev]);
   SelBuffers w;
+  w.status = nullptr;
   w.mean = reinterpret_cast<double *>(base);
   w.mean32 = reinterpret_cast<float *>(base + kStaticOffMean32);
   w.live = reinterpret_cast<int32_t *>(base + kStaticOffLive);

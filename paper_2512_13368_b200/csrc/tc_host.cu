@@ -33,10 +33,17 @@ int make_tensor_map(CUtensorMap *map, const void *base, const Shape &s, int box_
   const cuuint32_t box[4] = {(cuuint32_t)s.D, (cuuint32_t)box_rows, (cuuint32_t)box_heads, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUtensorMapSwizzle sw = s.D == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
-  CUresult rc = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box,
-                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return rc == CUDA_SUCCESS ? 0 : 1;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+      return 0;
+    // the driver call wants a current context, which a thread that has made no runtime call yet (autograd's)
+    // lacks: make the device's own current and try once more
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return 1;
+  }
+  return 1;
 }
 
 // Diagnostic kernel: the bounded-wait machinery of the attention kernels on a wait that cannot
