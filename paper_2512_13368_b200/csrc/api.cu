@@ -91,7 +91,7 @@ Workspace carve_workspace(const Shape &s, void *base) {
   w.sel_list = reinterpret_cast<int32_t *>(take((size_t)s.B * (s.pq ? (size_t)s.Hkv * s.L : (size_t)s.H * s.M) * sizeof(int32_t)));
   w.sel_count = reinterpret_cast<int32_t *>(take(256));
   w.delta = reinterpret_cast<float *>(take(2 * units * s.L * sizeof(float)));
-  w.dalpha = reinterpret_cast<double *>(take(units * s.M * sizeof(double)));
+  w.dalpha = reinterpret_cast<double *>(take(units * (size_t)((s.L + 15) / 16 > s.M ? (s.L + 15) / 16 : s.M) * sizeof(double)));
   w.qstats = reinterpret_cast<float4 *>(take(units * (size_t)((s.L + 63) / 64 * 64) * sizeof(float4)));
   w.cmean = reinterpret_cast<double *>(take(units * (size_t)s.Mc * s.D * sizeof(double)));
   w.clive = reinterpret_cast<int32_t *>(take(units * (size_t)s.Mc * sizeof(int32_t)));
@@ -311,6 +311,8 @@ int blossom_attn_fwd(const blossom_params *params, const void *q, const void *k,
     return tc::launch_fwd_tc(s, q, k, v, gate_logits, seq_lens, block_idx, out, out_lt, out_st, lse, ws,
                              st);
   }
+  if (!force_simt() && f32::supported(s, params->dtype))
+    return f32::launch_fwd(s, q, k, v, gate_logits, seq_lens, block_idx, out, out_lt, out_st, lse, st);
   return launch_fwd_simt(s, params->dtype, q, k, v, gate_logits, seq_lens, block_idx, out, out_lt,
                          out_st, lse, ws, st);
 }
@@ -356,6 +358,9 @@ int blossom_attn_bwd(const blossom_params *params, const void *q, const void *k,
       rc = tc::launch_bwd_tc(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout, dq,
                              dk, dv, dgate, ws, st);
     }
+  } else if (!force_simt() && f32::supported(s, params->dtype)) {
+    rc = f32::launch_bwd(s, q, k, v, gate_logits, seq_lens, block_idx, out_lt, out_st, lse, dout, dq, dk, dv, dgate, ws,
+                         st);
   } else {
     rc = launch_bwd_simt(s, params->dtype, q, k, v, gate_logits, seq_lens, block_idx, out_lt,
                          out_st, lse, dout, dq, dk, dv, dgate, ws, st);

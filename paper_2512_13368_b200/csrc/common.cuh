@@ -46,7 +46,7 @@ struct Workspace {
                      //               fp32 stage could not certify
   int32_t *sel_count;// [1]           length of that list
   float *delta;      // [2][B][H][L]  rowsum(G_branch o O_branch) for the backward
-  double *dalpha;    // [B][H][M]     per query block partial of d alpha
+  double *dalpha;    // [B][H][M], [B][H][ceil(L/16)] for the fp32 kernels: partials of d alpha
   float4 *qstats;    // [B][H][ceil(L/64)*64]  16 bytes per query row, laid out per pair of rows as
                      //   {nl_lt(2), -Delta_lt(2)} {nl_st(2), -Delta_st(2)} for the dK/dV kernel
   double *cmean;     // [B][H][Mc][D]  means of the overlapping compression blocks (cmp_l > 0)
@@ -274,6 +274,16 @@ int launch_bwd_short(const Shape &s, const void *q, const void *k, const void *v
                      const Workspace &ws, cudaStream_t st);
 constexpr int kCounterWord = 16;  // word of the status area: CTAs of the short backward that have finished
 }  // namespace sh
+
+namespace f32 {
+// Single-precision inputs: register-tiled products, a warp per 16 rows.
+bool supported(const Shape &s, int dtype);
+int launch_fwd(const Shape &s, const void *q, const void *k, const void *v, const float *gate, const int32_t *seq_lens,
+               const int32_t *idx, void *out, void *out_lt, void *out_st, float *lse, cudaStream_t st);
+int launch_bwd(const Shape &s, const void *q, const void *k, const void *v, const float *gate, const int32_t *seq_lens,
+               const int32_t *idx, const void *out_lt, const void *out_st, const float *lse, const void *dout, void *dq,
+               void *dk, void *dv, float *dgate, const Workspace &ws, cudaStream_t st);
+}  // namespace f32
 
 // BLOSSOM_FORCE_SIMT=1 in the environment routes every call to the fp32 CUDA-core kernels.
 bool force_simt();
