@@ -127,6 +127,30 @@ struct Acc {
         }
     }
   }
+  // += the accumulators the other warps of the tile left in shared memory, and leaving one there
+  __device__ __forceinline__ void put(float *b, int lane) const {
+    float2 *o = reinterpret_cast<float2 *>(b) + lane;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int n = 0; n < D / 16; ++n)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) o[32 * ((i * (D / 16) + n) * 2 + j)] = v[i][n][j];
+  }
+  __device__ __forceinline__ void take(const float *b, int lane) {
+    const float2 *o = reinterpret_cast<const float2 *>(b) + lane;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int n = 0; n < D / 16; ++n)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float2 x = o[32 * ((i * (D / 16) + n) * 2 + j)];
+          v[i][n][j].x += x.x;
+          v[i][n][j].y += x.y;
+        }
+  }
+  static constexpr int kFloats = 16 * D;  // of one accumulator in shared memory
   // rows r0 + gid, r0 + gid + 8 (those < hi) of a tensor
   __device__ __forceinline__ void store(float *base, int64_t sl, int r0, int hi, float f0, float f1, int gid, int tig) const {
 #pragma unroll
@@ -143,29 +167,37 @@ struct Acc {
 };
 
 // The chunks of 16 positions a warp visits, 64 at a time (bit = chunk): sets(w) fills L and S for chunks
-// 64 w ...; next() hands them out in ascending order, -1 at the end.
+// 64 w ...; next() hands out every split-th of them (the sub-th, ...) in ascending order, -1 at the end.
 template <typename F>
 struct Walk {
   F sets;
-  int w, nw, skip;
+  int w, nw, skip, sub, split, count;
   uint64_t L, S, todo;
-  __device__ __forceinline__ Walk(F f, int nw_, int skip_) : sets(f), w(-1), nw(nw_), skip(skip_), L(0), S(0), todo(0) {}
+  __device__ __forceinline__ Walk(F f, int nw_, int skip_, int sub_, int split_)
+      : sets(f), w(-1), nw(nw_), skip(skip_), sub(sub_), split(split_), count(0), L(0), S(0), todo(0) {}
   __device__ __forceinline__ int next(bool *inL, bool *inS) {
-    while (!todo) {
-      if (++w >= nw) return -1;
-      sets(w, L, S);
-      todo = L | S;
-      if (skip >= 0 && (skip >> 6) == w) todo &= ~(1ull << (skip & 63));
+    while (true) {
+      while (!todo) {
+        if (++w >= nw) return -1;
+        sets(w, L, S);
+        todo = L | S;
+        if (skip >= 0 && (skip >> 6) == w) todo &= ~(1ull << (skip & 63));
+      }
+      const int b = __ffsll((long long)todo) - 1;
+      todo &= todo - 1;
+      const bool mine = count == sub;
+      if (++count == split) count = 0;
+      if (!mine) continue;
+      *inL = (L >> b) & 1;
+      *inS = (S >> b) & 1;
+      return 64 * w + b;
     }
-    const int b = __ffsll((long long)todo) - 1;
-    todo &= todo - 1;
-    *inL = (L >> b) & 1;
-    *inS = (S >> b) & 1;
-    return 64 * w + b;
   }
 };
 template <typename F>
-__device__ __forceinline__ Walk<F> make_walk(F f, int nw, int skip) { return Walk<F>(f, nw, skip); }
+__device__ __forceinline__ Walk<F> make_walk(F f, int nw, int skip, int sub, int split) {
+  return Walk<F>(f, nw, skip, sub, split);
+}
 
 // chunk sets of a query tile: the blocks its block selected, the chunks its rows' window touches
 __device__ __forceinline__ void query_sets(const Shape &s, const int32_t *idxrow, int b, int t0, int t_last, int pad0, int w,
@@ -220,14 +252,15 @@ __global__ void __launch_bounds__(128) fwd_f32_kernel(Shape s, const float *__re
                                                       const float *__restrict__ v, const float *__restrict__ gate,
                                                       const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ idx,
                                                       float *__restrict__ out, float *__restrict__ out_lt,
-                                                      float *__restrict__ out_st, float *__restrict__ lse) {
+                                                      float *__restrict__ out_st, float *__restrict__ lse, int split) {
   grid_chain_enter();
   extern __shared__ __align__(16) float fsm[];
   constexpr int T = Geo<D>::kTile, kWarp = 5 * T + 2 * 16 * kPP;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   float *qt = fsm + warp * kWarp, *kv = qt + T, *pl = kv + 4 * T, *ps = pl + 16 * kPP;  // kv: [2 stages][K, V]
   const int units = s.B * s.H, ntile = (s.L + 15) >> 4;
-  const int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int sub = split > 1 ? warp : 0;  // with split > 1 the CTA's warps share one tile's chunks
+  const int64_t task = split > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (task >= (int64_t)units * ntile) return;
   const int u = (int)(task % units), t0 = (ntile - 1 - (int)(task / units)) * 16;  // late tiles first
   const int n = u / s.H, h = u % s.H, hk = h / s.G;
@@ -262,7 +295,7 @@ __global__ void __launch_bounds__(128) fwd_f32_kernel(Shape s, const float *__re
       inL = (L >> (own & 63)) & 1;
       inS = (S >> (own & 63)) & 1;
     }
-    auto walk = make_walk(sets, nw, own);
+    auto walk = make_walk(sets, nw, own, sub, split);
     int c = own, st = 0;
     bool first = true;
 #pragma unroll 1
@@ -292,6 +325,10 @@ __global__ void __launch_bounds__(128) fwd_f32_kernel(Shape s, const float *__re
           m[i] = x > -INFINITY ? x : 0.f;
         }
         first = false;
+        if (sub) {  // (every warp of the tile needs the reference; the first one adds the chunk)
+          inL = inS = false;
+          bL[0] = bL[1] = bS[0] = bS[1] = 0u;
+        }
       }
       float pL[2][4], pS[2][4];
 #pragma unroll
@@ -316,6 +353,23 @@ __global__ void __launch_bounds__(128) fwd_f32_kernel(Shape s, const float *__re
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) l[i] = quad_sum(l[i]);
+    if (split > 1) {
+      constexpr int F = Acc<D>::kFloats;
+      if (sub) {
+        aL.put(kv, lane);
+        aS.put(kv + F, lane);
+        *reinterpret_cast<float4 *>(kv + 2 * F + 4 * lane) = make_float4(l[0], l[1], l[2], l[3]);
+      }
+      __syncthreads();
+      if (sub) return;
+      for (int w = 1; w < split; ++w) {  // in warp order
+        const float *o = kv + w * kWarp;
+        aL.take(o, lane);
+        aS.take(o + F, lane);
+        const float4 x = *reinterpret_cast<const float4 *>(o + 2 * F + 4 * lane);
+        l[0] += x.x; l[1] += x.y; l[2] += x.z; l[3] += x.w;
+      }
+    }
     mL[0] = mS[0] = m[0];
     mL[1] = mS[1] = m[1];
     bool bad = false;
@@ -384,6 +438,7 @@ __global__ void __launch_bounds__(128) fwd_f32_kernel(Shape s, const float *__re
       }
     }
   }
+  if (sub) return;  // (a tile of padding)
   // normalise, mix (Eq. 19), store; padded rows are zeros
   float f[4];
 #pragma unroll
@@ -428,14 +483,15 @@ __global__ void __launch_bounds__(128) dq_f32_kernel(Shape s, const float *__res
                                                      const float *__restrict__ out_lt, const float *__restrict__ out_st,
                                                      const float *__restrict__ lse, const float *__restrict__ dout,
                                                      float *__restrict__ dq, float4 *__restrict__ records,
-                                                     double *__restrict__ dalpha_part) {
+                                                     double *__restrict__ dalpha_part, int split) {
   grid_chain_enter();
   extern __shared__ __align__(16) float fsm[];
   constexpr int T = Geo<D>::kTile, kWarp = 6 * T + 16 * kPP;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   float *qt = fsm + warp * kWarp, *gt = qt + T, *kv = gt + T, *pt = kv + 4 * T;
   const int units = s.B * s.H, ntile = (s.L + 15) >> 4;
-  const int64_t task = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  const int sub = split > 1 ? warp : 0;  // with split > 1 the CTA's warps share one tile's chunks
+  const int64_t task = split > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (task >= (int64_t)units * ntile) return;
   const int u = (int)(task % units), tile = ntile - 1 - (int)(task / units), t0 = tile * 16;
   const int n = u / s.H, h = u % s.H, hk = h / s.G, Lpad = (s.L + 63) / 64 * 64;
@@ -458,7 +514,7 @@ __global__ void __launch_bounds__(128) dq_f32_kernel(Shape s, const float *__res
     fetch<D>(qt, q + off, s.sl, t0, pad0, s.L, lane);
     fetch<D>(gt, dout + off, s.sl, t0, pad0, s.L, lane);
     cp_async_commit();
-    auto walk = make_walk(sets, (ntile + 63) >> 6, -1);
+    auto walk = make_walk(sets, (ntile + 63) >> 6, -1, sub, split);
     bool inL = false, inS = false;
     int c = walk.next(&inL, &inS), st = 0;
     if (c >= 0) load(c, 0);
@@ -481,7 +537,7 @@ __global__ void __launch_bounds__(128) dq_f32_kernel(Shape s, const float *__res
       const int64_t row = (int64_t)u * s.L + (ok ? t : t_last), BHL = (int64_t)s.B * s.H * s.L;
       float4 rec = make_float4(lse[row] * kLog2e, lse[BHL + row] * kLog2e, alpha * a, beta * c2);
       if (!ok) rec = make_float4(0.f, 0.f, 0.f, 0.f);
-      if ((lane & 1) == 0 && t < Lpad) records[(int64_t)u * Lpad + t] = rec;
+      if ((lane & 1) == 0 && t < Lpad && !sub) records[(int64_t)u * Lpad + t] = rec;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int src = 2 * (gid + 8 * i);
@@ -526,9 +582,23 @@ __global__ void __launch_bounds__(128) dq_f32_kernel(Shape s, const float *__res
       inS = nS;
       st ^= 1;
     }
+    if (split > 1) {
+      if (sub) {
+        acc.put(kv, lane);
+        kv[Acc<D>::kFloats + lane] = dal;
+      }
+      __syncthreads();
+      if (!sub)
+        for (int w = 1; w < split; ++w) {
+          const float *o = kv + w * kWarp;
+          acc.take(o, lane);
+          dal += o[Acc<D>::kFloats + lane];
+        }
+    }
   } else if (lane < 16 && t0 + lane < Lpad) {
     records[(int64_t)u * Lpad + t0 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  if (sub) return;
   acc.store(dq + off, s.sl, t0, s.L, s.scale, s.scale, gid, tig);
   double a = (double)dal;
 #pragma unroll
@@ -544,7 +614,8 @@ __global__ void __launch_bounds__(128) dkdv_f32_kernel(Shape s, const float *__r
                                                        const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ idx,
                                                        const float4 *__restrict__ records, const float *__restrict__ dout,
                                                        float *__restrict__ dk, float *__restrict__ dv,
-                                                       const double *__restrict__ dalpha_part, float *__restrict__ dgate) {
+                                                       const double *__restrict__ dalpha_part, float *__restrict__ dgate,
+                                                       int split) {
   grid_chain_enter();
   extern __shared__ __align__(16) float fsm[];
   constexpr int T = Geo<D>::kTile, kStage = 2 * T + 64, kWarp = 2 * T + 2 * kStage + 2 * 16 * kPP;
@@ -569,7 +640,8 @@ __global__ void __launch_bounds__(128) dkdv_f32_kernel(Shape s, const float *__r
   float *kt = fsm + warp * kWarp, *vt = kt + T, *stages = vt + T, *wt = stages + 2 * kStage, *dt = wt + 16 * kPP;
   const bool causal = PLAIN || s.causal;
   const int units = s.B * s.Hkv;
-  const int64_t task = (int64_t)(blockIdx.x - 1) * nwarp + warp;
+  const int sub = split > 1 ? warp : 0;  // with split > 1 the CTA's warps share one tile's chunks
+  const int64_t task = split > 1 ? (int64_t)blockIdx.x - 1 : (int64_t)(blockIdx.x - 1) * nwarp + warp;
   if (task >= (int64_t)units * ntile) return;
   const int uk = (int)(task % units), p0 = (int)(task / units) * 16;  // early keys (the most visitors) first
   const int n = uk / s.Hkv, hk = uk % s.Hkv, Lpad = (s.L + 63) / 64 * 64;
@@ -620,7 +692,7 @@ __global__ void __launch_bounds__(128) dkdv_f32_kernel(Shape s, const float *__r
         if (lane < 16) cp_async16(smem_addr(x + 2 * T + 4 * lane), records + u * Lpad + c * 16 + lane);
         cp_async_commit();
       };
-      auto walk = make_walk(sets, (ntile + 63) >> 6, -1);
+      auto walk = make_walk(sets, (ntile + 63) >> 6, -1, sub, split);
       bool inL = false, inS = false;
       int c = walk.next(&inL, &inS), st = 0;
       if (c >= 0) load(c, 0);
@@ -681,13 +753,30 @@ __global__ void __launch_bounds__(128) dkdv_f32_kernel(Shape s, const float *__r
       }
     }
     cp_async_wait<0>();
+    if (split > 1) {
+      if (sub) {
+        ak.put(stages, lane);
+        av.put(stages + Acc<D>::kFloats, lane);
+      }
+      __syncthreads();
+      if (!sub)
+        for (int w = 1; w < split; ++w) {
+          const float *o = stages + w * kWarp;
+          ak.take(o, lane);
+          av.take(o + Acc<D>::kFloats, lane);
+        }
+    }
   }
+  if (sub) return;
   av.store(dv + koff, s.ksl, p0, s.L, 1.f, 1.f, gid, tig);
   ak.store(dk + koff, s.ksl, p0, s.L, s.scale, s.scale, gid, tig);
 }
 
-// Warps per CTA: four, or one while that leaves SMs without work.
-int warps_per_cta(int64_t tasks) { return tasks < 148 * 8 ? 1 : 4; }
+// CTAs are four warps.  While the tiles leave SMs without work a CTA's warps share one tile's chunks
+// instead of taking a tile each: the tile with the most chunks is then the kernel's time.
+constexpr int kCtaWarps = 4;
+int chunk_split(int64_t tasks) { return tasks <= 148 * 6 ? kCtaWarps : 1; }
+unsigned ctas(int64_t tasks, int split) { return (unsigned)(split > 1 ? tasks : (tasks + kCtaWarps - 1) / kCtaWarps); }
 
 template <typename K>
 bool allow(K kern, size_t smem) {
@@ -701,12 +790,12 @@ int launch_fwd_t(const Shape &s, const float *q, const float *k, const float *v,
   const bool plain = s.causal && s.stis_mode == 0;
   auto kern = plain ? fwd_f32_kernel<D, true> : fwd_f32_kernel<D, false>;
   const int64_t tasks = (int64_t)s.B * s.H * ((s.L + 15) / 16);
-  const int wpc = warps_per_cta(tasks);
-  const size_t smem = (size_t)wpc * (5 * Geo<D>::kTile + 2 * 16 * kPP) * sizeof(float);
+  const int split = chunk_split(tasks);
+  const size_t smem = (size_t)kCtaWarps * (5 * Geo<D>::kTile + 2 * 16 * kPP) * sizeof(float);
   if (!allow(kern, smem)) return BLOSSOM_ERR_CUDA;
   LaunchScope ls(K_FWD_SIMT, st);
-  return launch_chained(kern, dim3((unsigned)((tasks + wpc - 1) / wpc)), dim3(32 * wpc), smem, st, s, q, k, v, gate, seq_lens,
-                        idx, out, out_lt, out_st, lse) == cudaSuccess
+  return launch_chained(kern, dim3(ctas(tasks, split)), dim3(32 * kCtaWarps), smem, st, s, q, k, v, gate, seq_lens, idx, out,
+                        out_lt, out_st, lse, split) == cudaSuccess
              ? BLOSSOM_OK
              : BLOSSOM_ERR_CUDA;
 }
@@ -720,20 +809,20 @@ int launch_bwd_t(const Shape &s, const float *q, const float *k, const float *v,
   auto kk = plain ? dkdv_f32_kernel<D, true> : dkdv_f32_kernel<D, false>;
   const int ntile = (s.L + 15) / 16;
   const int64_t tq = (int64_t)s.B * s.H * ntile, tk = (int64_t)s.B * s.Hkv * ntile;
-  const int wq = warps_per_cta(tq), wk = warps_per_cta(tk);
+  const int wq = chunk_split(tq), wk = chunk_split(tk);
   constexpr int T = Geo<D>::kTile;
-  const size_t sq = (size_t)wq * (6 * T + 16 * kPP) * sizeof(float);
-  const size_t sk = (size_t)wk * (2 * T + 2 * (2 * T + 64) + 2 * 16 * kPP) * sizeof(float);
+  const size_t sq = (size_t)kCtaWarps * (6 * T + 16 * kPP) * sizeof(float);
+  const size_t sk = (size_t)kCtaWarps * (2 * T + 2 * (2 * T + 64) + 2 * 16 * kPP) * sizeof(float);
   if (!allow(kq, sq) || !allow(kk, sk)) return BLOSSOM_ERR_CUDA;
   {
     LaunchScope ls(K_BWD_DQ_SIMT, st);
-    if (launch_chained(kq, dim3((unsigned)((tq + wq - 1) / wq)), dim3(32 * wq), sq, st, s, q, k, v, gate, seq_lens, idx, out_lt,
-                       out_st, lse, dout, dq, ws.qstats, ws.dalpha) != cudaSuccess)
+    if (launch_chained(kq, dim3(ctas(tq, wq)), dim3(32 * kCtaWarps), sq, st, s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse,
+                       dout, dq, ws.qstats, ws.dalpha, wq) != cudaSuccess)
       return BLOSSOM_ERR_CUDA;
   }
   LaunchScope ls(K_BWD_DKDV_SIMT, st);
-  return launch_chained(kk, dim3((unsigned)((tk + wk - 1) / wk) + 1), dim3(32 * wk), sk, st, s, q, k, v, gate, seq_lens, idx,
-                        (const float4 *)ws.qstats, dout, dk, dv, (const double *)ws.dalpha, dgate) == cudaSuccess
+  return launch_chained(kk, dim3(ctas(tk, wk) + 1), dim3(32 * kCtaWarps), sk, st, s, q, k, v, gate, seq_lens, idx,
+                        (const float4 *)ws.qstats, dout, dk, dv, (const double *)ws.dalpha, dgate, wk) == cudaSuccess
              ? BLOSSOM_OK
              : BLOSSOM_ERR_CUDA;
 }
