@@ -577,6 +577,7 @@ __global__ void __launch_bounds__(256) gate_param_grad_kernel(Shape s, const dou
   if (w >= s.H * GW) return;
   const int h = w / GW, d = w % GW, n_entries = s.B * s.M;
   double a = 0.0;
+#pragma unroll 16
   for (int e = lane; e < n_entries; e += 32) {
     const int n = e / s.M, qb = e % s.M;
     a += part[(((int64_t)n * s.H + h) * s.M + qb) * GW + d];

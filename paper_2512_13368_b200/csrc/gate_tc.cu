@@ -221,14 +221,12 @@ struct AddTensor {
 };
 __global__ void __launch_bounds__(256) grad_add_kernel(int B, int L, int D, AddTensor x, AddTensor y, AddTensor z) {
   grid_chain_enter();
-  const int cpr = D / 8;
-  const int64_t per = (int64_t)B * L * cpr, nx = per * x.heads, ny = per * y.heads, total = nx + 2 * ny;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+  // (32-bit counts: the tensors have fewer than 2^32 pieces of 16 bytes)
+  const uint32_t cpr = D / 8, per = (uint32_t)B * L * cpr, nx = per * x.heads, ny = per * y.heads, total = nx + 2 * ny;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const AddTensor &w = i < nx ? x : i < nx + ny ? y : z;
-    const int64_t e = i < nx ? i : i < nx + ny ? i - nx : i - nx - ny;
-    const int ch = (int)(e % cpr);
-    const int64_t row = e / cpr;
-    const int t = (int)(row % L), h = (int)((row / L) % w.heads), n = (int)(row / ((int64_t)L * w.heads));
+    const uint32_t e = i < nx ? i : i < nx + ny ? i - nx : i - nx - ny;
+    const uint32_t ch = e % cpr, row = e / cpr, t = row % L, uh = row / L, h = uh % w.heads, n = uh / w.heads;
     const int64_t off = (int64_t)n * w.sb + (int64_t)h * w.sh + (int64_t)t * w.sl + ch * 8;
     float a[8], b[8];
     unpack8(*reinterpret_cast<const uint4 *>(w.dst + off), a);

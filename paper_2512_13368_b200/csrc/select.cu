@@ -1092,8 +1092,8 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   // First stage: single precision with a bound; what it cannot certify goes on the work list.
   RowsGeom rg;
   size_t rsm = 0;
-  const bool rows = g.n > 0 && rows_geom(sh, g, &rg, &rsm);
   const int dtype = sizeof(T) == 2 ? BLOSSOM_DTYPE_BF16 : BLOSSOM_DTYPE_FP32;
+  const bool rows = g.n > 0 && rows_geom(sh, g, dtype, &rg, &rsm);
   if (sh.pq) {  // one selection per query position: block_idx is [B][Hkv][L][top_k]
     if (!rows && !g.plain && g.n > 128) return BLOSSOM_ERR_UNSUPPORTED;  // (see make_shape)
     const bool listed = rows && !exact_select_only();

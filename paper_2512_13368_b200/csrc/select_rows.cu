@@ -1,24 +1,27 @@
 // Certified single-precision scoring, a lane per query row: first stage of the selection (see
 // select.cu for the stages, the scored blocks and the promise) for up to 128 scored blocks.
 //
-// A CTA of four warps takes 128 consecutive positions of a (batch, key/value head); a lane owns a
-// row's logits, its norm, its softmax statistics and (in the per-position mode) its whole choice; rows of q
-// are in registers (two lanes share the products of two rows) and the candidates' means are broadcast
-// from shared memory, so that nothing of a row has to be staged.  The exponentials are taken relative to the bound
-// scale |q| max|mean| of the row's logits instead of their maximum, which needs no pass of its own; a row
-// for which that bound is so loose that its sum nearly vanishes is left to double precision.
-// The register-blocked product of 128 x 64 tiles that this replaces (it remains for more than 128
-// scored blocks) read every query row into shared memory as fp32 and computed 64 candidates whether
-// there were 64 or 5: 123 us at B 128, H 4, L 1024 (32 blocks), 149 us at B 16, H 8, L 4096 (64
-// blocks); 80 us (double precision throughout) without the causal mask at B 16, H 4, L 777, 122 us per
-// position at B 8, 8 heads on 2, L 1500.
+// A CTA of four warps takes 128 consecutive positions of a (batch, key/value head).  The logits of a warp's
+// rows come from warp-level matrix products for bf16 inputs, the means split into three bf16 values whose
+// sum they are exactly (a lane holding its row in registers and the means broadcast from shared memory took
+// 100 us at B 16, H 8, L 4096, 68 at B 128, H 4, L 1024; the shared-memory pipe bound it), and from
+// packed multiply-adds for fp32.  The exponentials, relative to the bound scale |q| max|mean| of the row's
+// logits instead of their maximum (which needs no pass of its own; a row for which that bound is so loose
+// that its sum nearly vanishes is left to double precision), go through a table in shared memory: a lane
+// per column sums them over the rows of a block, or, per position, a lane per row makes its row's choice.
+// The register-blocked product of 128 x 64 tiles in select.cu (more than 128 scored blocks) stages every
+// query row as fp32 and computes 64 candidates whether there are 64 or 5: 149 and 123 us at these sizes.
 //
-// Error bound, as in select.cu: with u = 2^-24 every logit is within E = (D + 4) u bound of its exact
-// value (bound = scale max|q| max|mean|); the exponentials add 2^-21 and 2^-22 per unit of logit range;
-// every addition of the normaliser and of the column sums, every head, every term of Eq. 11 one u each,
-// with a margin of 40.
-#include "select_geom.cuh"
+// Error bound, as in select.cu: with u = 2^-24 every logit is within E of its exact value, bound = scale
+// max|q| max|mean|: (D + 4) u bound for multiply-adds.  For the matrix products PTX guarantees exact
+// products and accumulation in at least single precision with unspecified rounding, so 2 u per addition; the
+// leading parts are accumulated 16 dimensions at a time from zero (16 additions, 32 u) and the D / 16
+// results added up, the smaller ones, at 2^-8 of their size, in one go (2 D additions): (32 + D / 16 + 0.1 D
+// + 6) u bound.  The exponentials add 2^-21 and 2^-22 per unit of logit range; sums of non-negative
+// terms add one u per addition that a term goes through (the normaliser, 16 rows, the 16-row groups of a
+// block, the heads, Eq. 11), with a margin of 40.
 #include "select_rows.cuh"
+#include "short_common.cuh"
 
 namespace blossom {
 namespace {
@@ -66,18 +69,22 @@ __device__ __forceinline__ float square(const float2 (&q)[N]) {
 
 // PQ: one selection per query position.
 template <typename T, int D, bool PQ>
-__global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_kernel(
     Shape sh, SelGeom g, RowsGeom rg, const T *__restrict__ q, const float *__restrict__ mean32,
     const float *__restrict__ norm, const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx,
     int32_t *__restrict__ worklist, int32_t *__restrict__ work_count) {
   grid_chain_enter();
-  constexpr int P = D + 4;  // pitch of the means (floats)
-  extern __shared__ __align__(16) float fsm[];
-  __shared__ float kn_w[kWarps], qn_w[kWarps], inv_s[kWarps][32], bound_s[8][2];
-  float *ms = fsm;                                     // [rg.cols][P] candidate means, candidate cmin first
+  constexpr bool kMma = sizeof(T) == 2;  // bf16: products on the warp-level matrix pipe
+  constexpr int P = D + 4;               // pitch of the means (floats; the fp32 form)
+  // rows of a warp that its table holds at a time
+  constexpr int kTab = kMma && !PQ ? 16 : 32;
+  extern __shared__ __align__(128) float fsm[];
+  __shared__ float kn_w[kWarps], inv_s[kWarps][32], rowq_s[kWarps][32], bound_s[8][2];
+  // candidate means, candidate cmin first: [rg.cols][P] floats, or bf16 tiles [hi, mid, lo][rg.cols][D]
+  float *ms = fsm, *tab = fsm + rg.means;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float *et = ms + rg.cols * P + warp * 32 * rg.pitch;  // [32][pitch] this warp's exponentials / scores
-  float *pt = et + kWarps * 32 * rg.pitch;              // (PQ with grouped heads) [32][pitch] probabilities summed over heads
+  float *et = tab + warp * kTab * rg.pitch;  // [kTab][pitch] this warp's exponentials / scores
+  float *pt = et + kWarps * 32 * rg.pitch;   // (PQ with grouped heads) [32][pitch] probabilities summed over heads
   const int M = sh.M, Bk = sh.Bk;
   const int ntiles = (sh.L + kRows - 1) / kRows, nU = sh.B * sh.Hkv;
   // late tiles have the most candidates: they go first (tile-major)
@@ -115,8 +122,34 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
 
   if (need) {
     const float *kb = mean32 + ((int64_t)u * g.n + cmin) * D;
-    for (int i = tid; i < ncol * (D / 4); i += kThreads)
-      *reinterpret_cast<float4 *>(ms + (i / (D / 4)) * P + (i % (D / 4)) * 4) = reinterpret_cast<const float4 *>(kb)[i];
+    if constexpr (kMma) {
+      // a mean of 24 significant bits as the exact sum of three bf16 values
+      uint8_t *tiles = reinterpret_cast<uint8_t *>(ms);
+      for (int i = tid; i < rg.cols * (D / 8); i += kThreads) {
+        const int c = i / (D / 8), ch = i % (D / 8);
+        float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (c < ncol) {
+          const float4 a = reinterpret_cast<const float4 *>(kb)[2 * i], e = reinterpret_cast<const float4 *>(kb)[2 * i + 1];
+          x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = e.x; x[5] = e.y; x[6] = e.z; x[7] = e.w;
+        }
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            w[e] = sh::pack2(x[2 * e], x[2 * e + 1]);
+            x[2 * e] -= sh::lo_bf(w[e]);
+            x[2 * e + 1] -= sh::hi_bf(w[e]);
+          }
+          *reinterpret_cast<uint4 *>(tiles + part * rg.cols * D * 2 + sh::tile_off<D>(c, ch)) =
+              make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      }
+      rowq_s[warp][lane] = 0.f;
+    } else {
+      for (int i = tid; i < ncol * (D / 4); i += kThreads)
+        *reinterpret_cast<float4 *>(ms + (i / (D / 4)) * P + (i % (D / 4)) * 4) = reinterpret_cast<const float4 *>(kb)[i];
+    }
     for (int c = tid; c < ncol; c += kThreads) kn = fmaxf(kn, norm[(int64_t)u * g.n + cmin + c]);
     kn = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(kn)));  // (non-negative floats order like integers)
     if (lane == 0) kn_w[warp] = kn;
@@ -128,8 +161,100 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
     const float sc2 = sh.scale * 1.4426950408889634f;
     float *er = et + lane * rg.pitch;
     const bool up = lane >= 16;
+    // column sums of 16 rows' probabilities (tables: exponentials and the rows' reciprocal normalisers)
+    auto sums = [&](int half, const float *e16, const float *inv16) {
+#pragma unroll 1
+      for (int x = 0; x < 4; ++x) {
+        const int c = lane + 32 * x;
+        if (32 * x >= nc_warp) break;
+        float a = 0.f;
+        if (c < nc_warp)
+#pragma unroll 8
+          for (int r = 0; r < 16; ++r) a = fmaf(e16[r * rg.pitch + c], inv16[r], a);
+        // (half and x are warp-uniform; the registers are selected by constants)
+        float(&cs)[4] = half ? colsum[1] : colsum[0];
+        if (x == 0) cs[0] += a;
+        else if (x == 1) cs[1] += a;
+        else if (x == 2) cs[2] += a;
+        else cs[3] += a;
+      }
+    };
 #pragma unroll 1
     for (int hg = 0; hg < sh.G; ++hg) {  // the heads of the group in ascending order (Eq. 12)
+      if constexpr (kMma) {
+        const int gid = lane >> 2, tig = lane & 3;
+        const uint32_t tiles = sh::smem_addr(ms) + sh::lane_off_nt<D>(lane), part_bytes = (uint32_t)rg.cols * D * 2;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {  // 16 rows at a time
+          const int tm = row0 + warp * 32 + 16 * mt;
+          uint32_t qa[D / 16][4];
+          sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg, 0), sh.sl, tm, pad0, sh.L, lane, qa);
+          float ref[2] = {0.f, 0.f}, den[2] = {0.f, 0.f}, qh[2];
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              ref[e & 1] = fmaf(sh::lo_bf(qa[k][e]), sh::lo_bf(qa[k][e]), ref[e & 1]);
+              ref[e & 1] = fmaf(sh::hi_bf(qa[k][e]), sh::hi_bf(qa[k][e]), ref[e & 1]);
+            }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            qh[i] = sqrtf(sh::quad_sum(ref[i])) * 1.0001f;
+            ref[i] = sc2 * qh[i] * kn;  // >= every logit of the row (log2 units)
+          }
+          const int t0 = tm + gid;
+          const bool ok0 = t0 >= pad0 && t0 < sh.L, ok1 = t0 + 8 >= pad0 && t0 + 8 < sh.L;
+          int ncm[2], skip[2];  // (blocks of 8: rows gid and gid + 8 lie in different ones)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int bm = min(t0 + 8 * i, sh.L - 1) / Bk;
+            ncm[i] = max(0, (causal ? n_candidates(sh, g, bm) : g.n) - cmin);
+            skip[i] = own ? bm - cmin : -1;
+          }
+          float *e0 = et + ((PQ ? 16 * mt : 0) + gid) * rg.pitch + 2 * tig, *e1 = e0 + 8 * rg.pitch;
+#pragma unroll 1
+          for (int c = 0; c < nc_warp; c += 16) {
+            const uint32_t chunk = tiles + c * D * 2;
+            float z[2][4];
+            sh::product_nt<D>(qa, chunk + 2 * part_bytes, z);       // the small parts first
+            sh::product_nt_add<D>(qa, chunk + part_bytes, z);
+            sh::product_nt_steps<D>(qa, chunk, z);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                const int cc = c + 8 * nt + 2 * tig + j;
+                z[nt][j] = ok0 && cc < ncm[0] && cc != skip[0] ? exp2f(fmaf(z[nt][j], sc2, -ref[0])) : 0.f;
+                z[nt][2 + j] = ok1 && cc < ncm[1] && cc != skip[1] ? exp2f(fmaf(z[nt][2 + j], sc2, -ref[1])) : 0.f;
+                e0[c + 8 * nt + j] = z[nt][j];
+                e1[c + 8 * nt + j] = z[nt][2 + j];
+              }
+            den[0] += (z[0][0] + z[0][1]) + (z[1][0] + z[1][1]);
+            den[1] += (z[0][2] + z[0][3]) + (z[1][2] + z[1][3]);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            den[i] = sh::quad_sum(den[i]);
+            if (tig == 0) {
+              const int r = 16 * mt + gid + 8 * i;
+              const bool bad = (i ? ok1 : ok0) && ncm[i] > own && !(den[i] > 1e-30f);  // the reference is too far away
+              inv_s[warp][r] = den[i] > 0.f ? 1.f / den[i] : 0.f;
+              rowq_s[warp][r] = fmaxf(rowq_s[warp][r], bad ? INFINITY : qh[i]);
+            }
+          }
+          __syncwarp();
+          if (!PQ) {
+            sums(mt, et, inv_s[warp] + 16 * mt);
+            __syncwarp();
+          }
+        }
+        if (PQ && sh.G > 1) {
+          float *pr = pt + lane * rg.pitch;
+          const float inv = inv_s[warp][lane];
+          for (int c = 0; c < nc_warp; ++c) pr[c] = hg == 0 ? er[c] * inv : fmaf(er[c], inv, pr[c]);
+          __syncwarp();
+        }
+      } else {
       // The products are shared by two lanes: lanes l and l + 16 hold the lower and the upper half of the
       // dimensions of rows l and l + 16, and exchange one partial sum per candidate, so that lane l ends up
       // with row l.  A broadcast load then feeds two rows (alone it took more cycles of the shared-memory
@@ -178,31 +303,22 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
       } else {
         inv_s[warp][lane] = inv;
         __syncwarp();
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-#pragma unroll 1
-          for (int x = 0; x < 4; ++x) {
-            const int c = lane + 32 * x;
-            if (32 * x >= nc_warp) break;
-            float a = 0.f;
-            if (c < nc_warp)
-#pragma unroll 8
-              for (int r = 0; r < 16; ++r) a = fmaf(et[(16 * half + r) * rg.pitch + c], inv_s[warp][16 * half + r], a);
-            // (x is a warp-uniform loop index; the registers are selected by constants)
-            if (x == 0) colsum[half][0] += a;
-            else if (x == 1) colsum[half][1] += a;
-            else if (x == 2) colsum[half][2] += a;
-            else colsum[half][3] += a;
-          }
-        }
+        sums(0, et, inv_s[warp]);
+        sums(1, et + 16 * rg.pitch, inv_s[warp] + 16);
         __syncwarp();
       }
+      }
+    }
+    if constexpr (kMma) {
+      qn = rowq_s[warp][lane];
+      loose = qn == INFINITY;
     }
   }
   const float uu = 5.9604645e-8f, bound0 = sh.scale * kn;
-  // relative distance of a score from its exact value, for query norms up to qmax and nsum additions
+  // relative distance of a score from its exact value, for query norms up to qmax and nsum additions in a row
+  const auto den_adds = [](int cols) { return kMma ? cols / 16 + 6 : cols / 2 + 2; };
   auto error = [&](float qmax, float nsum) {
-    const float bound = bound0 * qmax, E = (float)(D + 4) * uu * bound * 1.01f;
+    const float bound = bound0 * qmax, E = (kMma ? 32.f + 0.1f * D + (float)(D / 16) + 6.f : (float)(D + 4)) * uu * bound * 1.01f;
     return 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f + (nsum + 2.f * (float)sh.G + (float)(g.rs * g.rl) + 40.f) * uu;
   };
 
@@ -260,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
             else taken[3] |= bit;
           }
         }
-        certain = !rg.exact && !loose && (kept - dropped) > error(qn, (float)nc) * (kept + dropped) * 1.001f;
+        certain = !rg.exact && !loose && (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f;
       }
       if (certain) {
         int pos = 0;
@@ -279,10 +395,10 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
   // ---- per query block: column sums of its rows, Eq. 11, Eq. 13 and the certificate ----
   // Sc[i][cols]: the tables are free now; block i's rows are 16-row groups i Bk / 16 ...
   __syncthreads();
-  float *part = ms + rg.cols * P;            // [8 groups of 16 rows][128]
-  float *Sc = part + 8 * 128;                // [4 warps][128]
-  float *Sm = Sc + kWarps * 128;             // [4 warps][128] selection-block scores
-  uint8_t *taken = reinterpret_cast<uint8_t *>(Sm + kWarps * 128);  // [4 warps][128]
+  float *part = tab;                         // [8 groups of 16 rows][128]
+  float *Sc = part + 8 * 128;                // [4 warps][132]
+  float *Sm = Sc + kWarps * 132;             // [4 warps][132] selection-block scores
+  uint8_t *taken = reinterpret_cast<uint8_t *>(Sm + kWarps * 132);  // [4 warps][128]
 #pragma unroll
   for (int half = 0; half < 2; ++half)
 #pragma unroll
@@ -316,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
     } else if (live_cands(bb) == 0) {
       for (int j = jmin + lane; j < hi; j += 32) tk[j] = j - jmin < want ? 1 : 0;
     } else {
-      float *S = Sc + warp * 128, qmax = 0.f;
+      float *S = Sc + warp * 132, qmax = 0.f;
       for (int c = lane; c < ncb - cmin; c += 32) {
         float a = 0.f;
         for (int r = 0; r < gpb; ++r) a += part[(i * gpb + r) * 128 + c];
@@ -325,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
       for (int r = 0; r < gpb; ++r) qmax = fmaxf(qmax, bound_s[i * gpb + r][0]);
       __syncwarp();
       if (!g.plain) {
-        float *o = Sm + warp * 128;
+        float *o = Sm + warp * 132;
         for (int j = jmin + lane; j < hi; j += 32) {
           float a = 0.f;
           for (int m = 0; m < g.rs; ++m)
@@ -341,13 +457,21 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
       // by rank: block j is kept iff fewer than `want` others beat it (ties to the lower index)
       const int ns = hi - jmin, ob = own ? bb - jmin : -1;
       float kept = -1.f, dropped = -1.f;
+      if (lane < 4) S[ns + lane] = -1.f;
+      if (lane == 0 && ob >= 0) S[ob] = -1.f;
+      __syncwarp();
       for (int j = lane; j < ns; j += 32) {
         const float sj = S[j];
         int rank = 0;
-#pragma unroll 4
-        for (int x = 0; x < ns; ++x) {
-          const float sx = S[x];
-          rank += x != ob && (sx > sj || (sx == sj && x < j)) ? 1 : 0;
+        // (non-negative floats order like integers; the own block, -1, beats nobody; four at a time, the
+        // scores padded with -1)
+        const int kj = __float_as_int(sj);
+        for (int x = 0; x < ns; x += 4) {
+          const int4 k4 = *reinterpret_cast<const int4 *>(S + x);
+          rank += k4.x > kj || (k4.x == kj && x < j) ? 1 : 0;
+          rank += k4.y > kj || (k4.y == kj && x + 1 < j) ? 1 : 0;
+          rank += k4.z > kj || (k4.z == kj && x + 2 < j) ? 1 : 0;
+          rank += k4.w > kj || (k4.w == kj && x + 3 < j) ? 1 : 0;
         }
         tk[jmin + j] = j != ob && rank < want ? 1 : 0;
         if (j != ob && rank == want - 1) kept = sj;
@@ -356,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
       // (scores are non-negative: exactly one lane holds each)
       kept = __uint_as_float(__reduce_max_sync(0xffffffffu, kept < 0.f ? 0u : __float_as_uint(kept)));
       dropped = __uint_as_float(__reduce_max_sync(0xffffffffu, dropped < 0.f ? 0u : __float_as_uint(dropped)));
-      const float R = error(qmax, (float)(ncb - cmin) + (float)Bk * (float)sh.G);
+      const float R = error(qmax, (float)(den_adds(ncb - cmin) + 16 + gpb));
       certain = !rg.exact && (kept - dropped) > R * (kept + dropped) * 1.001f;  // (false for an infinite qmax)
     }
     if (own && lane == 0) tk[bb] = 1;
@@ -383,15 +507,17 @@ __global__ void __launch_bounds__(kThreads, 4) score_rows_kernel(
 
 }  // namespace
 
-bool rows_geom(const Shape &sh, const SelGeom &g, RowsGeom *rg, size_t *smem) {
+bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_t *smem) {
   if (g.n > 128 || sh.M > 128) return false;
-  rg->cols = (g.n + 1) / 2 * 2 + 2;
+  const bool mma = dtype == BLOSSOM_DTYPE_BF16;
+  rg->cols = mma ? (g.n + 15) / 16 * 16 : (g.n + 1) / 2 * 2 + 2;
+  rg->means = mma ? 3 * rg->cols * sh.D / 2 : rg->cols * (sh.D + 4);  // (a multiple of four)
   const int wide = sh.M > rg->cols ? sh.M : rg->cols;  // (per position the table also holds the scores of the selection blocks)
   rg->pitch = (sh.pq ? wide : rg->cols) | 1;
   const bool two = sh.pq && (sh.G > 1 || !g.plain);
-  const size_t tables = (size_t)(two ? 2 : 1) * kWarps * 32 * rg->pitch * 4;
-  const size_t tail = (size_t)(8 * 128 + 2 * kWarps * 128) * 4 + kWarps * 128;
-  *smem = (size_t)rg->cols * (sh.D + 4) * 4 + (tables > tail ? tables : tail) + 16;
+  const size_t tables = (size_t)(two ? 2 : 1) * kWarps * (mma && !sh.pq ? 16 : 32) * rg->pitch * 4;
+  const size_t tail = (size_t)(8 * 128 + 2 * kWarps * 132) * 4 + kWarps * 128;
+  *smem = (size_t)rg->means * 4 + (tables > tail ? tables : tail) + 16;
   return *smem <= 200 * 1024;
 }
 

@@ -5,11 +5,12 @@
 namespace blossom {
 
 struct RowsGeom {
-  int cols, pitch;  // rows of the table of means; pitch of a row's table of exponentials (floats)
+  int cols, pitch;  // candidates in the table of means; pitch of a row's table of exponentials (floats)
+  int means;        // floats of the table of means
   int exact;        // leave every choice to double precision
 };
 // Whether the kernel takes the problem (up to 128 scored and selection blocks), its plan and its shared memory.
-bool rows_geom(const Shape &sh, const SelGeom &g, RowsGeom *rg, size_t *smem);
+bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_t *smem);
 // Writes the certain index rows and appends the others to `list` (per block: unit * M + block; per
 // position: unit * L + position).
 int launch_score_rows(const Shape &sh, const SelGeom &g, const RowsGeom &rg, size_t smem, int dtype, const void *q,

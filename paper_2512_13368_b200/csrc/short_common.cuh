@@ -104,6 +104,33 @@ __device__ __forceinline__ void product_nt(const uint32_t (&a)[D / 16][4], uint3
     }
   }
 }
+// the same added to s
+template <int D>
+__device__ __forceinline__ void product_nt_add(const uint32_t (&a)[D / 16][4], uint32_t chunk, float (&s)[2][4]) {
+#pragma unroll
+  for (int k = 0; k < D / 16; ++k) {
+    uint32_t b[4];
+    ldsm4(chunk ^ (32 * k), b);
+    mma16816(s[0], a[k], b[0], b[1]);
+    mma16816(s[1], a[k], b[2], b[3]);
+  }
+}
+// the same with every 16 columns' product formed from zero and then added (fewer roundings in a row)
+template <int D>
+__device__ __forceinline__ void product_nt_steps(const uint32_t (&a)[D / 16][4], uint32_t chunk, float (&s)[2][4]) {
+#pragma unroll
+  for (int k = 0; k < D / 16; ++k) {
+    uint32_t b[4];
+    float x[2][4];
+    ldsm4(chunk ^ (32 * k), b);
+    mma16816_0(x[0], a[k], b[0], b[1]);
+    mma16816_0(x[1], a[k], b[2], b[3]);
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[nt][e] += x[nt][e];
+  }
+}
 // acc[16 rows x D] += A (16 x 16) times the 16 rows at `chunk` (tile address + row * 2 D + lane_off_nn)
 template <int D>
 __device__ __forceinline__ void product_nn(const uint32_t (&a)[4], uint32_t chunk, float (&acc)[D / 8][4]) {
