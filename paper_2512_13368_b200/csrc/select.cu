@@ -1099,7 +1099,7 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
     const bool listed = rows && !exact_select_only();
     if (listed) {
       rg.exact = 0;
-      if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, seq_lens, idx, w.list, w.count, st))
+      if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, w.mean, seq_lens, idx, w.list, w.count, st))
         return rc;
     }
     const size_t psm = (size_t)8 * ((5 * g.n + (g.plain ? 0 : sh.M) + 4 * D + 1) / 2 * 2) * sizeof(double) + (size_t)8 * sh.M + 16;
@@ -1120,7 +1120,8 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   const bool exact_only = exact_select_only() || (!use_rows && (fsm == 0 || !sh.causal));
   if (!exact_only && use_rows) {
     rg.exact = 0;
-    if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, seq_lens, idx, w.list, w.count, st)) return rc;
+    if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, w.mean, seq_lens, idx, w.list, w.count, st)) return rc;
+    if (!rg.list) return BLOSSOM_OK;
   } else if (!exact_only) {
     if (fsm > 48 * 1024 && cudaFuncSetAttribute(score_fast_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)fsm) != cudaSuccess)

@@ -67,12 +67,96 @@ __device__ __forceinline__ float square(const float2 (&q)[N]) {
   return (a0.x + a0.y) + (a1.x + a1.y);
 }
 
+// Eight elements as doubles.
+__device__ __forceinline__ void to_double(const uint4 &v, double (&x)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    x[2 * e] = (double)__uint_as_float(w[e] << 16);
+    x[2 * e + 1] = (double)__uint_as_float(w[e] & 0xffff0000u);
+  }
+}
+
+struct Columns {
+  double s[4];
+};
+// One warp's part of the column sums of a query block's probabilities in double precision: of the block's
+// rows (`nq` positions from `qlo` of G heads, head-major) taken 16 at a time the four rows 4 warp ...; a
+// lane forms the logits of one of them against every eighth candidate.  s[x]: candidate lane + 32 x of
+// ncol; candidate `skip` takes no part.  Out of line: its registers must not count against the common path.
+template <typename T, int D>
+__device__ __noinline__ Columns exact_columns(const T *q, int64_t sh, int64_t sl, int G, int nq, int qlo, double scale,
+                                              double *zd, int nz, const double *mean, int ncol, int skip, int warp,
+                                              int lane) {
+  const int r = lane & 3, pt = lane >> 2, nrows = nq * G;
+  Columns out = {{0.0, 0.0, 0.0, 0.0}};
+#pragma unroll 1
+  for (int r0 = 4 * warp; r0 < nrows; r0 += 16) {
+    const int x = r0 + r;
+    const bool on = x < nrows;
+    const T *row = q + (on ? (int64_t)(x / nq) * sh + (int64_t)(qlo + x % nq) * sl : (int64_t)qlo * sl);
+    double *z = zd + (4 * warp + r) * nz;
+    __syncwarp();
+    double mx = -INFINITY, den = 0.0;
+#pragma unroll 1
+    for (int c = pt; c < ncol; c += 16) {
+      const int c1 = c + 8 < ncol ? c + 8 : c;
+      const double2 *k0 = reinterpret_cast<const double2 *>(mean + (int64_t)c * D);
+      const double2 *k1 = reinterpret_cast<const double2 *>(mean + (int64_t)c1 * D);
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+      for (int e = 0; e < D / 8; ++e) {
+        double v[8];
+        if constexpr (sizeof(T) == 2) {
+          to_double(reinterpret_cast<const uint4 *>(row)[e], v);
+        } else {
+          const float4 f = reinterpret_cast<const float4 *>(row)[2 * e], g = reinterpret_cast<const float4 *>(row)[2 * e + 1];
+          v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w; v[4] = g.x; v[5] = g.y; v[6] = g.z; v[7] = g.w;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const double2 x0 = k0[4 * e + j], x1 = k1[4 * e + j];
+          a[0] = fma(v[2 * j], x0.x, a[0]);
+          a[1] = fma(v[2 * j + 1], x0.y, a[1]);
+          a[2] = fma(v[2 * j], x1.x, a[2]);
+          a[3] = fma(v[2 * j + 1], x1.y, a[3]);
+        }
+      }
+      const double z0 = c == skip ? -INFINITY : scale * (a[0] + a[1]), z1 = c1 == skip ? -INFINITY : scale * (a[2] + a[3]);
+      z[c] = z0;
+      if (c1 != c) z[c1] = z1;
+      mx = fmax(mx, fmax(z0, z1));
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+#pragma unroll 1
+    for (int c = pt; c < ncol; c += 8) {
+      const double e = exp(z[c] - mx);  // exp(-inf) = 0
+      z[c] = e;
+      den += e;
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    const double inv = on ? 1.0 / den : 0.0;
+    __syncwarp();
+#pragma unroll 1
+    for (int y = 0; y < 4; ++y) {
+      const double iv = __shfl_sync(0xffffffffu, inv, y);
+      const double *zy = zd + (4 * warp + y) * nz;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (lane + 32 * i < ncol) out.s[i] = fma(zy[lane + 32 * i], iv, out.s[i]);
+    }
+  }
+  return out;
+}
+
 // PQ: one selection per query position.
 template <typename T, int D, bool PQ>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_kernel(
     Shape sh, SelGeom g, RowsGeom rg, const T *__restrict__ q, const float *__restrict__ mean32,
-    const float *__restrict__ norm, const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx,
-    int32_t *__restrict__ worklist, int32_t *__restrict__ work_count) {
+    const float *__restrict__ norm, const double *__restrict__ mean, const int32_t *__restrict__ seq_lens,
+    int32_t *__restrict__ idx, int32_t *__restrict__ worklist, int32_t *__restrict__ work_count) {
   grid_chain_enter();
   constexpr bool kMma = sizeof(T) == 2;  // bf16: products on the warp-level matrix pipe
   constexpr int P = D + 4;               // pitch of the means (floats; the fp32 form)
@@ -80,6 +164,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
   constexpr int kTab = kMma && !PQ ? 16 : 32;
   extern __shared__ __align__(128) float fsm[];
   __shared__ float kn_w[kWarps], inv_s[kWarps][32], rowq_s[kWarps][32], bound_s[8][2];
+  __shared__ int n_uncertain, uncertain[8];
   // candidate means, candidate cmin first: [rg.cols][P] floats, or bf16 tiles [hi, mid, lo][rg.cols][D]
   float *ms = fsm, *tab = fsm + rg.means;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -114,6 +199,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
     int want;
     need |= max((qb0 + i) * Bk, pad0) < min((qb0 + i + 1) * Bk, sh.L) && choice(qb0 + i, &want) && live_cands(qb0 + i) > 0;
   }
+  if (tid == 0) n_uncertain = 0;
   float qn = 0.f, kn = 0.f;  // the lane's largest query norm over the group's heads; the largest mean norm
   bool loose = false;        // a row whose reference was too far from its logits
   float colsum[2][4];        // (per block) summed probabilities of candidates lane, lane + 32, ...: of rows 0..15, 16..31
@@ -500,8 +586,68 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
       }
       for (int x = pos + lane; x < sh.topk; x += 32) row[x] = -1;
     } else if (lane == 0) {
-      worklist[atomicAdd(work_count, 1)] = u * M + bb;
+      if (rg.list) worklist[atomicAdd(work_count, 1)] = u * M + bb;
+      else uncertain[atomicAdd(&n_uncertain, 1)] = bb;
     }
+  }
+  if (rg.list) return;
+  // ---- the blocks that could not be certified, in double precision by all warps ----
+  __syncthreads();
+  const int nun = n_uncertain;  // (in any order: every one is decided by itself)
+  const int nz = (g.n + 1) | 1;
+  double *zd = reinterpret_cast<double *>(fsm), *partd = zd + 16 * nz, *Sc2 = partd + kWarps * 128, *S2 = Sc2 + 128;
+  uint8_t *tk = reinterpret_cast<uint8_t *>(S2 + 128);
+  for (int i = 0; i < nun; ++i) {
+    const int bb = uncertain[i], hi = causal ? bb : M, ncb = causal ? n_candidates(sh, g, bb) : g.n;
+    const int qlo = max(bb * Bk, pad0), nq = min((bb + 1) * Bk, sh.L) - qlo;
+    int want;
+    choice(bb, &want);
+    const Columns c = exact_columns<T, D>(q + row_offset(sh, n, hk * sh.G, 0), sh.sh, sh.sl, sh.G, nq, qlo, sh.scale_d, zd, nz,
+                                          mean + ((int64_t)u * g.n + cmin) * D, ncb - cmin, own ? bb - cmin : -1, warp, lane);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) partd[warp * 128 + lane + 32 * x] = c.s[x];
+    __syncthreads();
+    Sc2[tid] = (partd[tid] + partd[128 + tid]) + (partd[256 + tid] + partd[384 + tid]);
+    __syncthreads();
+    const int j = jmin + tid;
+    const bool in = j < hi && !(own && j == bb);
+    if (j < hi) {
+      double a = 0.0;
+      for (int m = 0; m < g.rs; ++m)
+        for (int e = 0; e < g.rl; ++e) {
+          const int y = g.rs * j - m - e;
+          if (y >= cmin && y < ncb) a += Sc2[y - cmin];
+        }
+      S2[tid] = in ? a : -INFINITY;  // (the own block is not ranked: it is kept anyway)
+    }
+    __syncthreads();
+    if (j < hi) {
+      const double sj = S2[tid];
+      int rk = 0;
+#pragma unroll 4
+      for (int y = 0; y < hi - jmin; ++y) {
+        const double sy = S2[y];
+        rk += (sy > sj || (sy == sj && y < tid)) ? 1 : 0;
+      }
+      tk[tid] = !in || rk < want ? 1 : 0;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int32_t *row = idx + ((int64_t)u * M + bb) * sh.topk;
+      int pos = 0;
+      for (int base = 0; base < hi - jmin; base += 32) {
+        const bool f = base + lane < hi - jmin && tk[base + lane];
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (f) row[pos + __popc(m & ((1u << lane) - 1u))] = jmin + base + lane;
+        pos += __popc(m);
+      }
+      if (!own) {
+        if (lane == 0) row[pos] = bb;
+        ++pos;
+      }
+      for (int x = pos + lane; x < sh.topk; x += 32) row[x] = -1;
+    }
+    __syncthreads();
   }
 }
 
@@ -518,35 +664,42 @@ bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_
   const size_t tables = (size_t)(two ? 2 : 1) * kWarps * (mma && !sh.pq ? 16 : 32) * rg->pitch * 4;
   const size_t tail = (size_t)(8 * 128 + 2 * kWarps * 132) * 4 + kWarps * 128;
   *smem = (size_t)rg->means * 4 + (tables > tail ? tables : tail) + 16;
+  // What single precision cannot certify (some percent of the blocks) the kernel decides itself while that
+  // takes a CTA a few microseconds: no second launch (D 32, L 1024, block 32: 40 -> 32 us for both).  With
+  // more rows, candidates or dimensions the CTA that has such a block ends long after the others (D 64, L
+  // 900, block 32: 27 us either way; L 4096, block 64: 105 -> 147 us): a list, shared by clusters of CTAs.
+  rg->list = sh.pq || sh.G * sh.Bk > 128 || (int64_t)sh.G * sh.Bk * g.n * sh.D > 32768;
+  const size_t own = ((size_t)16 * ((g.n + 1) | 1) + kWarps * 128 + 128 + 128) * 8 + 128;
+  if (!rg->list && *smem < own) *smem = own;
   return *smem <= 200 * 1024;
 }
 
 template <typename T, int D>
 static int launch_t(const Shape &sh, const SelGeom &g, const RowsGeom &rg, size_t smem, const T *q, const float *mean32,
-                    const float *norm, const int32_t *seq_lens, int32_t *idx, int32_t *list, int32_t *count,
-                    cudaStream_t st) {
+                    const float *norm, const double *mean, const int32_t *seq_lens, int32_t *idx,
+                    int32_t *list, int32_t *count, cudaStream_t st) {
   auto kern = sh.pq ? score_rows_kernel<T, D, true> : score_rows_kernel<T, D, false>;
   if (smem > 40 * 1024 &&  // (static shared memory counts too)
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
   const unsigned grid = (unsigned)((sh.L + kRows - 1) / kRows) * (unsigned)(sh.B * sh.Hkv);
   LaunchScope ls(K_SCORE_FAST, st);
-  return launch_chained(kern, dim3(grid), dim3(kThreads), smem, st, sh, g, rg, q, mean32, norm, seq_lens, idx, list,
-                        count) == cudaSuccess
+  return launch_chained(kern, dim3(grid), dim3(kThreads), smem, st, sh, g, rg, q, mean32, norm, mean, seq_lens, idx,
+                        list, count) == cudaSuccess
              ? BLOSSOM_OK
              : BLOSSOM_ERR_CUDA;
 }
 
 int launch_score_rows(const Shape &sh, const SelGeom &g, const RowsGeom &rg, size_t smem, int dtype, const void *q,
-                      const float *mean32, const float *norm, const int32_t *seq_lens, int32_t *idx, int32_t *list,
-                      int32_t *count, cudaStream_t st) {
+                      const float *mean32, const float *norm, const double *mean, const int32_t *seq_lens, int32_t *idx,
+                      int32_t *list, int32_t *count, cudaStream_t st) {
   typedef __nv_bfloat16 bf;
   if (dtype == BLOSSOM_DTYPE_FP32) {
-    if (sh.D == 32) return launch_t<float, 32>(sh, g, rg, smem, (const float *)q, mean32, norm, seq_lens, idx, list, count, st);
-    return launch_t<float, 64>(sh, g, rg, smem, (const float *)q, mean32, norm, seq_lens, idx, list, count, st);
+    if (sh.D == 32) return launch_t<float, 32>(sh, g, rg, smem, (const float *)q, mean32, norm, mean, seq_lens, idx, list, count, st);
+    return launch_t<float, 64>(sh, g, rg, smem, (const float *)q, mean32, norm, mean, seq_lens, idx, list, count, st);
   }
-  if (sh.D == 32) return launch_t<bf, 32>(sh, g, rg, smem, (const bf *)q, mean32, norm, seq_lens, idx, list, count, st);
-  return launch_t<bf, 64>(sh, g, rg, smem, (const bf *)q, mean32, norm, seq_lens, idx, list, count, st);
+  if (sh.D == 32) return launch_t<bf, 32>(sh, g, rg, smem, (const bf *)q, mean32, norm, mean, seq_lens, idx, list, count, st);
+  return launch_t<bf, 64>(sh, g, rg, smem, (const bf *)q, mean32, norm, mean, seq_lens, idx, list, count, st);
 }
 
 }  // namespace blossom
