@@ -50,6 +50,17 @@ struct Raw8<__nv_bfloat16> {
       x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
     }
   }
+  // a[e] += x[e] * 2^-896, exactly: the bits of a bf16 moved into the exponent and mantissa fields of a double
+  // (for denormals too: the fields then hold a denormal).  `odd`: its bits 15 or 31 are set by an infinity or NaN.
+  __device__ __forceinline__ void add_scaled(double (&a)[8], uint32_t *odd) const {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      a[2 * e] += __hiloint2double(((int)(w[e] << 16) >> 3) & 0x8fffe000, 0);
+      a[2 * e + 1] += __hiloint2double(((int)w[e] >> 3) & 0x8fffe000, 0);
+      *odd |= (w[e] & 0x7f807f80u) + 0x00800080u;
+    }
+  }
 };
 template <>
 struct Raw8<float> {
@@ -67,8 +78,47 @@ struct Raw8<float> {
 // ---- Eq. 8 + 9: mean of the valid keys of every scored block (fp64) ------------------------
 // One warp per scored block, 8 blocks per CTA.  A lane owns eight columns (one 16-byte load of
 // bf16, two of fp32) of every (32 / (D / 8))-th row and sums them in a fixed order with eight rows
-// in flight (kept as loaded until they are added); the lanes that share columns are combined by
-// shuffles in a fixed tree.
+// in flight (kept as loaded until they are added); the lanes that share columns are combined in a fixed
+// tree in which each keeps half of the columns, so that a lane ends with the D / 32 it divides and writes.
+// Bound by instructions, not by the keys' 4 - 10 us: a conversion to double takes eight cycles of a
+// scheduler, so bf16 is widened by moving its bits (B 128, H 4, L 1024, D 64: 27 -> 24 us).
+template <typename T, int D, bool PHI, bool MOVE>  // MOVE: sums times 2^-896; phi: by position
+__device__ __forceinline__ void column_sums(const T *base, int64_t stride, int lo, int hi, const float *phi,
+                                            double (&a)[8], double *wsum, uint32_t *odd) {
+  constexpr int RPI = 32 / (D / 8);           // rows per warp iteration
+  constexpr int NF = sizeof(T) == 2 ? 8 : 2;  // rows in flight per lane
+#pragma unroll
+  for (int e = 0; e < 8; ++e) a[e] = 0.0;
+  for (int p = lo; p < hi; p += NF * RPI) {
+    Raw8<T> x[NF];
+#pragma unroll
+    for (int r = 0; r < NF; ++r) {
+      const int pp = p + r * RPI;
+      if (pp < hi) x[r].load(base + (int64_t)pp * stride);
+      else x[r].zero();
+    }
+#pragma unroll
+    for (int r = 0; r < NF; ++r) {
+      if constexpr (MOVE) {
+        x[r].add_scaled(a, odd);
+      } else {
+        const int pp = p + r * RPI;
+        float f[8];
+        x[r].unpack(f);
+        if (PHI) {  // learnable summary: weight exp(phi[i]) for position i of the block
+          const double w = pp < hi ? exp((double)phi[pp]) : 0.0;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) a[e] = fma(w, (double)f[e], a[e]);
+          *wsum += w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) a[e] += (double)f[e];
+        }
+      }
+    }
+  }
+}
+
 template <typename T, int D, bool PHI>
 __global__ void __launch_bounds__(256, PHI ? 2 : 4) summary_kernel(Shape sh, SelGeom g, const T *__restrict__ k,
                                                          const int32_t *__restrict__ seq_lens,
@@ -81,8 +131,6 @@ __global__ void __launch_bounds__(256, PHI ? 2 : 4) summary_kernel(Shape sh, Sel
   grid_chain_enter();
   if (status && blockIdx.x == 0 && threadIdx.x < 8) status[threadIdx.x] = 0;  // a new step's status words
   constexpr int LPR = D / 8;     // lanes per row
-  constexpr int RPI = 32 / LPR;  // rows per warp iteration
-  constexpr int NF = sizeof(T) == 2 ? 8 : 2;  // rows in flight per lane
   if (blockIdx.x == 0 && threadIdx.x == 0) *sel_count = 0;  // work list of the scoring kernel
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t blk = (int64_t)blockIdx.x * 8 + warp;  // (batch, key/value head, scored block)
@@ -94,65 +142,52 @@ __global__ void __launch_bounds__(256, PHI ? 2 : 4) summary_kernel(Shape sh, Sel
   const int lo = max(c * g.s, pad0), hi = min(c * g.s + g.l, sh.L);
   const int sub = lane / LPR, col = (lane % LPR) * 8;
   const T *base = k + row_offset_kv(sh, n, hk, 0) + col;
+  constexpr bool kMove = sizeof(T) == 2 && !PHI;  // widen by moving bits
   double a[8], wsum = 0.0;  // weighted column sums and the sum of the weights (Eq. 9)
-#pragma unroll
-  for (int e = 0; e < 8; ++e) a[e] = 0.0;
-  for (int p = lo + sub; p < hi; p += NF * RPI) {
-    Raw8<T> x[NF];
-#pragma unroll
-    for (int r = 0; r < NF; ++r) {
-      const int pp = p + r * RPI;
-      if (pp < hi) x[r].load(base + (int64_t)pp * sh.ksl);
-      else x[r].zero();
-    }
-    if (PHI) {  // learnable summary: weight exp(phi[i]) for position i of the block
-#pragma unroll
-      for (int r = 0; r < NF; ++r) {
-        const int pp = p + r * RPI;
-        const double w = pp < hi ? exp((double)sh.phi[pp - c * g.s]) : 0.0;
-        float f[8];
-        x[r].unpack(f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) a[e] = fma(w, (double)f[e], a[e]);
-        wsum += w;
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < NF; ++r) {
-        float f[8];
-        x[r].unpack(f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) a[e] += (double)f[e];
-      }
+  uint32_t odd = 0;
+  const int cnt = max(hi - lo, 0);
+  column_sums<T, D, PHI, kMove>(base, sh.ksl, lo + sub, hi, PHI ? sh.phi - c * g.s : nullptr, a, &wsum, &odd);
+  double unit = 1.0;
+  if (kMove) {
+    unit = 0x1p896;
+    if (__any_sync(0xffffffffu, (odd & 0x80008000u) != 0)) {  // infinities and NaNs are left to the conversion
+      unit = 1.0;
+      column_sums<T, D, PHI, false>(base, sh.ksl, lo + sub, hi, nullptr, a, &wsum, &odd);
     }
   }
-#pragma unroll
-  for (int o = LPR; o < 32; o <<= 1)  // the lanes that took other rows of the same columns
-#pragma unroll
-    for (int e = 0; e < 8; ++e) a[e] += __shfl_xor_sync(0xffffffffu, a[e], o);
-  const int cnt = max(hi - lo, 0);
   if (PHI) {
 #pragma unroll
     for (int o = LPR; o < 32; o <<= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
   } else {
     wsum = (double)cnt;
   }
-  float sq = 0.f;
-  if (sub == 0) {
-    double m[8];
-    float f[8];
+  // the lanes that took other rows of the same columns
+  constexpr int NC = D / 32;  // columns a lane ends with
+  int at = col;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      m[e] = cnt > 0 ? a[e] / wsum : 0.0;
-      f[e] = (float)m[e];
-      sq = fmaf(f[e], f[e], sq);
+  for (int o = LPR, h = 4; o < 32; o <<= 1, h >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int e = 0; e < h; ++e) {
+      const double send = up ? a[e] : a[e + h], keep = up ? a[e + h] : a[e];
+      a[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
     }
-    double2 *md = reinterpret_cast<double2 *>(mean + blk * D + col);
-    md[0] = make_double2(m[0], m[1]); md[1] = make_double2(m[2], m[3]);
-    md[2] = make_double2(m[4], m[5]); md[3] = make_double2(m[6], m[7]);
-    float4 *mf = reinterpret_cast<float4 *>(mean32 + blk * D + col);
-    mf[0] = make_float4(f[0], f[1], f[2], f[3]);
-    mf[1] = make_float4(f[4], f[5], f[6], f[7]);
+    at += up ? h : 0;
+  }
+  float sq = 0.f, f[NC];
+#pragma unroll
+  for (int e = 0; e < NC; ++e) {
+    a[e] = cnt > 0 ? a[e] * unit / wsum : 0.0;
+    f[e] = (float)a[e];
+    sq = fmaf(f[e], f[e], sq);
+  }
+  if constexpr (NC == 1) {
+    mean[blk * D + at] = a[0];
+    mean32[blk * D + at] = f[0];
+  } else {
+    static_assert(NC == 2, "head dimension");
+    *reinterpret_cast<double2 *>(mean + blk * D + at) = make_double2(a[0], a[1]);
+    *reinterpret_cast<float2 *>(mean32 + blk * D + at) = make_float2(f[0], f[1]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
