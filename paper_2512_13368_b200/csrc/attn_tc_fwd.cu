@@ -7,6 +7,15 @@
 // the same 64 positions of two heads of a group, which share their selection (Eq. 12), their window
 // tiles and their K/V: every tile on the list then has work for every row (template flag PACK).
 //
+// The kernel is persistent: two CTAs on every SM take 128-row tiles, long rows first, from a counter
+// until none is left.  A tile's fixed part (its lists, queries and first keys to wait for, the merges,
+// the staged rows to be read by the bulk stores, launching a CTA) was most of the time of a kernel with
+// a CTA per tile: with four items a tile 146 us for 4096 tiles of D 64, 98 - 104 us so; 11.5 items
+// 228 -> 204 us, 27 items (L 4096) 388 -> 365 us, D 32 97 -> 91 us.  The roles therefore run on from
+// tile to tile (item counters, stages and barrier phases continue), each as far ahead as its own inputs
+// allow, while the softmax warps merge.  What is left is bound by the softmax warps' instructions:
+// tensor pipe 21 %, 0.53 instructions a cycle and scheduler, four softmax warps each.
+//
 // CTA = 384 threads.  Warps 0..7 are softmax warps: a query row (= TMEM lane) is shared by two
 // threads, warp w and warp w + 4, which split the KEYS of every tile: group 0 (warps 0..3) takes
 // keys 0..31, group 1 keys 32..63.  Each group keeps its own running maximum and sum and its own
@@ -15,7 +24,8 @@
 // halves of an online softmax, when a phase ends.  Sixteen softmax warps per SM instead of eight
 // hide the latency of a thread's dependent chain (load, maximum, exponentials, store).
 // Warps 8, 9, 10 stay converged and one elected lane of each loads K/V tiles (TMA), issues
-// S = Q K^T, and issues the two O += P V products with P read from tensor memory.
+// S = Q K^T, and issues the two O += P V products with P read from tensor memory.  Warp 11 stores the
+// finished rows and fetches the next tile's lists and queries.
 //
 // Tensor memory (256 columns): two logits / probability buffers [0,64) [64,128), O_A [128,128+D),
 // O_B [192,192+D).  Item i uses buffer i % 2: S(i) lands there as fp32, a softmax thread reads its
@@ -31,10 +41,11 @@
 //              commit done[i%2], release the stage
 //
 // When the long-term phase ends the merged, normalised rows go (as bf16) to a staging tile in
-// shared memory, from where they are stored and read back for the gate mix of the epilogue
-// (Eq. 19); the short-term phase then starts both accumulators afresh.
-// Epilogue: merge, normalise, gate mix, stage the rows in shared memory and write out / out_lt /
-// out_st with whole-line TMA stores; lse directly.  Every wait is bounded (tc_common.cuh).
+// shared memory, from where they are stored; the short-term phase then starts both accumulators
+// afresh.  At its end the staged rows are read back for the gate mix (Eq. 19) and replaced by the
+// short-term rows; the mix goes over the tile's queries, which no product reads any more (the next
+// tile's lie in a second buffer).  Whole-line TMA stores; lse directly.  Every wait is bounded
+// (tc_common.cuh); the softmax warps, which meet at named barriers, agree on every tile they start.
 #include "tc_common.cuh"
 
 namespace blossom {
@@ -42,15 +53,15 @@ namespace tc {
 namespace {
 
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
-constexpr int kFwdThreads = 384;  // warps 0..7 softmax; 8 loader, 9 S issuer, 10 PV issuer, 11 spare
+constexpr int kFwdThreads = 384;  // warps 0..7 softmax; 8 loader, 9 S issuer, 10 PV issuer, 11 storer
 constexpr int kSoftmaxWarps = 8;
 // The kernel is compiled for 80 registers per thread (two CTAs of 384 threads per SM): the pool of
 // a CTA is 384 * 80 = 30720, and the two register counts must fit in it or the increase would
 // wait for registers that never come: 256 * 96 + 128 * 40 = 29696.
 constexpr int kProducerRegs = 40, kSoftmaxRegs = 96;
 static_assert(256 * kSoftmaxRegs + 128 * kProducerRegs <= kFwdThreads * 80, "register pool of a CTA");
-constexpr int kFwdStages = 4;
 constexpr uint32_t kFwdTmemCols = 256;
+__host__ __device__ constexpr int fwd_stages(int D) { return D == 64 ? 3 : 4; }
 
 // maximum of 32 logits (those whose mask bit is set, all of them when FULL)
 template <bool FULL>
@@ -130,14 +141,16 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     const __grid_constant__ CUtensorMap tmol, const __grid_constant__ CUtensorMap tmos, Shape s,
     const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
     const uint8_t *__restrict__ qmeta, int training, float *__restrict__ lse,
-    int32_t *__restrict__ status, int nT) {
+    int32_t *__restrict__ status, int32_t *__restrict__ tickets, int nT, int n_tiles, int n_meta) {
   grid_chain_enter();
   using C = Cfg<D>;
-  constexpr int STAGES = kFwdStages;
+  constexpr int STAGES = fwd_stages(D);
   constexpr int DC = D / 2;  // output columns a softmax thread merges and stages
   extern __shared__ uint8_t smem_raw[];
-  // barriers: full[STAGES], empty[STAGES], res, meta, then per buffer: s_full[2], t_full[group][2], done[2]
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 10];
+  // barriers: full[STAGES], empty[STAGES], then by tile res[2], meta[2], per buffer s_full[2],
+  // t_full[group][2], done[2], then staged, stored and by tile roles[2]
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 16];
+  __shared__ int softmax_tile, tile_id[2];  // the tile whose lists lie (or are about to) behind meta[.]; -1: no more
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ float2 stat[2][128];  // (maximum, sum) of each group's half of every row, exchanged at a phase end
@@ -147,33 +160,46 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   // long rows first, tile-major: every unit's last tile, then every unit's last but one, ...
   // (PACK: a unit is a pair of heads, a tile 64 positions; h = the pair's first head)
   const int nU = PACK ? s.B * (s.H / 2) : s.B * s.H, nQT = PACK ? nT : nST;
-  const int st = nQT - 1 - (int)(blockIdx.x / nU);
-  const int u = (int)(blockIdx.x % nU);
-  const int n = PACK ? u / (s.H / 2) : u / s.H, h = PACK ? 2 * (u % (s.H / 2)) : u % s.H;
-  int len = seq_lens ? seq_lens[n] : s.L;
-  len = min(max(len, 0), s.L);
-  const int pad0 = s.L - len;
-  const int row0 = PACK ? st * 64 : st * 128;
-
   const uint32_t raw_addr = smem_u32(smem_raw);
   uint8_t *tiles = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
-  uint8_t *q_tile = tiles;
-  uint8_t *kv_tiles = q_tile + C::kBigBytes;                  // [stage][K, V]
-  uint8_t *sl = kv_tiles + STAGES * 2 * C::kSmallBytes;       // the long-term rows, staged when their phase ends
-  uint8_t *meta = sl + C::kBigBytes;                          // image built by tc_meta_kernel
+  uint8_t *q_tiles = tiles;                                  // [2]: the tile's queries, then its staged rows of out
+  uint8_t *kv_tiles = q_tiles + 2 * C::kBigBytes;            // [stage][K, V]
+  uint8_t *sl = kv_tiles + STAGES * 2 * C::kSmallBytes;      // staged rows: the long-term branch, then the short-term one
+  uint8_t *metas = sl + C::kBigBytes;                        // [n_meta] images built by tc_meta_kernel
   const bool causal = PLAIN || s.causal;
   const int pq = PLAIN ? 0 : s.pq;
   const MetaLayout ml = meta_layout(nT, pq);
-  const uint8_t *selb = meta;
-  const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
-  const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
-  const uint8_t *icls = meta + ml.icls;                                         // [2 nT][4]
-  const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
-
+  const int meta_step = n_meta == 2 ? ml.bytes : 0;
+  // tile x of this grid: its rows (tile st of unit u; long rows first, every unit's last tile, then every
+  // unit's last but one, ...) and heads
+  auto tile_unit = [&](int x) { return x % nU; };
+  auto tile_row0 = [&](int x) { return (nQT - 1 - x / nU) * (PACK ? 64 : 128); };
+  auto unit_batch = [&](int u) { return PACK ? u / (s.H / 2) : u / s.H; };
+  auto unit_head = [&](int u) { return PACK ? 2 * (u % (s.H / 2)) : u % s.H; };
   const uint32_t b_full = smem_u32(&bars[0]), b_empty = smem_u32(&bars[STAGES]);
-  const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 1]);
-  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 2]), b_tfull = smem_u32(&bars[2 * STAGES + 4]);  // [group][buffer]
-  const uint32_t b_done = smem_u32(&bars[2 * STAGES + 8]);
+  const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 2]);
+  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 4]), b_tfull = smem_u32(&bars[2 * STAGES + 6]);  // [group][buffer]
+  const uint32_t b_done = smem_u32(&bars[2 * STAGES + 10]);
+  const uint32_t b_staged = smem_u32(&bars[2 * STAGES + 12]), b_stored = smem_u32(&bars[2 * STAGES + 13]);
+  const uint32_t b_roles = smem_u32(&bars[2 * STAGES + 14]);
+  // one thread: the lists (and which tile's they are) and the queries of this CTA's k-th tile, number x
+  auto fetch_meta = [&](int k, int x) {
+    tile_id[k & 1] = x;
+    const uint32_t bar = b_meta + 8 * (k & 1);
+    if (x < 0) {
+      mbar_arrive(bar);
+    } else {
+      mbar_expect_tx(bar, (uint32_t)ml.bytes);
+      bulk_load(smem_u32(metas) + (k & 1) * meta_step,
+                qmeta + ((size_t)tile_unit(x) * nQT + x / nU) * ml.bytes, (uint32_t)ml.bytes, bar);
+    }
+  };
+  auto fetch_queries = [&](int k, int x) {
+    const int u = tile_unit(x);
+    const uint32_t bar = b_res + 8 * (k & 1);
+    mbar_expect_tx(bar, C::kBigBytes);
+    tma_load_4d(smem_u32(q_tiles) + (k & 1) * C::kBigBytes, &tmq, bar, 0, tile_row0(x), unit_head(u), unit_batch(u));
+  };
 
   if (tid == 0) {
     abort_flag = (*status != 0) ? 1 : 0;  // an earlier CTA timed out: do not wait again
@@ -184,20 +210,20 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
     }
-    mbar_init(b_res, 1);
-    mbar_init(b_meta, 1);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(b_res + 8 * i, 1);
+      mbar_init(b_meta + 8 * i, 1);
+      mbar_init(b_roles + 8 * i, 3);
       mbar_init(b_sfull + 8 * i, 1);
       mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);        // group 0
       mbar_init(b_tfull + 8 * (2 + i), kSoftmaxWarps / 2);  // group 1
       mbar_init(b_done + 8 * i, 1);
     }
+    mbar_init(b_staged, kSoftmaxWarps);
+    mbar_init(b_stored, 1);
     mbar_fence_init();
-    // the CTA's tile lists and its query tile
-    mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
-    bulk_load(smem_u32(meta), qmeta + ((size_t)u * nQT + (nQT - 1 - st)) * ml.bytes, (uint32_t)ml.bytes, b_meta);
-    mbar_expect_tx(b_res, C::kBigBytes);
-    tma_load_4d(smem_u32(q_tile), &tmq, b_res, 0, row0, h, n);
+    fetch_meta(0, (int)blockIdx.x);
+    fetch_queries(0, (int)blockIdx.x);
   }
   if (warp == 0) {
     __syncwarp();
@@ -207,266 +233,285 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  mbar_wait(b_meta, 0, &abort_flag, 113);
-  const int nL = counts[1], nS = counts[2], nI = nL + nS;
   const uint32_t tmem_base = tmem_slot;
   const uint32_t tmem_oa = tmem_base + 128, tmem_ob = tmem_base + 192;  // buffers at tmem_base + 64 * (item % 2)
 
   if (warp >= kSoftmaxWarps) {
     // ===================== three single-thread roles, one warp each =====================
     setmaxnreg_dec<kProducerRegs>();
-    if (warp == kSoftmaxWarps && nI > 0) {
-      // ---- loader: K/V tiles, up to STAGES ahead of their consumers ----
-      for (int j = 0; j < nI; ++j) {
-        const int sj = j % STAGES;
-        if (j >= STAGES) mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 105);
-        const uint32_t bar = b_full + 8 * sj;
-        const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
-        const int row = (int)items[j] * 64;
-        if (elect_one()) {
-          mbar_expect_tx(bar, 2 * C::kSmallBytes);
-          tma_load_4d(kt, &tmk, bar, 0, row, h / s.G, n);  // the key/value head of this query head
-          tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, h / s.G, n);
+    if (warp == kSoftmaxWarps + 3) {
+      // ---- storer: the staged rows of a tile as whole-line bulk stores (rows past L are clipped by the
+      // hardware, padded rows were staged as zeros).  When the long-term rows are there it takes the CTA's
+      // next tile and fetches that one's lists and queries: late enough for the CTAs that are behind to take
+      // fewer tiles (taken a tile earlier, 768 tiles of L 1500: 72 us), early enough for both to be there
+      // when the last items are done ----
+      if (lane == 0) {
+        int cur = (int)blockIdx.x;
+        for (int k = 0; cur >= 0 && !*(volatile int *)&abort_flag; ++k) {
+          const int u = tile_unit(cur), row0 = tile_row0(cur), h = unit_head(u), n = unit_batch(u);
+          mbar_wait(b_staged, 0, &abort_flag, 114);
+          if (training) {
+            tma_store_4d(&tmol, smem_u32(sl), 0, row0, h, n);
+            tma_store_commit();
+          }
+          int next = (int)gridDim.x + atomicAdd(tickets, 1);
+          next = next < n_tiles ? next : -1;
+          if (n_meta == 2) fetch_meta(k + 1, next);
+          if (next >= 0) fetch_queries(k + 1, next);
+          if (training) tma_store_wait_read();
+          mbar_arrive(b_stored);
+          mbar_wait(b_staged, 1, &abort_flag, 115);
+          mbar_wait(b_roles + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 116);  // (of a tile without items nobody else waits for them)
+          if (n_meta == 1) fetch_meta(k + 1, next);
+          tma_store_4d(&tmo, smem_u32(q_tiles) + (k & 1) * C::kBigBytes, 0, row0, h, n);
+          if (training) tma_store_4d(&tmos, smem_u32(sl), 0, row0, h, n);
+          tma_store_commit();
+          tma_store_wait_read();
+          mbar_arrive(b_stored);
+          cur = next;
         }
-        __syncwarp();
       }
-    } else if (warp == kSoftmaxWarps + 1 && nI > 0) {
-      // ---- S(i) = Q K^T into buffer i % 2 once the products of item i - 2 have read that buffer ----
-      constexpr uint32_t idesc_s = instr_desc(128, 64, 0, 0);
-      const uint64_t dq = smem_desc(smem_u32(q_tile), 16, C::kAtomBytes, C::kSwizzle);
-      mbar_wait(b_res, 0, &abort_flag, 101);
-      for (int i = 0; i < nI; ++i) {
-        const int b = i & 1, ph = (i >> 1) & 1;
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 102);
-        if (i >= 2) mbar_wait(b_done + 8 * b, ph ^ 1, &abort_flag, 103);
-        tc_fence_after();
-        const uint64_t dk =
-            smem_desc(smem_u32(kv_tiles + (i % STAGES) * 2 * C::kSmallBytes), 16, C::kAtomBytes, C::kSwizzle);
-        const uint32_t ts = tmem_base + 64 * b;
-        if (elect_one()) {
+      __syncwarp();
+    } else {
+      int it = 0;              // items of the tiles before
+      int sj = 0, sph = 0;     // their stage and its phase
+      auto step = [&] { if (++sj == STAGES) { sj = 0; sph ^= 1; } };
+      for (int k = 0;; ++k) {
+        mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 113);
+        const int x = *(volatile int *)&tile_id[k & 1];
+        if (x < 0 || *(volatile int *)&abort_flag) break;
+        const uint8_t *meta = metas + (k & 1) * meta_step;
+        const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
+        const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
+        const int nL = counts[1], nI = nL + counts[2];
+        if (warp == kSoftmaxWarps) {
+          // ---- loader: K/V tiles, up to STAGES ahead of their consumers ----
+          const int u = tile_unit(x), n = unit_batch(u), hk = unit_head(u) / s.G;
+          for (int j = 0; j < nI; ++j, ++it, step()) {
+            const int row = (int)items[j] * 64;
+            if (it >= STAGES) mbar_wait(b_empty + 8 * sj, sph ^ 1, &abort_flag, 105);
+            const uint32_t bar = b_full + 8 * sj;
+            const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
+            if (elect_one()) {
+              mbar_expect_tx(bar, 2 * C::kSmallBytes);
+              tma_load_4d(kt, &tmk, bar, 0, row, hk, n);  // the key/value head of this query head
+              tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, hk, n);
+            }
+            __syncwarp();
+          }
+        } else if (warp == kSoftmaxWarps + 1) {
+          // ---- S(i) = Q K^T into buffer i % 2 once the products of item i - 2 have read that buffer ----
+          constexpr uint32_t idesc_s = instr_desc(128, 64, 0, 0);
+          const uint64_t dq = smem_desc(smem_u32(q_tiles) + (k & 1) * C::kBigBytes, 16, C::kAtomBytes, C::kSwizzle);
+          mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 101);
+          for (int i = 0; i < nI; ++i, ++it, step()) {
+            const int b = it & 1, ph = (it >> 1) & 1;
+            mbar_wait(b_full + 8 * sj, sph, &abort_flag, 102);
+            if (it >= 2) mbar_wait(b_done + 8 * b, ph ^ 1, &abort_flag, 103);
+            tc_fence_after();
+            const uint64_t dk = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes), 16, C::kAtomBytes, C::kSwizzle);
+            const uint32_t ts = tmem_base + 64 * b;
+            if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) umma_bf16(ts, dq + 2 * k, dk + 2 * k, idesc_s, k > 0);
-          umma_commit(b_sfull + 8 * b);
-        }
-        __syncwarp();
-      }
-    } else if (warp == kSoftmaxWarps + 2 && nI > 0) {
-      // ---- O_A += P(i)[:, 0:32] V[0:32], O_B += P(i)[:, 32:64] V[32:64] once that group's
-      // probabilities of item i are in tensor memory ----
-      constexpr uint32_t idesc_pv = instr_desc(128, D, 0, 1);
-      for (int i = 0; i < nI; ++i) {
-        const int b = i & 1, ph = (i >> 1) & 1;
-        const uint64_t dv = smem_desc(smem_u32(kv_tiles + (i % STAGES) * 2 * C::kSmallBytes + C::kSmallBytes),
-                                      C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
-        const uint32_t tp = tmem_base + 64 * b;
-        const uint32_t first = (i == 0 || i == nL) ? 0u : 1u;  // a phase starts the accumulators afresh
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 106);
-        mbar_wait(b_tfull + 8 * b, ph, &abort_flag, 104);
-        tc_fence_after();
-        if (elect_one()) {
+              for (int c = 0; c < D / 16; ++c) umma_bf16(ts, dq + 2 * c, dk + 2 * c, idesc_s, c > 0);
+              umma_commit(b_sfull + 8 * b);
+            }
+            __syncwarp();
+          }
+        } else {
+          // ---- O_A += P(i)[:, 0:32] V[0:32], O_B += P(i)[:, 32:64] V[32:64] once that group's
+          // probabilities of item i are in tensor memory ----
+          constexpr uint32_t idesc_pv = instr_desc(128, D, 0, 1);
+          for (int i = 0; i < nI; ++i, ++it, step()) {
+            const int b = it & 1, ph = (it >> 1) & 1;
+            const uint64_t dv = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes + C::kSmallBytes),
+                                          C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
+            const uint32_t tp = tmem_base + 64 * b;
+            const uint32_t first = (i == 0 || i == nL) ? 0u : 1u;  // a phase starts the accumulators afresh
+            mbar_wait(b_full + 8 * sj, sph, &abort_flag, 106);
+            mbar_wait(b_tfull + 8 * b, ph, &abort_flag, 104);
+            tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < 2; ++k)
-            umma_bf16_ts(tmem_oa, tp + 8 * k, dv + k * C::kKStep, idesc_pv, (first | (uint32_t)k) != 0u);
-        }
-        __syncwarp();
-        mbar_wait(b_tfull + 8 * (2 + b), ph, &abort_flag, 109);
-        tc_fence_after();
-        if (elect_one()) {
+              for (int c = 0; c < 2; ++c)
+                umma_bf16_ts(tmem_oa, tp + 8 * c, dv + c * C::kKStep, idesc_pv, (first | (uint32_t)c) != 0u);
+            }
+            __syncwarp();
+            mbar_wait(b_tfull + 8 * (2 + b), ph, &abort_flag, 109);
+            tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < 2; ++k)
-            umma_bf16_ts(tmem_ob, tp + 32 + 8 * k, dv + (2 + k) * C::kKStep, idesc_pv, (first | (uint32_t)k) != 0u);
-          umma_commit(b_done + 8 * b);
-          umma_commit(b_empty + 8 * (i % STAGES));  // S(i) completed before the softmax warps read it
+              for (int c = 0; c < 2; ++c)
+                umma_bf16_ts(tmem_ob, tp + 32 + 8 * c, dv + (2 + c) * C::kKStep, idesc_pv, (first | (uint32_t)c) != 0u);
+              umma_commit(b_done + 8 * b);
+              umma_commit(b_empty + 8 * sj);  // S(i) completed before the softmax warps read it
+            }
+            __syncwarp();
+          }
         }
-        __syncwarp();
+        warp_arrive(b_roles + 8 * (k & 1), lane);  // done with the lists
       }
     }
   } else {
     // ================================ softmax =================================
     setmaxnreg_inc<kSoftmaxRegs>();
     const int quarter = warp & 3, grp = warp >> 2;  // TMEM lane quarter; key half of every tile
-    const int r = quarter * 32 + lane, t = PACK ? row0 + (r & 63) : row0 + r, g = r / s.Bk;
-    const int hr = PACK ? h + (r >> 6) : h;  // this row's head
-    const bool row_ok = t < s.L;
+    const int r = quarter * 32 + lane, g = r / s.Bk;
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const uint32_t acc_own = (grp ? tmem_ob : tmem_oa) + lane_off;
-    float m = -INFINITY, l = 0.f;  // this group's running maximum (log2 units) and sum of the row
-    float lseL = 0.f, lseS = 0.f;
-    bool haveL = false, haveS = false;
-    int acc = 0;  // the current phase has written the accumulators
     const float sc2 = s.scale * kLog2e;
-    const float alpha = gate_alpha(gate, hr), beta = 1.f - alpha;
-    int jt_n = nI > 0 ? items[0] : 0, cls_n = nI > 0 ? icls[quarter] : 0;
-    uint8_t *so = kv_tiles, *ss = so + C::kBigBytes;  // staging of out / out_st (the K/V stages, free by then)
+    int it = 0;  // items of the tiles before
+    for (int k = 0;; ++k) {
+      if (warp == 0) {  // one warp decides for all: the named barriers below need every one of them
+        mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 117);
+        if (lane == 0) softmax_tile = *(volatile int *)&abort_flag ? -1 : *(volatile int *)&tile_id[k & 1];
+      }
+      named_bar_sync(2, kSoftmaxWarps * 32);
+      const int x = *(volatile int *)&softmax_tile;
+      if (x < 0) break;
+      mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 120);  // (complete: makes the lists visible to this warp)
+      const uint8_t *meta = metas + (k & 1) * meta_step;
+      const uint8_t *selb = meta;
+      const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
+      const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
+      const uint8_t *icls = meta + ml.icls;                                         // [2 nT][4]
+      const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
+      const int nL = counts[1], nI = nL + counts[2];
+      const int u = tile_unit(x), n = unit_batch(u);
+      const int pad0 = s.L - min(max(seq_lens ? seq_lens[n] : s.L, 0), s.L);
+      const int t = tile_row0(x) + (PACK ? r & 63 : r);
+      const int hr = unit_head(u) + (PACK ? r >> 6 : 0);  // this row's head
+      const bool row_ok = t < s.L;
+      float m = -INFINITY, l = 0.f;  // this group's running maximum (log2 units) and sum of the row
+      const float alpha = gate_alpha(gate, hr), beta = 1.f - alpha;
+      int jt_n = nI > 0 ? items[0] : 0, cls_n = nI > 0 ? icls[quarter] : 0;
+      uint8_t *so = q_tiles + (k & 1) * C::kBigBytes;  // the gate mix is staged over the queries, free by then
 
-    // End of a phase: the two groups' halves of every row are merged (maxima, sums, accumulators),
-    // normalised, and this thread's DC columns are staged: the long-term rows into sl; at the very
-    // end the short-term rows and the gate mix (Eq. 19) into ss and so, the long-term rows being
-    // read back from sl.  The caller has waited for the phase's last products.
-    auto merge = [&](bool long_term, bool final_phase) {
-      stat[grp][r] = make_float2(m, l);
-      named_bar_sync(1, kSoftmaxWarps * 32);
-      const float2 oth = stat[grp ^ 1][r];
-      const float mt = fmaxf(m, oth.x);
-      const float fo = l > 0.f ? exp2f(m - mt) : 0.f, fp = oth.y > 0.f ? exp2f(oth.x - mt) : 0.f;
-      const float lt = l * fo + oth.y * fp;
-      const float inv = (lt > 0.f && row_ok && t >= pad0) ? 1.f / lt : 0.f;
-      const float fa = (grp ? fp : fo) * inv, fb = (grp ? fo : fp) * inv;
-      const float lse_v = lt > 0.f ? (mt + log2f(lt)) * kLn2 : 0.f;
-      if (long_term) { lseL = lse_v; haveL = lt > 0.f; } else { lseS = lse_v; haveS = lt > 0.f; }
+      // End of a phase: the two groups' halves of every row are merged (maxima, sums, accumulators),
+      // normalised, and this thread's DC columns are staged: the long-term rows into sl; at the end of the
+      // short-term phase, which finds the long-term rows there, its rows into sl and the gate mix (Eq. 19)
+      // into so.  The caller has waited for the phase's last products and for sl to be free.
+      auto merge = [&](bool final_phase) {
+        stat[grp][r] = make_float2(m, l);
+        named_bar_sync(1, kSoftmaxWarps * 32);
+        const float2 oth = stat[grp ^ 1][r];
+        const float mt = fmaxf(m, oth.x);
+        const float fo = l > 0.f ? exp2f(m - mt) : 0.f, fp = oth.y > 0.f ? exp2f(oth.x - mt) : 0.f;
+        const float lt = l * fo + oth.y * fp;
+        const float inv = (lt > 0.f && row_ok && t >= pad0) ? 1.f / lt : 0.f;
+        const float fa = (grp ? fp : fo) * inv, fb = (grp ? fo : fp) * inv;
+        if (grp == 0 && row_ok && lse)
+          lse[((int64_t)((final_phase ? s.B : 0) + n) * s.H + hr) * s.L + t] = lt > 0.f ? (mt + log2f(lt)) * kLn2 : 0.f;
 #pragma unroll
-      for (int c0 = 0; c0 < DC; c0 += 16) {
-        float a[16], b[16];
-        tmem_ld16(tmem_oa + lane_off + DC * grp + c0, a);
-        tmem_ld16(tmem_ob + lane_off + DC * grp + c0, b);
-        tmem_wait_ld();
+        for (int c0 = 0; c0 < DC; c0 += 16) {
+          float a[16], b[16];
+          tmem_ld16(tmem_oa + lane_off + DC * grp + c0, a);
+          tmem_ld16(tmem_ob + lane_off + DC * grp + c0, b);
+          tmem_wait_ld();
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-          const int chunk = (DC * grp + c0) / 8 + ch;
-          float o[8];
+          for (int ch = 0; ch < 2; ++ch) {
+            const int chunk = (DC * grp + c0) / 8 + ch;
+            float o[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) o[e] = inv > 0.f ? a[ch * 8 + e] * fa + b[ch * 8 + e] * fb : 0.f;
-          if (long_term || nL == 0) {  // (no long-term phase at all: its rows are zeros)
+            for (int e = 0; e < 8; ++e) o[e] = inv > 0.f ? a[ch * 8 + e] * fa + b[ch * 8 + e] * fb : 0.f;
+            if (final_phase) {
+              const uint4 w = load_row_chunk<D>(sl, r, chunk);
+              const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+              uint32_t wo[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                wo[e] = pack_bf16(alpha * __uint_as_float(ww[e] << 16) + beta * o[2 * e],
+                                  alpha * __uint_as_float(ww[e] & 0xffff0000u) + beta * o[2 * e + 1]);
+              store_row_chunk<D>(so, r, chunk, make_uint4(wo[0], wo[1], wo[2], wo[3]));
+            }
             store_row_chunk<D>(sl, r, chunk, make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]),
                                                          pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7])));
           }
-          if (final_phase) {
-            float oL[8], oS[8];
-            if (long_term) {  // (no short-term items at all: the long-term rows are the last phase)
-#pragma unroll
-              for (int e = 0; e < 8; ++e) { oL[e] = o[e]; oS[e] = 0.f; }
-            } else {
-              const uint4 w = nL > 0 ? load_row_chunk<D>(sl, r, chunk) : make_uint4(0u, 0u, 0u, 0u);
-              const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                oL[2 * e] = __uint_as_float(ww[e] << 16);
-                oL[2 * e + 1] = __uint_as_float(ww[e] & 0xffff0000u);
-                oS[2 * e] = o[2 * e];
-                oS[2 * e + 1] = o[2 * e + 1];
-              }
-            }
-            uint32_t wo[4], ws[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              wo[e] = pack_bf16(alpha * oL[2 * e] + beta * oS[2 * e], alpha * oL[2 * e + 1] + beta * oS[2 * e + 1]);
-              ws[e] = pack_bf16(oS[2 * e], oS[2 * e + 1]);
-            }
-            store_row_chunk<D>(so, r, chunk, make_uint4(wo[0], wo[1], wo[2], wo[3]));
-            store_row_chunk<D>(ss, r, chunk, make_uint4(ws[0], ws[1], ws[2], ws[3]));
-          }
         }
-      }
-    };
-
-    for (int i = 0; i < nI; ++i) {
-      const bool isL = i < nL;
-      const int jt = jt_n, cls = cls_n, p0 = jt * 64;
-      if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
-        jt_n = items[i + 1];
-        cls_n = icls[(i + 1) * 4 + quarter];
-      }
-      const int b = i & 1, ph = (i >> 1) & 1;
-      const uint32_t b_prev = b_done + 8 * (b ^ 1), ph_prev = ((i - 1) >> 1) & 1;  // item i-1
-      if (i == nL && nL > 0) {
-        // End of the long-term phase: merge and stage its rows; the first products of the
-        // short-term phase overwrite the accumulators.
-        mbar_wait(b_prev, ph_prev, &abort_flag, 111);
-        __syncwarp();
-        tc_fence_after();
-        merge(true, false);
+        fence_async_smem();
         tc_fence_before();
-        // Both groups read both accumulators in the merge, and the first product of the next phase
-        // overwrites an accumulator as soon as ITS group has stored the next probabilities: no
-        // warp may go on before every warp has read.
+        warp_arrive(b_staged, lane);
+        // Both groups read both accumulators above, and the first product of the next phase (or tile)
+        // overwrites an accumulator as soon as ITS group has stored the next probabilities: no warp may go
+        // on before every warp has read.
         named_bar_sync(3, kSoftmaxWarps * 32);
         m = -INFINITY;
         l = 0.f;
-        acc = 0;
-      }
-      uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
-      bool doB = cls == 1, fullB = cls == 1;
-      if (cls == 2) {
-        if (row_ok && (causal || t >= pad0)) {  // (a padded row sees nothing; under the causal mask the bounds below say so)
-          uint64_t mask = cols_le((causal ? t : s.L - 1) - p0) & cols_ge(pad0 - p0);
-          mask &= isL ? expand_block_bits(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk) : st_key_cols(s, t, p0, causal);
-          hm = (uint32_t)(mask >> (32 * grp));
-        }
-        doB = __any_sync(0xffffffffu, hm != 0u);
-        fullB = __all_sync(0xffffffffu, hm == 0xffffffffu);
-      }
-      const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
+      };
+      // the products of the item before `it` (of either phase) have completed
+      auto products_done = [&](int site) {
+        mbar_wait(b_done + 8 * ((it - 1) & 1), ((it - 1) >> 1) & 1, &abort_flag, site);
+        __syncwarp();
+        tc_fence_after();
+      };
+      auto end_long_term = [&] {
+        if (nL > 0) products_done(111);
+        mbar_wait(b_stored, 1, &abort_flag, 118);  // sl: the tile before has been stored (at once for the first)
+        merge(false);
+      };
 
-      mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 107);
-      __syncwarp();
-      tc_fence_after();
-      uint32_t pk[16];
-      if (doB) {
-        float sv[32];
-        tmem_ld32(t_b, sv);
-        tmem_wait_ld();
-        float fac = 1.f;
-        const float mt = (fullB ? half_row_max<true>(sv, 0u) : half_row_max<false>(sv, hm)) * sc2;
-        const bool need = mt > m + kRescaleThreshold;  // also true on the row's first keys
-        if (need) {
-          fac = exp2f(m - mt);
-          l *= fac;
-          m = mt;
+      for (int i = 0; i < nI; ++i, ++it) {
+        const bool isL = i < nL;
+        const int jt = jt_n, cls = cls_n, p0 = jt * 64;
+        if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
+          jt_n = items[i + 1];
+          cls_n = icls[(i + 1) * 4 + quarter];
         }
-        if (fullB) half_row_probs<true>(sv, 0u, sc2, -m, l, pk);
-        else half_row_probs<false>(sv, hm, sc2, -m, l, pk);
-        if (acc && __any_sync(0xffffffffu, need)) {  // rescaling needs the products of item i-1
-          mbar_wait(b_prev, ph_prev, &abort_flag, 108);
-          __syncwarp();
-          tc_fence_after();
-          rescale_acc<D>(acc_own, fac);
+        const int b = it & 1, ph = (it >> 1) & 1;
+        if (i == nL) end_long_term();
+        uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
+        bool doB = cls == 1, fullB = cls == 1;
+        if (cls == 2) {
+          if (row_ok && (causal || t >= pad0)) {  // (a padded row sees nothing; under the causal mask the bounds below say so)
+            uint64_t mask = cols_le((causal ? t : s.L - 1) - p0) & cols_ge(pad0 - p0);
+            mask &= isL ? expand_block_bits(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk) : st_key_cols(s, t, p0, causal);
+            hm = (uint32_t)(mask >> (32 * grp));
+          }
+          doB = __any_sync(0xffffffffu, hm != 0u);
+          fullB = __all_sync(0xffffffffu, hm == 0xffffffffu);
         }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) pk[c] = 0u;
-      }
-      tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
-      tmem_wait_st();
-      tc_fence_before();
-      warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
-      acc = 1;
-    }
+        const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
 
-    // ---- epilogue ----
-    if (nI > 0) {
-      mbar_wait(b_done + 8 * ((nI - 1) & 1), ((nI - 1) >> 1) & 1, &abort_flag, 110);
-      __syncwarp();
-      tc_fence_after();
-      merge(nS == 0, true);
-    } else {
+        mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 107);
+        __syncwarp();
+        tc_fence_after();
+        uint32_t pk[16];
+        if (doB) {
+          float sv[32];
+          tmem_ld32(t_b, sv);
+          tmem_wait_ld();
+          float fac = 1.f;
+          const float mt = (fullB ? half_row_max<true>(sv, 0u) : half_row_max<false>(sv, hm)) * sc2;
+          const bool need = mt > m + kRescaleThreshold;  // also true on the row's first keys, before which
+          const bool scale_acc = need && l > 0.f;        // the accumulator holds sums of zero probabilities
+          if (need) {
+            fac = exp2f(m - mt);
+            l *= fac;
+            m = mt;
+          }
+          if (fullB) half_row_probs<true>(sv, 0u, sc2, -m, l, pk);
+          else half_row_probs<false>(sv, hm, sc2, -m, l, pk);
+          if (__any_sync(0xffffffffu, scale_acc)) {  // rescaling needs the products of item i-1
+            products_done(108);
+            rescale_acc<D>(acc_own, fac);
+          }
+        } else {
 #pragma unroll
-      for (int ch = 0; ch < DC / 8; ++ch) {
-        const int chunk = DC * grp / 8 + ch;
-        store_row_chunk<D>(so, r, chunk, make_uint4(0u, 0u, 0u, 0u));
-        store_row_chunk<D>(sl, r, chunk, make_uint4(0u, 0u, 0u, 0u));
-        store_row_chunk<D>(ss, r, chunk, make_uint4(0u, 0u, 0u, 0u));
+          for (int c = 0; c < 16; ++c) pk[c] = 0u;
+        }
+        tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
+        tmem_wait_st();
+        tc_fence_before();
+        warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
       }
-    }
-    // Whole-line bulk stores of the staged rows; rows past L are clipped by the hardware, padded
-    // rows were staged as zeros.
-    fence_async_smem();
-    named_bar_sync(2, kSoftmaxWarps * 32);
-    if (tid == 0) {
-      tma_store_4d(&tmo, smem_u32(so), 0, row0, h, n);
-      if (training) {
-        tma_store_4d(&tmol, smem_u32(sl), 0, row0, h, n);
-        tma_store_4d(&tmos, smem_u32(ss), 0, row0, h, n);
-      }
-      tma_store_commit_and_wait();
-    }
-    if (grp == 0 && row_ok && lse) {
-      const int64_t BHL = (int64_t)s.B * s.H * s.L;
-      const int64_t row = ((int64_t)n * s.H + hr) * s.L + t;
-      lse[row] = haveL ? lseL : 0.f;
-      lse[BHL + row] = haveS ? lseS : 0.f;
+
+      if (nI == 0) mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 112);  // (nothing else waited for the queries)
+      if (nL == nI) end_long_term();
+      if (nI > nL) products_done(110);
+      mbar_wait(b_stored, 0, &abort_flag, 119);  // sl: the long-term rows have been stored
+      merge(true);
     }
   }
-  if (nI == 0 && tid == 0) mbar_wait(b_res, 0, &abort_flag, 112);  // no load may outlive the CTA
   finish(warp, tmem_base, kFwdTmemCols, &abort_flag, status);
 }
 
@@ -487,20 +532,27 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
       make_tensor_map(&tos, training ? out_st : out, s, qrows, false, qheads))
     return BLOSSOM_ERR_CUDA;
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
-  const size_t smem = 1024 + 2 * C::kBigBytes + kFwdStages * 2 * C::kSmallBytes + meta_bytes(nT, s.pq);
+  // Two CTAs share an SM (228 KB with 1 KB for each and its static part): a second buffer for the lists as long
+  // as that stays so.
+  const size_t tiles = 1024 + 3 * C::kBigBytes + fwd_stages(D) * 2 * C::kSmallBytes, list = meta_bytes(nT, s.pq);
+  const size_t kPair = 110 * 1024;
+  const int n_meta = tiles + 2 * list <= kPair ? 2 : 1;
+  const size_t smem = tiles + n_meta * list;
   const bool plain = s.causal && !s.pq;
   auto kern = s.pack ? (plain ? fwd_tc_kernel<D, true, true> : fwd_tc_kernel<D, false, true>)
                      : (plain ? fwd_tc_kernel<D, true, false> : fwd_tc_kernel<D, false, false>);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
-  const unsigned grid = s.pack ? (unsigned)nT * (unsigned)(s.B * (s.H / 2)) : (unsigned)nST * (unsigned)(s.B * s.H);
+  const int n_tiles = s.pack ? nT * (s.B * (s.H / 2)) : nST * (s.B * s.H);
+  const int resident = 148 * (smem <= kPair ? 2 : 1);
+  const unsigned grid = (unsigned)(n_tiles < resident ? n_tiles : resident);
   // A training call also builds the backward's tile lists (the same launch: one warp per image):
   // a backward call told to reuse them (blossom_params::reuse_tile_lists) then builds none.
-  if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training ? ws.kmeta : nullptr, st, 3, 1)) return rc;
+  if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training ? ws.kmeta : nullptr, st, ws.status + kTicketWord, 3, 1)) return rc;
   {
     LaunchScope ls(K_FWD_TC, st);
     launch_chained(kern, dim3(grid), dim3(kFwdThreads), smem, st, tq, tk, tv, to, tol, tos, s, gate, seq_lens,
-                   (const uint8_t *)ws.qmeta, training, lse, ws.status, nT);
+                   (const uint8_t *)ws.qmeta, training, lse, ws.status, ws.status + kTicketWord, nT, n_tiles, n_meta);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

@@ -46,8 +46,10 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                                                                   uint8_t *__restrict__ kmeta, int nT,
                                                                   int n_query_ctas, int image0, int image_end,
                                                                   int branches, int with_fwd,
-                                                                  uint32_t *__restrict__ inv_bits) {
+                                                                  uint32_t *__restrict__ inv_bits,
+                                                                  int32_t *__restrict__ tickets) {
   grid_chain_enter();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *tickets = 0;  // of the persistent kernel behind
   constexpr int NT = 32 * NW;  // threads per image
   auto sync = [] {
     if (NW == 1) __syncwarp();
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
 }  // namespace
 
 int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, uint8_t *qmeta,
-                   uint8_t *kmeta, cudaStream_t st, int branches, int with_fwd) {
+                   uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches, int with_fwd) {
   if (with_fwd < 0) with_fwd = kmeta == nullptr;
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
@@ -438,7 +440,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   auto launch = [&](int image0, int image_end, uint32_t *inv_bits) {
     LaunchScope ls(K_TC_META, st);
     launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,
-                   seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits);
+                   seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits, tickets);
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it

@@ -111,9 +111,12 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, uint32_t sr
       "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// the shared memory of every committed store of this thread has been read
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_commit_and_wait() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  tma_store_commit();
+  tma_store_wait_read();
 }
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -502,8 +505,9 @@ int make_tensor_map(CUtensorMap *map, const void *base, const Shape &s, int box_
 // with_fwd: 1 = the query-major images carry the forward's items, 0 = not, -1 = only when no
 // key-major images are asked for (a forward call builds the forward's part, a backward call the
 // rest; a training forward may build everything at once for a backward that reuses it).
+constexpr int kTicketWord = 20;  // word of the status area: tiles the CTAs of a persistent kernel have taken
 int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, uint8_t *qmeta,
-                   uint8_t *kmeta, cudaStream_t st, int branches = 3, int with_fwd = -1);
+                   uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches = 3, int with_fwd = -1);
 
 // per-file launchers behind launch_fwd_tc / launch_bwd_tc
 template <int D>
