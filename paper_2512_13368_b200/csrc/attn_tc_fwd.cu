@@ -382,6 +382,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       const int t = tile_row0(x) + (PACK ? r & 63 : r);
       const int hr = unit_head(u) + (PACK ? r >> 6 : 0);  // this row's head
       const bool row_ok = t < s.L;
+      // the last key this row may see (a padded row sees nothing; under the causal mask its keys lie behind t)
+      const int t_last = row_ok && (causal || t >= pad0) ? (causal ? t : s.L - 1) : -1;
       float m = -INFINITY, l = 0.f;  // this group's running maximum (log2 units) and sum of the row
       const float alpha = gate_alpha(gate, hr), beta = 1.f - alpha;
       int jt_n = nI > 0 ? items[0] : 0, cls_n = nI > 0 ? icls[quarter] : 0;
@@ -462,11 +464,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
         bool doB = cls == 1, fullB = cls == 1;
         if (cls == 2) {
-          if (row_ok && (causal || t >= pad0)) {  // (a padded row sees nothing; under the causal mask the bounds below say so)
-            uint64_t mask = cols_le((causal ? t : s.L - 1) - p0) & cols_ge(pad0 - p0);
-            mask &= isL ? expand_block_bits(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk) : st_key_cols(s, t, p0, causal);
-            hm = (uint32_t)(mask >> (32 * grp));
-          }
+          const int c0 = p0 + 32 * grp;
+          hm = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
+          if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, 32 * grp);
+          else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> (32 * grp)) : st_window32(s, t, c0, causal);
           doB = __any_sync(0xffffffffu, hm != 0u);
           fullB = __all_sync(0xffffffffu, hm == 0xffffffffu);
         }

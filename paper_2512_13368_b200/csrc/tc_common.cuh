@@ -356,6 +356,21 @@ __device__ __forceinline__ uint64_t expand_block_bits(uint32_t bits, int bk) {
 // the smallest power of two >= x (1 for x <= 1)
 __device__ __forceinline__ int pow2_at_least(int x) { return x <= 1 ? 1 : 1 << (32 - __clz(x - 1)); }
 
+// ---- 32-column masks (half the instructions; shifts clamp at 32) ----------------------------
+__device__ __forceinline__ uint32_t cols32_ge(int lo) {  // columns c >= lo
+  uint32_t m;
+  asm("shl.b32 %0, 0xffffffff, %1;" : "=r"(m) : "r"(max(lo, 0)));
+  return m;
+}
+__device__ __forceinline__ uint32_t cols32_le(int hi) { return ~cols32_ge(hi + 1); }  // columns c <= hi
+// expand_block_bits for the 32 columns from column c0 (a multiple of 16) of the tile: bits past the tile's
+// 64 columns are not asked for
+__device__ __forceinline__ uint32_t expand_block_bits32(uint32_t bits, int bk, int c0) {
+  if (bk >= 32) return ((bits >> (c0 / bk)) & 1u) ? 0xffffffffu : 0u;  // (16 columns from 16: the low ones count)
+  const uint32_t b = bits >> (c0 >> 4);
+  return ((b & 1u) ? 0xffffu : 0u) | ((b & 2u) ? 0xffff0000u : 0u);
+}
+
 // Short-term mask of Eq. 15 over the 64 keys p0 ... p0 + 63 for query t, without the causal and
 // the padding condition (the caller ANDs those): the window, and with the power-law mask the key
 // blocks at power-of-two block distances and the last block.  `causal` is the caller's (often
@@ -383,6 +398,12 @@ __device__ __forceinline__ uint64_t st_key_cols(const Shape &s, int t, int p0, b
       }
     }
   }
+  return m;
+}
+// The window's part of it over 32 keys (all of it with stis_mode = 0)
+__device__ __forceinline__ uint32_t st_window32(const Shape &s, int t, int p0, bool causal) {
+  uint32_t m = cols32_ge(t - s.window + 1 - p0);
+  if (!causal) m &= cols32_le(t + s.window - 1 - p0);
   return m;
 }
 // The same mask seen from key p over the 64 queries t0 ... t0 + 63 (again without causality and
