@@ -109,7 +109,7 @@ typedef struct {
                         * broadcast over the head's channels in Eq. 19.  The out_lt, out_st that
                         * enter F_o are the rows as stored (bf16 roundings for bf16 tensors on
                         * the tensor-core kernels, which then run the backward once per branch
-                        * and need about seven q-sized scratch tensors in the workspace)          */
+                        * and need about four q-sized scratch tensors in the workspace)           */
   float rope_theta;    /* 0 = q and k are used as given.  > 0 (>= 1, e.g. 10000): rotary position
                         * embedding inside the library: q and k are rotated by position before the
                         * selection and both branches (pairs (x[2i], x[2i+1]), angle

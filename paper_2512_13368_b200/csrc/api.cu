@@ -111,15 +111,13 @@ Workspace carve_workspace(const Shape &s, void *base) {
     // input-dependent gate on the tensor-core kernels (bf16): scratch tensors of the two passes
     const bool on = s.gate_mode && s.esz == 2;
     const size_t qspan = (size_t)((s.B - 1) * s.sb + (s.H - 1) * s.sh + (int64_t)(s.L - 1) * s.sl + s.D);
-    const size_t kspan = (size_t)((s.B - 1) * s.ksb + (s.Hkv - 1) * s.ksh + (int64_t)(s.L - 1) * s.ksl + s.D);
     w.gate_glt = take(on ? qspan * 2 : 0);
     w.gate_gst = take(on ? qspan * 2 : 0);
-    w.gate_dq = take(on ? qspan * 2 : 0);
     w.gate_olt = take(on ? qspan * 2 : 0);
     w.gate_ost = take(on ? qspan * 2 : 0);
-    w.gate_dk = take(on ? kspan * 2 : 0);
-    w.gate_dv = take(on ? kspan * 2 : 0);
     w.qstats2 = reinterpret_cast<float4 *>(take(on ? units * (size_t)((s.L + 63) / 64 * 64) * sizeof(float4) : 0));
+    w.qmeta2 = reinterpret_cast<uint8_t *>(take(on ? tc::tc_meta_bytes(s) : 0));
+    w.kmeta2 = reinterpret_cast<uint8_t *>(take(on ? tc::tc_meta_bytes(s) + tc::tc_inv_bits_bytes(s) : 0));
   }
   w.qmeta = reinterpret_cast<uint8_t *>(take(tc::tc_meta_bytes(s)));
   w.kmeta = reinterpret_cast<uint8_t *>(take(tc::tc_meta_bytes(s) + tc::tc_inv_bits_bytes(s)));

@@ -570,21 +570,24 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(Shape s, const float *__
 // over batch entries and query blocks in a fixed order.  One warp per (head, parameter): lane i
 // adds the entries i, i + 32, ... in ascending order, then a fixed shuffle tree joins the lanes.
 __global__ void __launch_bounds__(256) gate_param_grad_kernel(Shape s, const double *__restrict__ part,
-                                                              float *__restrict__ dgate) {
-  grid_chain_enter();
+                                                              float *__restrict__ dgate, int beside) {
+  if (beside) grid_release();  // beside the kernel before it, which has waited for what this one reads
+  else grid_chain_enter();
   const int GW = 2 * s.D + 1;
   const int w = (int)blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (w >= s.H * GW) return;
-  const int h = w / GW, d = w % GW, n_entries = s.B * s.M;
-  double a = 0.0;
+  if (w < s.H * GW) {
+    const int h = w / GW, d = w % GW, n_entries = s.B * s.M;
+    double a = 0.0;
 #pragma unroll 16
-  for (int e = lane; e < n_entries; e += 32) {
-    const int n = e / s.M, qb = e % s.M;
-    a += part[(((int64_t)n * s.H + h) * s.M + qb) * GW + d];
-  }
+    for (int e = lane; e < n_entries; e += 32) {
+      const int n = e / s.M, qb = e % s.M;
+      a += part[(((int64_t)n * s.H + h) * s.M + qb) * GW + d];
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  if (lane == 0) dgate[(int64_t)h * GW + d] = (float)a;
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) dgate[(int64_t)h * GW + d] = (float)a;
+  }
+  if (beside && threadIdx.x == 0) grid_wait();
 }
 
 namespace {
@@ -640,7 +643,7 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
   }
   if (s.gate_mode) {
     LaunchScope ls(K_GATE_GRAD, st);
-    gate_param_grad_kernel<<<(unsigned)((s.H * (2 * s.D + 1) + 7) / 8), 256, 0, st>>>(s, ws.dgate_part, dgate);
+    gate_param_grad_kernel<<<(unsigned)((s.H * (2 * s.D + 1) + 7) / 8), 256, 0, st>>>(s, ws.dgate_part, dgate, 0);
     return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
   }
   return launch_gate_grad(s, gate, ws, dgate, st);
@@ -648,11 +651,11 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
 
 }  // namespace
 
-int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st) {
+int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st, int beside) {
   {
     LaunchScope ls(K_GATE_GRAD, st);
     launch_chained(gate_param_grad_kernel, dim3((unsigned)((s.H * (2 * s.D + 1) + 7) / 8)), dim3(256), 0, st, s,
-                   (const double *)ws.dgate_part, dgate);
+                   (const double *)ws.dgate_part, dgate, beside);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

@@ -124,6 +124,16 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(Shape s, const float *__r
   }
 }
 
+// eight bf16 of a row += the eight at p (of the pass before), one rounding
+__device__ __forceinline__ void add_row_chunk(uint32_t (&w)[4], const __nv_bfloat16 *p) {
+  const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
+  const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    w[e] = pack_bf16(__uint_as_float(w[e] << 16) + __uint_as_float(x[e] << 16),
+                     __uint_as_float(w[e] & 0xffff0000u) + __uint_as_float(x[e] & 0xffff0000u));
+}
+
 // ---------------------------------------------------------------------------- backward dQ
 // 16 columns of one tile for one row: dS packed to bf16 pairs, partial sums of P' dP.
 // nlL / nlS = -(lse * log2e - log2 alpha) resp. beta: the branch weight rides in the exponent, so
@@ -162,21 +172,24 @@ __device__ __forceinline__ void dq_tile(const float (&sv)[16], const float (&dp)
   }
 }
 
-// PLAIN (both kernels below): the causal mask, one selection per query block and both branches: the other
-// modes' tests fold away at compile time, and a masked tile is taken for both branches at once (tiles
+// MODE of both kernels below.  kPlain: the causal mask, one selection per query block and both branches: the
+// other modes' tests fold away at compile time, and a masked tile is taken for both branches at once (tiles
 // with the masks of one branch only are rare there, and the code for them cost 2 %; in the other modes
 // it saves 5 - 12 %: selection per position, L 1500: dQ 63 -> 55 us, dK/dV 76 -> 72 us; a pass for one
-// branch of a gate that depends on the input: 27 -> 25 us).
+// branch of a gate that depends on the input: 27 -> 25 us).  kPass: a pass for one branch, the second of
+// which adds to what the first has written.
+constexpr int kGeneral = 0, kPlain = 1, kPass = 2;
 // PACK (dQ kernel): rows 0..63 and 64..127 of the CTA are the same 64 positions of two query heads
 // with a common key/value head, as in the forward kernel.
-template <int D, bool PLAIN, bool PACK>
+template <int D, int MODE, bool PACK>
 __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
     const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
     const uint8_t *__restrict__ qmeta, const __grid_constant__ CUtensorMap tmdq,
     const float4 *__restrict__ qstats, double *__restrict__ dalpha_part, int32_t *__restrict__ status,
-    int nT) {
+    int nT, const __nv_bfloat16 *add_dq) {
+  constexpr bool PLAIN = MODE == kPlain, ADDS = MODE == kPass;
   grid_wait();
   grid_release();  // (the dK/dV kernel depends on nothing of this one)
   using C = Cfg<D>;
@@ -451,6 +464,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
           const int c = ch * 8 + e * 2;
           w[e] = live ? pack_bf16(o[c] * s.scale, o[c + 1] * s.scale) : 0u;
         }
+        if (ADDS && add_dq && live) add_row_chunk(w, add_dq + row_offset(s, n, hr, t) + half * OC + ch * 8);
         store_row_chunk<D>(kv_tiles, r, half * (OC / 8) + ch, make_uint4(w[0], w[1], w[2], w[3]));
       }
       fence_async_smem();
@@ -560,15 +574,16 @@ __device__ __forceinline__ void reduce_gate(const Shape &s, const float *gate, c
   }
 }
 
-template <int D, bool PLAIN>
+template <int D, int MODE>
 __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
     const int32_t *__restrict__ seq_lens, const uint8_t *__restrict__ kmeta,
     const float4 *__restrict__ qstats, const __grid_constant__ CUtensorMap tmdk,
     const __grid_constant__ CUtensorMap tmdv, int32_t *__restrict__ status, int nT, int hs,
-    __nv_bfloat16 *__restrict__ dk, __nv_bfloat16 *__restrict__ dv, const float *__restrict__ gate,
-    const double *__restrict__ dalpha_part, float *__restrict__ dgate) {
+    __nv_bfloat16 *dk, __nv_bfloat16 *dv, const float *__restrict__ gate,
+    const double *__restrict__ dalpha_part, float *__restrict__ dgate, int accumulate) {
+  constexpr bool PLAIN = MODE == kPlain, ADDS = MODE == kPass;
   using C = Cfg<D>;
   constexpr int STAGES = kKvStages;
   constexpr int OC = D / 2;
@@ -843,6 +858,11 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
           wv[e] = live ? pack_bf16(ov[c], ov[c + 1]) : 0u;
           wk[e] = live ? pack_bf16(okk[c] * s.scale, okk[c + 1] * s.scale) : 0u;
         }
+        if (ADDS && accumulate && live) {
+          const int64_t off = row_offset_kv(s, n, hk, p) + half * OC + ch * 8;
+          add_row_chunk(wv, dv + off);
+          add_row_chunk(wk, dk + off);
+        }
         store_row_chunk<D>(sv_t, r, half * (OC / 8) + ch, make_uint4(wv[0], wv[1], wv[2], wv[3]));
         store_row_chunk<D>(sk_t, r, half * (OC / 8) + ch, make_uint4(wk[0], wk[1], wk[2], wk[3]));
       }
@@ -876,9 +896,11 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
           x[0] += a.x; x[1] += a.y; x[2] += a.z; x[3] += a.w; x[4] += b.x; x[5] += b.y; x[6] += b.z; x[7] += b.w;
         }
         const float f = which ? s.scale : 1.f;
-        *reinterpret_cast<uint4 *>((which ? dk : dv) + row_offset_kv(s, n, hk, p) + ch * 8) =
-            make_uint4(pack_bf16(x[0] * f, x[1] * f), pack_bf16(x[2] * f, x[3] * f), pack_bf16(x[4] * f, x[5] * f),
-                       pack_bf16(x[6] * f, x[7] * f));
+        __nv_bfloat16 *row = (which ? dk : dv) + row_offset_kv(s, n, hk, p) + ch * 8;
+        uint32_t w[4] = {pack_bf16(x[0] * f, x[1] * f), pack_bf16(x[2] * f, x[3] * f), pack_bf16(x[4] * f, x[5] * f),
+                         pack_bf16(x[6] * f, x[7] * f)};
+        if (ADDS && accumulate) add_row_chunk(w, row);
+        *reinterpret_cast<uint4 *>(row) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
     __syncwarp();
@@ -913,14 +935,21 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   const size_t smem_dq = 1024 + 2 * C::kBigBytes + kDqStages * 2 * C::kSmallBytes + meta_bytes(nT, s.pq);
   const size_t smem_kv =
       1024 + 2 * C::kBigBytes + kKvStages * (2 * C::kSmallBytes + kStatBytes) + meta_bytes(nT, s.pq);
-  const bool plain = s.causal && !s.pq && branches == 3;
-  auto kern_dq = s.pack ? (plain ? bwd_dq_tc_kernel<D, true, true> : bwd_dq_tc_kernel<D, false, true>)
-                        : (plain ? bwd_dq_tc_kernel<D, true, false> : bwd_dq_tc_kernel<D, false, false>);
-  auto kern_kv = plain ? bwd_dkdv_tc_kernel<D, true> : bwd_dkdv_tc_kernel<D, false>;
+  auto kern_dq = bwd_dq_tc_kernel<D, kGeneral, false>;
+  auto kern_kv = bwd_dkdv_tc_kernel<D, kGeneral>;
+  if (branches != 3) {
+    kern_dq = s.pack ? bwd_dq_tc_kernel<D, kPass, true> : bwd_dq_tc_kernel<D, kPass, false>;
+    kern_kv = bwd_dkdv_tc_kernel<D, kPass>;
+  } else if (s.causal && !s.pq) {
+    kern_dq = s.pack ? bwd_dq_tc_kernel<D, kPlain, true> : bwd_dq_tc_kernel<D, kPlain, false>;
+    kern_kv = bwd_dkdv_tc_kernel<D, kPlain>;
+  } else if (s.pack) {
+    kern_dq = bwd_dq_tc_kernel<D, kGeneral, true>;
+  }
   if (cudaFuncSetAttribute(kern_dq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_dq) != cudaSuccess ||
       cudaFuncSetAttribute(kern_kv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kv) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
-  if (!(s.reuse_lists && branches == 3 && !records))  // (the passes of the input-dependent gate build their own)
+  if (!records && !s.reuse_lists)  // (the passes of the input-dependent gate have got theirs)
     if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, ws.kmeta, st, ws.status + kTicketWord, branches)) return rc;
   const float4 *rec = records ? records : ws.qstats;
   if (!records) {
@@ -934,8 +963,12 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     LaunchScope ls(K_BWD_DQ_TC, st);
     const unsigned grid_q = s.pack ? (unsigned)nT * (unsigned)(s.B * (s.H / 2)) : grid;
     launch_chained(kern_dq, dim3(grid_q), dim3(kKvThreads), smem_dq, st, q128, k64, v64, g128, s, gate, seq_lens,
-                   (const uint8_t *)ws.qmeta, tdq, rec, ws.dalpha, ws.status_bwd, nT);
+                   (const uint8_t *)ws.qmeta, tdq, rec, ws.dalpha, ws.status_bwd, nT,
+                   branches == 2 ? (const bf *)dq : nullptr);
   }
+  if (dgate && branches != 3)  // between the two: it depends on neither, and its latency disappears
+    if (int rc = launch_gate_param_grad(s, ws, dgate, st, 1)) return rc;
+  float *dgate_here = branches == 3 ? dgate : nullptr;
   {
     LaunchScope ls(K_BWD_DKDV_TC, st);
     // Grouped heads: a CTA walks its tile list once per head, so with few CTAs the one with the first keys
@@ -944,15 +977,15 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     const unsigned ctas = (unsigned)nST * (unsigned)(s.B * s.Hkv);
     unsigned hs = 1;
     while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < 592) hs *= 2;
-    const dim3 grid_k((ctas + (dgate ? 1 : 0)) * hs);
+    const dim3 grid_k((ctas + (dgate_here ? 1 : 0)) * hs);
     if (hs > 1)
       launch_chained_cluster(kern_kv, grid_k, dim3(kKvThreads), smem_kv, hs, st, q64, k128, v128, g64, s, seq_lens,
                              (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, (int)hs, (bf *)dk, (bf *)dv, gate,
-                             (const double *)ws.dalpha, dgate);
+                             (const double *)ws.dalpha, dgate_here, branches == 2);
     else
       launch_chained(kern_kv, grid_k, dim3(kKvThreads), smem_kv, st, q64, k128, v128, g64, s, seq_lens,
                      (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, 1, (bf *)dk, (bf *)dv, gate,
-                     (const double *)ws.dalpha, dgate);
+                     (const double *)ws.dalpha, dgate_here, branches == 2);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

@@ -47,7 +47,8 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                                                                   int n_query_ctas, int image0, int image_end,
                                                                   int branches, int with_fwd,
                                                                   uint32_t *__restrict__ inv_bits,
-                                                                  int32_t *__restrict__ tickets) {
+                                                                  int32_t *__restrict__ tickets,
+                                                                  uint8_t *qmeta2, uint8_t *kmeta2) {
   grid_chain_enter();
   if (blockIdx.x == 0 && threadIdx.x == 0) *tickets = 0;  // of the persistent kernel behind
   constexpr int NT = 32 * NW;  // threads per image
@@ -59,8 +60,12 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   const MetaLayout ml = meta_layout(nT, s.pq);
   const int lane = threadIdx.x & 31, tid = threadIdx.x % NT, sub = threadIdx.x / NT;
   const bool scans = tid < 32;  // the warp that compacts
-  const int image = image0 + (int)blockIdx.x * (kMetaWarps / NW) + sub;  // this launch builds [image0, image_end)
+  int image = image0 + (int)blockIdx.x * (kMetaWarps / NW) + sub;  // this launch builds [image0, image_end)
   if (image >= image_end) return;
+  if (qmeta2) {  // one set of images per branch
+    branches = image < image_end / 2 ? 1 : 2;
+    if (branches == 2) image -= image_end / 2, qmeta = qmeta2, kmeta = kmeta2;
+  }
   const int Lw = (s.L + 31) >> 5;  // words per key block of the bit table
   const int slice = ml.bytes + ((3 * nT + 15) / 16) * 16;  // the image and a scratch list behind it
   uint8_t *meta = meta_all + (size_t)sub * slice;
@@ -423,14 +428,19 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
 }  // namespace
 
 int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, uint8_t *qmeta,
-                   uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches, int with_fwd) {
+                   uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches, int with_fwd, uint8_t *qmeta2,
+                   uint8_t *kmeta2) {
   if (with_fwd < 0) with_fwd = kmeta == nullptr;
+  if (qmeta2 && s.pq) {  // (a selection per position takes two launches for each set)
+    if (int rc = launch_tc_meta(s, seq_lens, idx, qmeta, kmeta, st, tickets, 1, with_fwd)) return rc;
+    return launch_tc_meta(s, seq_lens, idx, qmeta2, kmeta2, st, tickets, 2, with_fwd);
+  }
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
   // Four warps per image while its loops are long (a selection per position: 46 -> 28 us for 960 images at
   // L 1500) or the images do not fill the SMs (11 -> 10 us for 256 images at L 4096); at 4096 images of L 1024
   // four warps took 26 us and one 17.
-  const bool wide = n_images <= 148 * (s.pq ? 48 : 8);
+  const bool wide = n_images * (qmeta2 ? 2 : 1) <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;
   const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((3 * nT + 15) / 16) * 16);
   auto kern = wide ? tc_meta_kernel<kMetaWarps> : tc_meta_kernel<1>;
@@ -440,7 +450,8 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   auto launch = [&](int image0, int image_end, uint32_t *inv_bits) {
     LaunchScope ls(K_TC_META, st);
     launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,
-                   seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits, tickets);
+                   seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits, tickets, qmeta2,
+                   kmeta2);
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it
@@ -449,7 +460,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
     launch(0, nq, inv_bits);
     launch(nq, n_images, inv_bits);
   } else {
-    launch(0, n_images, nullptr);
+    launch(0, n_images * (qmeta2 ? 2 : 1), nullptr);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

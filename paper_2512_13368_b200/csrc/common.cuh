@@ -61,10 +61,11 @@ struct Workspace {
   // tensors, the second pass's gradients (added to the first pass's afterwards), its records, and
   // the branch outputs of a forward call that does not return them; q-shaped ones laid out with
   // q's strides, k-shaped ones with k's
-  void *gate_glt, *gate_gst, *gate_dq, *gate_dk, *gate_dv, *gate_olt, *gate_ost;
+  void *gate_glt, *gate_gst, *gate_olt, *gate_ost;
   float4 *qstats2;
   uint8_t *qmeta;    // per query-major CTA of the tensor-core kernels: tile lists (tc_meta_kernel)
   uint8_t *kmeta;    // per key-major CTA (dK/dV kernel): tile lists
+  uint8_t *qmeta2, *kmeta2;  // the same for the second pass of the input-dependent gate's backward
   size_t bytes;
 };
 
@@ -230,7 +231,8 @@ size_t select_static_capacity_bytes();
 int launch_gate_grad(const Shape &s, const float *gate, const Workspace &ws, float *dgate,
                      cudaStream_t st);
 // input-dependent gate: fixed-order reduction of ws.dgate_part into dgate [H][2 D + 1]
-int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st);
+// beside: between a kernel that has waited for the pre-pass (and released) and one that waits before it exits
+int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cudaStream_t st, int beside);
 int launch_rope(const Shape &s, int dtype, int dir, const void *qs, void *qd, const void *ks, void *kd, void *table,
                 bool have_table, cudaStream_t st);
 

@@ -12,7 +12,7 @@
 //             so the backward kernels run once per branch: pass 1 with the tensor G + kL w_lt in
 //             place of dO, tile lists of the long-term branch only and records that carry alpha_t
 //             in the exponent and switch the short-term branch off; pass 2 likewise for the
-//             short-term branch into scratch tensors; a third kernel adds the two results.  The
+//             short-term branch, adding to the first pass's gradients as it writes them.  The
 //             gradient of F_o's parameters is row-local (dw_lt = sum_t c_t O_lt,t, dw_st likewise,
 //             db = sum_t c_t) and is accumulated here in double precision, per query block, for the
 //             fixed-order reduction of gate_param_grad_kernel.
@@ -212,31 +212,6 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
   }
 }
 
-// ---- dst += src over the three gradients, one rounding --------------------------------------------
-struct AddTensor {
-  bf *dst;
-  const bf *src;
-  int heads;
-  int64_t sb, sh, sl;
-};
-__global__ void __launch_bounds__(256) grad_add_kernel(int B, int L, int D, AddTensor x, AddTensor y, AddTensor z) {
-  grid_chain_enter();
-  // (32-bit counts: the tensors have fewer than 2^32 pieces of 16 bytes)
-  const uint32_t cpr = D / 8, per = (uint32_t)B * L * cpr, nx = per * x.heads, ny = per * y.heads, total = nx + 2 * ny;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const AddTensor &w = i < nx ? x : i < nx + ny ? y : z;
-    const uint32_t e = i < nx ? i : i < nx + ny ? i - nx : i - nx - ny;
-    const uint32_t ch = e % cpr, row = e / cpr, t = row % L, uh = row / L, h = uh % w.heads, n = uh / w.heads;
-    const int64_t off = (int64_t)n * w.sb + (int64_t)h * w.sh + (int64_t)t * w.sl + ch * 8;
-    float a[8], b[8];
-    unpack8(*reinterpret_cast<const uint4 *>(w.dst + off), a);
-    unpack8(*reinterpret_cast<const uint4 *>(w.src + off), b);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) a[j] += b[j];
-    *reinterpret_cast<uint4 *>(w.dst + off) = pack8(a);
-  }
-}
-
 }  // namespace
 
 int launch_fwd_tc_gate(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
@@ -267,22 +242,19 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
                    ws.qstats, ws.qstats2, ws.dgate_part, Lpad, ws.status_bwd);
     if (cudaGetLastError() != cudaSuccess) return BLOSSOM_ERR_CUDA;
   }
-  int rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, nullptr, ws, st, 1,
-                         ws.qstats);
+  // The lists of both passes in one launch; the second pass adds to the first one's gradients as it writes them
+  // (three scratch tensors, an addition kernel and a launch of lists less: 234 -> 204 us for a step of B 16,
+  // H 4, L 900, D 64 with rotary positions).
+  int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, ws.kmeta, st, ws.status + kTicketWord, 3, 0, ws.qmeta2, ws.kmeta2);
   if (rc) return rc;
-  rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_gst, ws.gate_dq, ws.gate_dk,
-                     ws.gate_dv, nullptr, ws, st, 2, ws.qstats2);
+  rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, dgate, ws, st, 1,
+                     ws.qstats);
   if (rc) return rc;
-  {
-    const AddTensor x = {(bf *)dq, (const bf *)ws.gate_dq, s.H, s.sb, s.sh, s.sl};
-    const AddTensor y = {(bf *)dk, (const bf *)ws.gate_dk, s.Hkv, s.ksb, s.ksh, s.ksl};
-    const AddTensor z = {(bf *)dv, (const bf *)ws.gate_dv, s.Hkv, s.ksb, s.ksh, s.ksl};
-    const int64_t ctas = ((int64_t)s.B * (s.H + 2 * s.Hkv) * s.L * (s.D / 8) + 255) / 256;
-    LaunchScope ls(K_GATE_GRAD, st);
-    launch_chained(grad_add_kernel, dim3((unsigned)(ctas < 148 * 16 ? ctas : 148 * 16)), dim3(256), 0, st, s.B, s.L, s.D, x, y,
-                   z);
-  }
-  return launch_gate_param_grad(s, ws, dgate, st);
+  Workspace second = ws;
+  second.qmeta = ws.qmeta2;
+  second.kmeta = ws.kmeta2;
+  return launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_gst, dq, dk, dv, nullptr, second, st, 2,
+                       ws.qstats2);
 }
 
 }  // namespace tc
