@@ -229,7 +229,8 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
   }
 
   // ============================================================ query CTA: dQ, d alpha of some tiles
-  const int x = (int)blockIdx.x - bg.nkey_ctas, u = x / bg.nq, sp = x % bg.nq, n = u / s.H, h = u % s.H, hk = h / s.G;
+  // the last positions' CTAs first: they have the most keys, and the early ones may be all padding
+  const int nQ = s.B * s.H, x = (int)blockIdx.x - bg.nkey_ctas, u = x % nQ, sp = bg.nq - 1 - x / nQ, n = u / s.H, h = u % s.H, hk = h / s.G;
   int len = seq_lens ? seq_lens[n] : s.L;
   len = min(max(len, 0), s.L);
   const int pad0 = s.L - len;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
   if (lane == 0) red[warp] = dal;
   __syncthreads();
   if (tid == 0) {
-    part[x] = (red[0] + red[1]) + (red[2] + red[3]);
+    part[u * bg.nq + sp] = (red[0] + red[1]) + (red[2] + red[3]);
     __threadfence();
     const int total = s.B * s.H * bg.nq;
     last = atomicAdd(counter, 1) == total - 1;
@@ -338,22 +339,17 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
   if (!last) return;
   __threadfence();
   if (tid == 0) *counter = 0;  // (a repeated backward on this workspace starts from zero again)
+  // A warp per head, its lanes in ascending order and a fixed tree: this tail is a chain of latencies.
   const int per_head = s.B * bg.nq;
-  for (int hh = 0; hh < s.H; ++hh) {
+  for (int hh = warp; hh < s.H; hh += kWarps) {
     double a = 0.0;
 #pragma unroll 8
-    for (int i = tid; i < per_head; i += kThreads)
-      a += __ldcg(part + ((int64_t)(i / bg.nq) * s.H + hh) * bg.nq + i % bg.nq);
-    __syncthreads();
-    red[tid] = a;
-    __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-      if (tid < o) red[tid] += red[tid + o];
-      __syncthreads();
-    }
-    if (tid == 0) {
+    for (int i = lane; i < per_head; i += 32) a += __ldcg(part + ((int64_t)(i / bg.nq) * s.H + hh) * bg.nq + i % bg.nq);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) {
       const double al = 1.0 / (1.0 + exp(-((double)gate[hh * 2 + 0] - (double)gate[hh * 2 + 1])));
-      const double g0 = al * (1.0 - al) * red[0];
+      const double g0 = al * (1.0 - al) * a;
       dgate[hh * 2 + 0] = (float)g0;
       dgate[hh * 2 + 1] = (float)(-g0);
     }

@@ -29,7 +29,7 @@ namespace sh {
 namespace {
 
 struct ShortGeom {
-  int nsplit, per;  // CTAs per (batch, key/value head); query blocks per CTA
+  int nsplit, per, longer;  // CTAs per (batch, key/value head); query blocks of each, one more for the first `longer`
   int rows;         // rows of the shared K / V tiles
   int zp;           // pitch of a warp's score table (floats)
   int o_v, o_warp, warp_bytes, o_mean, o_mean32, o_sel;  // byte offsets in shared memory
@@ -235,11 +235,12 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) fwd_short_kernel(
   const bool causal = PLAIN || s.causal;
 
   if (blockIdx.x == 0 && tid < 32) status[tid] = 0;  // status words of a new step, and the backward's CTA counter
-  const int uk = (int)(blockIdx.x / sg.nsplit), sp = (int)(blockIdx.x % sg.nsplit), n = uk / s.Hkv, hk = uk % s.Hkv;
+  // the last positions' CTAs first: they have the most keys, and the early ones may be all padding
+  const int nU = s.B * s.Hkv, uk = (int)blockIdx.x % nU, sp = sg.nsplit - 1 - (int)blockIdx.x / nU, n = uk / s.Hkv, hk = uk % s.Hkv;
   int len = seq_lens ? seq_lens[n] : s.L;
   len = min(max(len, 0), s.L);
   const int pad0 = s.L - len;
-  const int qb0 = sp * sg.per, qb1 = min(s.M, qb0 + sg.per);
+  const int qb0 = sp * sg.per + min(sp, sg.longer), qb1 = qb0 + sg.per + (sp < sg.longer ? 1 : 0);
   const int q0 = qb0 * s.Bk, q1 = min(s.L, qb1 * s.Bk);  // this CTA's query positions
   const int p_lo = pad0 & ~15, p_hi = causal ? q1 : s.L;  // keys it may need
   const bool live = q1 > pad0;
@@ -737,9 +738,9 @@ int short_geom(const Shape &s, const SelGeom &g, ShortGeom *o) {
   // heads on 2; without them a finer split only repeats the loads and means: 12 -> 16 us at B 32, L 100).
   const int units = s.B * s.Hkv, want = 444 * (s.G < 2 ? 1 : 2);
   int nsplit = units >= want ? 1 : (want + units - 1) / units;
-  if (nsplit > s.M) nsplit = s.M;
-  o->per = (s.M + nsplit - 1) / nsplit;
-  o->nsplit = (s.M + o->per - 1) / o->per;
+  o->nsplit = nsplit > s.M ? s.M : nsplit;
+  o->per = s.M / o->nsplit;
+  o->longer = s.M % o->nsplit;
   return off;
 }
 
