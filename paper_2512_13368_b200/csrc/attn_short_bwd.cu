@@ -384,6 +384,7 @@ static int launch_t(const Shape &s, const void *q, const void *k, const void *v,
   bg.nkey_ctas = s.B * s.Hkv * bg.nkt;
   bg.per = s.B * s.H >= 296 ? 8 : 4;
   bg.nq = (ntiles + bg.per - 1) / bg.per;
+  bg.per = (ntiles + bg.nq - 1) / bg.nq;  // of equal size
   bg.o_b = rows * D * 2;
   bg.o_rec = 2 * rows * D * 2;
   bg.o_stage = bg.o_rec + rows * 16;

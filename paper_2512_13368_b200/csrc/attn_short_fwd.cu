@@ -733,10 +733,12 @@ int short_geom(const Shape &s, const SelGeom &g, ShortGeom *o) {
   off += g.n * (s.D + 4) * 4;
   o->o_sel = off;
   off += 32 * 4;
-  // With fewer (batch, head) pairs than fill the SMs three times the query blocks are split over CTAs
-  // (six times with grouped heads, whose CTAs have several heads' rows to do: 87 -> 75 us at B 128, 8
-  // heads on 2; without them a finer split only repeats the loads and means: 12 -> 16 us at B 32, L 100).
-  const int units = s.B * s.Hkv, want = 444 * (s.G < 2 ? 1 : 2);
+  // With fewer (batch, head) pairs than fill the SMs three times the query blocks are split over CTAs (a finer
+  // split of few pairs only repeats the loads and means: 12 -> 16 us at B 32, L 100); with up to twice as many
+  // every pair's blocks go to two CTAs, so that the long ones start first and the rest fills up (512 pairs,
+  // L 200: 38 -> 34 us).  Nine times with grouped heads, whose CTAs have several heads' rows to do (B 128, 8 heads
+  // on 2: three times 83, six 61, nine 57, eighteen 62 us).
+  const int units = s.B * s.Hkv, want = s.G > 1 ? 1332 : units >= 444 ? 888 : 444;
   int nsplit = units >= want ? 1 : (want + units - 1) / units;
   o->nsplit = nsplit > s.M ? s.M : nsplit;
   o->per = s.M / o->nsplit;
