@@ -91,8 +91,16 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   uint8_t *jcls = meta + ml.jcls;
   int *counts = reinterpret_cast<int *>(meta + ml.counts);
   const unsigned lt = (1u << lane) - 1u;
-  const int G = 128 / s.Bk, nb = 64 / s.Bk;
-  const int bk_shift = __ffs(s.Bk) - 1;  // Bk is a power of two
+  const int bk_shift = __ffs(s.Bk) - 1, nb_shift = 6 - bk_shift;  // Bk is a power of two
+  const int G = 128 >> bk_shift, nb = 1 << nb_shift;  // query blocks of a CTA, blocks of a tile
+  // index rows: entry i of a run is slot i % topk of row i / topk; a thread's next entry lies NT further
+  const int step_row = NT / s.topk, step_slot = NT % s.topk;
+  auto next_entry = [&](int &row, int &slot) {
+    row += step_row;
+    slot += step_slot;
+    if (slot >= s.topk) slot -= s.topk, ++row;
+  };
+  const int row_0 = tid / s.topk, slot_0 = tid % s.topk;
 
   for (int i = tid; i < ml.bytes / 4; i += NT) selw[i] = 0u;  // the whole image
   sync();
@@ -109,27 +117,27 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       uint32_t *roww = reinterpret_cast<uint32_t *>(meta + ml.rows);
       // the bit table is per key/value head: the group's first query head (or pair of heads) fills it
       const bool fills = inv_bits && (pack ? (2 * (u % (s.H / 2))) % s.G == 0 : (u % s.H) % s.G == 0);
-      for (int i = tid; i < 128 * s.topk; i += NT) {
-        const int r = i / s.topk, slot = i % s.topk, t = pack ? row0 + (r & 63) : row0 + r;
+      for (int r = row_0, slot = slot_0; r < 128; next_entry(r, slot)) {
+        const int t = pack ? row0 + (r & 63) : row0 + r;
         if (t < s.L) {
           const int blk = idx[((int64_t)uk * s.L + t) * s.topk + slot];
           if (blk >= 0 && blk <= (t >> bk_shift)) {
-            const int a = (r >> bk_shift) * nT + blk / nb, b2 = r * nT + blk / nb;
-            atomicOr(&selw[a >> 2], (1u << (blk % nb)) << ((a & 3) * 8));
-            atomicOr(&roww[b2 >> 2], (1u << (blk % nb)) << ((b2 & 3) * 8));
+            const int a = (r >> bk_shift) * nT + (blk >> nb_shift), b2 = r * nT + (blk >> nb_shift);
+            atomicOr(&selw[a >> 2], (1u << (blk & (nb - 1))) << ((a & 3) * 8));
+            atomicOr(&roww[b2 >> 2], (1u << (blk & (nb - 1))) << ((b2 & 3) * 8));
             if (fills && (!pack || r < 64))
               atomicOr(&inv_bits[((int64_t)uk * s.M + blk) * Lw + (t >> 5)], 1u << (t & 31));
           }
         }
       }
     } else {
-    for (int i = tid; i < G * s.topk; i += NT) {  // the selections of the CTA's query blocks
-      const int g = i / s.topk, slot = i % s.topk, qb = pack ? st * nb + g % nb : st * G + g;
+    for (int g = row_0, slot = slot_0; g < G; next_entry(g, slot)) {  // the selections of the CTA's query blocks
+      const int qb = pack ? st * nb + (g & (nb - 1)) : st * G + g;
       if (qb < s.M) {
         const int blk = idx[((int64_t)uk * s.M + qb) * s.topk + slot];
         if (blk >= 0 && blk < s.M && (blk <= qb || !s.causal)) {
-          const int a = g * nT + blk / nb;
-          atomicOr(&selw[a >> 2], (1u << (blk % nb)) << ((a & 3) * 8));
+          const int a = g * nT + (blk >> nb_shift);
+          atomicOr(&selw[a >> 2], (1u << (blk & (nb - 1))) << ((a & 3) * 8));
         }
       }
     }
@@ -170,10 +178,17 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       for (int base = 0; base < nv; base += 32) {
         const int j = base + lane;
         int c = 0;
-        if (j < nv && (lflags[j] & 1)) {
-          const int jt = list[j];
-          for (int g = 0; g < G; ++g)
-            if (selb[g * nT + jt]) c |= g < gh ? 1 : 2;
+        if (j < nv) {
+          if (pass == 0) {
+            if (lflags[j] & 1) {
+              const int jt = list[j];
+              for (int g = 0; g < G; ++g)
+                if (selb[g * nT + jt]) c |= g < gh ? 1 : 2;
+            }
+            icls[j] = (uint8_t)c;  // (for the second pass; the classes come later)
+          } else {
+            c = icls[j];
+          }
         }
         const unsigned bA = __ballot_sync(0xffffffffu, c == 1), bB = __ballot_sync(0xffffffffu, c == 2),
                        bC = __ballot_sync(0xffffffffu, c == 3);
@@ -216,7 +231,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     // Class of every (item, softmax warp): 0 = no row of the warp needs the tile, 1 = every row
     // sees all 64 keys, 2 = mixed (the warp builds per-lane column masks).
     const bool uni = s.Bk >= 32;  // a warp's 32 rows share one query block
-    const uint32_t allbits = (1u << (64 / s.Bk)) - 1u;
+    const uint32_t allbits = (1u << nb) - 1u;
     for (int e = tid; e < count * 4; e += NT) {
       const int it = e >> 2, w = e & 3;
       const int jt = items[it], p0 = jt * 64, t_lo = quarter_row0(w);
@@ -228,7 +243,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         if (it < nl) {
           if (!uni) cls = 2;
           else {
-            const uint32_t bits = selb[((w * 32) / s.Bk) * nT + jt];
+            const uint32_t bits = selb[((w * 32) >> bk_shift) * nT + jt];
             cls = bits == 0u ? 0 : ((!s.pq && inner && bits == allbits) ? 1 : 2);  // (per position: the rows differ)
           }
         } else if (st_ranges_touch(s, t_lo, t_lo + 31, p0, p0 + 63)) {
@@ -252,7 +267,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         for (int base = 0; base < nv; base += 32) {
           const int j = base + lane;
           int c = 0;
-          if (j < nv) {
+          if (j < nv && pass == 1) {
+            c = jcls[j];
+          } else if (j < nv) {
             const int jt = list[j], p0 = jt * 64;
             if (lflags[j] & 1)
               for (int g = 0; g < G; ++g)
@@ -263,6 +280,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                     st_ranges_touch(s, half_row0(hf), half_row0(hf) + 63, p0, p0 + 63))
                   c |= 1 << hf;
             if (c == 0) c = 3;
+            jcls[j] = (uint8_t)c;  // (for the second pass)
           }
           const unsigned bA = __ballot_sync(0xffffffffu, c == 1), bB = __ballot_sync(0xffffffffu, c == 2),
                          bC = __ballot_sync(0xffffffffu, c == 3);
@@ -349,6 +367,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       // (without the causal mask every query block may have selected them: the rows start at block 0)
       const int qb0 = kt * G, qb_first = s.causal ? qb0 : 0, total = (s.M - qb_first) * s.topk;
       const int32_t *rows = idx + ((int64_t)uk * s.M + qb_first) * s.topk;
+      int row = row_0, slot = slot_0;
       for (int base = 0; base < total; base += 8 * NT) {
         int blk[8];
 #pragma unroll
@@ -358,10 +377,11 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
         }
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int i = base + e * NT + tid, qb = qb_first + i / s.topk;
+          const int qb = qb_first + row;
+          next_entry(row, slot);
           if (blk[e] >= qb0 && blk[e] < qb0 + G && (blk[e] <= qb || !s.causal)) {
-            const int a = (blk[e] - qb0) * nT + qb / nb;
-            atomicOr(&selw[a >> 2], (1u << (qb % nb)) << ((a & 3) * 8));
+            const int a = (blk[e] - qb0) * nT + (qb >> nb_shift);
+            atomicOr(&selw[a >> 2], (1u << (qb & (nb - 1))) << ((a & 3) * 8));
           }
         }
       }
