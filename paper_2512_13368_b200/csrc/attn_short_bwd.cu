@@ -52,27 +52,33 @@ __device__ __forceinline__ void key_pairs(bool inL, bool inS, const float (&z)[2
       }
     }
 }
-// A thread's 8 (query row, key column) pairs: dS and the sums behind d alpha.  nl, nD: {long-term rows
-// gid, gid + 8, short-term rows gid, gid + 8}.
+// A thread's 8 (query row, key column) pairs: dS and d alpha = sum (P_lt - P_st) dP.  nl = -lse (log2 units)
+// and nD = -weight Delta: {long-term rows gid, gid + 8, short-term rows gid, gid + 8}.  The probabilities are
+// unweighted and subtracted pair by pair, so that pairs which both branches see alike (the same keys, hence the
+// same bits of lse) add exactly nothing: as two sums, subtracted at the end, histories shorter than the window
+// left their rounding in the place of a zero.  (The same instructions: the weights ride in an addition.)
 __device__ __forceinline__ void query_pairs(bool inL, bool inS, const float (&z)[2][4], const float (&dp)[2][4],
-                                            const uint32_t (&bL)[2], const uint32_t (&bS)[2], float sc2,
-                                            const float (&nl)[4], const float (&nD)[4], float &dalL, float &dalS,
+                                            const uint32_t (&bL)[2], const uint32_t (&bS)[2], float sc2, float alpha,
+                                            float beta, const float (&nl)[4], const float (&nD)[4], float &dal,
                                             float (&d)[2][4]) {
+  float diff[2][4];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) d[e >> 2][e & 3] = 0.f;
+  for (int e = 0; e < 8; ++e) d[e >> 2][e & 3] = diff[e >> 2][e & 3] = 0.f;
 #pragma unroll
   for (int br = 0; br < 2; ++br)
     if (br ? inS : inL) {
+      const float weight = br ? beta : alpha;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int i = (e >> 1) & 1, c = (e >> 2) * 8 + (e & 1);
         const uint32_t b = br ? bS[i] : bL[i];
         const float y = ((b >> c) & 1u) ? exp2f(fmaf(z[e >> 2][e & 3], sc2, nl[2 * br + i])) : 0.f;
-        if (br) dalS = fmaf(y, dp[e >> 2][e & 3], dalS);
-        else dalL = fmaf(y, dp[e >> 2][e & 3], dalL);
-        d[e >> 2][e & 3] = fmaf(y, dp[e >> 2][e & 3] + nD[2 * br + i], d[e >> 2][e & 3]);
+        diff[e >> 2][e & 3] = br ? diff[e >> 2][e & 3] - y : y;
+        d[e >> 2][e & 3] = fmaf(y, fmaf(weight, dp[e >> 2][e & 3], nD[2 * br + i]), d[e >> 2][e & 3]);
       }
     }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) dal = fmaf(diff[e >> 2][e & 3], dp[e >> 2][e & 3], dal);
 }
 
 template <int D, bool PLAIN>
@@ -237,7 +243,7 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
   const int ntiles = (s.L + 15) >> 4, tile0 = sp * bg.per, tile1 = min(ntiles, tile0 + bg.per);
   const int q1 = min(s.L, tile1 * 16), p_lo = pad0 & ~15, p_hi = causal ? q1 : s.L;
   const int64_t off = row_offset(s, n, h, 0), koff = row_offset_kv(s, n, hk, 0);
-  const float alpha = head_alpha(gate, h), beta = 1.f - alpha, la = log2f(alpha), lb = log2f(beta);
+  const float alpha = head_alpha(gate, h), beta = 1.f - alpha;
   if (q1 > pad0) {
     const int hi16 = (p_hi + 15) & ~15;
     stage_rows<D>(ta, k + koff, s.ksl, p_lo, hi16, pad0, p_hi, tid, kThreads);
@@ -275,9 +281,9 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
       const int r0 = t0 + gid;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        nD[i] = -quad_sum(nD[i]);
+        nD[i] = -(i < 2 ? alpha : beta) * quad_sum(nD[i]);
         const int t = r0 + 8 * (i & 1);
-        nl[i] = t >= pad0 && t < s.L ? (i < 2 ? la : lb) - lse[(i < 2 ? 0 : BHL) + (int64_t)u * s.L + t] * kLog2e : 0.f;
+        nl[i] = t >= pad0 && t < s.L ? -(lse[(i < 2 ? 0 : BHL) + (int64_t)u * s.L + t] * kLog2e) : 0.f;
       }
       const uint32_t sb = sel[t0 >> bsh];
       uint64_t setL, setS;
@@ -294,7 +300,7 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
         setS = ballot64(fs[0], fs[1]);
       }
       const bool rows_in = t0 >= pad0 && t0 + 15 < s.L;
-      float dalL = 0.f, dalS = 0.f;
+      float dal_t = 0.f;
 #pragma unroll 1
       for (uint64_t todo = setL | setS; todo; todo &= todo - 1) {
         const int c = __ffsll((long long)todo) - 1, p0 = c * 16;
@@ -314,13 +320,12 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
         if (inS && !(past && t0 + 15 - p0 < s.window && (causal || p0 + 15 - t0 < s.window)))
 #pragma unroll
           for (int i = 0; i < 2; ++i) bS[i] &= st_keys16<PLAIN>(s, r0 + 8 * i, p0, causal) >> (2 * tig);
-        query_pairs(inL, inS, z, dp, bL, bS, sc2, nl, nD, dalL, dalS, d);
+        query_pairs(inL, inS, z, dp, bL, bS, sc2, alpha, beta, nl, nD, dal_t, d);
         uint32_t pa[4];
         to_a(d, pa);
         product_nn<D>(pa, ta_a + co + onn, acc);
       }
-      // d alpha = sum (P_lt - P_st) dP; a weight of exactly 0 makes its branch's sum 0
-      dal += (double)((alpha > 0.f ? dalL / alpha : 0.f) - (beta > 0.f ? dalS / beta : 0.f));
+      dal += (double)dal_t;
     }
     store_rows<D>(dq + off, s.sl, t0, s.L, acc, s.scale, s.scale, stage, lane);
   }

@@ -22,12 +22,12 @@
 //         columns (half tile x uses buffer x % 2: S in its first 32 columns, dP in the other 32),
 //         Q and dO as first operands of the first-stage products [128,128+D/2), [160,160+D/2)
 //         (read from shared memory they cost 4 KB per product, more than the data pipe delivers
-//         in the product's run time), and dQ [192,192+D).  S = Q K^T, dP = dO V^T; P'_x = weight_x exp(S - lse_x);
-//         dS = P'_lt (dP - Delta_lt) + P'_st (dP - Delta_st) (one tile for both branches, they share
-//         K).  A thread owns 16 of the 32 columns and writes its dS (bf16 pairs) over the first 8
+//         in the product's run time), and dQ [192,192+D).  S = Q K^T, dP = dO V^T; P_x = exp(S - lse_x);
+//         dS = P_lt (alpha dP - alpha Delta_lt) + P_st (beta dP - beta Delta_st) (one tile for both
+//         branches, they share K).  A thread owns 16 of the 32 columns and writes its dS (bf16 pairs) over the first 8
 //         of its own S columns, from where dQ += dS K reads it: the compute warps wait for one
 //         thing per half tile (its S and dP), and the first stage of the next two half tiles runs
-//         meanwhile.  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities.
+//         meanwhile.  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities, subtracted pair by pair.
 //  dK/dV  transposed: resident K, V of 128 keys, streams Q, dO 64-query tiles (and their row
 //         records, by bulk copy) that selected one of its key blocks or whose window reaches them.
 //         It works through them in half tiles of 32 queries.  Tensor memory: two buffers of 64
@@ -135,28 +135,31 @@ __device__ __forceinline__ void add_row_chunk(uint32_t (&w)[4], const __nv_bfloa
 }
 
 // ---------------------------------------------------------------------------- backward dQ
-// 16 columns of one tile for one row: dS packed to bf16 pairs, partial sums of P' dP.
-// nlL / nlS = -(lse * log2e - log2 alpha) resp. beta: the branch weight rides in the exponent, so
-// P' = alpha P_lt (beta P_st) comes straight out of the exponential; nDL / nDS = -Delta.
-// Two columns per FMA / ADD / MUL instruction.
+// 16 columns of one tile for one row: dS packed to bf16 pairs, and this row's part of d alpha = sum (P_lt -
+// P_st) dP.  nlL / nlS = -lse (log2 units), wL / wS: the branches' weights, nDL / nDS = -weight Delta.  The
+// unweighted probabilities are subtracted pair by pair, so that pairs which both branches see alike (the same
+// keys, hence the same bits of lse) add exactly nothing; with the weights in the exponent and a sum per
+// branch, subtracted at the end, rows whose window holds the whole history left their rounding instead of a
+// zero.  (The same instructions: the weight rides in what was the addition of -Delta.)  dalS collects what
+// only the short-term branch sees.  Two columns per FMA / ADD / MUL instruction.
 template <bool HAS_L, bool HAS_S, bool FULL>
 __device__ __forceinline__ void dq_tile(const float (&sv)[16], const float (&dp)[16], uint32_t hL,
-                                        uint32_t hS, float sc2, float nlL, float nlS, float nDL,
-                                        float nDS, float2 &dalL, float2 &dalS, uint32_t (&dw)[8]) {
+                                        uint32_t hS, float sc2, float nlL, float nlS, float wL, float wS,
+                                        float nDL, float nDS, float2 &dalL, float2 &dalS, uint32_t (&dw)[8]) {
   const float2 sc = make_float2(sc2, sc2);
 #pragma unroll
   for (int c = 0; c < 16; c += 2) {
     const float2 s2 = make_float2(sv[c], sv[c + 1]), dp2 = make_float2(dp[c], dp[c + 1]);
-    float2 acc = make_float2(0.f, 0.f);
+    float2 acc = make_float2(0.f, 0.f), pL = acc;
     if (HAS_L) {
       const float2 x = ffma2(s2, sc, make_float2(nlL, nlL));
-      float2 p = make_float2(exp2f(x.x), exp2f(x.y));
+      pL = make_float2(exp2f(x.x), exp2f(x.y));
       if (!FULL) {
-        p.x = bit(hL, c) ? p.x : 0.f;
-        p.y = bit(hL, c + 1) ? p.y : 0.f;
+        pL.x = bit(hL, c) ? pL.x : 0.f;
+        pL.y = bit(hL, c + 1) ? pL.y : 0.f;
       }
-      dalL = ffma2(p, dp2, dalL);
-      acc = fmul2(p, fadd2(dp2, make_float2(nDL, nDL)));
+      if (!HAS_S) dalL = ffma2(pL, dp2, dalL);
+      acc = fmul2(pL, ffma2(dp2, make_float2(wL, wL), make_float2(nDL, nDL)));
     }
     if (HAS_S) {
       const float2 x = ffma2(s2, sc, make_float2(nlS, nlS));
@@ -165,8 +168,9 @@ __device__ __forceinline__ void dq_tile(const float (&sv)[16], const float (&dp)
         p.x = bit(hS, c) ? p.x : 0.f;
         p.y = bit(hS, c + 1) ? p.y : 0.f;
       }
-      dalS = ffma2(p, dp2, dalS);
-      acc = ffma2(p, fadd2(dp2, make_float2(nDS, nDS)), acc);
+      if (HAS_L) dalL = ffma2(ffma2(p, make_float2(-1.f, -1.f), pL), dp2, dalL);
+      else dalS = ffma2(p, dp2, dalS);
+      acc = ffma2(p, ffma2(dp2, make_float2(wS, wS), make_float2(nDS, nDS)), acc);
     }
     dw[c >> 1] = pack_bf16(acc.x, acc.y);
   }
@@ -185,7 +189,7 @@ template <int D, int MODE, bool PACK>
 __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
-    const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
+    const float *__restrict__ gate, const int32_t *__restrict__ seq_lens, const float *__restrict__ lse,
     const uint8_t *__restrict__ qmeta, const __grid_constant__ CUtensorMap tmdq,
     const float4 *__restrict__ qstats, double *__restrict__ dalpha_part, int32_t *__restrict__ status,
     int nT, const __nv_bfloat16 *add_dq) {
@@ -362,18 +366,19 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     const bool row_ok = t < s.L, row_valid = row_ok && t >= pad0;
     const int t_last = row_valid ? (causal ? t : s.L - 1) : -1;  // the last key this row may see
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-    const float alpha = gate_alpha(gate, hr), beta = 1.f - alpha;
+    // kPass: the row's weight rides in its record's exponents (the gate's gradient is not formed here)
+    const float alpha = ADDS ? 1.f : gate_alpha(gate, hr), beta = ADDS ? 1.f : 1.f - alpha;
     // this row's record from the pre-pass: nl = -(lse * log2e - log2 weight), nD = -Delta
     float nlL = 0.f, nlS = 0.f, nDL = 0.f, nDS = 0.f;
     if (row_valid) {
-      const float *rec =
-          reinterpret_cast<const float *>(qstats) + (((int64_t)n * s.H + hr) * Lpad + (t & ~1)) * 4 + (t & 1);
-      nlL = rec[0];
-      nDL = rec[2];
-      nlS = rec[4];
-      nDS = rec[6];
+      const int64_t hrow = (int64_t)n * s.H + hr;
+      const float *rec = reinterpret_cast<const float *>(qstats) + (hrow * Lpad + (t & ~1)) * 4 + (t & 1);
+      nlL = ADDS ? rec[0] : -(lse[hrow * s.L + t] * kLog2e);
+      nDL = alpha * rec[2];
+      nlS = ADDS ? rec[4] : -(lse[((int64_t)s.B * s.H + hrow) * s.L + t] * kLog2e);
+      nDS = beta * rec[6];
     }
-    float2 dalL = make_float2(0.f, 0.f), dalS = make_float2(0.f, 0.f);  // sums of P' dP per branch
+    float2 dalL = make_float2(0.f, 0.f), dalS = make_float2(0.f, 0.f);  // see dq_tile
     const float sc2 = s.scale * kLog2e;
     int b = 0, ph = 0;  // buffer x % 2 of half tile x = 2 i + hh and the parity (x / 2) & 1
     if (nvis > 0) {
@@ -421,12 +426,12 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         tmem_ld16(tb, sv);
         tmem_ld16(tb + 32, dp);
         tmem_wait_ld();
-        if (!full && (PLAIN || (anyL && anyS))) dq_tile<true, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
-        else if (!full && anyL) dq_tile<true, false, false>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
-        else if (!full) dq_tile<false, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
-        else if (anyL && anyS) dq_tile<true, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
-        else if (anyL) dq_tile<true, false, true>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
-        else dq_tile<false, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, nDL, nDS, dalL, dalS, dw);
+        if (!full && (PLAIN || (anyL && anyS))) dq_tile<true, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        else if (!full && anyL) dq_tile<true, false, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        else if (!full) dq_tile<false, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        else if (anyL && anyS) dq_tile<true, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        else if (anyL) dq_tile<true, false, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        else dq_tile<false, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
       } else {
 #pragma unroll
         for (int c = 0; c < 8; ++c) dw[c] = 0u;
@@ -474,9 +479,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         tma_store_commit_and_wait();
       }
     }
-    // d alpha = sum (P_lt - P_st) dP; a weight of exactly 0 makes its branch's sum 0 and the gate
-    // gradient alpha (1 - alpha) d alpha 0 whatever d alpha is
-    const float dal = (alpha > 0.f ? (dalL.x + dalL.y) / alpha : 0.f) - (beta > 0.f ? (dalS.x + dalS.y) / beta : 0.f);
+    const float dal = (dalL.x + dalL.y) - (dalS.x + dalS.y);
     double a = row_valid ? (double)dal : 0.0;  // fixed-shape tree over the warp, then over the warps
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
@@ -962,7 +965,7 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   {
     LaunchScope ls(K_BWD_DQ_TC, st);
     const unsigned grid_q = s.pack ? (unsigned)nT * (unsigned)(s.B * (s.H / 2)) : grid;
-    launch_chained(kern_dq, dim3(grid_q), dim3(kKvThreads), smem_dq, st, q128, k64, v64, g128, s, gate, seq_lens,
+    launch_chained(kern_dq, dim3(grid_q), dim3(kKvThreads), smem_dq, st, q128, k64, v64, g128, s, gate, seq_lens, lse,
                    (const uint8_t *)ws.qmeta, tdq, rec, ws.dalpha, ws.status_bwd, nT,
                    branches == 2 ? (const bf *)dq : nullptr);
   }
