@@ -62,8 +62,8 @@ __device__ __forceinline__ double bf_double(uint32_t f) {
 }
 
 // Eq. 13 by rank over the (at most 32) selection blocks, lane j = block j: the `want` best blocks of
-// [jmin, hi) (the own block b left out without the causal mask), ties to the lower index.  kept /
-// dropped: the smallest kept and the largest dropped score.
+// [jmin, hi) (the own block b left out without the causal mask), ties to the lower index.  S: rankable scores,
+// -infinity outside.  kept / dropped: the smallest kept and the largest dropped score.
 template <typename F>
 __device__ __forceinline__ uint32_t rank32(F S, bool in, int lo, int hi, int want, int lane, F *kept, F *dropped) {
   int rank = 0;
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) fwd_short_kernel(
         scf[lane + 32] = sc1;
         __syncwarp();
         float kept, dropped;
-        const float S = in ? map32(g, scf, cmin, nc, lane) : -INFINITY;
+        const float S = in ? rankable(map32(g, scf, cmin, nc, lane)) : -INFINITY;
         mask = rank32<float>(S, in, jmin, hi, want, lane, &kept, &dropped);
         qn = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(qn)));
         // The bound of select.cu, with the roundings of the mean's sum (g.l / 2 + 2 of them, relative to the
@@ -465,7 +465,8 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) fwd_short_kernel(
         const float E = ((float)(D + 6) * bound + (float)(g.l / 2 + 2) * s.scale * qn * krms) * uu * 1.01f;
         const float R_ = 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f +
                          (float)(ncol + s.Bk * s.G + 2 * s.G + g.rs * g.rl + 40) * uu;
-        const bool certain = !exact && (kept - dropped) > R_ * (kept + dropped) * 1.001f;
+        // (a negative score is no number: left to double precision)
+        const bool certain = !exact && dropped >= 0.f && (kept - dropped) > R_ * (kept + dropped) * 1.001f;
         if (!certain) {  // decided in double precision below, by all warps
           if (lane == 0) uncertain[atomicAdd(&n_uncertain, 1)] = b;
           __syncwarp();
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) fwd_short_kernel(
         __syncwarp();
         const bool in = lane >= jmin && lane < hi && !(own && lane == b);
         double kept, dropped;
-        const double S = in ? map32(g, scd, cmin, nc, lane) : -INFINITY;
+        const double S = in ? rankable(map32(g, scd, cmin, nc, lane)) : -INFINITY;
         emit(b, rank32<double>(S, in, jmin, hi, want, lane, &kept, &dropped));
       }
       __syncthreads();

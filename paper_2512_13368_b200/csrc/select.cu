@@ -217,10 +217,12 @@ __device__ __forceinline__ void map_scores(const SelGeom &g, const F *Sc, int cm
 
 // Eq. 13 by rank: block j in [jmin, b) is kept iff fewer than `want` selectable blocks beat it
 // (larger score, or equal score and lower index).  One warp; `bound` receives the smallest kept
-// and the largest dropped score.
+// and the largest dropped score.  Scores that are no number (queries or keys that are not finite) count
+// as -1, below every other one: each would have rank 0 otherwise, and the row would take them all.
 template <typename F>
-__device__ __forceinline__ void rank_select(const F *S, int jmin, int b, int want, uint8_t *taken, F *bound,
-                                            int lane) {
+__device__ __forceinline__ void rank_select(F *S, int jmin, int b, int want, uint8_t *taken, F *bound, int lane) {
+  for (int j = jmin + lane; j < b; j += 32) S[j] = rankable(S[j]);
+  __syncwarp();
   for (int j = jmin + lane; j < b; j += 32) {
     const F sj = S[j];
     int rank = 0;
@@ -599,7 +601,7 @@ __global__ void __launch_bounds__(kFastThreads, 3) score_fast_kernel(
       const float R = 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f +
                       (16.f * nchunks + (float)(Bk / 4) + 2.f + (float)sh.G + (float)(g.rs * g.rl) + 40.f) * uu;
       const float smin = bound_s[i][0], umax = bound_s[i][1];
-      certain = (smin - umax) > R * (smin + umax) * 1.001f;
+      certain = umax >= 0.f && (smin - umax) > R * (smin + umax) * 1.001f;  // (a negative one is no number)
     }
     __syncwarp();
     if (certain) emit_row(row, tk, jmin, b, sh.topk, lane);
@@ -954,7 +956,7 @@ __global__ void __launch_bounds__(128) score_exact16_kernel(
             const int i = g.rs * j - m - e;
             if (i >= cmin && i < nc) acc += Sc[i - cmin];
           }
-        S[j] = own && j == b ? -INFINITY : acc;  // the own block is not ranked: it is kept anyway
+        S[j] = own && j == b ? -INFINITY : rankable(acc);  // the own block is not ranked: it is kept anyway
       }
       __syncthreads();
       for (int j = jmin + tid; j < hi; j += 128) {  // Eq. 13 by rank
@@ -1089,7 +1091,7 @@ __global__ void __launch_bounds__(256) score_per_query_kernel(
         }
       }
       __syncwarp();
-      const double *S = P;
+      double *S = P;
       if (!g.plain) {
         map_scores<double>(g, P, cmin, nc, jmin, b, Smap, lane);
         __syncwarp();

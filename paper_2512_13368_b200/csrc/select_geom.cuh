@@ -33,5 +33,10 @@ __device__ __forceinline__ int n_candidates(const Shape &sh, const SelGeom &g, i
 __device__ __forceinline__ int first_live_scored(const SelGeom &g, int pad0) {
   return pad0 < g.l ? 0 : (pad0 - g.l) / g.s + 1;
 }
+// A score as the rankings take it: sums of probabilities are not negative, and what is no number ranks
+// below all of them (but above the own block's -infinity), so that a ranking is an order whatever the inputs
+// and a row never gets more blocks than it has room for.
+template <typename F>
+__device__ __forceinline__ F rankable(F x) { return x == x ? x : (F)-1; }
 
 }  // namespace blossom

@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
           const int y = g.rs * j - m - e;
           if (y >= cmin && y < ncb) a += Sc2[y - cmin];
         }
-      S2[tid] = in ? a : -INFINITY;  // (the own block is not ranked: it is kept anyway)
+      S2[tid] = in ? rankable(a) : -INFINITY;  // (the own block is not ranked: it is kept anyway)
     }
     __syncthreads();
     if (j < hi) {
