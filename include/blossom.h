@@ -22,8 +22,8 @@
  *     the selected key blocks in ascending order, -1 padded.  The query block's own block is
  *     always one of them.  (select_mode 1: a row per query position, [B][H][L][top_k].)
  *   - Inputs are expected to be finite, padded rows included.  A value that is not spoils the outputs
- *     and gradients of its own sequence (and dgate); block_idx keeps the form above: scores that are
- *     no number rank below all others, ties to the lower index.
+ *     and gradients of its own sequence (and dgate).  Which blocks that sequence selects is then not
+ *     specified (entry points and sizes may differ), but its block_idx rows keep the form above.
  *   - lse is float [2][B][H][L]: plane 0 long-term branch, plane 1 short-term branch; natural log
  *     of the sum over the branch's visible keys of exp(sm_scale * <q, k>).
  *   - gate_logits is float [H][2]: column 0 long-term, column 1 short-term logit;

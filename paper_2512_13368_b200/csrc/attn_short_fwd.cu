@@ -54,7 +54,9 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 
 // the double of a bf16 value given as fp32 bits (denormals count as zero, as they do in this build's
 // fp32 arithmetic), by rebiasing the exponent: the conversion instruction runs at a fraction of the
-// integer rate
+// integer rate.  An infinity or NaN becomes a number of 2^128 and more: it weighs like one in the sums, where
+// the general path's scores of its block are no numbers; either way the row is a valid one (testing every
+// value here made the whole kernel 2.6 % slower at B 64, L 200, a probe of every row and mean 0.7 %).
 __device__ __forceinline__ double bf_double(uint32_t f) {
   const uint32_t e = f & 0x7f800000u;
   const uint32_t hi = e ? (f & 0x80000000u) | (((f & 0x7fffffffu) >> 3) + ((1023u - 127u) << 20)) : 0u;
