@@ -37,7 +37,7 @@ def test_index_rows_of_non_finite_inputs(dtype, H, Hkv, L, D, block, topk, opts,
     w.cmp_block, w.cmp_stride = opts.get("cmp", (0, 0))
     p = runner.DeviceProblem(w, training=False)
     p.forward()
-    want = p.idx.clone()
+    want, out = p.idx.clone(), p.out.clone()
     n = p.idx.numel()
     guarded = torch.full((n + 4096,), -7, dtype=torch.int32, device=p.idx.device)
     p.idx = guarded[:n].view(p.idx.shape)
@@ -76,4 +76,4 @@ def test_index_rows_of_non_finite_inputs(dtype, H, Hkv, L, D, block, topk, opts,
                     assert kept[0] >= first and kept[-1] <= last, (seq, h, r, got)
                     assert len(kept) == min(topk, last - first + 1), (seq, h, r, got)
         for seq in (0, 4):
-            assert torch.equal(p.idx[seq], want[seq])
+            assert torch.equal(p.idx[seq], want[seq]) and torch.equal(p.out[seq], out[seq])
