@@ -231,12 +231,17 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const int64_t rows = p.select_mode ? L : (L + p.block_size - 1) / p.block_size;
     Tensor out = like(q), idx = fresh({B, Hkv, rows, p.top_k}, at::kInt, dev);
     const blossom_stream_t st = (blossom_stream_t)c10::cuda::getCurrentCUDAStream(dev.index()).stream();
+    // Every address is taken before the interpreter is let go: a tensor without memory of its own (a batched
+    // one inside vmap) throws here, and an exception must not leave the block below.
+    const void *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr();
+    const float *gp = gate.data_ptr<float>();
+    const int32_t *np = lens.defined() ? lens.data_ptr<int32_t>() : nullptr;
+    int32_t *ip = idx.data_ptr<int32_t>();
+    void *op = out.data_ptr(), *lp = grad ? s.out_lt() : nullptr, *sp = grad ? s.out_st() : nullptr, *wp = s.workspace();
+    float *ep = grad ? s.lse() : nullptr;
     int rc;
     Py_BEGIN_ALLOW_THREADS;
-    rc = blossom_attn_fwd(&p, q.data_ptr(), k.data_ptr(), v.data_ptr(), gate.data_ptr<float>(),
-                          lens.defined() ? lens.data_ptr<int32_t>() : nullptr, idx.data_ptr<int32_t>(), 0,
-                          out.data_ptr(), grad ? s.out_lt() : nullptr, grad ? s.out_st() : nullptr,
-                          grad ? s.lse() : nullptr, s.workspace(), ws_bytes, st);
+    rc = blossom_attn_fwd(&p, qp, kp, vp, gp, np, ip, 0, op, lp, sp, ep, wp, ws_bytes, st);
     Py_END_ALLOW_THREADS;
     if (rc) return raise_blossom(rc, "blossom_attn_fwd");
     if (grad) {

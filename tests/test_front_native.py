@@ -53,3 +53,24 @@ def test_calls_without_a_gradient_and_partial_gradients(dtype, L, lens):
         blossom_attention(d[0], d[1], d[2], mk(3, 2), 16, 3, 9)
     with pytest.raises(RuntimeError):   # BlossomError: the library does not take top_k = 0
         blossom_attention(*d, 16, 0, 9)
+
+
+@pytest.mark.gpu
+def test_transforms_without_a_rule_are_refused():
+    """Batched tensors (vmap) and those of functional gradients have no memory that the library could read."""
+    import torch
+    from paper_2512_13368_b200.autograd import blossom_attention
+    g = torch.Generator(device="cuda").manual_seed(1)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda")  # noqa: E731
+    q, k, v, gate = mk(2, 2, 70, 32), mk(2, 2, 70, 32), mk(2, 2, 70, 32), mk(2, 2)
+    n = torch.tensor([70, 9], dtype=torch.int32, device="cuda")
+    call = lambda a, b, c, d, e: blossom_attention(a, b, c, d, 16, 3, 9, seq_lens=e)  # noqa: E731
+    args = [q, k, v, gate, n]
+    for i, x in enumerate(args):
+        f = lambda t: call(*args[:i], t, *args[i + 1:])  # noqa: E731,B023
+        with pytest.raises(RuntimeError):
+            torch.func.vmap(f)(torch.stack([x, x]))
+        if i < 4:
+            with pytest.raises(RuntimeError):
+                torch.func.grad(lambda t: f(t).sum())(x)  # noqa: B023
+    assert call(*args).shape == q.shape     # (and the interpreter is in order)
