@@ -188,6 +188,13 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
     Tensor phi;
     if (a[5] != Py_None) phi = THPVariable_Unpack(a[5]);  // (checked by the caller)
 
+    // (the tangents would be dropped without a word)
+    for (const Tensor *t : {&q0, &k0, &v0, &gate0})
+      if (t->_fw_grad(/*level=*/0).defined()) {
+        PyErr_SetString(PyExc_NotImplementedError, "blossom_attention has no forward-mode derivative");
+        return nullptr;
+      }
+
     c10::cuda::CUDAGuard guard(q0.device());
     Tensor q = q0, k = k0, v = v0, gate = gate0;
     {

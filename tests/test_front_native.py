@@ -74,3 +74,22 @@ def test_transforms_without_a_rule_are_refused():
             with pytest.raises(RuntimeError):
                 torch.func.grad(lambda t: f(t).sum())(x)  # noqa: B023
     assert call(*args).shape == q.shape     # (and the interpreter is in order)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("train", [False, True])
+def test_forward_mode_is_refused(train):
+    """There is no forward-mode rule: a tangent is an error, never dropped."""
+    import torch
+    import torch.autograd.forward_ad as fwd
+    from paper_2512_13368_b200.autograd import blossom_attention
+    g = torch.Generator(device="cuda").manual_seed(1)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda").requires_grad_(train)  # noqa: E731
+    args = [mk(2, 2, 70, 32), mk(2, 2, 70, 32), mk(2, 2, 70, 32), mk(2, 2)]
+    with fwd.dual_level():
+        for i in range(4):
+            a = list(args)
+            a[i] = fwd.make_dual(a[i], torch.ones_like(a[i]))
+            with pytest.raises(NotImplementedError):
+                blossom_attention(*a, 16, 3, 9)
+    assert blossom_attention(*args, 16, 3, 9).shape == args[0].shape
