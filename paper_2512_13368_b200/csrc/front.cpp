@@ -59,17 +59,18 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 // What the backward needs beside q, k, v, the gate and the indices: one allocation
 // [out_lt | out_st | lse | workspace].
 struct Scratch {
-  Tensor buf;
   size_t span, lse_bytes, ws_bytes;
-  char *base() const { return static_cast<char *>(buf.data_ptr()); }
-  void *out_lt() const { return base(); }
-  void *out_st() const { return base() + span; }
-  float *lse() const { return reinterpret_cast<float *>(base() + 2 * span); }
-  void *workspace() const { return base() + 2 * span + lse_bytes; }
+  size_t bytes() const { return 2 * span + lse_bytes + ws_bytes; }
+  void *out_lt(char *base) const { return base; }
+  void *out_st(char *base) const { return base + span; }
+  float *lse(char *base) const { return reinterpret_cast<float *>(base + 2 * span); }
+  void *workspace(char *base) const { return base + 2 * span + lse_bytes; }
 };
 
 struct BlossomAttentionBackward : public Node {
-  SavedVariable q_, k_, v_, gate_, idx_;
+  // (the scratch buffer, the largest of them, goes through the saved-tensor hooks like the rest: offloading and
+  // checkpointing free it between the passes)
+  SavedVariable q_, k_, v_, gate_, idx_, buf_;
   Tensor lens_, phi_;  // (the params hold phi's address)
   Scratch scratch_;
   blossom_params params_;
@@ -82,13 +83,17 @@ struct BlossomAttentionBackward : public Node {
     v_.reset_data();
     gate_.reset_data();
     idx_.reset_data();
-    scratch_.buf.reset();
+    buf_.reset_data();
   }
   variable_list apply(variable_list &&grads) override {
     at::NoGradGuard no_grad;
     variable_list res(4);
     if (!grads[0].defined()) return res;
-    const Tensor q = q_.unpack(), k = k_.unpack(), v = v_.unpack(), gate = gate_.unpack(), idx = idx_.unpack();
+    const Tensor q = q_.unpack(), k = k_.unpack(), v = v_.unpack(), gate = gate_.unpack(), idx = idx_.unpack(),
+                 buf = buf_.unpack();
+    if (buf.device() != q.device() || (size_t)buf.nbytes() != scratch_.bytes() || !buf.is_contiguous())
+      throw std::runtime_error("blossom_attention: a saved-tensor hook returned another tensor than it was given");
+    char *const base = static_cast<char *>(buf.data_ptr());
     c10::cuda::CUDAGuard guard(q.device());
     Tensor dout = grads[0];
     if (dout.strides() != q.strides() || dout.scalar_type() != q.scalar_type())  // the library wants q's layout
@@ -101,9 +106,9 @@ struct BlossomAttentionBackward : public Node {
     p.reuse_tile_lists = 1;
     const int rc = blossom_attn_bwd(
         &p, q.data_ptr(), k.data_ptr(), v.data_ptr(), gate.data_ptr<float>(),
-        lens_.defined() ? lens_.data_ptr<int32_t>() : nullptr, idx.data_ptr<int32_t>(), scratch_.out_lt(),
-        scratch_.out_st(), scratch_.lse(), dout.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(),
-        dgate.data_ptr<float>(), scratch_.workspace(), scratch_.ws_bytes,
+        lens_.defined() ? lens_.data_ptr<int32_t>() : nullptr, idx.data_ptr<int32_t>(), scratch_.out_lt(base),
+        scratch_.out_st(base), scratch_.lse(base), dout.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(),
+        dgate.data_ptr<float>(), scratch_.workspace(base), scratch_.ws_bytes,
         (blossom_stream_t)c10::cuda::getCurrentCUDAStream(q.device().index()).stream());
     if (rc) throw std::runtime_error(failure("blossom_attn_bwd", rc));
     res[0] = dq;
@@ -234,7 +239,8 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
     s.span = grad ? align256((size_t)q.numel() * q.element_size()) : 0;
     s.lse_bytes = grad ? align256((size_t)2 * B * H * L * sizeof(float)) : 0;
     s.ws_bytes = ws_bytes;
-    s.buf = fresh({(int64_t)(2 * s.span + s.lse_bytes + ws_bytes)}, at::kByte, dev);
+    const Tensor buf = fresh({(int64_t)s.bytes()}, at::kByte, dev);
+    char *const base = static_cast<char *>(buf.data_ptr());
     const int64_t rows = p.select_mode ? L : (L + p.block_size - 1) / p.block_size;
     Tensor out = like(q), idx = fresh({B, Hkv, rows, p.top_k}, at::kInt, dev);
     const blossom_stream_t st = (blossom_stream_t)c10::cuda::getCurrentCUDAStream(dev.index()).stream();
@@ -244,8 +250,9 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const float *gp = gate.data_ptr<float>();
     const int32_t *np = lens.defined() ? lens.data_ptr<int32_t>() : nullptr;
     int32_t *ip = idx.data_ptr<int32_t>();
-    void *op = out.data_ptr(), *lp = grad ? s.out_lt() : nullptr, *sp = grad ? s.out_st() : nullptr, *wp = s.workspace();
-    float *ep = grad ? s.lse() : nullptr;
+    void *op = out.data_ptr(), *lp = grad ? s.out_lt(base) : nullptr, *sp = grad ? s.out_st(base) : nullptr,
+         *wp = s.workspace(base);
+    float *ep = grad ? s.lse(base) : nullptr;
     int rc;
     Py_BEGIN_ALLOW_THREADS;
     rc = blossom_attn_fwd(&p, qp, kp, vp, gp, np, ip, 0, op, lp, sp, ep, wp, ws_bytes, st);
@@ -259,6 +266,7 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
       node->v_ = SavedVariable(v, false);
       node->gate_ = SavedVariable(gate.is_same(gate0) ? gate : gate.detach(), false);
       node->idx_ = SavedVariable(idx, false);
+      node->buf_ = SavedVariable(buf, false);
       node->lens_ = lens;
       node->phi_ = phi;
       node->scratch_ = s;

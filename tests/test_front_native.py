@@ -93,3 +93,46 @@ def test_forward_mode_is_refused(train):
             with pytest.raises(NotImplementedError):
                 blossom_attention(*a, 16, 3, 9)
     assert blossom_attention(*args, 16, 3, 9).shape == args[0].shape
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L,D,rope", [(70, 32, 0.0), (600, 64, 100.0)])
+def test_everything_the_backward_needs_goes_through_the_saved_tensor_hooks(L, D, rope):
+    """Offloaded to the host and brought back, or thrown away and computed again: the same gradients, and
+    nothing of the call's size stays on the GPU between the passes."""
+    import torch
+    from torch.utils.checkpoint import checkpoint
+    from paper_2512_13368_b200.autograd import blossom_attention
+    g = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda")  # noqa: E731
+    args = [mk(8, 2, L, D).bfloat16().requires_grad_(True) for _ in range(3)] + [mk(2, 2).requires_grad_(True)]
+    dout = mk(8, 2, L, D).bfloat16()
+    f = lambda *a: blossom_attention(*a, 32, 3, 40, rope_theta=rope)  # noqa: E731
+    want = torch.autograd.grad(f(*args), args, dout)
+    torch.cuda.synchronize()
+    tensor = dout.nbytes
+
+    def kept(make):
+        before = torch.cuda.memory_allocated()
+        out = make()
+        return out, torch.cuda.memory_allocated() - before
+
+    plain, size = kept(lambda: f(*args))
+    assert size > 3 * tensor                # the output, both branches' rows, the workspace
+    del plain
+    with torch.autograd.graph.save_on_cpu():
+        out, size = kept(lambda: f(*args))
+    assert size < 2 * tensor                # the output alone
+    for a, b in zip(want, torch.autograd.grad(out, args, dout, retain_graph=True)):
+        assert torch.equal(a, b)
+    for a, b in zip(want, torch.autograd.grad(out, args, dout)):
+        assert torch.equal(a, b)
+    del out
+    out, size = kept(lambda: checkpoint(f, *args, use_reentrant=False))
+    assert size < 2 * tensor
+    for a, b in zip(want, torch.autograd.grad(out, args, dout)):
+        assert torch.equal(a, b)
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t, lambda t: t[:1] if t.dtype == torch.uint8 else t):
+        out = f(*args)
+    with pytest.raises(RuntimeError):
+        torch.autograd.grad(out, args, dout)
