@@ -15,24 +15,22 @@ _DT = {torch.float32: "fp32", torch.bfloat16: "bf16"}
 
 
 def _dense(t) -> bool:
-    """True if the tensor's elements tile its storage span without gaps or overlap, so that a
-    buffer of ``numel`` elements laid out with the same strides holds every element."""
-    span = 1 + sum((n - 1) * st for n, st in zip(t.shape, t.stride()) if n > 0)
-    return t.numel() > 0 and span == t.numel() and all(st > 0 for st in t.stride())
+    """The native front end's test of a layout (``dense`` in ``csrc/front.cpp``): True if the tensor's elements
+    tile its storage span without gaps or overlap."""
+    return _module().dense(t)
 
 
 def _like(t):
-    """An uninitialised tensor with exactly t's shape AND strides (``empty_like`` does not keep the
-    strides of a non-dense view; the library writes every q-shaped buffer with the strides passed
-    in the params)."""
-    return torch.empty_strided(t.shape, t.stride(), dtype=t.dtype, device=t.device)
+    """The native front end's output allocation (``like`` in ``csrc/front.cpp``): an uninitialised tensor with
+    exactly t's shape AND strides."""
+    return _module().like(t)
 
 
 def check_arguments(q, k, v, gate_logits, seq_lens, require_cuda=True, gate_mode=0):
-    """Host-side validation before anything is launched: the library receives raw addresses, so a
-    host tensor, a tensor on another device, a wrong integer width or a wrong shape would become a
-    device memory fault instead of a Python error.  Returns seq_lens as the int32 CUDA tensor the
-    library reads (or None).  ``require_cuda=False`` (host-side tests only) skips the test that
+    """Why the native front end, which makes the same tests, would not take the arguments: raises for what
+    is wrong with them (the library receives raw addresses, so a host tensor, a tensor on another device, a
+    wrong integer width or a wrong shape would become a device memory fault instead of a Python error).
+    Returns seq_lens as the int32 tensor that the front end makes of it (or None).  ``require_cuda=False`` (host-side tests only) skips the test that
     the tensors are CUDA tensors and keeps every other check, the same-device one included."""
     if q.dtype not in _DT or k.dtype != q.dtype or v.dtype != q.dtype:
         raise TypeError("q, k, v must share one dtype, float32 or bfloat16")
@@ -64,19 +62,24 @@ def check_arguments(q, k, v, gate_logits, seq_lens, require_cuda=True, gate_mode
 _native = None
 
 
+def _module():
+    """``csrc/front.cpp`` as a module; the library it links is loaded first (the same instance, and its own
+    message if it is missing)."""
+    binding.load()
+    try:
+        from . import _front as m
+    except ImportError as e:
+        raise RuntimeError("_front.so is missing or stale: build it with "
+                           "`python -m paper_2512_13368_b200.build`") from e
+    return m
+
+
 def _front():
-    """The native front end (``csrc/front.cpp``), loaded on first use: it validates, allocates the
-    outputs and one scratch buffer, calls ``blossom_attn_fwd`` and puts a C++ node into the autograd
-    graph that calls ``blossom_attn_bwd``."""
+    """The native front end, loaded on first use: it validates, allocates the outputs and one scratch buffer,
+    calls ``blossom_attn_fwd`` and puts a C++ node into the autograd graph that calls ``blossom_attn_bwd``."""
     global _native
     if _native is None:
-        binding.load()  # the same instance of the library, and its own message if it is missing
-        try:
-            from . import _front as m
-        except ImportError as e:
-            raise RuntimeError("_front.so is missing or stale: build it with "
-                               "`python -m paper_2512_13368_b200.build`") from e
-        _native = m.attention
+        _native = _module().attention
     return _native
 
 

@@ -32,7 +32,8 @@ using torch::autograd::Node;
 using torch::autograd::SavedVariable;
 using torch::autograd::variable_list;
 
-// the tensor's elements tile its storage span without gaps or overlap
+// the tensor's elements tile its storage span without gaps or overlap, so that a buffer of numel elements laid
+// out with the same strides holds every one
 bool dense(const Tensor &t) {
   int64_t span = 1;
   for (int64_t i = 0; i < t.dim(); ++i) {
@@ -42,8 +43,10 @@ bool dense(const Tensor &t) {
   return t.numel() > 0 && span == t.numel();
 }
 
-// an uninitialised tensor with t's shape and strides
+// an uninitialised tensor with exactly t's shape and strides (empty_like does not keep those of a view that is
+// not dense, and the library writes every q-shaped buffer with the strides it is given)
 Tensor like(const Tensor &t) {
+  if (!t.is_cuda()) return at::empty_strided(t.sizes(), t.strides(), t.options());
   return at::detail::empty_strided_cuda(t.sizes(), t.strides(), t.scalar_type(), t.device());
 }
 Tensor fresh(at::IntArrayRef sizes, at::ScalarType type, const at::Device &dev) {
@@ -285,7 +288,24 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
   }
 }
 
+// dense(tensor) -> bool, like(tensor) -> tensor: the two rules above, for the host-side tests
+PyObject *py_dense(PyObject *, PyObject *t) {
+  if (!THPVariable_Check(t)) return PyErr_Format(PyExc_TypeError, "dense() takes a tensor");
+  return PyBool_FromLong(dense(THPVariable_Unpack(t)));
+}
+PyObject *py_like(PyObject *, PyObject *t) {
+  if (!THPVariable_Check(t)) return PyErr_Format(PyExc_TypeError, "like() takes a tensor");
+  try {
+    return THPVariable_Wrap(like(THPVariable_Unpack(t)));
+  } catch (const std::exception &e) {
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
 PyMethodDef methods[] = {
+    {"dense", py_dense, METH_O, nullptr},
+    {"like", py_like, METH_O, nullptr},
     {"attention", (PyCFunction)(void (*)(void))attention, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };

@@ -136,3 +136,64 @@ def test_everything_the_backward_needs_goes_through_the_saved_tensor_hooks(L, D,
         out = f(*args)
     with pytest.raises(RuntimeError):
         torch.autograd.grad(out, args, dout)
+
+
+def test_layout_rules():
+    import torch
+    build.build()
+    from paper_2512_13368_b200 import binding
+    binding.load()
+    from paper_2512_13368_b200 import _front
+    x = torch.zeros(2, 3, 8, 32)
+    for t, dense in ((x, True), (x.transpose(1, 2), True), (x.permute(3, 2, 0, 1), True), (x[:, :1], False),
+                     (x[:1], True), (x[:, :, ::2], False), (x[:1].expand(2, 3, 8, 32), False), (x[:0], False),
+                     (x[:, :, :1], False), (torch.zeros(5), True), (torch.zeros(5).expand(4, 5), False)):
+        assert _front.dense(t) == dense, (t.shape, t.stride())
+        if t.numel() and 0 not in t.stride():
+            assert _front.like(t).stride() == t.stride() and _front.like(t).shape == t.shape
+    for f in (_front.dense, _front.like):
+        with pytest.raises(TypeError):
+            f(3)
+
+
+@pytest.mark.gpu
+def test_every_layout_gives_what_the_dense_tensors_give():
+    """Transposed, packed, strided and broadcast inputs, k and v in layouts of their own, transposed and
+    broadcast upstream gradients; outputs and gradients keep the strides of a dense input."""
+    import torch
+    from paper_2512_13368_b200.autograd import blossom_attention
+    B, H, L, D = 2, 3, 70, 32
+    g = torch.Generator(device="cuda").manual_seed(5)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda").bfloat16()  # noqa: E731
+    gate = torch.randn((H, 2), generator=g, device="cuda")
+
+    def views(x):       # the same numbers [B, H, L, D] in other layouts
+        yield x.transpose(1, 2).contiguous().transpose(1, 2)
+        p = torch.zeros(B, L, 3, H, D, dtype=x.dtype, device="cuda")
+        p[:, :, 1] = x.transpose(1, 2)
+        yield p[:, :, 1].transpose(1, 2)
+        w = torch.zeros(B, H, 2 * L, D, dtype=x.dtype, device="cuda")
+        w[:, :, ::2] = x
+        yield w[:, :, ::2]
+        yield x.permute(3, 2, 1, 0).contiguous().permute(3, 2, 1, 0)    # the last dimension is not contiguous
+
+    def step(q, k, v, dout):
+        leaves = [t.detach().requires_grad_(True) for t in (q, k, v)]
+        out = blossom_attention(*leaves, gate, 16, 3, 9)
+        return [out.detach()] + list(torch.autograd.grad(out, leaves, dout))
+
+    q, k, v, dout = mk(B, H, L, D), mk(B, H, L, D), mk(B, H, L, D), mk(B, H, L, D)
+    want = step(q, k, v, dout)
+    for i, x in enumerate((q, k, v, dout)):
+        for t in views(x):
+            a = [q, k, v, dout]
+            a[i] = t
+            assert torch.equal(t, x)
+            got = step(*a)
+            for y, z in zip(want, got):
+                assert torch.equal(y, z), (i, t.stride())
+    qt = next(views(q))
+    assert step(qt, next(views(k)), next(views(v)), dout)[0].stride() == qt.stride()
+    k1, d1 = mk(1, 1, L, D).expand(B, H, L, D), mk(1, 1, 1, D).expand(B, H, L, D)   # (strides of zero)
+    for y, z in zip(step(q, k1.contiguous(), v, d1.contiguous()), step(q, k1, v, d1)):
+        assert torch.equal(y, z)
