@@ -21,14 +21,6 @@ namespace {
 
 using namespace sh;
 
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)),
-        "l"(*reinterpret_cast<uint64_t *>(&c)));
-  return *reinterpret_cast<float2 *>(&d);
-}
 __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
 
 constexpr int kPP = 20;  // pitch of a 16 x 16 tile in shared memory (floats)

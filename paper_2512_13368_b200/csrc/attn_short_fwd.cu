@@ -35,23 +35,6 @@ struct ShortGeom {
   int o_v, o_warp, warp_bytes, o_mean, o_mean32, o_sel;  // byte offsets in shared memory
 };
 
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)),
-        "l"(*reinterpret_cast<uint64_t *>(&c)));
-  return *reinterpret_cast<float2 *>(&d);
-}
-
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  uint64_t d;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)));
-  return *reinterpret_cast<float2 *>(&d);
-}
-
 // the double of a bf16 value given as fp32 bits (denormals count as zero, as they do in this build's
 // fp32 arithmetic), by rebiasing the exponent: the conversion instruction runs at a fraction of the
 // integer rate.  An infinity or NaN becomes a number of 2^128 and more: it weighs like one in the sums, where

@@ -301,16 +301,6 @@ __device__ __forceinline__ void emit_flags(int32_t *row, const uint8_t *taken, i
 // when a - b > R (a + b).
 constexpr int kFastThreads = 128;
 
-// d = a * b + c on two packed fp32 values: two IEEE fused multiply-adds in one instruction (the
-// same rounding, and the same flush of denormals, as the scalar fmaf of this build)
-__device__ __forceinline__ float2 fma_pair(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)),
-        "l"(*reinterpret_cast<uint64_t *>(&c)));
-  return *reinterpret_cast<float2 *>(&d);
-}
 constexpr int kRowTile = 128;  // positions per CTA
 constexpr int kChunk = 64;     // candidates per product
 
@@ -480,10 +470,10 @@ __global__ void __launch_bounds__(kFastThreads, 3) score_fast_kernel(
 #pragma unroll
                 for (int a = 0; a < 8; ++a) {
                   float2 r = acc2[a][e2];
-                  r = fma_pair(make_float2(qa[a].x, qa[a].x), make_float2(kb[e2][0].x, kb[e2][0].y), r);
-                  r = fma_pair(make_float2(qa[a].y, qa[a].y), make_float2(kb[e2][0].z, kb[e2][0].w), r);
-                  r = fma_pair(make_float2(qa[a].z, qa[a].z), make_float2(kb[e2][1].x, kb[e2][1].y), r);
-                  r = fma_pair(make_float2(qa[a].w, qa[a].w), make_float2(kb[e2][1].z, kb[e2][1].w), r);
+                  r = fma2(make_float2(qa[a].x, qa[a].x), make_float2(kb[e2][0].x, kb[e2][0].y), r);
+                  r = fma2(make_float2(qa[a].y, qa[a].y), make_float2(kb[e2][0].z, kb[e2][0].w), r);
+                  r = fma2(make_float2(qa[a].z, qa[a].z), make_float2(kb[e2][1].x, kb[e2][1].y), r);
+                  r = fma2(make_float2(qa[a].w, qa[a].w), make_float2(kb[e2][1].z, kb[e2][1].w), r);
                   acc2[a][e2] = r;
                 }
               }

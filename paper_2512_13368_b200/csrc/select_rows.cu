@@ -28,14 +28,6 @@ namespace {
 
 constexpr int kRows = 128, kThreads = 128, kWarps = 4;
 
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  uint64_t d;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;"
-      : "=l"(d)
-      : "l"(*reinterpret_cast<uint64_t *>(&a)), "l"(*reinterpret_cast<uint64_t *>(&b)),
-        "l"(*reinterpret_cast<uint64_t *>(&c)));
-  return *reinterpret_cast<float2 *>(&d);
-}
 // N consecutive elements as float pairs (zeros where !ok)
 template <int N>
 __device__ __forceinline__ void load_part(const __nv_bfloat16 *p, bool ok, float2 (&q)[N / 2]) {

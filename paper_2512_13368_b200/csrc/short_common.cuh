@@ -142,19 +142,6 @@ __device__ __forceinline__ void product_nn(const uint32_t (&a)[4], uint32_t chun
     mma16816(acc[2 * n2 + 1], a, b[2], b[3]);
   }
 }
-// the same product added to two accumulators (two branches that share every pair of the chunk)
-template <int D>
-__device__ __forceinline__ void product_nn2(const uint32_t (&a)[4], uint32_t chunk, float (&x)[D / 8][4], float (&y)[D / 8][4]) {
-#pragma unroll
-  for (int n2 = 0; n2 < D / 16; ++n2) {
-    uint32_t b[4];
-    ldsm4t(chunk ^ (32 * n2), b);
-    mma16816(x[2 * n2], a, b[0], b[1]);
-    mma16816(x[2 * n2 + 1], a, b[2], b[3]);
-    mma16816(y[2 * n2], a, b[0], b[1]);
-    mma16816(y[2 * n2 + 1], a, b[2], b[3]);
-  }
-}
 // Probabilities (accumulator layout, 16 x 16) -> first operand of the next product.
 __device__ __forceinline__ void to_a(const float (&p)[2][4], uint32_t (&a)[4]) {
   a[0] = pack2(p[0][0], p[0][1]);

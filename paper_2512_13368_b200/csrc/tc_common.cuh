@@ -237,18 +237,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-      "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-      "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-      "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-      "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-      "r"(__float_as_uint(v[15]))
-      : "memory");
-}
 // packed words (two bf16 per 32-bit column) -> tensor memory
 __device__ __forceinline__ void tmem_st32u(uint32_t taddr, const uint32_t *v) {
   asm volatile(
@@ -306,11 +294,6 @@ template <int N>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float *v) {
   static_assert(N == 16 || N == 32, "16 or 32 columns");
   if constexpr (N == 32) tmem_ld32(taddr, v); else tmem_ld16(taddr, v);
-}
-template <int N>
-__device__ __forceinline__ void tmem_st(uint32_t taddr, const float *v) {
-  static_assert(N == 16 || N == 32, "16 or 32 columns");
-  if constexpr (N == 32) tmem_st32(taddr, v); else tmem_st16(taddr, v);
 }
 
 // ---- descriptors --------------------------------------------------------------------------
@@ -433,12 +416,6 @@ __device__ __forceinline__ uint64_t st_query_cols(const Shape &s, int p, int t0,
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t *>(&h);
-}
-
-// Store one 64-column bf16 row (row r of a [rows][64] tile with 128-byte rows, 128-byte swizzle:
-// 16-byte chunk ch lands at chunk position ch ^ (r & 7)).  `tile` must be 1024-byte aligned.
-__device__ __forceinline__ void store_row_sw128(uint8_t *tile, int r, int ch, uint4 v) {
-  *reinterpret_cast<uint4 *>(tile + r * 128 + ((ch ^ (r & 7)) << 4)) = v;
 }
 
 // ---- pieces shared by the forward and backward kernels ------------------------------------
