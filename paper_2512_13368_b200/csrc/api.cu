@@ -153,8 +153,9 @@ static int make_shape(const blossom_params *p, Shape *out) {
   if ((int64_t)p->batch * p->heads * M > 0x7fffffffLL) return BLOSSOM_ERR_UNSUPPORTED;
   Shape s;
   s.B = p->batch; s.H = p->heads; s.L = p->seq_len; s.D = p->head_dim; s.Bk = p->block_size;
-  s.topk = p->top_k; s.window = p->window; s.M = (int)M;
-  s.stis_mode = p->stis_mode; s.stis_blk = p->stis_block > 0 ? p->stis_block : 1;
+  // (a window or mask block past the sequence changes no mask; unclamped, sums like position + window overflow)
+  s.topk = p->top_k; s.window = p->window < p->seq_len ? p->window : p->seq_len; s.M = (int)M;
+  s.stis_mode = p->stis_mode; s.stis_blk = p->stis_block > 0 ? (p->stis_block < p->seq_len ? p->stis_block : p->seq_len) : 1;
   s.cmp_l = s.cmp_s = s.Mc = 0;
   if (p->cmp_block < 0 || p->cmp_stride < 0) return BLOSSOM_ERR_INVALID_ARG;
   if (p->cmp_block > 0 || p->cmp_stride > 0) {
