@@ -23,13 +23,11 @@ CASES = [  # dtype, H, Hkv, L, D, block, lengths, options
 ]
 
 
-@pytest.mark.parametrize("what", ["window", "mask_block"])
-@pytest.mark.parametrize("dtype,H,Hkv,L,D,block,lens,opts", CASES)
+@pytest.mark.parametrize("dtype,H,Hkv,L,D,block,lens,opts,what", [c + ("window",) for c in CASES] +
+                         [c + ("mask_block",) for c in CASES if c[-1].get("power_law")])
 def test_limits_past_the_sequence(dtype, H, Hkv, L, D, block, lens, opts, what):
     import torch
     from paper_2512_13368_b200 import runner
-    if what == "mask_block" and not opts.get("power_law"):
-        pytest.skip("the window alone has no mask block")
     first = None
     for x in (L, L + 1, 2 * L, INT_MAX - 16, INT_MAX):
         w = workloads.make("limits", dtype, 2, H, L, D, block, 3, x if what == "window" else 9, seed=L, lengths=lens,
