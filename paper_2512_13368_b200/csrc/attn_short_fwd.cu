@@ -445,13 +445,14 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) fwd_short_kernel(
         // The bound of select.cu, with the roundings of the mean's sum (g.l / 2 + 2 of them, relative to the
         // block's keys and not to their mean) added to E: E on every logit, 2^-21 and 2^-22 per unit of logit range for the
         // exponentials and the division, one rounding per addition of the normaliser (ncol) and of
-        // the column sums (rows and heads of the block), per term of Eq. 11, and a margin of 40.
+        // the column sums (rows and heads of the block), per term of Eq. 11, and a margin of 40; 1e-30 for what is
+        // flushed below 2^-126 of a row's largest exponential.
         const float uu = 5.9604645e-8f, bound = s.scale * qn * kn;
         const float E = ((float)(D + 6) * bound + (float)(g.l / 2 + 2) * s.scale * qn * krms) * uu * 1.01f;
         const float R_ = 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f +
                          (float)(ncol + s.Bk * s.G + 2 * s.G + g.rs * g.rl + 40) * uu;
         // (a negative score is no number: left to double precision)
-        const bool certain = !exact && dropped >= 0.f && (kept - dropped) > R_ * (kept + dropped) * 1.001f;
+        const bool certain = !exact && dropped >= 0.f && (kept - dropped) > R_ * (kept + dropped) * 1.001f + 1e-30f;
         if (!certain) {  // decided in double precision below, by all warps
           if (lane == 0) uncertain[atomicAdd(&n_uncertain, 1)] = b;
           __syncwarp();

@@ -298,7 +298,7 @@ __device__ __forceinline__ void emit_flags(int32_t *row, const uint8_t *taken, i
 // division), 2^-22 per unit of logit range, and one u per addition: 16 per candidate chunk for
 // the normaliser, 2 + Bk / 4 for the column sum, one per head of the group, one per term of
 // Eq. 11, and a margin of 40.  R is the total, relative; two scores a > b are in certain order
-// when a - b > R (a + b).
+// when a - b > R (a + b) + 1e-30 (what is flushed below 2^-126 of a row's largest exponential).
 constexpr int kFastThreads = 128;
 
 constexpr int kRowTile = 128;  // positions per CTA
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kFastThreads, 3) score_fast_kernel(
       const float R = 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f +
                       (16.f * nchunks + (float)(Bk / 4) + 2.f + (float)sh.G + (float)(g.rs * g.rl) + 40.f) * uu;
       const float smin = bound_s[i][0], umax = bound_s[i][1];
-      certain = umax >= 0.f && (smin - umax) > R * (smin + umax) * 1.001f;  // (a negative one is no number)
+      certain = umax >= 0.f && (smin - umax) > R * (smin + umax) * 1.001f + 1e-30f;  // (a negative one is no number)
     }
     __syncwarp();
     if (certain) emit_row(row, tk, jmin, b, sh.topk, lane);

@@ -19,7 +19,11 @@
 // results added up, the smaller ones, at 2^-8 of their size, in one go (2 D additions): (32 + D / 16 + 0.1 D
 // + 6) u bound.  The exponentials add 2^-21 and 2^-22 per unit of logit range; sums of non-negative
 // terms add one u per addition that a term goes through (the normaliser, 16 rows, the 16-row groups of a
-// block, the heads, Eq. 11), with a margin of 40.
+// block, the heads, Eq. 11), with a margin of 40.  One loss is not relative to the scores: exponentials (and
+// products) below 2^-126 are flushed to zero.  A row is left to double precision unless its sum exceeds
+// kMinDen = 2^-63, so each costs a probability less than 2^-62, and the certificate allows the dropped block
+// one of them per row, head and term of Eq. 11.  (2^-100 would accept looser references, but then
+// scores less than 1e-8 apart were never certain; 2^-63 is a reference 43 above the row's largest logit.)
 #include "select_rows.cuh"
 #include "short_common.cuh"
 
@@ -27,6 +31,7 @@ namespace blossom {
 namespace {
 
 constexpr int kRows = 128, kThreads = 128, kWarps = 4;
+constexpr float kMinDen = 1.0842022e-19f, kLost = 2.f * 2.1684043e-19f;  // 2^-63; twice 2^-62
 
 // N consecutive elements as float pairs (zeros where !ok)
 template <int N>
@@ -315,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
             den[i] = sh::quad_sum(den[i]);
             if (tig == 0) {
               const int r = 16 * mt + gid + 8 * i;
-              const bool bad = (i ? ok1 : ok0) && ncm[i] > own && !(den[i] > 1e-30f);  // the reference is too far away
+              const bool bad = (i ? ok1 : ok0) && ncm[i] > own && !(den[i] > kMinDen);  // the reference is too far away
               inv_s[warp][r] = den[i] > 0.f ? 1.f / den[i] : 0.f;
               rowq_s[warp][r] = fmaxf(rowq_s[warp][r], bad ? INFINITY : qh[i]);
             }
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
         er[c + 1] = e1;
         den += e0 + e1;
       }
-      loose |= nc > own && !(den > 1e-30f);
+      loose |= nc > own && !(den > kMinDen);
       const float inv = den > 0.f ? 1.f / den : 0.f;
       if (PQ) {
         if (sh.G > 1) {
@@ -399,6 +404,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
     const float bound = bound0 * qmax, E = (kMma ? 32.f + 0.1f * D + (float)(D / 16) + 6.f : (float)(D + 4)) * uu * bound * 1.01f;
     return 2.f * E + 4.77e-7f + 2.f * bound * 2.39e-7f + (nsum + 2.f * (float)sh.G + (float)(g.rs * g.rl) + 40.f) * uu;
   };
+
+  // what flushed exponentials of so many rows can take from a score
+  auto lost = [&](int rows) { return (float)(rows * sh.G * g.rs * g.rl) * kLost; };
 
   if (PQ) {
     // ---- Eq. 11, Eq. 13 and the certificate for this lane's own row ----
@@ -454,7 +462,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
             else taken[3] |= bit;
           }
         }
-        certain = !rg.exact && !loose && (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f;
+        certain = !rg.exact && !loose &&
+                  (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f + lost(1);
       }
       if (certain) {
         int pos = 0;
@@ -559,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
       kept = __uint_as_float(__reduce_max_sync(0xffffffffu, kept < 0.f ? 0u : __float_as_uint(kept)));
       dropped = __uint_as_float(__reduce_max_sync(0xffffffffu, dropped < 0.f ? 0u : __float_as_uint(dropped)));
       const float R = error(qmax, (float)(den_adds(ncb - cmin) + 16 + gpb));
-      certain = !rg.exact && (kept - dropped) > R * (kept + dropped) * 1.001f;  // (false for an infinite qmax)
+      certain = !rg.exact && (kept - dropped) > R * (kept + dropped) * 1.001f + lost(Bk);  // (false for an infinite qmax)
     }
     if (own && lane == 0) tk[bb] = 1;
     __syncwarp();
