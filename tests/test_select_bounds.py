@@ -86,3 +86,18 @@ def test_scores_that_no_bound_separates(B, H, Hkv, L, D, block, dtype, opts):
     w.q = workloads.quantize(w.q * np.float32(1e-5), dtype)
     a, b = _both(runner.DeviceProblem(w))
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("H,Hkv,L,block,dtype", [(2, 1, 8 * 1024, 8, "bf16"), (5, 1, 16 * 655, 16, "bf16"),
+                                                 (5, 1, 16 * 670, 16, "bf16"), (1, 1, 16 * 1024, 16, "fp32")])
+def test_per_position_selection_of_very_many_blocks(H, Hkv, L, block, dtype):
+    """Around the number of blocks from which a warp keeps one head's logits at a time, and the largest number."""
+    import torch
+    from paper_2512_13368_b200 import binding, runner
+    w = workloads.make("many", dtype, 1, H, L, 32, block, 4, 16, seed=H, kv_heads=Hkv if Hkv != H else 0)
+    w.per_query = 1
+    p = runner.DeviceProblem(w, training=False)
+    p.select()
+    torch.cuda.synchronize()
+    check_indices(w, p.idx.cpu().numpy())
+    assert binding.blossom_device_status(p.workspace) == 0
