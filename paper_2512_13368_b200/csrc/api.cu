@@ -7,7 +7,7 @@
 
 namespace blossom {
 
-unsigned long long g_launches = 0;
+std::atomic<unsigned long long> g_launches{0};
 
 // ---- optional per-launch event profile (process-wide, off by default) ---------------------
 static cudaEvent_t *g_prof_events = nullptr;  // [2 * cap]: before / after each launch
@@ -464,6 +464,6 @@ const char *blossom_kernel_name(int id) {
   return (id >= 0 && id < K_COUNT) ? names[id] : "unknown";
 }
 
-uint64_t blossom_launch_count(void) { return g_launches; }
+uint64_t blossom_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 }  // extern "C"

@@ -770,12 +770,6 @@ constexpr int kCtaWarps = 4;
 int chunk_split(int64_t tasks) { return tasks <= 148 * 6 ? kCtaWarps : 1; }
 unsigned ctas(int64_t tasks, int split) { return (unsigned)(split > 1 ? tasks : (tasks + kCtaWarps - 1) / kCtaWarps); }
 
-template <typename K>
-bool allow(K kern, size_t smem) {
-  return smem <= 48 * 1024 ||
-         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
-}
-
 template <int D>
 int launch_fwd_t(const Shape &s, const float *q, const float *k, const float *v, const float *gate, const int32_t *seq_lens,
                  const int32_t *idx, float *out, float *out_lt, float *out_st, float *lse, cudaStream_t st) {
@@ -784,7 +778,7 @@ int launch_fwd_t(const Shape &s, const float *q, const float *k, const float *v,
   const int64_t tasks = (int64_t)s.B * s.H * ((s.L + 15) / 16);
   const int split = chunk_split(tasks);
   const size_t smem = (size_t)kCtaWarps * (5 * Geo<D>::kTile + 2 * 16 * kPP) * sizeof(float);
-  if (!allow(kern, smem)) return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
   LaunchScope ls(K_FWD_SIMT, st);
   return launch_chained(kern, dim3(ctas(tasks, split)), dim3(32 * kCtaWarps), smem, st, s, q, k, v, gate, seq_lens, idx, out,
                         out_lt, out_st, lse, split) == cudaSuccess
@@ -805,7 +799,7 @@ int launch_bwd_t(const Shape &s, const float *q, const float *k, const float *v,
   constexpr int T = Geo<D>::kTile;
   const size_t sq = (size_t)kCtaWarps * (6 * T + 16 * kPP) * sizeof(float);
   const size_t sk = (size_t)kCtaWarps * (2 * T + 2 * (2 * T + 64) + 2 * 16 * kPP) * sizeof(float);
-  if (!allow(kq, sq) || !allow(kk, sk)) return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kq, sq) || !allow_smem(kk, sk)) return BLOSSOM_ERR_CUDA;
   {
     LaunchScope ls(K_BWD_DQ_SIMT, st);
     if (launch_chained(kq, dim3(ctas(tq, wq)), dim3(32 * kCtaWarps), sq, st, s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse,

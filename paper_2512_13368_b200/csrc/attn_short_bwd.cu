@@ -397,9 +397,7 @@ static int launch_t(const Shape &s, const void *q, const void *k, const void *v,
   const int smem = bg.o_sel + 128;
   const bool plain = s.causal && s.stis_mode == 0;
   auto kern = plain ? bwd_short_kernel<D, true> : bwd_short_kernel<D, false>;
-  if (smem > 40 * 1024 &&  // (static shared memory counts too)
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, (size_t)smem)) return BLOSSOM_ERR_CUDA;
   LaunchScope ls(K_BWD_SHORT, st);
   if (launch_chained(kern, dim3((unsigned)(bg.nkey_ctas + s.B * s.H * bg.nq)), dim3(128), (size_t)smem, st, s, bg,
                      (const bf *)q, (const bf *)k, (const bf *)v, gate, seq_lens, idx, (const bf *)out_lt,

@@ -771,9 +771,7 @@ static int launch_t(const Shape &s, const void *q, const void *k, const void *v,
   const int smem = short_geom(s, g, &sg);
   const bool plain = s.causal && s.stis_mode == 0;
   auto kern = plain ? fwd_short_kernel<D, true> : fwd_short_kernel<D, false>;
-  if (smem > 40 * 1024 &&  // (static shared memory counts too)
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, (size_t)smem)) return BLOSSOM_ERR_CUDA;
   LaunchScope ls(K_FWD_TC, st);
   if (launch_chained(kern, dim3((unsigned)(s.B * s.Hkv * sg.nsplit)), dim3(128), (size_t)smem, st, s, g, sg, (const bf *)q,
                      (const bf *)k, (const bf *)v, gate, seq_lens, idx, idx_is_input, exact_select_only() ? 1 : 0,

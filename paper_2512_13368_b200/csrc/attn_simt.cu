@@ -599,10 +599,7 @@ int launch_fwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
   const unsigned grid = (unsigned)s.M * (unsigned)(s.B * s.H);
   const size_t rowsel = s.pq ? (size_t)s.Bk * ((s.M + 31) / 32) * sizeof(uint32_t) : 0;
   const size_t smem = (size_t)2 * s.Bk * D * sizeof(float) + (size_t)s.M * sizeof(int) + rowsel;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(fwd_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(fwd_simt_kernel<T, D>, smem)) return BLOSSOM_ERR_CUDA;
   {
     LaunchScope ls(K_FWD_SIMT, st);
     fwd_simt_kernel<T, D><<<grid, s.Bk * 4, smem, st>>>(s, q, k, v, gate, seq_lens, idx, out, out_lt,
@@ -620,10 +617,7 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
   const size_t rowsel = s.pq ? (size_t)s.Bk * ((s.M + 31) / 32) * sizeof(uint32_t) : 0;
   const size_t smem_q = (size_t)2 * s.Bk * D * sizeof(float) +
                         (size_t)(s.M + (s.M & 1)) * sizeof(int) + (size_t)s.Bk * sizeof(double) + rowsel;
-  if (smem_q > 48 * 1024 &&
-      cudaFuncSetAttribute(bwd_dq_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_q) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(bwd_dq_simt_kernel<T, D>, smem_q)) return BLOSSOM_ERR_CUDA;
   {
     LaunchScope ls(K_BWD_DQ_SIMT, st);
     bwd_dq_simt_kernel<T, D><<<grid, s.Bk * 4, smem_q, st>>>(s, q, k, v, gate, seq_lens, idx, out_lt,
@@ -631,10 +625,7 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
                                                              ws.dalpha, ws.gate_ac, ws.dgate_part);
   }
   const size_t smem_k = (size_t)(2 * s.Bk * D + 6 * s.Bk) * sizeof(float) + (size_t)(s.M + s.Bk) * sizeof(int);
-  if (smem_k > 48 * 1024 &&
-      cudaFuncSetAttribute(bwd_dkdv_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem_k) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(bwd_dkdv_simt_kernel<T, D>, smem_k)) return BLOSSOM_ERR_CUDA;
   {
     LaunchScope ls(K_BWD_DKDV_SIMT, st);
     const unsigned grid_k = (unsigned)s.M * (unsigned)(s.B * s.Hkv);

@@ -949,9 +949,7 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   } else if (s.pack) {
     kern_dq = bwd_dq_tc_kernel<D, kGeneral, true>;
   }
-  if (cudaFuncSetAttribute(kern_dq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_dq) != cudaSuccess ||
-      cudaFuncSetAttribute(kern_kv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_kv) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern_dq, smem_dq) || !allow_smem(kern_kv, smem_kv)) return BLOSSOM_ERR_CUDA;
   if (!records && !s.reuse_lists)  // (the passes of the input-dependent gate have got theirs)
     if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, ws.kmeta, st, ws.status + kTicketWord, branches)) return rc;
   const float4 *rec = records ? records : ws.qstats;

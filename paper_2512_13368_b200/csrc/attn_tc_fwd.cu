@@ -542,8 +542,7 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   const bool plain = s.causal && !s.pq;
   auto kern = s.pack ? (plain ? fwd_tc_kernel<D, true, true> : fwd_tc_kernel<D, false, true>)
                      : (plain ? fwd_tc_kernel<D, true, false> : fwd_tc_kernel<D, false, false>);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
   const int n_tiles = s.pack ? nT * (s.B * (s.H / 2)) : nST * (s.B * s.H);
   const int resident = 148 * (smem <= kPair ? 2 : 1);
   const unsigned grid = (unsigned)(n_tiles < resident ? n_tiles : resident);

@@ -464,9 +464,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   const int per_cta = wide ? 1 : kMetaWarps;
   const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((3 * nT + 15) / 16) * 16);
   auto kern = wide ? tc_meta_kernel<kMetaWarps> : tc_meta_kernel<1>;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
   auto launch = [&](int image0, int image_end, uint32_t *inv_bits) {
     LaunchScope ls(K_TC_META, st);
     launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "../../include/blossom.h"
@@ -71,7 +72,7 @@ struct Workspace {
 
 Workspace carve_workspace(const Shape &s, void *base);
 
-extern unsigned long long g_launches;  // host-side launch counter
+extern std::atomic<unsigned long long> g_launches;  // host-side launch counter
 
 // Kernel identifiers reported by the optional per-launch event profile.
 enum KernelId {
@@ -85,7 +86,7 @@ void prof_mark(int id, int phase, cudaStream_t st);  // no-op unless a profile i
 struct LaunchScope {
   int id;
   cudaStream_t st;
-  LaunchScope(int id_, cudaStream_t st_) : id(id_), st(st_) { ++g_launches; prof_mark(id, 0, st); }
+  LaunchScope(int id_, cudaStream_t st_) : id(id_), st(st_) { g_launches.fetch_add(1, std::memory_order_relaxed); prof_mark(id, 0, st); }
   ~LaunchScope() { prof_mark(id, 1, st); }
 };
 
@@ -109,6 +110,17 @@ __device__ __forceinline__ void grid_chain_enter() {
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 bool chained_launches();  // blossom_debug_switch(2, ...) / BLOSSOM_SERIAL_LAUNCH
+
+// Dynamic shared memory beyond 48 KB (less what a kernel has of its own) takes an attribute of the function,
+// which host threads share: set to each call's own size, one thread's launch is refused when another has
+// just lowered it.  So every call that needs it sets the same value, the most any kernel here can ask for.
+constexpr size_t kMaxDynamicSmem = 224 * 1024;
+template <typename K>
+inline bool allow_smem(K kern, size_t bytes) {
+  return bytes <= 40 * 1024 ||
+         (bytes <= kMaxDynamicSmem &&
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem) == cudaSuccess);
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -1154,11 +1154,9 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
         return rc;
     }
     const auto need = [&](int hp) { return (size_t)8 * per_query_doubles(sh, g, D, hp) * sizeof(double) + (size_t)8 * sh.M + 16; };
-    const int hp = need(4) <= 220 * 1024 ? 4 : 1;
+    const int hp = need(4) <= kMaxDynamicSmem ? 4 : 1;
     const size_t psm = need(hp);
-    if (psm > 40 * 1024 && cudaFuncSetAttribute(score_per_query_kernel<T, D>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm) != cudaSuccess)
-      return BLOSSOM_ERR_CUDA;
+    if (!allow_smem(score_per_query_kernel<T, D>, psm)) return BLOSSOM_ERR_CUDA;
     LaunchScope ls(K_SCORE_SELECT, st);
     const int64_t ctas = (units * sh.L + 7) / 8;
     launch_chained(score_per_query_kernel<T, D>, dim3((unsigned)(listed && ctas > 592 ? 592 : ctas)), dim3(256), psm, st, sh,
@@ -1176,9 +1174,7 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
     if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, w.mean, seq_lens, idx, w.list, w.count, st)) return rc;
     if (!rg.list) return BLOSSOM_OK;
   } else if (!exact_only) {
-    if (fsm > 48 * 1024 && cudaFuncSetAttribute(score_fast_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)fsm) != cudaSuccess)
-      return BLOSSOM_ERR_CUDA;
+    if (!allow_smem(score_fast_kernel<T, D>, fsm)) return BLOSSOM_ERR_CUDA;
     const unsigned ntiles = (unsigned)((sh.L + kRowTile - 1) / kRowTile);
     LaunchScope ls(K_SCORE_FAST, st);
     launch_chained(score_fast_kernel<T, D>, dim3(ntiles * (unsigned)units), dim3(kFastThreads), fsm, st, sh, g, q,
@@ -1210,9 +1206,7 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
     auto exact = score_exact16_kernel<T, D>;
     const size_t esm = ((size_t)(g.n + 1 + 16) * (D + 2) + (size_t)16 * ((g.n + 1) | 1) + 4 * 128 + 128 + sh.M) * sizeof(double) +
                        (size_t)sh.M + 16;
-    if (esm > 40 * 1024 &&
-        cudaFuncSetAttribute(exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm) != cudaSuccess)
-      return BLOSSOM_ERR_CUDA;
+    if (!allow_smem(exact, esm)) return BLOSSOM_ERR_CUDA;
     plan(16, 1184);
     cfg.blockDim = dim3(128);
     cfg.dynamicSmemBytes = esm;
@@ -1223,9 +1217,7 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   }
   const size_t esm = exact_smem_bytes(sh, g, D, &sc_len);
   auto exact = score_exact_kernel<T, D>;
-  if (esm > 48 * 1024 &&
-      cudaFuncSetAttribute(exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(exact, esm)) return BLOSSOM_ERR_CUDA;
   plan(64, 592);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = esm;

@@ -680,9 +680,7 @@ static int launch_t(const Shape &sh, const SelGeom &g, const RowsGeom &rg, size_
                     const float *norm, const double *mean, const int32_t *seq_lens, int32_t *idx,
                     int32_t *list, int32_t *count, cudaStream_t st) {
   auto kern = sh.pq ? score_rows_kernel<T, D, true> : score_rows_kernel<T, D, false>;
-  if (smem > 40 * 1024 &&  // (static shared memory counts too)
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return BLOSSOM_ERR_CUDA;
+  if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
   const unsigned grid = (unsigned)((sh.L + kRows - 1) / kRows) * (unsigned)(sh.B * sh.Hkv);
   LaunchScope ls(K_SCORE_FAST, st);
   return launch_chained(kern, dim3(grid), dim3(kThreads), smem, st, sh, g, rg, q, mean32, norm, mean, seq_lens, idx,
