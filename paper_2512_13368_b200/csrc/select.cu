@@ -1149,7 +1149,6 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
     if (!rows && !g.plain && g.n > 128) return BLOSSOM_ERR_UNSUPPORTED;  // (see make_shape)
     const bool listed = rows && !exact_select_only();
     if (listed) {
-      rg.exact = 0;
       if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, w.mean, seq_lens, idx, w.list, w.count, st))
         return rc;
     }
@@ -1170,7 +1169,6 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
   const bool use_rows = rows && sh.Bk >= 16;  // (it sums the columns in groups of 16 rows)
   const bool exact_only = exact_select_only() || (!use_rows && (fsm == 0 || !sh.causal));
   if (!exact_only && use_rows) {
-    rg.exact = 0;
     if (int rc = launch_score_rows(sh, g, rg, rsm, dtype, q, w.mean32, w.norm, w.mean, seq_lens, idx, w.list, w.count, st)) return rc;
     if (!rg.list) return BLOSSOM_OK;
   } else if (!exact_only) {

@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
             else taken[3] |= bit;
           }
         }
-        certain = !rg.exact && !loose &&
+        certain = !loose &&
                   (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f + lost(1);
       }
       if (certain) {
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
       kept = __uint_as_float(__reduce_max_sync(0xffffffffu, kept < 0.f ? 0u : __float_as_uint(kept)));
       dropped = __uint_as_float(__reduce_max_sync(0xffffffffu, dropped < 0.f ? 0u : __float_as_uint(dropped)));
       const float R = error(qmax, (float)(den_adds(ncb - cmin) + 16 + gpb));
-      certain = !rg.exact && (kept - dropped) > R * (kept + dropped) * 1.001f + lost(Bk);  // (false for an infinite qmax)
+      certain = (kept - dropped) > R * (kept + dropped) * 1.001f + lost(Bk);  // (false for an infinite qmax)
     }
     if (own && lane == 0) tk[bb] = 1;
     __syncwarp();
@@ -666,10 +666,15 @@ bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_
   const size_t tail = (size_t)(8 * 128 + 2 * kWarps * 132) * 4 + kWarps * 128;
   *smem = (size_t)rg->means * 4 + (tables > tail ? tables : tail) + 16;
   // What single precision cannot certify (some percent of the blocks) the kernel decides itself while that
-  // takes a CTA a few microseconds: no second launch (D 32, L 1024, block 32: 40 -> 32 us for both).  With
-  // more rows, candidates or dimensions the CTA that has such a block ends long after the others (D 64, L
-  // 900, block 32: 27 us either way; L 4096, block 64: 105 -> 147 us): a list, shared by clusters of CTAs.
-  rg->list = sh.pq || sh.G * sh.Bk > 128 || (int64_t)sh.G * sh.Bk * g.n * sh.D > 32768;
+  // takes a CTA a few microseconds: no second launch.  With more rows, candidates or dimensions the CTA that
+  // has such a block ends long after the others, unless there are waves of others behind it: a list, shared by
+  // clusters of CTAs.  Time with a list / without one over 176 shapes (D 32 and 64, blocks of 16 - 64, L 256 -
+  // 2048, 8 - 512 units), by the block's products x and the CTAs (740 fit on the GPU):
+  //     x up to              16384   24576   32768   45056   65536  131072
+  //     fewer than 1480 CTAs  1.07    1.05    0.95    0.99    0.85    0.73
+  //     1480 CTAs and more    1.13    1.08    1.04    1.01    1.01    0.94
+  const int64_t x = (int64_t)sh.G * sh.Bk * g.n * sh.D, ctas = (int64_t)((sh.L + kRows - 1) / kRows) * sh.B * sh.Hkv;
+  rg->list = sh.pq || sh.G * sh.Bk > 128 || x > (ctas >= 1480 ? 65536 : 24576);
   const size_t own = ((size_t)16 * ((g.n + 1) | 1) + kWarps * 128 + 128 + 128) * 8 + 128;
   if (!rg->list && *smem < own) *smem = own;
   return *smem <= 200 * 1024;
