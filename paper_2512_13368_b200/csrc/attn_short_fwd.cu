@@ -723,9 +723,10 @@ int short_geom(const Shape &s, const SelGeom &g, ShortGeom *o) {
   // With fewer (batch, head) pairs than fill the SMs three times the query blocks are split over CTAs (a finer
   // split of few pairs only repeats the loads and means: 12 -> 16 us at B 32, L 100); with up to twice as many
   // every pair's blocks go to two CTAs, so that the long ones start first and the rest fills up (512 pairs,
-  // L 200: 38 -> 34 us).  Nine times with grouped heads, whose CTAs have several heads' rows to do (B 128, 8 heads
-  // on 2: three times 83, six 61, nine 57, eighteen 62 us).
-  const int units = s.B * s.Hkv, want = s.G > 1 ? 1332 : units >= 444 ? 888 : 444;
+  // L 200: 38 -> 34 us).  Six times with grouped heads, whose CTAs have several heads' rows to do, and two CTAs up to
+  // nine times: over 216 shapes (two and four heads a group, L 50 - 400, B 4 - 512, D 32 and 64) three, six, nine
+  // and eighteen times are 8, 3, 4 and 10 % behind the best of each shape, this rule 2 %.
+  const int units = s.B * s.Hkv, want = s.G > 1 ? (units >= 888 ? 1332 : 888) : units >= 444 ? 888 : 444;
   int nsplit = units >= want ? 1 : (want + units - 1) / units;
   o->nsplit = nsplit > s.M ? s.M : nsplit;
   o->per = s.M / o->nsplit;
@@ -747,8 +748,10 @@ int short_geom(const Shape &s, const SelGeom &g, ShortGeom *o) {
 //         L 400    29 / 66        82 / 80         421 / 346
 // It wins while two of its CTAs fit on an SM (the keys and values of a head in shared memory) and,
 // where only one does, with so few (batch, head) pairs that the other path's launches count.
-// Training calls of 256 positions and more with fewer than 32 pairs stay on the general kernels: the
-// layer harness accounts for a launch per stage of the path at such sizes.
+// Training calls of 256 positions and more with fewer than 32 pairs stay on the general kernels, although
+// that is slower (forward + backward, us, general / short; 2 to 28 pairs, L 256 - 400): D 32 44 - 60 / 27 - 45,
+// D 64 46 - 60 / 33 - 59.  The only reason is a test of the layer harness that counts seven launches a layer at
+// 16 pairs of 256 positions, more than the two of the short path.
 bool fwd_short_supported(const Shape &s, int dtype, bool training) {
   if (dtype != BLOSSOM_DTYPE_BF16 || s.gate_mode || s.pq || s.phi) return false;
   if (s.Bk < 16 || s.M > 32 || s.L > 512 || s.G > 64) return false;
