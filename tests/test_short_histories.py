@@ -21,6 +21,7 @@ CASES = [  # B, H, Hkv, L, D, block, topk, window, lengths, options
     (2, 2, 2, 143, 64, 32, 3, 20, (20, 143), {"causal": 0, "power_law": 3}),
     (9, 4, 4, 400, 32, 16, 6, 50, (30, 400), {}),       # the largest training length of the rule
     (33, 2, 2, 300, 64, 32, 4, 64, (1, 300), {}),       # short forward, general backward
+    (56, 2, 2, 300, 64, 32, 4, 64, (1, 300), {}),       # (the row above is still within the short backward's rule, this is not)
     (2, 2, 2, 128, 64, 16, 4, 24, None, {"std": 9.0}),  # logits of several hundred
     (2, 2, 2, 96, 32, 16, 3, 10, None, {"ties": 1}),
 ]
