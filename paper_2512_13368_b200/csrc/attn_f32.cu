@@ -1,8 +1,9 @@
 // Single-precision forward and backward of the fused two-branch attention (blocks of 16 and more, one
 // selection per query block, per-head gate).
 //
-// The tolerance of fp32 inputs rules out tensor-core products, so the products are register tiles of
-// packed fp32 multiply-adds.  A warp owns 16 query rows (forward, dQ) or 16 keys (dK/dV) of a head and
+// The tolerance of fp32 inputs rules out a tensor-core product of rounded operands (one of bf16 or TF32; three
+// bf16 parts per operand, six products, would do, and have not been tried), so the products are register tiles
+// of packed fp32 multiply-adds.  A warp owns 16 query rows (forward, dQ) or 16 keys (dK/dV) of a head and
 // walks the 16-position chunks that its block selected (or was selected by) or its window reaches, with the
 // next chunk's rows on their way by cp.async: no barrier between warps, any number of warps per CTA.  A
 // chunk in both branches costs one S product and, in the forward, one exponential per pair (as in
