@@ -723,10 +723,13 @@ int short_geom(const Shape &s, const SelGeom &g, ShortGeom *o) {
   // With fewer (batch, head) pairs than fill the SMs three times the query blocks are split over CTAs (a finer
   // split of few pairs only repeats the loads and means: 12 -> 16 us at B 32, L 100); with up to twice as many
   // every pair's blocks go to two CTAs, so that the long ones start first and the rest fills up (512 pairs,
-  // L 200: 38 -> 34 us).  Six times with grouped heads, whose CTAs have several heads' rows to do, and two CTAs up to
-  // nine times: over 216 shapes (two and four heads a group, L 50 - 400, B 4 - 512, D 32 and 64) three, six, nine
-  // and eighteen times are 8, 3, 4 and 10 % behind the best of each shape, this rule 2 %.
-  const int units = s.B * s.Hkv, want = s.G > 1 ? (units >= 888 ? 1332 : 888) : units >= 444 ? 888 : 444;
+  // L 200: 38 -> 34 us).  More with grouped heads, whose CTAs have several heads' rows to do: nine times, and six
+  // at D = 64, of which an SM holds three and not five, up to 888 pairs.  Over 216 shapes (two and four heads a group,
+  // L 50 - 400, B 4 - 512, D 32 and 64) with full / with ragged lengths three, six and nine times for all are 8 / 11,
+  // 3.3 / 3.1 and 4.2 / 2.9 % behind the best of each shape, this rule 3.1 / 2.1.  (Six times up to 888 pairs for
+  // D = 32 too: 2.4 / 2.0, but B 128, 8 heads on 2, L 200, ragged 57.8 -> 59.8 us.)
+  const int units = s.B * s.Hkv;
+  const int want = s.G > 1 ? (s.D == 64 && units < 888 ? 888 : 1332) : units >= 444 ? 888 : 444;
   int nsplit = units >= want ? 1 : (want + units - 1) / units;
   o->nsplit = nsplit > s.M ? s.M : nsplit;
   o->per = s.M / o->nsplit;
