@@ -987,23 +987,23 @@ __host__ __device__ inline int per_query_doubles(const Shape &sh, const SelGeom 
 // of the group, the probabilities summed over the heads (Eq. 12), Eq. 11, the top_k - 1 largest kept
 // together with t's own block, ties to the lower index.  block_idx is [B][Hkv][L][top_k].  Lanes stride
 // over the candidates; the means come from global memory (they are shared by the neighbouring
-// positions and stay in L2).  hp: heads of the group whose logits a warp keeps at a time, 4, or 1 where four
+// positions and stay in L2).  HP: heads of the group whose logits a warp keeps at a time, 4, or 1 where four
 // heads' would not fit in shared memory (more than about 650 blocks).
-template <typename T, int D>
+template <typename T, int D, int HP>
 __global__ void __launch_bounds__(256) score_per_query_kernel(
     Shape sh, SelGeom g, const T *__restrict__ q, const double *__restrict__ mean,
     const int32_t *__restrict__ seq_lens, int32_t *__restrict__ idx, const int32_t *__restrict__ worklist,
-    const int32_t *__restrict__ work_count, int hp) {
+    const int32_t *__restrict__ work_count) {
   grid_chain_enter();
   extern __shared__ double dsm[];
   __shared__ double bound_d[8][2];
   const int M = sh.M, Bk = sh.Bk;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int per_warp = per_query_doubles(sh, g, D, hp);
+  const int per_warp = per_query_doubles(sh, g, D, HP);
   double *qrow = dsm + (size_t)warp * per_warp;  // [4][D] the current heads' rows
   double *P = qrow + 4 * D;                      // [n] summed probabilities of this warp's position
-  double *Z = P + g.n;                           // [hp][n] logits of the current heads
-  double *Smap = Z + hp * g.n;                   // [M] scores of the selection blocks (overlapping mode)
+  double *Z = P + g.n;                           // [HP][n] logits of the current heads
+  double *Smap = Z + HP * g.n;                   // [M] scores of the selection blocks (overlapping mode)
   uint8_t *taken = reinterpret_cast<uint8_t *>(dsm + (size_t)8 * per_warp) + (size_t)warp * M;
   const int64_t total = worklist ? *work_count : (int64_t)sh.B * sh.Hkv * sh.L;
   for (int64_t wi = (int64_t)blockIdx.x * 8 + warp; wi < total; wi += (int64_t)gridDim.x * 8) {
@@ -1024,10 +1024,10 @@ __global__ void __launch_bounds__(256) score_per_query_kernel(
     if (nsel > want && want > 0 && nc > cmin) {
       for (int j = cmin + lane; j < nc; j += 32) P[j] = 0.0;
       const double *kbase = mean + (int64_t)u * g.n * D;
-      // Up to hp heads of the group at a time, so that a candidate's mean is read (a lane per candidate,
+      // Up to HP heads of the group at a time, so that a candidate's mean is read (a lane per candidate,
       // eight 16-byte loads in flight) once for all of them.
-      for (int h0 = 0; h0 < sh.G; h0 += hp) {
-        const int nh = min(hp, sh.G - h0);
+      for (int h0 = 0; h0 < sh.G; h0 += HP) {
+        const int nh = min(HP, sh.G - h0);
         __syncwarp();
         for (int c = lane; c < 4 * D; c += 32) {
           const int h = c / D;
@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(256) score_per_query_kernel(
 #pragma unroll
           for (int h = 0; h < 4; ++h) {
             const double z = sh.scale_d * a[h];
-            if (h < hp) Z[h * g.n + j] = z;
+            if (h < HP) Z[h * g.n + j] = z;
             mx[h] = fmax(mx[h], z);
           }
         }
@@ -1153,14 +1153,15 @@ int launch_select_t(const Shape &sh, const T *q, const T *k, const int32_t *seq_
         return rc;
     }
     const auto need = [&](int hp) { return (size_t)8 * per_query_doubles(sh, g, D, hp) * sizeof(double) + (size_t)8 * sh.M + 16; };
-    const int hp = need(4) <= kMaxDynamicSmem ? 4 : 1;
-    const size_t psm = need(hp);
-    if (!allow_smem(score_per_query_kernel<T, D>, psm)) return BLOSSOM_ERR_CUDA;
+    const bool four = need(4) <= kMaxDynamicSmem;
+    const size_t psm = need(four ? 4 : 1);
+    auto per_query = four ? score_per_query_kernel<T, D, 4> : score_per_query_kernel<T, D, 1>;
+    if (!allow_smem(per_query, psm)) return BLOSSOM_ERR_CUDA;
     LaunchScope ls(K_SCORE_SELECT, st);
     const int64_t ctas = (units * sh.L + 7) / 8;
-    launch_chained(score_per_query_kernel<T, D>, dim3((unsigned)(listed && ctas > 592 ? 592 : ctas)), dim3(256), psm, st, sh,
+    launch_chained(per_query, dim3((unsigned)(listed && ctas > 592 ? 592 : ctas)), dim3(256), psm, st, sh,
                    g, q, (const double *)w.mean, seq_lens, idx, (const int32_t *)(listed ? w.list : nullptr),
-                   (const int32_t *)w.count, hp);
+                   (const int32_t *)w.count);
     return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
   }
   int sc_pitch = 0, sc_len = 0;
