@@ -8,37 +8,46 @@
 //            weights alpha, beta ride in the exponent, alpha P_lt = exp2(s*log2e + nl_lt); the dQ kernel
 //            needs unweighted probabilities and takes the log-sum-exps themselves.
 //
-// Main kernels: CTA = 384 threads.  Warps 0..7 compute; warps 8, 9, 10 stay converged and one
-// elected lane of each issues the TMA loads, the first-stage MMAs and the second-stage MMAs;
-// registers move from those warps to the compute warps (setmaxnreg).  A CTA owns a resident
-// 128-row tile (rows = TMEM lanes) and streams 64-row tiles past it.  Row r of the 128 is shared by
-// two compute threads: warp w and warp w + 4 both address TMEM lane quarter w % 4; the first takes
-// columns 0..31 of a 64-column tile, the second columns 32..63.  The tile arithmetic runs in
+// Main kernels: CTA = 384 threads.  Warps 0..7 compute; warps 8, 9 stay converged and one elected lane
+// of each issues the TMA loads and the MMAs (10 and 11 are spare); registers move from those warps to the
+// compute warps (setmaxnreg).  A CTA owns a resident 128-row tile (rows = TMEM lanes) and streams 64-row
+// tiles past it in two half tiles of 32 columns, each with a buffer in tensor memory and four compute warps of
+// its own: warps w and w + 4 both address TMEM lane quarter w % 4; the first takes columns 0..31 of every
+// tile, the second columns 32..63, so the two halves never wait for each other.  The tile arithmetic runs in
 // 16-column passes, two columns per FMA / ADD / MUL (packed f32x2); outputs are staged in shared
 // memory and written with whole-line TMA stores.
 //
+// What the products of a half tile wait for is one thing, its second operand in tensor memory: the warp that
+// issues them puts the first stage of the next half tile behind the second stage of this one, into the same
+// buffer, without waiting in between (products of one thread run in the order of their issue).  With eight
+// warps on every half tile (16 columns each, twice the hand-offs and their instructions), a warp for each
+// stage and without the uniform registers of tc_common.cuh the kernels took 197 and 232 us at B 128, H 4,
+// L 1024, D 64 (now 181 and 223), 384 and 479 at B 16, H 8, L 4096 (353 and 453), 64 and 80 with a selection
+// per position at B 8, L 1500 (50 and 73).  What is left is the chain of a half tile: arithmetic 1300 cycles,
+// from there to the next logits 700, while the issue slots are 42 % and the tensor pipe 30 % busy; and the
+// 8000 - 10000 cycles that a CTA spends outside its loop.
+//
 //  dQ     resident Q, dO (128 queries: 128 positions of a head, or with grouped heads 64 positions
 //         of two heads of a group, as in the forward); streams K, V 64-key tiles (same walk as the forward) and
-//         works through them in half tiles of 32 keys.  Tensor memory: two buffers of 64
-//         columns (half tile x uses buffer x % 2: S in its first 32 columns, dP in the other 32),
+//         works through them in half tiles of 32 keys.  Tensor memory: a buffer of 64 columns
+//         for each half (S in its first 32 columns, dP in the other 32),
 //         Q and dO as first operands of the first-stage products [128,128+D/2), [160,160+D/2)
 //         (read from shared memory they cost 4 KB per product, more than the data pipe delivers
 //         in the product's run time), and dQ [192,192+D).  S = Q K^T, dP = dO V^T; P_x = exp(S - lse_x);
 //         dS = P_lt (alpha dP - alpha Delta_lt) + P_st (beta dP - beta Delta_st) (one tile for both
-//         branches, they share K).  A thread owns 16 of the 32 columns and writes its dS (bf16 pairs) over the first 8
-//         of its own S columns, from where dQ += dS K reads it: the compute warps wait for one
-//         thing per half tile (its S and dP), and the first stage of the next two half tiles runs
-//         meanwhile.  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities, subtracted pair by pair.
+//         branches, they share K).  A thread writes the dS (bf16 pairs) of a pass's 16 columns over the first 8
+//         of them in S, from where dQ += dS K reads it: the compute warps wait for one
+//         thing per half tile (its S and dP).  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities, subtracted pair by pair.
 //  dK/dV  transposed: resident K, V of 128 keys, streams Q, dO 64-query tiles (and their row
 //         records, by bulk copy) that selected one of its key blocks or whose window reaches them.
-//         It works through them in half tiles of 32 queries.  Tensor memory: two buffers of 64
-//         columns (half tile x uses buffer x % 2: S^T in its first 32 columns, dP^T in the other
+//         It works through them in half tiles of 32 queries.  Tensor memory: a buffer of 64
+//         columns for each half (S^T in its first 32 columns, dP^T in the other
 //         32), dV [128,128+D), dK [192,192+D).  S^T = K Q^T, dP^T = V dO^T; thread = key row and
-//         16 of the 32 query columns; it writes W^T = P'_lt + P'_st and dS^T (bf16 pairs) over the
-//         first 8 of its own S^T / dP^T columns, from where dV += W^T dO and dK += dS^T Q read
+//         32 query columns; it writes W^T = P'_lt + P'_st and dS^T (bf16 pairs) of a pass's 16 columns over
+//         the first 8 of them in S^T / dP^T, from where dV += W^T dO and dK += dS^T Q read
 //         their first operand: nothing of a tile's arithmetic goes through shared memory, whose
 //         data pipe (operand reads of the products, row records) is the busiest unit of this
-//         kernel, and the first stage of the next half tile runs during the arithmetic of this one.
+//         kernel.
 // Every wait is bounded (tc_common.cuh).
 #include "tc_common.cuh"
 
@@ -49,7 +58,7 @@ namespace tc {
 namespace cg = cooperative_groups;
 namespace {
 
-// warps 0..7 compute; 8 loader, 9 first-stage issuer, 10 second-stage issuer, 11 spare
+// warps 0..7 compute; 8 loader, 9 issuer of the products; 10, 11 spare
 constexpr int kKvThreads = 384;
 constexpr int kProducerRegs = 64, kKvComputeRegs = 88;  // 256 * 88 + 128 * 64 = 384 * 80 (measured: the issuing warps spill below 48)
 constexpr int kComputeWarps = 8;
@@ -204,13 +213,13 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   constexpr int OC = D / 2;  // accumulator columns per thread
   extern __shared__ uint8_t smem_raw[];
   // barriers: full[STAGES], empty[STAGES], res, meta, a_ready, then one per buffer: s_full[2],
-  // t_full[2], mma_done[2]
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 9];
+  // t_full[2]; all_done
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 8];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ double red[kComputeWarps];
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int nST = (s.L + 127) >> 7;
   // long rows first, tile-major: every unit's last tile, then every unit's last but one, ...
   // (PACK: a unit is a pair of heads, a tile 64 positions; h = the pair's first head)
@@ -243,7 +252,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 1]);
   const uint32_t b_aready = smem_u32(&bars[2 * STAGES + 2]);
   const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 3]), b_tfull = smem_u32(&bars[2 * STAGES + 5]);
-  const uint32_t b_done = smem_u32(&bars[2 * STAGES + 7]);
+  const uint32_t b_all = smem_u32(&bars[2 * STAGES + 7]);
 
   if (tid == 0) {
     abort_flag = (*status != 0) ? 1 : 0;
@@ -259,10 +268,10 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     mbar_init(b_aready, kComputeWarps);
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_sfull + 8 * i, 1);
-      mbar_init(b_tfull + 8 * i, kComputeWarps);
-      mbar_init(b_done + 8 * i, 1);
+      mbar_init(b_tfull + 8 * i, kComputeWarps / 2);
     }
     mbar_init(b_meta, 1);
+    mbar_init(b_all, 1);
     mbar_fence_init();
     // the CTA's tile lists and its resident tiles
     mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
@@ -280,14 +289,14 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   __syncthreads();
   tc_fence_after();
   mbar_wait(b_meta, 0, &abort_flag, 223);
-  const int nvis = *reinterpret_cast<const int *>(meta + ml.counts);
-  const uint32_t tmem_base = tmem_slot;
+  const int nvis = uniform(*reinterpret_cast<const int *>(meta + ml.counts));
+  const uint32_t tmem_base = (uint32_t)uniform((int)tmem_slot);
   // buffers at tmem_base + 64 * (half tile % 2); Q and dO as first operands (bf16 pairs, D / 2
   // columns each) at 128 and 160; the dQ accumulator at 192
   const uint32_t tmem_qa = tmem_base + 128, tmem_ga = tmem_base + 160, tmem_dq = tmem_base + 192;
 
   if (warp >= kComputeWarps) {
-    // ============ three single-thread roles, one converged warp each ============
+    // ============ two single-thread roles, one converged warp each ============
     setmaxnreg_dec<kProducerRegs>();
     if (warp == kComputeWarps && nvis > 0) {
       // ---- loader: Q, dO once; K/V tiles up to STAGES ahead of their consumers ----
@@ -305,60 +314,53 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         __syncwarp();
       }
     } else if (warp == kComputeWarps + 1 && nvis > 0) {
-      // ---- S = Q K^T and dP = dO V^T of a half tile (32 keys) into buffer x % 2 once
-      // dQ += dS K of half tile x-2 has read that buffer.  Q and dO are read from tensor memory
-      // (the compute warps copied the resident tiles there), so a product fetches only its 32
-      // keys from shared memory instead of 128 rows of Q or dO as well ----
-      constexpr uint32_t idesc_s = instr_desc(128, 32, 0, 0);
-      mbar_wait(b_aready, 0, &abort_flag, 201);
-      tc_fence_after();
-      for (int i = 0, x = 0, b = 0, ph = 0; i < nvis; ++i) {  // x = 2 i + hh, b = x % 2, ph = (x / 2) & 1
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 202);
-        for (int hh = 0; hh < 2; ++hh, ++x) {
-          if (x >= 2) mbar_wait(b_done + 8 * b, ph ^ 1, &abort_flag, 203);
-          tc_fence_after();
-          const uint32_t kt = smem_u32(kv_tiles + (i % STAGES) * 2 * C::kSmallBytes) + hh * 32 * C::kRowBytes;
-          const uint64_t dkd = smem_desc(kt, 16, C::kAtomBytes, C::kSwizzle);
-          const uint64_t dvd = smem_desc(kt + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
-          const uint32_t ts = tmem_base + 64 * b;
-          if (elect_one()) {
+      // ---- S = Q K^T and dP = dO V^T of a half tile (32 keys) into buffer x % 2, then, once its dS is in
+      // tensor memory, dQ += dS K (K MN-major) and behind it the first stage of half tile x + 2 into the same
+      // buffer: products of one thread run in the order of their issue, so nothing has to wait in between for
+      // the second stage to have read the buffer.  Q and dO are read from tensor memory (the compute warps
+      // copied the resident tiles there), so a product fetches only its 32 keys from shared memory instead
+      // of 128 rows of Q or dO as well ----
+      constexpr uint32_t idesc_s = instr_desc(128, 32, 0, 0), idesc_dq = instr_desc(128, D, 0, 1);
+      auto first_stage = [&](int sj, int hh) {
+        const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes) + hh * 32 * C::kRowBytes;
+        const uint64_t dkd = smem_desc(kt, 16, C::kAtomBytes, C::kSwizzle);
+        const uint64_t dvd = smem_desc(kt + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
+        const uint32_t ts = tmem_base + 64 * hh;
+        if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts, tmem_qa + 8 * k, dkd + 2 * k, idesc_s, k > 0);
+          for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts, tmem_qa + 8 * k, dkd + 2 * k, idesc_s, k > 0);
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts + 32, tmem_ga + 8 * k, dvd + 2 * k, idesc_s, k > 0);
-            umma_commit(b_sfull + 8 * b);
-          }
-          __syncwarp();
-          if (++b == 2) {
-            b = 0;
-            ph ^= 1;
-          }
+          for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts + 32, tmem_ga + 8 * k, dvd + 2 * k, idesc_s, k > 0);
+          umma_commit(b_sfull + 8 * hh);
         }
-      }
-    } else if (warp == kComputeWarps + 2 && nvis > 0) {
-      // ---- dQ += dS K of a half tile (dS from tensor memory, K MN-major) ----
-      constexpr uint32_t idesc_dq = instr_desc(128, D, 0, 1);
-      for (int i = 0, b = 0, ph = 0; i < nvis; ++i) {
-        const uint64_t dkm = smem_desc(smem_u32(kv_tiles + (i % STAGES) * 2 * C::kSmallBytes), C::kSmallBytes,
-                                       C::kAtomBytes, C::kSwizzle);
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 206);
+        __syncwarp();
+      };
+      mbar_wait(b_aready, 0, &abort_flag, 201);
+      mbar_wait(b_full, 0, &abort_flag, 202);
+      tc_fence_after();
+      first_stage(0, 0);
+      first_stage(0, 1);
+      for (int i = 0, sj = 0; i < nvis; ++i) {
+        const int sn = sj + 1 == STAGES ? 0 : sj + 1;
+        const uint64_t dkm = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes), C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
+#pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          mbar_wait(b_tfull + 8 * b, ph, &abort_flag, 204);
+          mbar_wait(b_tfull + 8 * hh, i & 1, &abort_flag, 204);
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              umma_bf16_ts(tmem_dq, tmem_base + 64 * b + 16 * kk, dkm + (2 * hh + kk) * C::kKStep, idesc_dq,
+              umma_bf16_ts(tmem_dq, tmem_base + 64 * hh + 16 * kk, dkm + (2 * hh + kk) * C::kKStep, idesc_dq,
                            (i | hh | kk) != 0);
-            umma_commit(b_done + 8 * b);
-            if (hh == 1) umma_commit(b_empty + 8 * (i % STAGES));  // every product on this stage has completed
+            if (hh == 1) umma_commit(i + 1 < nvis ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
           }
           __syncwarp();
-          if (++b == 2) {
-            b = 0;
-            ph ^= 1;
+          if (i + 1 < nvis) {
+            if (hh == 0) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 206);
+            first_stage(sn, hh);
           }
         }
+        sj = sn;
       }
     }
   } else {
@@ -383,7 +385,6 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     }
     float2 dalL = make_float2(0.f, 0.f), dalS = make_float2(0.f, 0.f);  // see dq_tile
     const float sc2 = s.scale * kLog2e;
-    int b = 0, ph = 0;  // buffer x % 2 of half tile x = 2 i + hh and the parity (x / 2) & 1
     if (nvis > 0) {
       // The resident tiles become first operands in tensor memory: row r of Q (warps 0..3) or of dO
       // (warps 4..7) goes to lane r as it is stored, two bf16 per 32-bit column.
@@ -403,54 +404,62 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
       warp_arrive(b_aready, lane);
     }
 
-    int cls_n = nvis > 0 ? jcls[warp] : 0;
-    for (int x = 0; x < 2 * nvis; ++x) {  // half tile x: keys 32 (x % 2) ... of tile list[x / 2]
-      const int cls = cls_n;
-      if (x + 1 < 2 * nvis) cls_n = jcls[(x + 1) * kComputeWarps + warp];  // ahead of its use
-      uint32_t hL = 0u, hS = 0u;  // this thread's 16 keys: keys 32 (x % 2) + 16 half ... of the tile
-      bool anyL = cls & 1, anyS = cls & 2, full = true;
-      if (cls & 8) {  // mixed: per-lane column masks
-        const int i = x >> 1, jt = list[i], f = lflags[i], p0 = jt * 64, col = 32 * (x & 1) + 16 * half, c0 = p0 + col;
-        const uint32_t mc = cols32_le(t_last - c0) & cols32_ge(pad0 - c0) & 0xffffu;
+    // Keys 32 half ... of every tile belong to the four warps of group `half`, which have a buffer of their own:
+    // a thread takes all 32 columns, in two passes of 16.
+    const uint32_t tb = tmem_base + 64 * half + lane_off;  // S; dP 32 columns further
+    const uint8_t *jc = jcls + 8 * half + quarter;  // classes of the half tile's two column halves: [0], [4]
+    int c0_n = nvis > 0 ? jc[0] : 0, c1_n = nvis > 0 ? jc[4] : 0;
+    for (int i = 0; i < nvis; ++i) {
+      const int cls0 = c0_n, cls1 = c1_n;
+      if (i + 1 < nvis) {  // ahead of their use
+        c0_n = jc[(i + 1) * 16];
+        c1_n = jc[(i + 1) * 16 + 4];
+      }
+      uint32_t hL = 0u, hS = 0u;  // this thread's 32 keys
+      if ((cls0 | cls1) & 8) {  // mixed: per-lane column masks
+        const int jt = list[i], f = lflags[i], p0 = jt * 64, col = 32 * half, c0 = p0 + col;
+        const uint32_t mc = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
         if (f & 1) hL = mc & expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, col);
         if (f & 2) hS = mc & (s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> col) : st_window32(s, t, c0, causal));
-        anyL = __any_sync(0xffffffffu, hL != 0u);
-        anyS = __any_sync(0xffffffffu, hS != 0u);
-        full = __all_sync(0xffffffffu, (!anyL || hL == 0xffffu) && (!anyS || hS == 0xffffu));
       }
-      const uint32_t tb = tmem_base + 64 * b + lane_off + 16 * half;  // S; dP 32 columns further
-
-      mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 207);
+      mbar_wait(b_sfull + 8 * half, i & 1, &abort_flag, 207);
       __syncwarp();
       tc_fence_after();
-      uint32_t dw[8];
-      if (anyL || anyS) {
-        float sv[16], dp[16];
-        tmem_ld16(tb, sv);
-        tmem_ld16(tb + 32, dp);
-        tmem_wait_ld();
-        if (!full && (PLAIN || (anyL && anyS))) dq_tile<true, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-        else if (!full && anyL) dq_tile<true, false, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-        else if (!full) dq_tile<false, true, false>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-        else if (anyL && anyS) dq_tile<true, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-        else if (anyL) dq_tile<true, false, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-        else dq_tile<false, true, true>(sv, dp, hL, hS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-      } else {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) dw[c] = 0u;
+      for (int ps = 0; ps < 2; ++ps) {
+        const int cls = ps ? cls1 : cls0;
+        const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
+        bool anyL = cls & 1, anyS = cls & 2, full = true;
+        if (cls & 8) {
+          anyL = __any_sync(0xffffffffu, xL != 0u);
+          anyS = __any_sync(0xffffffffu, xS != 0u);
+          full = __all_sync(0xffffffffu, (!anyL || xL == 0xffffu) && (!anyS || xS == 0xffffu));
+        }
+        uint32_t dw[8];
+        if (anyL || anyS) {
+          float sv[16], dp[16];
+          tmem_ld16(tb + 16 * ps, sv);
+          tmem_ld16(tb + 32 + 16 * ps, dp);
+          tmem_wait_ld();
+          if (!full && (PLAIN || (anyL && anyS))) dq_tile<true, true, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          else if (!full && anyL) dq_tile<true, false, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          else if (!full) dq_tile<false, true, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          else if (anyL && anyS) dq_tile<true, true, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          else if (anyL) dq_tile<true, false, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          else dq_tile<false, true, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) dw[c] = 0u;
+        }
+        tmem_st8u(tb + 16 * ps, dw);  // dS (bf16 pairs) over the first 8 of the pass's 16 S columns
       }
-      tmem_st8u(tb, dw);  // dS (bf16 pairs) over the first 8 of this thread's own 16 S columns
       tmem_wait_st();
       tc_fence_before();
-      warp_arrive(b_tfull + 8 * b, lane);
-      if (++b == 2) {
-        b = 0;
-        ph ^= 1;
-      }
+      warp_arrive(b_tfull + 8 * half, lane);
     }
 
     if (nvis > 0) {
-      mbar_wait(b_done + 8, (nvis - 1) & 1, &abort_flag, 209);  // the last half tile used buffer 1
+      mbar_wait(b_all, 0, &abort_flag, 209);
       __syncwarp();
       tc_fence_after();
     }
@@ -595,12 +604,12 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   constexpr int OC = D / 2;
   constexpr int kStageBytes = 2 * C::kSmallBytes + kStatBytes;  // Q, dO, row records
   extern __shared__ uint8_t smem_raw[];
-  // barriers: full[STAGES], empty[STAGES], res, meta, and per buffer s_full[2], t_full[2], done[2]
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 8];
+  // barriers: full[STAGES], empty[STAGES], res, meta, per buffer s_full[2], t_full[2]; all_done
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 7];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   grid_release();
   const int nKT = (s.L + 127) >> 7;
   // A CTA owns 128 keys of one (batch, key/value head) and collects from every query head of the
@@ -641,7 +650,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   const uint32_t b_full = smem_u32(&bars[0]), b_empty = smem_u32(&bars[STAGES]);
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 1]);
   const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 2]), b_tfull = smem_u32(&bars[2 * STAGES + 4]);
-  const uint32_t b_done = smem_u32(&bars[2 * STAGES + 6]);
+  const uint32_t b_all = smem_u32(&bars[2 * STAGES + 6]);
 
   if (tid == 0) {
     abort_flag = (*status != 0) ? 1 : 0;
@@ -656,10 +665,10 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     mbar_init(b_res, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_sfull + 8 * i, 1);
-      mbar_init(b_tfull + 8 * i, kComputeWarps);
-      mbar_init(b_done + 8 * i, 1);
+      mbar_init(b_tfull + 8 * i, kComputeWarps / 2);
     }
     mbar_init(b_meta, 1);
+    mbar_init(b_all, 1);
     mbar_fence_init();
     // the CTA's tile lists and its resident tiles
     mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
@@ -679,14 +688,14 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   mbar_wait(b_meta, 0, &abort_flag, 224);
   // The tile list is the same for every query head of the group (one selection per group): the
   // kernel walks it once per head, item x = (head x / nlist, tile list[x % nlist]).
-  const int nlist = *reinterpret_cast<const int *>(meta + ml.counts);
+  const int nlist = uniform(*reinterpret_cast<const int *>(meta + ml.counts));
   const int nvis = nlist * Gs;
-  const uint32_t tmem_base = tmem_slot;
-  // half tile x uses buffer x % 2 at column 64 (x % 2): S^T in its first 32 columns, dP^T behind
+  const uint32_t tmem_base = (uint32_t)uniform((int)tmem_slot);
+  // the half tile of group hh uses the buffer at column 64 hh: S^T in its first 32 columns, dP^T behind
   const uint32_t tmem_dv = tmem_base + 128, tmem_dk = tmem_base + 192;
 
   if (warp >= kComputeWarps) {
-    // ===================== three single-thread roles, one warp each =====================
+    // ===================== two single-thread roles, one warp each =====================
     setmaxnreg_dec<kProducerRegs>();
     if (warp == kComputeWarps && nvis > 0) {
       // ---- loader: K, V once; Q, dO tiles and their row records up to STAGES ahead ----
@@ -707,59 +716,58 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
         __syncwarp();
       }
     } else if (warp == kComputeWarps + 1 && nvis > 0) {
-      // ---- S^T = K Q^T, dP^T = V dO^T of half tile x into buffer x % 2 once the products of half
-      // tile x - 2 have read that buffer ----
-      constexpr uint32_t idesc_s = instr_desc(128, 32, 0, 0);
+      // ---- S^T = K Q^T, dP^T = V dO^T of half tile x into buffer x % 2, then, once its W^T and dS^T are in
+      // tensor memory, dV += W^T dO, dK += dS^T Q and behind them the first stage of half tile x + 2 (see the
+      // dQ kernel) ----
+      constexpr uint32_t idesc_s = instr_desc(128, 32, 0, 0), idesc_o = instr_desc(128, D, 0, 1);
       const uint64_t dkd = smem_desc(smem_u32(k_tile), 16, C::kAtomBytes, C::kSwizzle);
       const uint64_t dvd = smem_desc(smem_u32(v_tile), 16, C::kAtomBytes, C::kSwizzle);
+      auto first_stage = [&](int sj, int hh) {
+        const uint32_t qt_ = smem_u32(qg_tiles + sj * kStageBytes) + hh * 32 * C::kRowBytes;
+        const uint64_t dqd = smem_desc(qt_, 16, C::kAtomBytes, C::kSwizzle);
+        const uint64_t dgd = smem_desc(qt_ + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
+        const uint32_t ts = tmem_base + 64 * hh;
+        if (elect_one()) {
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k) umma_bf16(ts, dkd + 2 * k, dqd + 2 * k, idesc_s, k > 0);
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k) umma_bf16(ts + 32, dvd + 2 * k, dgd + 2 * k, idesc_s, k > 0);
+          umma_commit(b_sfull + 8 * hh);
+        }
+        __syncwarp();
+      };
       mbar_wait(b_res, 0, &abort_flag, 210);
-      for (int i = 0, x = 0; i < nvis; ++i) {
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 213);
-        for (int hh = 0; hh < 2; ++hh, ++x) {
-          const int b = x & 1, ph = (x >> 1) & 1;
-          if (x >= 2) mbar_wait(b_done + 8 * b, ph ^ 1, &abort_flag, 212);
-          tc_fence_after();
-          const uint32_t qt_ = smem_u32(qg_tiles + (i % STAGES) * kStageBytes) + hh * 32 * C::kRowBytes;
-          const uint64_t dqd = smem_desc(qt_, 16, C::kAtomBytes, C::kSwizzle);
-          const uint64_t dgd = smem_desc(qt_ + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
-          const uint32_t ts = tmem_base + 64 * b;
-          if (elect_one()) {
+      mbar_wait(b_full, 0, &abort_flag, 213);
+      tc_fence_after();
+      first_stage(0, 0);
+      first_stage(0, 1);
+      for (int i = 0, sj = 0; i < nvis; ++i) {
+        const int sn = sj + 1 == STAGES ? 0 : sj + 1;
+        const uint32_t q_tile = smem_u32(qg_tiles + sj * kStageBytes);
+        const uint64_t dgm = smem_desc(q_tile + C::kSmallBytes, C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
+        const uint64_t dqm = smem_desc(q_tile, C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) umma_bf16(ts, dkd + 2 * k, dqd + 2 * k, idesc_s, k > 0);
-#pragma unroll
-            for (int k = 0; k < D / 16; ++k) umma_bf16(ts + 32, dvd + 2 * k, dgd + 2 * k, idesc_s, k > 0);
-            umma_commit(b_sfull + 8 * b);
-          }
-          __syncwarp();
-        }
-      }
-    } else if (warp == kComputeWarps + 2 && nvis > 0) {
-      // ---- dV += W^T dO, dK += dS^T Q of a half tile; W^T and dS^T are read from tensor memory,
-      // where the compute warps wrote them over the half tile's logits ----
-      constexpr uint32_t idesc_o = instr_desc(128, D, 0, 1);
-      for (int i = 0, x = 0; i < nvis; ++i) {
-        uint8_t *q_tile = qg_tiles + (i % STAGES) * kStageBytes, *g_tile = q_tile + C::kSmallBytes;
-        const uint64_t dgm = smem_desc(smem_u32(g_tile), C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
-        const uint64_t dqm = smem_desc(smem_u32(q_tile), C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
-        mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 215);
-        for (int hh = 0; hh < 2; ++hh, ++x) {
-          const int b = x & 1, ph = (x >> 1) & 1;
-          mbar_wait(b_tfull + 8 * b, ph, &abort_flag, 211);
+        for (int hh = 0; hh < 2; ++hh) {
+          const uint32_t tb = tmem_base + 64 * hh;
+          mbar_wait(b_tfull + 8 * hh, i & 1, &abort_flag, 211);
           tc_fence_after();
-          const uint32_t tb = tmem_base + 64 * b;
           if (elect_one()) {
-            // 16 queries per step: the bf16 pairs of the warps of column half kk, 8 columns
+            // 16 queries per step: the bf16 pairs of column half kk, 8 columns
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              umma_bf16_ts(tmem_dv, tb + 16 * kk, dgm + (2 * hh + kk) * C::kKStep, idesc_o, (x | kk) != 0);
+              umma_bf16_ts(tmem_dv, tb + 16 * kk, dgm + (2 * hh + kk) * C::kKStep, idesc_o, (i | hh | kk) != 0);
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              umma_bf16_ts(tmem_dk, tb + 32 + 16 * kk, dqm + (2 * hh + kk) * C::kKStep, idesc_o, (x | kk) != 0);
-            umma_commit(b_done + 8 * b);
-            if (hh == 1) umma_commit(b_empty + 8 * (i % STAGES));  // every product on this stage has completed
+              umma_bf16_ts(tmem_dk, tb + 32 + 16 * kk, dqm + (2 * hh + kk) * C::kKStep, idesc_o, (i | hh | kk) != 0);
+            if (hh == 1) umma_commit(i + 1 < nvis ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
           }
           __syncwarp();
+          if (i + 1 < nvis) {
+            if (hh == 0) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 215);
+            first_stage(sn, hh);
+          }
         }
+        sj = sn;
       }
     }
   } else {
@@ -770,68 +778,68 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const float sc2 = s.scale * kLog2e;
 
+    // Half tile hh of every tile (32 queries) belongs to the four warps of group hh = half, which have a buffer of
+    // their own: a thread takes all 32 columns, in two passes of 16.
+    const uint32_t tb = tmem_base + 64 * half + lane_off;
+    const int q0 = 32 * half;
     int li = 0;
-    for (int i = 0, x = 0; i < nvis; ++i) {
+    for (int i = 0; i < nvis; ++i) {
       if (li == nlist) li = 0;
-      const int qt = list[li], f = lflags[li], t0 = qt * 64;
-      const uint8_t *cls2 = kcls + li * 16 + warp;  // classes of the tile's two half tiles for this warp
+      const int qt = list[li], f = lflags[li], t0 = qt * 64 + q0;
+      const uint8_t *cls2 = kcls + li * 16 + 8 * half + quarter;  // classes of the half tile's two column halves
+      const int cls0 = cls2[0], cls1 = cls2[4];
       ++li;
-      uint64_t maskL = 0ull, maskS = 0ull;
-      if (cls2[0] == 8 || cls2[8] == 8) {  // a mixed half tile: per-lane column masks
+      uint32_t hL = 0u, hS = 0u;
+      if ((cls0 | cls1) & 8) {  // a mixed half: per-lane column masks
         if (row_valid) {
-          const uint64_t mc = cols_ge((causal ? p : pad0) - t0) & cols_le(s.L - 1 - t0);
-          if (f & 1) maskL = mc & (pq ? inv64[g * nT + qt] : expand_block_bits(invb[g * nT + qt], s.Bk));
-          if (f & 2) maskS = mc & st_query_cols(s, p, t0, causal);
+          const uint32_t mc = cols32_ge((causal ? p : pad0) - t0) & cols32_le(s.L - 1 - t0);
+          if (f & 1) hL = mc & (pq ? (uint32_t)(inv64[g * nT + qt] >> q0) : expand_block_bits32(invb[g * nT + qt], s.Bk, q0));
+          if (f & 2) hS = mc & (uint32_t)(st_query_cols(s, p, qt * 64, causal) >> q0);
         }
       }
       mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 216);  // the row records have landed
       const float4 *stt = reinterpret_cast<const float4 *>(qg_tiles + (i % STAGES) * kStageBytes + 2 * C::kSmallBytes);
-      // A half tile = 32 queries; this thread's 16 columns of it are queries 32 hh + 16 half ...
-      // W^T and dS^T go, as bf16 pairs, over the first 8 of the thread's own 16 columns of S^T / dP^T.
+      mbar_wait(b_sfull + 8 * half, i & 1, &abort_flag, 217);
+      __syncwarp();
+      tc_fence_after();
+      // W^T and dS^T of the 16 columns of a pass go, as bf16 pairs, over the first 8 of them in S^T / dP^T.
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh, ++x) {
-        const int b = x & 1, ph = (x >> 1) & 1, c0 = 32 * hh + 16 * half;
-        const int cls = cls2[8 * hh];
-        uint32_t hL = 0u, hS = 0u;
+      for (int ps = 0; ps < 2; ++ps) {
+        const int cls = ps ? cls1 : cls0;
+        const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
         bool anyL = (cls & 1) != 0, anyS = (cls & 2) != 0, full = true;
         if (cls == 8) {
-          hL = (uint32_t)(maskL >> c0) & 0xffffu;
-          hS = (uint32_t)(maskS >> c0) & 0xffffu;
-          anyL = __any_sync(0xffffffffu, hL != 0u);
-          anyS = __any_sync(0xffffffffu, hS != 0u);
-          full = __all_sync(0xffffffffu, (!anyL || hL == 0xffffu) && (!anyS || hS == 0xffffu));
+          anyL = __any_sync(0xffffffffu, xL != 0u);
+          anyS = __any_sync(0xffffffffu, xS != 0u);
+          full = __all_sync(0xffffffffu, (!anyL || xL == 0xffffu) && (!anyS || xS == 0xffffu));
         }
-        const uint32_t tb = tmem_base + 64 * b + lane_off + 16 * half;
-        mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 217);
-        __syncwarp();
-        tc_fence_after();
         uint32_t ww[8], dw[8];
         if (anyL || anyS) {
           float sv[16], dp[16];
-          tmem_ld16(tb, sv);
-          tmem_ld16(tb + 32, dp);
+          tmem_ld16(tb + 16 * ps, sv);
+          tmem_ld16(tb + 32 + 16 * ps, dp);
           tmem_wait_ld();
-          const float4 *sq = stt + c0;  // 8 pairs x 2 float4
-          if (!full && (PLAIN || (anyL && anyS))) dkdv_tile<true, true, false>(sv, dp, hL, hS, sc2, sq, ww, dw);
-          else if (!full && anyL) dkdv_tile<true, false, false>(sv, dp, hL, hS, sc2, sq, ww, dw);
-          else if (!full) dkdv_tile<false, true, false>(sv, dp, hL, hS, sc2, sq, ww, dw);
-          else if (anyL && anyS) dkdv_tile<true, true, true>(sv, dp, hL, hS, sc2, sq, ww, dw);
-          else if (anyL) dkdv_tile<true, false, true>(sv, dp, hL, hS, sc2, sq, ww, dw);
-          else dkdv_tile<false, true, true>(sv, dp, hL, hS, sc2, sq, ww, dw);
+          const float4 *sq = stt + q0 + 16 * ps;  // 8 pairs x 2 float4
+          if (!full && (PLAIN || (anyL && anyS))) dkdv_tile<true, true, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else if (!full && anyL) dkdv_tile<true, false, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else if (!full) dkdv_tile<false, true, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else if (anyL && anyS) dkdv_tile<true, true, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else if (anyL) dkdv_tile<true, false, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else dkdv_tile<false, true, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
         } else {
 #pragma unroll
           for (int c = 0; c < 8; ++c) { ww[c] = 0u; dw[c] = 0u; }
         }
-        tmem_st8u(tb, ww);
-        tmem_st8u(tb + 32, dw);
-        tmem_wait_st();
-        tc_fence_before();
-        warp_arrive(b_tfull + 8 * b, lane);
+        tmem_st8u(tb + 16 * ps, ww);
+        tmem_st8u(tb + 32 + 16 * ps, dw);
       }
+      tmem_wait_st();
+      tc_fence_before();
+      warp_arrive(b_tfull + 8 * half, lane);
     }
 
     if (nvis > 0) {
-      mbar_wait(b_done + 8, (nvis - 1) & 1, &abort_flag, 218);  // the last half tile used buffer 1
+      mbar_wait(b_all, 0, &abort_flag, 218);
       __syncwarp();
       tc_fence_after();
     }

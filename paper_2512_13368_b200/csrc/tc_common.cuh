@@ -78,6 +78,10 @@ __device__ __forceinline__ void setmaxnreg_dec() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
 
+// A value that is the same in all lanes of a converged warp, in a form the compiler knows to be so: roles chosen
+// by it are convergent code, and what is computed from it can live in uniform registers, from which the
+// asynchronous instructions take their operands.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 // True in exactly one lane of a converged warp.  The single-thread roles keep their whole warp
 // converged (every lane waits on the barriers and computes the uniform addresses) and put only the
 // asynchronous instructions under this predicate, so that descriptors and addresses can live in
