@@ -14,7 +14,12 @@
 // 228 -> 204 us, 27 items (L 4096) 388 -> 365 us, D 32 97 -> 91 us.  The roles therefore run on from
 // tile to tile (item counters, stages and barrier phases continue), each as far ahead as its own inputs
 // allow, while the softmax warps merge.  What is left is bound by the softmax warps' instructions:
-// tensor pipe 21 %, 0.53 instructions a cycle and scheduler, four softmax warps each.
+// tensor pipe 24 %, 0.56 instructions a cycle and scheduler, four softmax warps each.
+//
+// One warp issues both products of an item.  With a warp for each, S(i + 2) waited for the products of item
+// i to be reported complete; products of one thread run in the order of their issue, so it can follow them
+// at once.  That, and roles, loop bounds and addresses in uniform registers (tc_common.cuh), took the kernel
+// from 199 to 179 us at B 128, H 4, L 1024, D 64 and from 360 to 332 at B 16, H 8, L 4096.
 //
 // CTA = 384 threads.  Warps 0..7 are softmax warps: a query row (= TMEM lane) is shared by two
 // threads, warp w and warp w + 4, which split the KEYS of every tile: group 0 (warps 0..3) takes
@@ -33,12 +38,12 @@
 // products read their first operand:
 //
 //   loader   : stage j <- K, V of item j once the products of item j - STAGES have completed
-//   S issuer : wait K(i) and "products of item i-2 done" (the buffer is free) -> S(i) -> s_full[i%2]
 //   softmax  : wait s_full -> tcgen05.ld 32 logits -> online softmax of the half row (maximum
 //              raised, and the group's accumulator rescaled, only when it grows by > 2^8) ->
 //              tcgen05.st P -> arrive t_full[group][i%2]
-//   PV issuer: wait t_full[0] -> O_A += P_A V[0:32]; wait t_full[1] -> O_B += P_B V[32:64] ->
-//              commit done[i%2], release the stage
+//   issuer   : (S(0) -> s_full[0], S(1) -> s_full[1] of a tile;) wait t_full[0] -> O_A += P_A V[0:32];
+//              wait t_full[1] -> O_B += P_B V[32:64] -> commit done[i%2], release the stage; wait
+//              K(i+2) -> S(i+2) into the same buffer -> s_full[i%2]
 //
 // When the long-term phase ends the merged, normalised rows go (as bf16) to a staging tile in
 // shared memory, from where they are stored; the short-term phase then starts both accumulators
@@ -53,7 +58,7 @@ namespace tc {
 namespace {
 
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
-constexpr int kFwdThreads = 384;  // warps 0..7 softmax; 8 loader, 9 S issuer, 10 PV issuer, 11 storer
+constexpr int kFwdThreads = 384;  // warps 0..7 softmax; 8 loader, 9 issuer of the products, 11 storer
 constexpr int kSoftmaxWarps = 8;
 // The kernel is compiled for 80 registers per thread (two CTAs of 384 threads per SM): the pool of
 // a CTA is 384 * 80 = 30720, and the two register counts must fit in it or the increase would
@@ -155,7 +160,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   __shared__ int abort_flag;
   __shared__ float2 stat[2][128];  // (maximum, sum) of each group's half of every row, exchanged at a phase end
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const int nST = (s.L + 127) >> 7;
   // long rows first, tile-major: every unit's last tile, then every unit's last but one, ...
   // (PACK: a unit is a pair of heads, a tile 64 positions; h = the pair's first head)
@@ -213,7 +218,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_res + 8 * i, 1);
       mbar_init(b_meta + 8 * i, 1);
-      mbar_init(b_roles + 8 * i, 3);
+      mbar_init(b_roles + 8 * i, 2);
       mbar_init(b_sfull + 8 * i, 1);
       mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);        // group 0
       mbar_init(b_tfull + 8 * (2 + i), kSoftmaxWarps / 2);  // group 1
@@ -233,11 +238,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = tmem_slot;
+  const uint32_t tmem_base = (uint32_t)uniform((int)tmem_slot);
   const uint32_t tmem_oa = tmem_base + 128, tmem_ob = tmem_base + 192;  // buffers at tmem_base + 64 * (item % 2)
 
   if (warp >= kSoftmaxWarps) {
-    // ===================== three single-thread roles, one warp each =====================
+    // ===================== three single-thread roles, one warp each (warp 10 is spare) =====================
     setmaxnreg_dec<kProducerRegs>();
     if (warp == kSoftmaxWarps + 3) {
       // ---- storer: the staged rows of a tile as whole-line bulk stores (rows past L are clipped by the
@@ -272,18 +277,18 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         }
       }
       __syncwarp();
-    } else {
+    } else if (warp < kSoftmaxWarps + 2) {
       int it = 0;              // items of the tiles before
       int sj = 0, sph = 0;     // their stage and its phase
       auto step = [&] { if (++sj == STAGES) { sj = 0; sph ^= 1; } };
       for (int k = 0;; ++k) {
         mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 113);
-        const int x = *(volatile int *)&tile_id[k & 1];
-        if (x < 0 || *(volatile int *)&abort_flag) break;
+        const int x = uniform(*(volatile int *)&abort_flag ? -1 : *(volatile int *)&tile_id[k & 1]);
+        if (x < 0) break;
         const uint8_t *meta = metas + (k & 1) * meta_step;
         const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
         const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
-        const int nL = counts[1], nI = nL + counts[2];
+        const int nL = uniform(counts[1]), nI = nL + uniform(counts[2]);
         if (warp == kSoftmaxWarps) {
           // ---- loader: K/V tiles, up to STAGES ahead of their consumers ----
           const int u = tile_unit(x), n = unit_batch(u), hk = unit_head(u) / s.G;
@@ -299,36 +304,34 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
             }
             __syncwarp();
           }
-        } else if (warp == kSoftmaxWarps + 1) {
-          // ---- S(i) = Q K^T into buffer i % 2 once the products of item i - 2 have read that buffer ----
-          constexpr uint32_t idesc_s = instr_desc(128, 64, 0, 0);
+        } else {
+          // ---- S(i) = Q K^T into buffer i % 2; once a group's probabilities of item i are in tensor memory,
+          // O_A += P(i)[:, 0:32] V[0:32], O_B += P(i)[:, 32:64] V[32:64], and behind them S(i + 2) into the same
+          // buffer: products of one thread run in the order of their issue, so nothing has to wait in between
+          // for the probabilities to have been read ----
+          constexpr uint32_t idesc_s = instr_desc(128, 64, 0, 0), idesc_pv = instr_desc(128, D, 0, 1);
           const uint64_t dq = smem_desc(smem_u32(q_tiles) + (k & 1) * C::kBigBytes, 16, C::kAtomBytes, C::kSwizzle);
-          mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 101);
-          for (int i = 0; i < nI; ++i, ++it, step()) {
-            const int b = it & 1, ph = (it >> 1) & 1;
-            mbar_wait(b_full + 8 * sj, sph, &abort_flag, 102);
-            if (it >= 2) mbar_wait(b_done + 8 * b, ph ^ 1, &abort_flag, 103);
-            tc_fence_after();
-            const uint64_t dk = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes), 16, C::kAtomBytes, C::kSwizzle);
-            const uint32_t ts = tmem_base + 64 * b;
+          auto logits = [&](int b, int stage, int phase) {
+            mbar_wait(b_full + 8 * stage, phase, &abort_flag, 102);
+            const uint64_t dk = smem_desc(smem_u32(kv_tiles + stage * 2 * C::kSmallBytes), 16, C::kAtomBytes, C::kSwizzle);
             if (elect_one()) {
 #pragma unroll
-              for (int c = 0; c < D / 16; ++c) umma_bf16(ts, dq + 2 * c, dk + 2 * c, idesc_s, c > 0);
+              for (int c = 0; c < D / 16; ++c) umma_bf16(tmem_base + 64 * b, dq + 2 * c, dk + 2 * c, idesc_s, c > 0);
               umma_commit(b_sfull + 8 * b);
             }
             __syncwarp();
-          }
-        } else {
-          // ---- O_A += P(i)[:, 0:32] V[0:32], O_B += P(i)[:, 32:64] V[32:64] once that group's
-          // probabilities of item i are in tensor memory ----
-          constexpr uint32_t idesc_pv = instr_desc(128, D, 0, 1);
+          };
+          mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 101);
+          tc_fence_after();
+          int ss = sj, sp = sph;  // stage and phase of the next logits
+          auto step_s = [&] { if (++ss == STAGES) { ss = 0; sp ^= 1; } };
+          for (int i = 0; i < 2 && i < nI; ++i, step_s()) logits((it + i) & 1, ss, sp);
           for (int i = 0; i < nI; ++i, ++it, step()) {
             const int b = it & 1, ph = (it >> 1) & 1;
             const uint64_t dv = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes + C::kSmallBytes),
                                           C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
             const uint32_t tp = tmem_base + 64 * b;
             const uint32_t first = (i == 0 || i == nL) ? 0u : 1u;  // a phase starts the accumulators afresh
-            mbar_wait(b_full + 8 * sj, sph, &abort_flag, 106);
             mbar_wait(b_tfull + 8 * b, ph, &abort_flag, 104);
             tc_fence_after();
             if (elect_one()) {
@@ -347,6 +350,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
               umma_commit(b_empty + 8 * sj);  // S(i) completed before the softmax warps read it
             }
             __syncwarp();
+            if (i + 2 < nI) {
+              logits(b, ss, sp);
+              step_s();
+            }
           }
         }
         warp_arrive(b_roles + 8 * (k & 1), lane);  // done with the lists
@@ -367,7 +374,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         if (lane == 0) softmax_tile = *(volatile int *)&abort_flag ? -1 : *(volatile int *)&tile_id[k & 1];
       }
       named_bar_sync(2, kSoftmaxWarps * 32);
-      const int x = *(volatile int *)&softmax_tile;
+      const int x = uniform(*(volatile int *)&softmax_tile);
       if (x < 0) break;
       mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 120);  // (complete: makes the lists visible to this warp)
       const uint8_t *meta = metas + (k & 1) * meta_step;
@@ -376,7 +383,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
       const uint8_t *icls = meta + ml.icls;                                         // [2 nT][4]
       const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
-      const int nL = counts[1], nI = nL + counts[2];
+      const int nL = uniform(counts[1]), nI = nL + uniform(counts[2]);
       const int u = tile_unit(x), n = unit_batch(u);
       const int pad0 = s.L - min(max(seq_lens ? seq_lens[n] : s.L, 0), s.L);
       const int t = tile_row0(x) + (PACK ? r & 63 : r);
@@ -441,6 +448,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         l = 0.f;
       };
       // the products of the item before `it` (of either phase) have completed
+      // (A parity only tells a barrier's last two phases apart.  The one before, item it - 3's, has passed: this
+      // warp has seen the logits of item it - 1, which were issued behind those products, and reported behind them.)
       auto products_done = [&](int site) {
         mbar_wait(b_done + 8 * ((it - 1) & 1), ((it - 1) >> 1) & 1, &abort_flag, site);
         __syncwarp();
