@@ -254,12 +254,22 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 3]), b_tfull = smem_u32(&bars[2 * STAGES + 5]);
   const uint32_t b_all = smem_u32(&bars[2 * STAGES + 7]);
 
-  if (tid == 0) {
-    abort_flag = (*status != 0) ? 1 : 0;
-    tma_prefetch_desc(&tmq);
-    tma_prefetch_desc(&tmk);
-    tma_prefetch_desc(&tmv);
-    tma_prefetch_desc(&tmg);
+  // this thread's row (compute warps) and its record from the pre-pass: asked for here, used after the set-up
+  const int quarter = warp & 3, half = warp >> 2;
+  const int r = quarter * 32 + lane, t = PACK ? row0 + (r & 63) : row0 + r;
+  const int hr = PACK ? h + (r >> 6) : h;  // this row's head
+  const bool row_ok = t < s.L;
+  float rec0 = 0.f, rec2 = 0.f, rec4 = 0.f, rec6 = 0.f;
+  if (row_ok && warp < kComputeWarps) {
+    const int64_t hrow = (int64_t)n * s.H + hr;
+    const float *rec = reinterpret_cast<const float *>(qstats) + (hrow * Lpad + (t & ~1)) * 4 + (t & 1);
+    rec0 = ADDS ? rec[0] : lse[hrow * s.L + t];
+    rec2 = rec[2];
+    rec4 = ADDS ? rec[4] : lse[((int64_t)s.B * s.H + hrow) * s.L + t];
+    rec6 = rec[6];
+  }
+  // The set-up is shared out so that the first loads leave at once: nothing before them waits for memory.
+  if (warp == kComputeWarps && lane == 0) {
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
@@ -273,18 +283,20 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     mbar_init(b_meta, 1);
     mbar_init(b_all, 1);
     mbar_fence_init();
-    // the CTA's tile lists and its resident tiles
+    // the CTA's tile lists (the streamed tiles wait for them) and its resident tiles
     mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
     bulk_load(smem_u32(meta), qmeta + ((size_t)u * nQT + (nQT - 1 - st)) * ml.bytes, (uint32_t)ml.bytes, b_meta);
     mbar_expect_tx(b_res, 2 * C::kBigBytes);
     tma_load_4d(smem_u32(q_tile), &tmq, b_res, 0, row0, h, n);
     tma_load_4d(smem_u32(g_tile), &tmg, b_res, 0, row0, h, n);
+    tma_prefetch_desc(&tmk);
+    tma_prefetch_desc(&tmv);
   }
-  if (warp == 0) {
-    __syncwarp();
+  if (warp == kComputeWarps + 1) {
     tmem_alloc(smem_u32(&tmem_slot), kBwdTmemCols);
     tmem_relinquish();
   }
+  if (warp == kComputeWarps + 2 && lane == 0) abort_flag = (*status != 0) ? 1 : 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -326,25 +338,27 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         const uint64_t dkd = smem_desc(kt, 16, C::kAtomBytes, C::kSwizzle);
         const uint64_t dvd = smem_desc(kt + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
         const uint32_t ts = tmem_base + 64 * hh;
-        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts, tmem_qa + 8 * k, dkd + 2 * k, idesc_s, k > 0);
+        for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts, tmem_qa + 8 * k, dkd + 2 * k, idesc_s, k > 0);
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts + 32, tmem_ga + 8 * k, dvd + 2 * k, idesc_s, k > 0);
-          umma_commit(b_sfull + 8 * hh);
-        }
-        __syncwarp();
+        for (int k = 0; k < D / 16; ++k) umma_bf16_ts(ts + 32, tmem_ga + 8 * k, dvd + 2 * k, idesc_s, k > 0);
+        umma_commit(b_sfull + 8 * hh);
       };
       mbar_wait(b_aready, 0, &abort_flag, 201);
       mbar_wait(b_full, 0, &abort_flag, 202);
       tc_fence_after();
-      first_stage(0, 0);
-      first_stage(0, 1);
+      if (elect_one()) {
+        first_stage(0, 0);
+        first_stage(0, 1);
+      }
+      __syncwarp();
       for (int i = 0, sj = 0; i < nvis; ++i) {
         const int sn = sj + 1 == STAGES ? 0 : sj + 1;
+        const bool more = i + 1 < nvis;
         const uint64_t dkm = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes), C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
+          if (hh == 0 && more) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 206);
           mbar_wait(b_tfull + 8 * hh, i & 1, &abort_flag, 204);
           tc_fence_after();
           if (elect_one()) {
@@ -352,23 +366,18 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
             for (int kk = 0; kk < 2; ++kk)
               umma_bf16_ts(tmem_dq, tmem_base + 64 * hh + 16 * kk, dkm + (2 * hh + kk) * C::kKStep, idesc_dq,
                            (i | hh | kk) != 0);
-            if (hh == 1) umma_commit(i + 1 < nvis ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
+            if (hh == 1) umma_commit(more ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
+            if (more) first_stage(sn, hh);
           }
           __syncwarp();
-          if (i + 1 < nvis) {
-            if (hh == 0) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 206);
-            first_stage(sn, hh);
-          }
         }
         sj = sn;
       }
     }
   } else {
     setmaxnreg_inc<kKvComputeRegs>();
-    const int quarter = warp & 3, half = warp >> 2;
-    const int r = quarter * 32 + lane, t = PACK ? row0 + (r & 63) : row0 + r, g = r / s.Bk;
-    const int hr = PACK ? h + (r >> 6) : h;  // this row's head
-    const bool row_ok = t < s.L, row_valid = row_ok && t >= pad0;
+    const int g = r / s.Bk;
+    const bool row_valid = row_ok && t >= pad0;
     const int t_last = row_valid ? (causal ? t : s.L - 1) : -1;  // the last key this row may see
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     // kPass: the row's weight rides in its record's exponents (the gate's gradient is not formed here)
@@ -376,12 +385,10 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     // this row's record from the pre-pass: nl = -(lse * log2e - log2 weight), nD = -Delta
     float nlL = 0.f, nlS = 0.f, nDL = 0.f, nDS = 0.f;
     if (row_valid) {
-      const int64_t hrow = (int64_t)n * s.H + hr;
-      const float *rec = reinterpret_cast<const float *>(qstats) + (hrow * Lpad + (t & ~1)) * 4 + (t & 1);
-      nlL = ADDS ? rec[0] : -(lse[hrow * s.L + t] * kLog2e);
-      nDL = alpha * rec[2];
-      nlS = ADDS ? rec[4] : -(lse[((int64_t)s.B * s.H + hrow) * s.L + t] * kLog2e);
-      nDS = beta * rec[6];
+      nlL = ADDS ? rec0 : -(rec0 * kLog2e);
+      nDL = alpha * rec2;
+      nlS = ADDS ? rec4 : -(rec4 * kLog2e);
+      nDS = beta * rec6;
     }
     float2 dalL = make_float2(0.f, 0.f), dalS = make_float2(0.f, 0.f);  // see dq_tile
     const float sc2 = s.scale * kLog2e;
@@ -458,6 +465,13 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
       warp_arrive(b_tfull + 8 * half, lane);
     }
 
+    {
+      const float dal = (dalL.x + dalL.y) - (dalS.x + dalS.y);
+      double a = row_valid ? (double)dal : 0.0;  // fixed-shape tree over the warp, then over the warps
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) red[warp] = a;
+    }
     if (nvis > 0) {
       mbar_wait(b_all, 0, &abort_flag, 209);
       __syncwarp();
@@ -488,14 +502,9 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
       named_bar_sync(5, kComputeWarps * 32);
       if (tid == 0) {
         tma_store_4d(&tmdq, smem_u32(kv_tiles), 0, row0, h, n);
-        tma_store_commit_and_wait();
+        tma_store_commit();
       }
     }
-    const float dal = (dalL.x + dalL.y) - (dalS.x + dalS.y);
-    double a = row_valid ? (double)dal : 0.0;  // fixed-shape tree over the warp, then over the warps
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) red[warp] = a;
   }
   tc_fence_before();
   __syncthreads();
@@ -520,6 +529,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     }
   }
   if (nvis == 0 && tid == 0) mbar_wait(b_res, 0, &abort_flag, 221);  // no load may outlive the CTA
+  if (tid == 0) tma_store_wait_read();
   finish(warp, tmem_base, kBwdTmemCols, &abort_flag, status);
 }
 
@@ -727,28 +737,30 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
         const uint64_t dqd = smem_desc(qt_, 16, C::kAtomBytes, C::kSwizzle);
         const uint64_t dgd = smem_desc(qt_ + C::kSmallBytes, 16, C::kAtomBytes, C::kSwizzle);
         const uint32_t ts = tmem_base + 64 * hh;
-        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) umma_bf16(ts, dkd + 2 * k, dqd + 2 * k, idesc_s, k > 0);
+        for (int k = 0; k < D / 16; ++k) umma_bf16(ts, dkd + 2 * k, dqd + 2 * k, idesc_s, k > 0);
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) umma_bf16(ts + 32, dvd + 2 * k, dgd + 2 * k, idesc_s, k > 0);
-          umma_commit(b_sfull + 8 * hh);
-        }
-        __syncwarp();
+        for (int k = 0; k < D / 16; ++k) umma_bf16(ts + 32, dvd + 2 * k, dgd + 2 * k, idesc_s, k > 0);
+        umma_commit(b_sfull + 8 * hh);
       };
       mbar_wait(b_res, 0, &abort_flag, 210);
       mbar_wait(b_full, 0, &abort_flag, 213);
       tc_fence_after();
-      first_stage(0, 0);
-      first_stage(0, 1);
+      if (elect_one()) {
+        first_stage(0, 0);
+        first_stage(0, 1);
+      }
+      __syncwarp();
       for (int i = 0, sj = 0; i < nvis; ++i) {
         const int sn = sj + 1 == STAGES ? 0 : sj + 1;
+        const bool more = i + 1 < nvis;
         const uint32_t q_tile = smem_u32(qg_tiles + sj * kStageBytes);
         const uint64_t dgm = smem_desc(q_tile + C::kSmallBytes, C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
         const uint64_t dqm = smem_desc(q_tile, C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const uint32_t tb = tmem_base + 64 * hh;
+          if (hh == 0 && more) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 215);
           mbar_wait(b_tfull + 8 * hh, i & 1, &abort_flag, 211);
           tc_fence_after();
           if (elect_one()) {
@@ -759,13 +771,10 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
               umma_bf16_ts(tmem_dk, tb + 32 + 16 * kk, dqm + (2 * hh + kk) * C::kKStep, idesc_o, (i | hh | kk) != 0);
-            if (hh == 1) umma_commit(i + 1 < nvis ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
+            if (hh == 1) umma_commit(more ? b_empty + 8 * sj : b_all);  // every product on this stage has completed
+            if (more) first_stage(sn, hh);
           }
           __syncwarp();
-          if (i + 1 < nvis) {
-            if (hh == 0) mbar_wait(b_full + 8 * sn, ((i + 1) / STAGES) & 1, &abort_flag, 215);
-            first_stage(sn, hh);
-          }
         }
         sj = sn;
       }
