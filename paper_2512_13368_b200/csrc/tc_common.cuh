@@ -353,11 +353,57 @@ __device__ __forceinline__ uint32_t cols32_le(int hi) { return ~cols32_ge(hi + 1
 // expand_block_bits for the 32 columns from column c0 (a multiple of 16) of the tile: bits past the tile's
 // 64 columns are not asked for
 __device__ __forceinline__ uint32_t expand_block_bits32(uint32_t bits, int bk, int c0) {
-  if (bk >= 32) return ((bits >> (c0 / bk)) & 1u) ? 0xffffffffu : 0u;  // (16 columns from 16: the low ones count)
+  // (16 columns from 16: the low ones count; no division by bk)
+  if (bk >= 32) return ((bk == 64 ? bits : bits >> (c0 >> 5)) & 1u) ? 0xffffffffu : 0u;
   const uint32_t b = bits >> (c0 >> 4);
   return ((b & 1u) ? 0xffffu : 0u) | ((b & 2u) ? 0xffff0000u : 0u);
 }
 
+// Links at power-of-two distances for mask blocks of one position (the paper's), over 64 columns.  kPow2: bits 1, 2, 4, 8,
+// 16, 32; a tile further away than 64 holds one column at most.
+constexpr uint64_t kPow2 = 0x0000000100010116ull, kPow2Rev = 0x6880800080000000ull;  // (bit b of one is bit 63 - b of the other)
+__device__ __forceinline__ uint64_t pow2_keys(int d0) {  // columns c with d0 - c a power of two
+  if (d0 < 64) return d0 < 1 ? 0ull : kPow2Rev >> (63 - d0);
+  if (d0 < 96) return (kPow2Rev << (d0 - 63)) | (1ull << (d0 - 64));
+  const int c = d0 - (1 << (31 - __clz(d0)));
+  return c < 64 ? 1ull << c : 0ull;
+}
+__device__ __forceinline__ uint64_t pow2_queries(int e0) {  // columns c with e0 + c a power of two
+  if (e0 <= 0) return e0 > -64 ? kPow2 << -e0 : 0ull;
+  if (e0 < 64) return (kPow2 >> e0) | (1ull << (64 - e0));
+  const int c = pow2_at_least(e0) - e0;
+  return c < 64 ? 1ull << c : 0ull;
+}
+
+// The links part of the masks below, out of line: the kernels' own instructions have to be fetched by every CTA and
+// warp, which is felt (inline, windows alone: forward 175 -> 172 us at B 128, H 4, L 1024, D 64, dK/dV 100 -> 98 at D 32;
+// with links and a selection per position at B 8, L 1500 dK/dV 70 -> 72).  For mask blocks of one position in closed
+// form: a walk over the powers of two took forward, dQ and dK/dV 55, 47 and 74 us there, now 50, 43 and 70.
+static __device__ __noinline__ uint64_t link_key_cols(int L, int blk, int t, int p0, bool causal) {
+  uint64_t m = cols_ge(L - blk - p0);
+  if (blk == 1) {
+    m |= pow2_keys(t - p0);
+    return causal ? m : m | pow2_queries(p0 - t);
+  }
+  const int bq = t / blk;
+  // key block bq - d, d a power of two: later d lie further left.  The walk starts at the first d
+  // that can reach the tile from the right, the smallest power of two >= bq - (last block of the
+  // tile), instead of at 1: a far tile then costs one or two steps, not log2 of its distance.
+  const int dmin = bq - (p0 + 63) / blk;
+  for (int d = pow2_at_least(dmin); d <= bq; d <<= 1) {
+    const int a = (bq - d) * blk;
+    if (a + blk - 1 < p0) break;
+    if (a <= p0 + 63) m |= cols_ge(a - p0) & cols_le(a + blk - 1 - p0);
+  }
+  if (!causal) {
+    for (int d = pow2_at_least(p0 / blk - bq);; d <<= 1) {  // and key block bq + d: later d lie further right
+      const int a = (bq + d) * blk;
+      if (a > p0 + 63 || a >= L) break;
+      if (a + blk - 1 >= p0) m |= cols_ge(a - p0) & cols_le(a + blk - 1 - p0);
+    }
+  }
+  return m;
+}
 // Short-term mask of Eq. 15 over the 64 keys p0 ... p0 + 63 for query t, without the causal and
 // the padding condition (the caller ANDs those): the window, and with the power-law mask the key
 // blocks at power-of-two block distances and the last block.  `causal` is the caller's (often
@@ -365,27 +411,7 @@ __device__ __forceinline__ uint32_t expand_block_bits32(uint32_t bits, int bk, i
 __device__ __forceinline__ uint64_t st_key_cols(const Shape &s, int t, int p0, bool causal) {
   uint64_t m = cols_ge(t - s.window + 1 - p0);
   if (!causal) m &= cols_le(t + s.window - 1 - p0);  // (without the causal mask the window has two sides)
-  if (s.stis_mode) {
-    m |= cols_ge(s.L - s.stis_blk - p0);
-    const int bq = t / s.stis_blk;
-    // key block bq - d, d a power of two: later d lie further left.  The walk starts at the first d
-    // that can reach the tile from the right, the smallest power of two >= bq - (last block of the
-    // tile), instead of at 1: a far tile then costs one or two steps, not log2 of its distance.
-    const int dmin = bq - (p0 + 63) / s.stis_blk;
-    for (int d = pow2_at_least(dmin); d <= bq; d <<= 1) {
-      const int a = (bq - d) * s.stis_blk;
-      if (a + s.stis_blk - 1 < p0) break;
-      if (a <= p0 + 63) m |= cols_ge(a - p0) & cols_le(a + s.stis_blk - 1 - p0);
-    }
-    if (!causal) {
-      for (int d = pow2_at_least(p0 / s.stis_blk - bq);; d <<= 1) {  // and key block bq + d: later d lie further right
-        const int a = (bq + d) * s.stis_blk;
-        if (a > p0 + 63 || a >= s.L) break;
-        if (a + s.stis_blk - 1 >= p0) m |= cols_ge(a - p0) & cols_le(a + s.stis_blk - 1 - p0);
-      }
-    }
-  }
-  return m;
+  return s.stis_mode ? m | link_key_cols(s.L, s.stis_blk, t, p0, causal) : m;
 }
 // The window's part of it over 32 keys (all of it with stis_mode = 0)
 __device__ __forceinline__ uint32_t st_window32(const Shape &s, int t, int p0, bool causal) {
@@ -393,28 +419,31 @@ __device__ __forceinline__ uint32_t st_window32(const Shape &s, int t, int p0, b
   if (!causal) m &= cols32_le(t + s.window - 1 - p0);
   return m;
 }
+static __device__ __noinline__ uint64_t link_query_cols(int L, int blk, int p, int t0, bool causal) {
+  if (p >= L - blk) return ~0ull;
+  if (blk == 1) return causal ? pow2_queries(t0 - p) : pow2_queries(t0 - p) | pow2_keys(p - t0);
+  uint64_t m = 0ull;
+  const int bk = p / blk;
+  for (int d = pow2_at_least(t0 / blk - bk);; d <<= 1) {  // query block bk + d: later d lie further right
+    const int a = (bk + d) * blk;
+    if (a > t0 + 63 || a >= L) break;
+    if (a + blk - 1 >= t0) m |= cols_ge(a - t0) & cols_le(a + blk - 1 - t0);
+  }
+  if (!causal) {
+    for (int d = pow2_at_least(bk - (t0 + 63) / blk); d <= bk; d <<= 1) {  // and query block bk - d
+      const int a = (bk - d) * blk;
+      if (a + blk - 1 < t0) break;
+      if (a <= t0 + 63) m |= cols_ge(a - t0) & cols_le(a + blk - 1 - t0);
+    }
+  }
+  return m;
+}
 // The same mask seen from key p over the 64 queries t0 ... t0 + 63 (again without causality and
 // padding).
 __device__ __forceinline__ uint64_t st_query_cols(const Shape &s, int p, int t0, bool causal) {
   uint64_t m = cols_le(p + s.window - 1 - t0);
   if (!causal) m &= cols_ge(p - s.window + 1 - t0);
-  if (s.stis_mode) {
-    if (p >= s.L - s.stis_blk) return ~0ull;
-    const int bk = p / s.stis_blk;
-    for (int d = pow2_at_least(t0 / s.stis_blk - bk);; d <<= 1) {  // query block bk + d: later d lie further right
-      const int a = (bk + d) * s.stis_blk;
-      if (a > t0 + 63 || a >= s.L) break;
-      if (a + s.stis_blk - 1 >= t0) m |= cols_ge(a - t0) & cols_le(a + s.stis_blk - 1 - t0);
-    }
-    if (!causal) {
-      for (int d = pow2_at_least(bk - (t0 + 63) / s.stis_blk); d <= bk; d <<= 1) {  // and query block bk - d
-        const int a = (bk - d) * s.stis_blk;
-        if (a + s.stis_blk - 1 < t0) break;
-        if (a <= t0 + 63) m |= cols_ge(a - t0) & cols_le(a + s.stis_blk - 1 - t0);
-      }
-    }
-  }
-  return m;
+  return s.stis_mode ? m | link_query_cols(s.L, s.stis_blk, p, t0, causal) : m;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
