@@ -20,6 +20,11 @@
 // i to be reported complete; products of one thread run in the order of their issue, so it can follow them
 // at once.  That, and roles, loop bounds and addresses in uniform registers (tc_common.cuh), took the kernel
 // from 199 to 179 us at B 128, H 4, L 1024, D 64 and from 360 to 332 at B 16, H 8, L 4096.
+// One code serves all items, masked or not, and both phases' ends: the logits that a row does not see become
+// -infinity before the maximum is taken.  With variants for masked items, a vote which to take and the merge inlined three
+// times the instructions did not come fast enough: 176 -> 165 us, 330 -> 310, D 32 78 -> 74, a selection per position
+// at B 8, L 1500 51 -> 45 (2 - 4 us of each by classes per half of the keys, which leave out masks where one of two
+// blocks of 32 was selected).
 //
 // CTA = 384 threads.  Warps 0..7 are softmax warps: a query row (= TMEM lane) is shared by two
 // threads, warp w and warp w + 4, which split the KEYS of every tile: group 0 (warps 0..3) takes
@@ -68,42 +73,28 @@ static_assert(256 * kSoftmaxRegs + 128 * kProducerRegs <= kFwdThreads * 80, "reg
 constexpr uint32_t kFwdTmemCols = 256;
 __host__ __device__ constexpr int fwd_stages(int D) { return D == 64 ? 3 : 4; }
 
-// maximum of 32 logits (those whose mask bit is set, all of them when FULL)
-template <bool FULL>
-__device__ __forceinline__ float half_row_max(const float (&v)[32], uint32_t mask) {
+// maximum of 32 logits
+__device__ __forceinline__ float half_row_max(const float (&v)[32]) {
   float a[4];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) a[e] = -INFINITY;
+  for (int e = 0; e < 4; ++e) a[e] = fmaxf(v[2 * e], v[2 * e + 1]);
 #pragma unroll
-  for (int c = 0; c < 32; c += 8) {
-    float x[8];
+  for (int c = 8; c < 32; c += 8)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) x[e] = (FULL || ((mask >> (c + e)) & 1u)) ? v[c + e] : -INFINITY;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) a[e] = max3(a[e], x[2 * e], x[2 * e + 1]);
-  }
+    for (int e = 0; e < 4; ++e) a[e] = max3(a[e], v[c + 2 * e], v[c + 2 * e + 1]);
   return fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3]));
 }
 
 // probabilities of 32 logits relative to the running maximum (nm = -m, log2 units), packed as
 // bf16 pairs; their sum is added to l.  Two logits per FMA / ADD instruction.
-template <bool FULL>
-__device__ __forceinline__ void half_row_probs(const float (&sv)[32], uint32_t mask, float sc2, float nm,
-                                               float &l, uint32_t (&pk)[16]) {
+__device__ __forceinline__ void half_row_probs(const float (&sv)[32], float sc2, float nm, float &l, uint32_t (&pk)[16]) {
   const float2 sc = make_float2(sc2, sc2), nn = make_float2(nm, nm);
   float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
 #pragma unroll
   for (int c = 0; c < 32; c += 4) {
     const float2 x0 = ffma2(make_float2(sv[c], sv[c + 1]), sc, nn);
     const float2 x1 = ffma2(make_float2(sv[c + 2], sv[c + 3]), sc, nn);
-    float2 e0 = make_float2(exp2f(x0.x), exp2f(x0.y)), e1 = make_float2(exp2f(x1.x), exp2f(x1.y));
-    if (!FULL) {
-      const uint32_t w = mask >> c;
-      e0.x = (w & 1u) ? e0.x : 0.f;
-      e0.y = (w & 2u) ? e0.y : 0.f;
-      e1.x = (w & 4u) ? e1.x : 0.f;
-      e1.y = (w & 8u) ? e1.y : 0.f;
-    }
+    const float2 e0 = make_float2(exp2f(x0.x), exp2f(x0.y)), e1 = make_float2(exp2f(x1.x), exp2f(x1.y));
     s0 = fadd2(s0, e0);
     s1 = fadd2(s1, e1);
     pk[c >> 1] = pack_bf16(e0.x, e0.y);
@@ -455,30 +446,27 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         __syncwarp();
         tc_fence_after();
       };
-      auto end_long_term = [&] {
-        if (nL > 0) products_done(111);
-        mbar_wait(b_stored, 1, &abort_flag, 118);  // sl: the tile before has been stored (at once for the first)
-        merge(false);
-      };
-
-      for (int i = 0; i < nI; ++i, ++it) {
-        const bool isL = i < nL;
-        const int jt = jt_n, cls = cls_n, p0 = jt * 64;
+      int i = 0;
+#pragma unroll 1
+      for (int phase = 0; phase < 2; ++phase) {  // the long-term items, the short-term items
+      const int phase_end = phase ? nI : nL;
+      const bool isL = phase == 0;
+#pragma unroll 1
+      for (; i < phase_end; ++i, ++it) {
+        const int jt = jt_n, cls = (cls_n >> (2 * grp)) & 3, p0 = jt * 64;
         if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
           jt_n = items[i + 1];
           cls_n = icls[(i + 1) * 4 + quarter];
         }
         const int b = it & 1, ph = (it >> 1) & 1;
-        if (i == nL) end_long_term();
         uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
-        bool doB = cls == 1, fullB = cls == 1;
+        bool doB = cls == 1;
         if (cls == 2) {
           const int c0 = p0 + 32 * grp;
           hm = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
           if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, 32 * grp);
           else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> (32 * grp)) : st_window32(s, t, c0, causal);
           doB = __any_sync(0xffffffffu, hm != 0u);
-          fullB = __all_sync(0xffffffffu, hm == 0xffffffffu);
         }
         const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
 
@@ -491,7 +479,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           tmem_ld32(t_b, sv);
           tmem_wait_ld();
           float fac = 1.f;
-          const float mt = (fullB ? half_row_max<true>(sv, 0u) : half_row_max<false>(sv, hm)) * sc2;
+          if (cls == 2)  // (one code behind it for all items: the instructions have to be fetched, and that is felt)
+#pragma unroll
+            for (int c = 0; c < 32; ++c) sv[c] = (hm >> c) & 1u ? sv[c] : -INFINITY;
+          const float mt = half_row_max(sv) * sc2;
           const bool need = mt > m + kRescaleThreshold;  // also true on the row's first keys, before which
           const bool scale_acc = need && l > 0.f;        // the accumulator holds sums of zero probabilities
           if (need) {
@@ -499,8 +490,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
             l *= fac;
             m = mt;
           }
-          if (fullB) half_row_probs<true>(sv, 0u, sc2, -m, l, pk);
-          else half_row_probs<false>(sv, hm, sc2, -m, l, pk);
+          half_row_probs(sv, sc2, m == -INFINITY ? 0.f : -m, l, pk);  // (no key yet: all logits are -infinity)
           if (__any_sync(0xffffffffu, scale_acc)) {  // rescaling needs the products of item i-1
             products_done(108);
             rescale_acc<D>(acc_own, fac);
@@ -515,11 +505,12 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
       }
 
-      if (nI == 0) mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 112);  // (nothing else waited for the queries)
-      if (nL == nI) end_long_term();
-      if (nI > nL) products_done(110);
-      mbar_wait(b_stored, 0, &abort_flag, 119);  // sl: the long-term rows have been stored
-      merge(true);
+      if (phase_end > (phase ? nL : 0)) products_done(110 + phase);
+      if (phase && nI == 0) mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 112);  // (nothing else waited for the queries)
+      // sl: the tile before has been stored (at once for the first); the long-term rows have been stored
+      mbar_wait(b_stored, phase ^ 1, &abort_flag, 118 + phase);
+      merge(phase == 1);
+      }
     }
   }
   finish(warp, tmem_base, kFwdTmemCols, &abort_flag, status);

@@ -13,7 +13,7 @@
 //   list[nT], flags[nT]       the tiles any row of the CTA needs, ascending; bit 0: some selected
 //                             block lies in the tile, bit 1: the window of some row reaches it
 //   items[2 nT], icls[2 nT][4] (forward) the long-term tiles, then the short-term tiles, and the
-//                             class of every (item, softmax warp)
+//                             classes of every (item, row quarter), two bits per half of the keys
 //   jcls[nT][2][8]            (dQ) class of every (listed tile, half tile, compute warp)
 //   counts                    {tiles on the list, long-term items, short-term items}
 // Head-packed variant (Shape::pack): the CTA's rows 0..63 and 64..127 are the same 64 positions of
@@ -228,27 +228,30 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
     sync();
     const int nl = counts[1], count = nl + counts[2];
-    // Class of every (item, softmax warp): 0 = no row of the warp needs the tile, 1 = every row
-    // sees all 64 keys, 2 = mixed (the warp builds per-lane column masks).
-    const bool uni = s.Bk >= 32;  // a warp's 32 rows share one query block
-    const uint32_t allbits = (1u << nb) - 1u;
+    // Class of every (item, row quarter, key half), two bits each in a byte per (item, quarter): 0 = no row of the
+    // quarter needs the 32 keys, 1 = every row sees all of them, 2 = mixed (the warp builds per-lane column masks).
+    const bool uni = s.Bk >= 32;  // a quarter's 32 rows share one query block
     for (int e = tid; e < count * 4; e += NT) {
       const int it = e >> 2, w = e & 3;
-      const int jt = items[it], p0 = jt * 64, t_lo = quarter_row0(w);
-      const bool some = (p0 <= t_lo + 31 || !s.causal) && p0 + 63 >= pad0 && t_lo + 31 >= pad0 && t_lo < s.L;
-      // every row of the warp may see every key of the tile as far as validity and causality go
-      const bool inner = t_lo >= pad0 && t_lo + 31 < s.L && p0 >= pad0 && (s.causal ? p0 + 63 <= t_lo : p0 + 63 < s.L);
+      const int jt = items[it], t_lo = quarter_row0(w), t_hi = t_lo + 31;
+      const bool rows = t_hi >= pad0 && t_lo < s.L, rows_in = t_lo >= pad0 && t_hi < s.L;
+      const uint32_t bits = it < nl && uni ? selb[((w * 32) >> bk_shift) * nT + jt] : 0u;
       int cls = 0;
-      if (some) {
-        if (it < nl) {
-          if (!uni) cls = 2;
-          else {
-            const uint32_t bits = selb[((w * 32) >> bk_shift) * nT + jt];
-            cls = bits == 0u ? 0 : ((!s.pq && inner && bits == allbits) ? 1 : 2);  // (per position: the rows differ)
+#pragma unroll 1
+      for (int hf = 0; hf < 2; ++hf) {
+        const int k_lo = jt * 64 + 32 * hf, k_hi = k_lo + 31;
+        int c = 0;
+        if (rows && (k_lo <= t_hi || !s.causal) && k_hi >= pad0 && k_lo < s.L) {
+          // every row of the quarter may see every key of the half as far as validity and causality go
+          const bool inner = rows_in && k_lo >= pad0 && (s.causal ? k_hi <= t_lo : k_hi < s.L);
+          if (it < nl) {
+            if (!uni) c = 2;
+            else if ((bits >> ((32 * hf) >> bk_shift)) & 1u) c = !s.pq && inner ? 1 : 2;  // (per position: the rows differ)
+          } else if (st_ranges_touch(s, t_lo, t_hi, k_lo, k_hi)) {
+            c = (inner && k_lo >= t_hi - s.window + 1 && (s.causal || k_hi <= t_lo + s.window - 1)) ? 1 : 2;  // 1: inside every row's window
           }
-        } else if (st_ranges_touch(s, t_lo, t_lo + 31, p0, p0 + 63)) {
-          cls = (inner && p0 >= t_lo + 31 - s.window + 1 && (s.causal || p0 + 63 <= t_lo + s.window - 1)) ? 1 : 2;  // 1: inside every row's window
         }
+        cls |= c << (2 * hf);
       }
       icls[e] = (uint8_t)cls;
     }
