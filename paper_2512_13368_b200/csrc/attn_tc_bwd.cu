@@ -23,9 +23,11 @@
 // warps on every half tile (16 columns each, twice the hand-offs and their instructions), a warp for each
 // stage and without the uniform registers of tc_common.cuh the kernels took 197 and 232 us at B 128, H 4,
 // L 1024, D 64 (now 181 and 223), 384 and 479 at B 16, H 8, L 4096 (353 and 453), 64 and 80 with a selection
-// per position at B 8, L 1500 (50 and 73).  What is left is the chain of a half tile: arithmetic 1300 cycles,
-// from there to the next logits 700, while the issue slots are 42 % and the tensor pipe 30 % busy; and the
-// 8000 - 10000 cycles that a CTA spends outside its loop.
+// per position at B 8, L 1500 (50 and 73).  Then the code: half tiles of one branch without masks are one code for
+// either branch, everything else goes through one masked code; with a code for each branch, both, and masked tiles the
+// instructions did not come fast enough (173 and 221 -> 166 and 212 us; 341 and 450 -> 331 and 435; D 32 82 and 98 -> 78
+// and 93).  What is left is the chain of a half tile: arithmetic 1300 cycles, from there to the next logits 700, while
+// the issue slots are 42 % and the tensor pipe 30 % busy; and the 8000 cycles that a CTA spends outside its loop.
 //
 //  dQ     resident Q, dO (128 queries: 128 positions of a head, or with grouped heads 64 positions
 //         of two heads of a group, as in the forward); streams K, V 64-key tiles (same walk as the forward) and
@@ -52,6 +54,7 @@
 #include "tc_common.cuh"
 
 #include <cooperative_groups.h>
+#include <type_traits>
 
 namespace blossom {
 namespace tc {
@@ -165,35 +168,34 @@ __device__ __forceinline__ void add_row_chunk(uint32_t (&w)[4], const __nv_bfloa
 // zero.  (As many instructions: the weight rides in what was the addition of -Delta; the kernel went from
 // 0.381 to 0.388 ms at B 16, H 8, L 4096.)  dalS collects what only the short-term branch sees.  Two columns
 // per FMA / ADD / MUL instruction.
-template <bool HAS_L, bool HAS_S, bool FULL>
-__device__ __forceinline__ void dq_tile(const float (&sv)[16], const float (&dp)[16], uint32_t hL,
-                                        uint32_t hS, float sc2, float nlL, float nlS, float wL, float wS,
-                                        float nDL, float nDS, float2 &dalL, float2 &dalS, uint32_t (&dw)[8]) {
+// BOTH: both branches see columns of the tile; else the one whose record, weight and mask come as the first ones
+// (one code for either branch: the instructions of the variants have to be fetched, and that is felt).
+template <bool BOTH, bool FULL>
+__device__ __forceinline__ void dq_tile(const float (&sv)[16], const float (&dp)[16], uint32_t hL, uint32_t hS, float sc2,
+                                        float nlL, float nlS, float wL, float wS, float nDL, float nDS, float2 &dal,
+                                        uint32_t (&dw)[8]) {
   const float2 sc = make_float2(sc2, sc2);
 #pragma unroll
   for (int c = 0; c < 16; c += 2) {
     const float2 s2 = make_float2(sv[c], sv[c + 1]), dp2 = make_float2(dp[c], dp[c + 1]);
-    float2 acc = make_float2(0.f, 0.f), pL = acc;
-    if (HAS_L) {
-      const float2 x = ffma2(s2, sc, make_float2(nlL, nlL));
-      pL = make_float2(exp2f(x.x), exp2f(x.y));
-      if (!FULL) {
-        pL.x = bit(hL, c) ? pL.x : 0.f;
-        pL.y = bit(hL, c + 1) ? pL.y : 0.f;
-      }
-      if (!HAS_S) dalL = ffma2(pL, dp2, dalL);
-      acc = fmul2(pL, ffma2(dp2, make_float2(wL, wL), make_float2(nDL, nDL)));
+    const float2 x = ffma2(s2, sc, make_float2(nlL, nlL));
+    float2 pL = make_float2(exp2f(x.x), exp2f(x.y));
+    if (!FULL) {
+      pL.x = bit(hL, c) ? pL.x : 0.f;
+      pL.y = bit(hL, c + 1) ? pL.y : 0.f;
     }
-    if (HAS_S) {
-      const float2 x = ffma2(s2, sc, make_float2(nlS, nlS));
-      float2 p = make_float2(exp2f(x.x), exp2f(x.y));
+    float2 acc = fmul2(pL, ffma2(dp2, make_float2(wL, wL), make_float2(nDL, nDL)));
+    if (BOTH) {
+      const float2 y = ffma2(s2, sc, make_float2(nlS, nlS));
+      float2 p = make_float2(exp2f(y.x), exp2f(y.y));
       if (!FULL) {
         p.x = bit(hS, c) ? p.x : 0.f;
         p.y = bit(hS, c + 1) ? p.y : 0.f;
       }
-      if (HAS_L) dalL = ffma2(ffma2(p, make_float2(-1.f, -1.f), pL), dp2, dalL);
-      else dalS = ffma2(p, dp2, dalS);
+      dal = ffma2(ffma2(p, make_float2(-1.f, -1.f), pL), dp2, dal);
       acc = ffma2(p, ffma2(dp2, make_float2(wS, wS), make_float2(nDS, nDS)), acc);
+    } else {
+      dal = ffma2(pL, dp2, dal);
     }
     dw[c >> 1] = pack_bf16(acc.x, acc.y);
   }
@@ -434,42 +436,51 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         c1_n = jc[(i + 1) * 16 + 4];
       }
       uint32_t hL = 0u, hS = 0u;  // this thread's 32 keys
+      const bool masked = ((cls0 | cls1) & 8) || (cls0 & 3) == 3 || (cls1 & 3) == 3;
       if ((cls0 | cls1) & 8) {  // mixed: per-lane column masks
         const int jt = list[i], f = lflags[i], p0 = jt * 64, col = 32 * half, c0 = p0 + col;
         const uint32_t mc = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
         if (f & 1) hL = mc & expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, col);
         if (f & 2) hS = mc & (s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> col) : st_window32(s, t, c0, causal));
+      } else if (masked) {
+        hL = (cls0 & 1 ? 0xffffu : 0u) | (cls1 & 1 ? 0xffff0000u : 0u);
+        hS = (cls0 & 2 ? 0xffffu : 0u) | (cls1 & 2 ? 0xffff0000u : 0u);
       }
       mbar_wait(b_sfull + 8 * half, i & 1, &abort_flag, 207);
       __syncwarp();
       tc_fence_after();
-#pragma unroll
-      for (int ps = 0; ps < 2; ++ps) {
-        const int cls = ps ? cls1 : cls0;
-        const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
-        bool anyL = cls & 1, anyS = cls & 2, full = true;
-        if (cls & 8) {
-          anyL = __any_sync(0xffffffffu, xL != 0u);
-          anyS = __any_sync(0xffffffffu, xS != 0u);
-          full = __all_sync(0xffffffffu, (!anyL || xL == 0xffffu) && (!anyS || xS == 0xffffu));
-        }
+      // dS (bf16 pairs) goes over the first 8 of a pass's 16 S columns
+      auto pass = [&](auto full_tag, int ps, bool anyL, bool anyS, uint32_t xL, uint32_t xS) {
+        constexpr bool FULL = decltype(full_tag)::value;
         uint32_t dw[8];
         if (anyL || anyS) {
           float sv[16], dp[16];
           tmem_ld16(tb + 16 * ps, sv);
           tmem_ld16(tb + 32 + 16 * ps, dp);
           tmem_wait_ld();
-          if (!full && (PLAIN || (anyL && anyS))) dq_tile<true, true, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-          else if (!full && anyL) dq_tile<true, false, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-          else if (!full) dq_tile<false, true, false>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-          else if (anyL && anyS) dq_tile<true, true, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-          else if (anyL) dq_tile<true, false, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
-          else dq_tile<false, true, true>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dalS, dw);
+          if (!FULL && (PLAIN || (anyL && anyS))) {
+            dq_tile<true, FULL>(sv, dp, xL, xS, sc2, nlL, nlS, alpha, beta, nDL, nDS, dalL, dw);
+          } else {
+            float2 dal = make_float2(0.f, 0.f);
+            dq_tile<false, FULL>(sv, dp, anyL ? xL : xS, 0u, sc2, anyL ? nlL : nlS, 0.f, anyL ? alpha : beta, 0.f, anyL ? nDL : nDS, 0.f, dal, dw);
+            if (anyL) dalL = fadd2(dalL, dal);
+            else dalS = fadd2(dalS, dal);
+          }
         } else {
 #pragma unroll
           for (int c = 0; c < 8; ++c) dw[c] = 0u;
         }
-        tmem_st8u(tb + 16 * ps, dw);  // dS (bf16 pairs) over the first 8 of the pass's 16 S columns
+        tmem_st8u(tb + 16 * ps, dw);
+      };
+      if (masked) {
+#pragma unroll 2
+        for (int ps = 0; ps < 2; ++ps) {
+          const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
+          pass(std::false_type(), ps, __any_sync(0xffffffffu, xL != 0u), __any_sync(0xffffffffu, xS != 0u), xL, xS);
+        }
+      } else {
+        pass(std::true_type(), 0, cls0 & 1, cls0 & 2, 0u, 0u);
+        pass(std::true_type(), 1, cls1 & 1, cls1 & 2, 0u, 0u);
       }
       tmem_wait_st();
       tc_fence_before();
@@ -549,7 +560,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
 // the records of these 8 query pairs: {nl_lt(2), -Delta_lt(2)} {nl_st(2), -Delta_st(2)} per pair
 // (nl = -(lse * log2e - log2 weight): the branch weight rides in the exponent).  Two columns per
 // FMA / ADD / MUL instruction.
-template <bool HAS_L, bool HAS_S, bool FULL>
+// BOTH as in dq_tile: with one branch st points at that branch's half of the records.
+template <bool BOTH, bool FULL>
 __device__ __forceinline__ void dkdv_tile(const float (&sv)[16], const float (&dp)[16], uint32_t hL,
                                           uint32_t hS, float sc2, const float4 *st, uint32_t (&ww)[8],
                                           uint32_t (&dw)[8]) {
@@ -557,28 +569,24 @@ __device__ __forceinline__ void dkdv_tile(const float (&sv)[16], const float (&d
 #pragma unroll
   for (int c = 0; c < 16; c += 2) {
     const float2 s2 = make_float2(sv[c], sv[c + 1]), dp2 = make_float2(dp[c], dp[c + 1]);
-    float2 w = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
-    if (HAS_L) {
-      const float4 r = st[c];  // pair c / 2, long-term half of the record
-      const float2 x = ffma2(s2, sc, make_float2(r.x, r.y));
-      float2 p = make_float2(exp2f(x.x), exp2f(x.y));
-      if (!FULL) {
-        p.x = bit(hL, c) ? p.x : 0.f;
-        p.y = bit(hL, c + 1) ? p.y : 0.f;
-      }
-      w = p;
-      d = fmul2(p, fadd2(dp2, make_float2(r.z, r.w)));
+    const float4 r = st[c];  // pair c / 2
+    const float2 x = ffma2(s2, sc, make_float2(r.x, r.y));
+    float2 w = make_float2(exp2f(x.x), exp2f(x.y));
+    if (!FULL) {
+      w.x = bit(hL, c) ? w.x : 0.f;
+      w.y = bit(hL, c + 1) ? w.y : 0.f;
     }
-    if (HAS_S) {
-      const float4 r = st[c + 1];  // short-term half
-      const float2 x = ffma2(s2, sc, make_float2(r.x, r.y));
-      float2 p = make_float2(exp2f(x.x), exp2f(x.y));
+    float2 d = fmul2(w, fadd2(dp2, make_float2(r.z, r.w)));
+    if (BOTH) {
+      const float4 q = st[c + 1];  // short-term half
+      const float2 y = ffma2(s2, sc, make_float2(q.x, q.y));
+      float2 p = make_float2(exp2f(y.x), exp2f(y.y));
       if (!FULL) {
         p.x = bit(hS, c) ? p.x : 0.f;
         p.y = bit(hS, c + 1) ? p.y : 0.f;
       }
-      w = HAS_L ? fadd2(w, p) : p;
-      d = ffma2(p, fadd2(dp2, make_float2(r.z, r.w)), d);
+      w = fadd2(w, p);
+      d = ffma2(p, fadd2(dp2, make_float2(q.z, q.w)), d);
     }
     ww[c >> 1] = pack_bf16(w.x, w.y);
     dw[c >> 1] = pack_bf16(d.x, d.y);
@@ -810,12 +818,16 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
       const int cls0 = cls2[0], cls1 = cls2[4];
       ++li;
       uint32_t hL = 0u, hS = 0u;
+      const bool masked = ((cls0 | cls1) & 8) || (cls0 & 3) == 3 || (cls1 & 3) == 3;
       if ((cls0 | cls1) & 8) {  // a mixed half: per-lane column masks
         if (row_valid) {
           const uint32_t mc = cols32_ge((causal ? p : pad0) - t0) & cols32_le(s.L - 1 - t0);
           if (f & 1) hL = mc & (pq ? (uint32_t)(inv64[g * nT + qt] >> q0) : expand_block_bits32(invb[g * nT + qt], s.Bk, q0));
           if (f & 2) hS = mc & (uint32_t)(st_query_cols(s, p, qt * 64, causal) >> q0);
         }
+      } else if (masked) {
+        hL = (cls0 & 1 ? 0xffffu : 0u) | (cls1 & 1 ? 0xffff0000u : 0u);
+        hS = (cls0 & 2 ? 0xffffu : 0u) | (cls1 & 2 ? 0xffff0000u : 0u);
       }
       mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 216);  // the row records have landed
       const float4 *stt = reinterpret_cast<const float4 *>(qg_tiles + (i % STAGES) * kStageBytes + 2 * C::kSmallBytes);
@@ -823,16 +835,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
       __syncwarp();
       tc_fence_after();
       // W^T and dS^T of the 16 columns of a pass go, as bf16 pairs, over the first 8 of them in S^T / dP^T.
-#pragma unroll
-      for (int ps = 0; ps < 2; ++ps) {
-        const int cls = ps ? cls1 : cls0;
-        const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
-        bool anyL = (cls & 1) != 0, anyS = (cls & 2) != 0, full = true;
-        if (cls == 8) {
-          anyL = __any_sync(0xffffffffu, xL != 0u);
-          anyS = __any_sync(0xffffffffu, xS != 0u);
-          full = __all_sync(0xffffffffu, (!anyL || xL == 0xffffu) && (!anyS || xS == 0xffffu));
-        }
+      auto pass = [&](auto full_tag, int ps, bool anyL, bool anyS, uint32_t xL, uint32_t xS) {
+        constexpr bool FULL = decltype(full_tag)::value;
         uint32_t ww[8], dw[8];
         if (anyL || anyS) {
           float sv[16], dp[16];
@@ -840,18 +844,24 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
           tmem_ld16(tb + 32 + 16 * ps, dp);
           tmem_wait_ld();
           const float4 *sq = stt + q0 + 16 * ps;  // 8 pairs x 2 float4
-          if (!full && (PLAIN || (anyL && anyS))) dkdv_tile<true, true, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
-          else if (!full && anyL) dkdv_tile<true, false, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
-          else if (!full) dkdv_tile<false, true, false>(sv, dp, xL, xS, sc2, sq, ww, dw);
-          else if (anyL && anyS) dkdv_tile<true, true, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
-          else if (anyL) dkdv_tile<true, false, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
-          else dkdv_tile<false, true, true>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          if (!FULL && (PLAIN || (anyL && anyS))) dkdv_tile<true, FULL>(sv, dp, xL, xS, sc2, sq, ww, dw);
+          else dkdv_tile<false, FULL>(sv, dp, anyL ? xL : xS, 0u, sc2, sq + (anyL ? 0 : 1), ww, dw);
         } else {
 #pragma unroll
           for (int c = 0; c < 8; ++c) { ww[c] = 0u; dw[c] = 0u; }
         }
         tmem_st8u(tb + 16 * ps, ww);
         tmem_st8u(tb + 32 + 16 * ps, dw);
+      };
+      if (masked) {
+#pragma unroll 2
+        for (int ps = 0; ps < 2; ++ps) {
+          const uint32_t xL = (hL >> (16 * ps)) & 0xffffu, xS = (hS >> (16 * ps)) & 0xffffu;
+          pass(std::false_type(), ps, __any_sync(0xffffffffu, xL != 0u), __any_sync(0xffffffffu, xS != 0u), xL, xS);
+        }
+      } else {
+        pass(std::true_type(), 0, cls0 & 1, cls0 & 2, 0u, 0u);
+        pass(std::true_type(), 1, cls1 & 1, cls1 & 2, 0u, 0u);
       }
       tmem_wait_st();
       tc_fence_before();
