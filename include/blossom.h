@@ -230,6 +230,16 @@ int blossom_attn_bwd(const blossom_params *params /* host */, const void *q, con
                      float *dgate, void *workspace, size_t workspace_bytes,
                      blossom_stream_t stream);
 
+/* Copies rows between layouts (no counterpart in the paper): row (b, h, l) of row_bytes bytes from
+ * src + b * src_strides[0] + h * src_strides[1] + l * src_strides[2] to the place that dst_strides give,
+ * for callers whose tensors do not have the layout that the other entry points want.  Strides in bytes
+ * (host arrays of 3; 0 in src_strides repeats, the destination's rows must not overlap).  row_bytes is 16
+ * times a power of two, at most 4096; addresses and strides are multiples of 16 and strides are not
+ * negative, and there are at most 2^30 rows: BLOSSOM_ERR_UNSUPPORTED otherwise, and nothing is copied. */
+int blossom_copy_rows(int32_t batch, int32_t heads, int32_t seq_len, int32_t row_bytes, const void *src,
+                      const int64_t *src_strides /* host */, void *dst,
+                      const int64_t *dst_strides /* host */, blossom_stream_t stream);
+
 /* Synchronises the stream and copies the workspace's device status to *host_out (host): 0 = no
  * device-side error, else a blossom_status.  The workspace holds one status word for the forward
  * (blossom_select_blocks and blossom_attn_fwd clear both words when they start: a new step) and

@@ -29,7 +29,7 @@ EXPORTS = (
     "blossom_device_status", "blossom_status_string", "blossom_version", "blossom_launch_count",
     "blossom_profile_start", "blossom_profile_every", "blossom_profile_stop", "blossom_kernel_name",
     "blossom_debug_switch",
-    "blossom_selftest_wait_timeout",
+    "blossom_selftest_wait_timeout", "blossom_copy_rows",
 )
 
 

@@ -53,6 +53,25 @@ Tensor fresh(at::IntArrayRef sizes, at::ScalarType type, const at::Device &dev) 
   return at::detail::empty_cuda(sizes, type, dev, std::nullopt);
 }
 
+// src's values in `dst` (same sizes, another layout).  Rows in 16-byte pieces go through the library's copy, every
+// other form (types, strides of the last dimension, views that have to be resolved, empty tensors) through PyTorch's.
+Tensor copied(const Tensor &src, Tensor dst) {
+  if (src.is_cuda() && src.dim() == 4 && src.scalar_type() == dst.scalar_type() && src.device() == dst.device() &&
+      src.sizes() == dst.sizes() && src.numel() > 0 && src.stride(3) == 1 && dst.stride(3) == 1 && !src.is_neg() &&
+      !src._is_zerotensor() && src.size(0) <= INT32_MAX && src.size(1) <= INT32_MAX && src.size(2) <= INT32_MAX &&
+      src.size(3) <= 1024) {
+    const int64_t e = src.element_size();
+    const int64_t ss[3] = {src.stride(0) * e, src.stride(1) * e, src.stride(2) * e},
+                  ds[3] = {dst.stride(0) * e, dst.stride(1) * e, dst.stride(2) * e};
+    if (blossom_copy_rows((int32_t)src.size(0), (int32_t)src.size(1), (int32_t)src.size(2), (int32_t)(src.size(3) * e),
+                          src.data_ptr(), ss, dst.data_ptr(), ds,
+                          (blossom_stream_t)c10::cuda::getCurrentCUDAStream(dst.device().index()).stream()) == BLOSSOM_OK)
+      return dst;
+  }
+  return dst.copy_(src);
+}
+Tensor packed(const Tensor &t) { return t.is_contiguous() ? t : copied(t, at::empty(t.sizes(), t.options())); }
+
 std::string failure(const char *where, int rc) {
   return std::string(where) + ": " + blossom_status_string(rc) + " (status " + std::to_string(rc) + ")";
 }
@@ -100,7 +119,7 @@ struct BlossomAttentionBackward : public Node {
     c10::cuda::CUDAGuard guard(q.device());
     Tensor dout = grads[0];
     if (dout.strides() != q.strides() || dout.scalar_type() != q.scalar_type())  // the library wants q's layout
-      dout = like(q).copy_(dout);
+      dout = copied(dout, like(q));
     Tensor dq = like(q), dk = like(k), dv = like(k);
     Tensor dgate = fresh(gate.sizes(), at::kFloat, q.device());
     // The workspace is this call's own and its last user was the training forward (or an earlier
@@ -209,14 +228,14 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
       at::NoGradGuard no_grad;
       // The library addresses every q-shaped buffer with q's strides and every k-shaped one with k's:
       // views that are not dense (a slice of a packed projection) are copied first.
-      if (!(dense(q) && q.stride(3) == 1)) q = q.contiguous();
+      if (!(dense(q) && q.stride(3) == 1)) q = packed(q);
       if (!(dense(k) && k.stride(3) == 1 && k.strides() == v.strides())) {
-        k = k.contiguous();
-        v = v.contiguous();
+        k = packed(k);
+        v = packed(v);
       }
       if (Hkv == H && k.strides() != q.strides()) {
-        k = like(q).copy_(k);
-        v = like(q).copy_(v);
+        k = copied(k, like(q));
+        v = copied(v, like(q));
       }
       if (gate.scalar_type() != at::kFloat || !gate.is_contiguous()) gate = gate.to(at::kFloat).contiguous();
     }
