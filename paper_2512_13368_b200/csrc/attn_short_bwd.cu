@@ -11,9 +11,13 @@
 //   query CTAs  some 16-row tiles of a (batch, head): K, V rows in shared memory, a warp per tile,
 //               dQ += dS K; they also produce d alpha from the fp32 probabilities, and the last of
 //               them to finish adds the partial sums in a fixed order into dgate.
+// With grouped heads and few (batch, key/value head) pairs a cluster of CTAs shares a key tile, each with its part of
+// the heads, and adds dK and dV over the cluster (head_split).
 // Key CTAs come first in the grid, those of the early keys (the most visitors) before the others.
 // Both kinds recompute Delta = rowsum(dO o O_x) of the rows they need: 3 more row reads out of L2
 // instead of a launch.  No gradient is written by more than one warp: no atomics on results.
+#include <cooperative_groups.h>
+
 #include "short_common.cuh"
 
 namespace blossom {
@@ -21,7 +25,8 @@ namespace sh {
 namespace {
 
 struct BwdGeom {
-  int nkey_ctas, nkt;  // key CTAs of the grid; key CTAs per (batch, key/value head)
+  int nkey_ctas, nkt;  // key CTAs of the grid; tiles of 64 keys per (batch, key/value head)
+  int split, heads;    // CTAs of a cluster that share a key tile's heads (1: no clusters); heads of each
   int per, nq;         // tiles per query CTA; query CTAs per (batch, head)
   int o_b, o_rec, o_stage, o_sel;  // byte offsets in shared memory
 };
@@ -83,7 +88,7 @@ __device__ __forceinline__ void query_pairs(bool inL, bool inS, const float (&z)
   for (int e = 0; e < 8; ++e) dal = fmaf(diff[e >> 2][e & 3], dp[e >> 2][e & 3], dal);
 }
 
-template <int D, bool PLAIN>
+template <int D, bool PLAIN, bool SPLIT>
 __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
     Shape s, BwdGeom bg, const __nv_bfloat16 *__restrict__ q, const __nv_bfloat16 *__restrict__ k,
     const __nv_bfloat16 *__restrict__ v, const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
@@ -124,7 +129,8 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
   if ((int)blockIdx.x < bg.nkey_ctas) {
     // ============================================================ key CTA: dK, dV of 64 keys
     float4 *rec = reinterpret_cast<float4 *>(smem + bg.o_rec);  // {nl_lt, -Delta_lt, nl_st, -Delta_st} per query
-    const int kt = (int)blockIdx.x / nU, uk = (int)blockIdx.x % nU, n = uk / s.Hkv, hk = uk % s.Hkv;
+    const int rank = SPLIT ? (int)blockIdx.x % bg.split : 0, kc = SPLIT ? (int)blockIdx.x / bg.split : (int)blockIdx.x;
+    const int kt = kc / nU, uk = kc % nU, n = uk / s.Hkv, hk = uk % s.Hkv;
     int len = seq_lens ? seq_lens[n] : s.L;
     len = min(max(len, 0), s.L);
     const int pad0 = s.L - len;
@@ -143,8 +149,8 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
       load_a_rows<D>(k + koff, s.ksl, p0, pad0, s.L, lane, ka);
       load_a_rows<D>(v + koff, s.ksl, p0, pad0, s.L, lane, va);
       uint64_t setL = 0ull, setS = 0ull;
-      for (int hg = 0; hg < s.G; ++hg) {
-        const int h = hk * s.G + hg;
+      for (int hg = 0; hg < (SPLIT ? bg.heads : s.G); ++hg) {
+        const int h = hk * s.G + (SPLIT ? rank * bg.heads : 0) + hg;
         const int64_t off = row_offset(s, n, h, 0);
         if (hg) __syncthreads();  // the previous head's rows are no longer read
         stage_rows<D>(ta, q + off, s.sl, q_lo, q_hi, pad0, s.L, tid, kThreads);
@@ -228,6 +234,44 @@ __global__ void __launch_bounds__(128, D == 32 ? 5 : 3) bwd_short_kernel(
           product_nn<D>(pa, ta_a + co + onn, ak);
         }
       }
+    }
+    if (SPLIT) {  // rank 0 adds dV over the cluster and writes it, rank 1 dK; in rank order
+      if (cta_live) {    // (the same for all of a cluster)
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        float4 *own = reinterpret_cast<float4 *>(smem) + tid;
+        __syncthreads();  // the last head's rows are no longer read
+#pragma unroll
+        for (int e = 0; e < D / 8; ++e) {
+          own[e * kThreads] = make_float4(av[e][0], av[e][1], av[e][2], av[e][3]);
+          own[(D / 8 + e) * kThreads] = make_float4(ak[e][0], ak[e][1], ak[e][2], ak[e][3]);
+        }
+        cluster.sync();
+        if (rank < 2) {
+#pragma unroll
+          for (int e = 0; e < D / 8; ++e)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) av[e][i] = 0.f;
+#pragma unroll 1
+          for (int r = 0; r < bg.split; ++r) {
+            const float4 *o = cluster.map_shared_rank(own, r) + rank * (D / 8) * kThreads;
+#pragma unroll
+            for (int e = 0; e < D / 8; ++e) {
+              const float4 x = o[e * kThreads];
+              av[e][0] += x.x;
+              av[e][1] += x.y;
+              av[e][2] += x.z;
+              av[e][3] += x.w;
+            }
+          }
+        }
+        cluster.sync();  // nobody leaves while its sums are being read
+      }
+      if (rank < 2 && p0 < s.L) {
+        const float f = rank ? s.scale : 1.f;
+        store_rows<D>((rank ? dk : dv) + koff, s.ksl, p0, s.L, av, f, f, stage, lane);
+      }
+      return;
     }
     if (p0 < s.L) {
       store_rows<D>(dv + koff, s.ksl, p0, s.L, av, 1.f, 1.f, stage, lane);
@@ -380,6 +424,21 @@ bool bwd_short_supported(const Shape &s, int dtype) {
   return s.L <= (s.D == 32 ? 300 : 128) || rows <= (s.L * s.D <= 25000 ? 32768 : 8192);
 }
 
+// CTAs of a cluster that share the heads of a key tile.  A key CTA with all heads of a group is a chain (stage, wait,
+// walk, a head after the other) that sets the time of a small batch: with four heads on one at L 200, D 32 the backward
+// took 46 us at B 4 and 54 at B 16, against 83 at B 128; split, forward + backward 68 -> 41, 84 -> 49 (B 32: 88 -> 64).
+// The chip full, the copies of the fixed part (selection, K and V rows, the sums over the cluster) cost 3 - 17 %: B 128
+// 141 -> 146 with two CTAs and 163 with four.  The lines, from 178 shapes (two to eight heads a group, L 50 - 300,
+// B 2 - 256): as many CTAs as divide the heads while (batch, key/value head) pairs x CTAs stay below them.
+static int head_split(const Shape &s) {
+  const int64_t units = (int64_t)s.B * s.Hkv;
+  for (int split = 8; split > 1; split /= 2) {
+    const int line = split == s.G ? (s.D == 32 ? 256 : 192) : (s.D == 32 ? 384 : 256);
+    if (s.G % split == 0 && units * split <= line) return split;
+  }
+  return 1;
+}
+
 template <int D>
 static int launch_t(const Shape &s, const void *q, const void *k, const void *v, const float *gate, const int32_t *seq_lens,
                     const int32_t *idx, const void *out_lt, const void *out_st, const float *lse, const void *dout, void *dq,
@@ -388,23 +447,31 @@ static int launch_t(const Shape &s, const void *q, const void *k, const void *v,
   BwdGeom bg;
   const int ntiles = (s.L + 15) / 16, rows = ntiles * 16;
   bg.nkt = (s.L + 63) / 64;
-  bg.nkey_ctas = s.B * s.Hkv * bg.nkt;
+  bg.split = head_split(s);
+  bg.heads = s.G / bg.split;
+  bg.nkey_ctas = s.B * s.Hkv * bg.nkt * bg.split;
   bg.per = s.B * s.H >= 296 ? 8 : 4;
   bg.nq = (ntiles + bg.per - 1) / bg.per;
   bg.per = (ntiles + bg.nq - 1) / bg.nq;  // of equal size
   bg.o_b = rows * D * 2;
   bg.o_rec = 2 * rows * D * 2;
   bg.o_stage = bg.o_rec + rows * 16;
+  const int sums = 2 * (D / 8) * 128 * 16;  // a CTA's dV and dK, over the tiles
+  if (bg.split > 1 && bg.o_stage < sums) bg.o_stage = sums;
   bg.o_sel = bg.o_stage + 4 * 16 * D * 2;
   const int smem = bg.o_sel + 128;
   const bool plain = s.causal && s.stis_mode == 0;
-  auto kern = plain ? bwd_short_kernel<D, true> : bwd_short_kernel<D, false>;
+  auto kern = bg.split > 1 ? (plain ? bwd_short_kernel<D, true, true> : bwd_short_kernel<D, false, true>)
+                           : (plain ? bwd_short_kernel<D, true, false> : bwd_short_kernel<D, false, false>);
   if (!allow_smem(kern, (size_t)smem)) return BLOSSOM_ERR_CUDA;
   LaunchScope ls(K_BWD_SHORT, st);
-  if (launch_chained(kern, dim3((unsigned)(bg.nkey_ctas + s.B * s.H * bg.nq)), dim3(128), (size_t)smem, st, s, bg,
-                     (const bf *)q, (const bf *)k, (const bf *)v, gate, seq_lens, idx, (const bf *)out_lt,
-                     (const bf *)out_st, lse, (const bf *)dout, (bf *)dq, (bf *)dk, (bf *)dv, dgate, ws.dalpha,
-                     ws.status + kCounterWord) != cudaSuccess)
+  const dim3 grid((unsigned)(bg.nkey_ctas + s.B * s.H * bg.nq));
+  auto launch = [&](auto... args) {
+    return bg.split > 1 ? launch_chained_cluster(kern, grid, dim3(128), (size_t)smem, (unsigned)bg.split, st, args...)
+                        : launch_chained(kern, grid, dim3(128), (size_t)smem, st, args...);
+  };
+  if (launch(s, bg, (const bf *)q, (const bf *)k, (const bf *)v, gate, seq_lens, idx, (const bf *)out_lt, (const bf *)out_st,
+             lse, (const bf *)dout, (bf *)dq, (bf *)dk, (bf *)dv, dgate, ws.dalpha, ws.status + kCounterWord) != cudaSuccess)
     return BLOSSOM_ERR_CUDA;
   return BLOSSOM_OK;
 }
