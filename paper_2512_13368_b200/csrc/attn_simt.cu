@@ -566,21 +566,21 @@ __global__ void __launch_bounds__(256) gate_grad_kernel(Shape s, const float *__
   }
 }
 
-// Gradient of F_o's parameters (input-dependent gate): the per-query-block partial sums added
-// over batch entries and query blocks in a fixed order.  One warp per (head, parameter): lane i
+// Gradient of F_o's parameters (input-dependent gate): the partial sums ([B][H][M][2 D + 1], `parts` of the M places
+// of a (batch, head) in use) added over batch entries and parts in a fixed order.  One warp per (head, parameter): lane i
 // adds the entries i, i + 32, ... in ascending order, then a fixed shuffle tree joins the lanes.
-__global__ void __launch_bounds__(256) gate_param_grad_kernel(Shape s, const double *__restrict__ part,
+__global__ void __launch_bounds__(256) gate_param_grad_kernel(Shape s, const double *__restrict__ part, int parts,
                                                               float *__restrict__ dgate, int beside) {
   if (beside) grid_release();  // beside the kernel before it, which has waited for what this one reads
   else grid_chain_enter();
   const int GW = 2 * s.D + 1;
   const int w = (int)blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w < s.H * GW) {
-    const int h = w / GW, d = w % GW, n_entries = s.B * s.M;
+    const int h = w / GW, d = w % GW, n_entries = s.B * parts;
     double a = 0.0;
 #pragma unroll 16
     for (int e = lane; e < n_entries; e += 32) {
-      const int n = e / s.M, qb = e % s.M;
+      const int n = e / parts, qb = e % parts;
       a += part[(((int64_t)n * s.H + h) * s.M + qb) * GW + d];
     }
 #pragma unroll
@@ -634,7 +634,7 @@ int launch_bwd_t(const Shape &s, const T *q, const T *k, const T *v, const float
   }
   if (s.gate_mode) {
     LaunchScope ls(K_GATE_GRAD, st);
-    gate_param_grad_kernel<<<(unsigned)((s.H * (2 * s.D + 1) + 7) / 8), 256, 0, st>>>(s, ws.dgate_part, dgate, 0);
+    gate_param_grad_kernel<<<(unsigned)((s.H * (2 * s.D + 1) + 7) / 8), 256, 0, st>>>(s, ws.dgate_part, s.M, dgate, 0);
     return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
   }
   return launch_gate_grad(s, gate, ws, dgate, st);
@@ -646,7 +646,7 @@ int launch_gate_param_grad(const Shape &s, const Workspace &ws, float *dgate, cu
   {
     LaunchScope ls(K_GATE_GRAD, st);
     launch_chained(gate_param_grad_kernel, dim3((unsigned)((s.H * (2 * s.D + 1) + 7) / 8)), dim3(256), 0, st, s,
-                   (const double *)ws.dgate_part, dgate, beside);
+                   (const double *)ws.dgate_part, (s.L + gate_prep_rows(s) - 1) / gate_prep_rows(s), dgate, beside);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

@@ -57,7 +57,7 @@ struct Workspace {
   void *rope_table;     // [L][D / 2] (cos, sin) in double precision (rope_theta > 0)
   void *q_rot, *k_rot;  // rotated copies of q and k (rope_theta > 0), laid out with the originals' strides
   float *gate_ac;    // [2][B][H][L]  input-dependent gate: alpha_t and c_t of every row (backward)
-  double *dgate_part;// [B][H][M][2 D + 1]  per query block partial of the gradient of F_o's parameters
+  double *dgate_part;// [B][H][M][2 D + 1]  partials of the gradient of F_o's parameters, one per query block or fewer
   // input-dependent gate on the tensor-core kernels (bf16 only): the two branches' upstream
   // tensors, the second pass's gradients (added to the first pass's afterwards), its records, and
   // the branch outputs of a forward call that does not return them; q-shaped ones laid out with
@@ -241,6 +241,17 @@ __device__ __forceinline__ bool st_ranges_touch(const Shape &s, int t0, int t1, 
   const int dmax = stis_block_of(s, t1) - stis_block_of(s, p0);
   const int dmin = max(1, stis_block_of(s, t0) - stis_block_of(s, p1));
   return dmax >= dmin && (1 << (31 - __clz(dmax))) >= dmin;  // largest power of two <= dmax
+}
+
+// Rows that one CTA of the tensor-core path's gate pre-pass takes (gate_prep_kernel, which leaves a partial sum of the
+// parameters' gradient per CTA): up to four passes over its 256 threads' rows while there are CTAs for two per SM (eight
+// passes: B 64, H 4, L 900, D 64 43 -> 41 us, but B 64, L 200 12.7 -> 15.2).  Not less than a query block, so that the
+// partials fit their place in the workspace.
+inline int gate_prep_rows(const Shape &s) {
+  const int rpb = 2048 / s.D;
+  const int64_t tiles = (int64_t)s.B * s.H * ((s.L + rpb - 1) / rpb), it = tiles / (2 * 148);
+  const int rows = rpb * (int)(it < 1 ? 1 : it > 4 ? 4 : it);
+  return rows > s.Bk ? rows : s.Bk;
 }
 
 // launchers (one translation unit each)

@@ -92,7 +92,11 @@ __global__ void __launch_bounds__(256) gate_mix_kernel(Shape s, const float *__r
 }
 
 // ---- backward pre-pass --------------------------------------------------------------------------
-// One CTA per (batch, head, query block).  Per row: alpha_t, c_t, the two upstream tensors (bf16,
+// One CTA per (batch, head, gate_prep_rows rows).  Bound by the tail of a CTA (the double-precision sums of the
+// parameters' gradient, 2 D + 1 of them, over lanes and warps) and then by memory: with a CTA per query block a thread
+// had one row for each such tail, and 129 partial sums per 32 rows went to memory and back (B 16, H 4, L 900, D 64
+// 19.0 us and 8.5 in the kernel that adds the partials; four rows a thread, the next loaded ahead, 13.3 and 4.2; B 64
+// 72 and 40 -> 43 and 13; three CTAs an SM instead of two spill: 19.1).  Per row: alpha_t, c_t, the two upstream tensors (bf16,
 // zeros in padded rows: the attention kernels multiply them by exact zeros, which must stay
 // zeros), the records of the two passes (layout of bwd_prep_kernel; Delta of a pass is taken with
 // the rounded tensor the pass multiplies with, and the branch a pass leaves out gets the exponent
@@ -104,13 +108,13 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
                                                         const float *__restrict__ lse, const bf *__restrict__ dout,
                                                         bf *__restrict__ g_lt, bf *__restrict__ g_st,
                                                         float4 *__restrict__ rec_lt, float4 *__restrict__ rec_st,
-                                                        double *__restrict__ dgate_part, int Lpad,
+                                                        double *__restrict__ dgate_part, int Lpad, int rows, int parts,
                                                         int32_t *__restrict__ status) {
   grid_chain_enter();
   if (blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;  // the backward's status words
   constexpr int LPR = D / 8, RPB = 256 / LPR, GW = 2 * D + 1;
   __shared__ double red[8][GW];
-  const int u = blockIdx.x / s.M, qb = blockIdx.x % s.M, n = u / s.H, h = u % s.H;
+  const int u = blockIdx.x / parts, qb = blockIdx.x % parts, n = u / s.H, h = u % s.H;
   const int lr = threadIdx.x / LPR, ch = threadIdx.x % LPR;
   int len = seq_lens ? seq_lens[n] : s.L;
   len = min(max(len, 0), s.L);
@@ -124,20 +128,29 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
   double acc[16], accB = 0.0;  // eight columns of O_lt, eight of O_st
 #pragma unroll
   for (int e = 0; e < 16; ++e) acc[e] = 0.0;
-  // the last query block also writes the (zero) records of the rows that pad L to a multiple of 64
-  const int t_end = qb == s.M - 1 ? Lpad : min((qb + 1) * s.Bk, s.L);
-  for (int t0 = qb * s.Bk; t0 < t_end; t0 += RPB) {
+  // the last CTA of a head also writes the (zero) records of the rows that pad L to a multiple of 64
+  const int t_end = qb == parts - 1 ? Lpad : (qb + 1) * rows;
+  uint4 next[3];  // the next row's pieces of dO, O_lt, O_st, loaded a row ahead
+  auto load = [&](int t) {
+    next[0] = next[1] = next[2] = make_uint4(0u, 0u, 0u, 0u);
+    if (t >= pad0 && t < min(t_end, s.L)) {
+      const int64_t off = row_offset(s, n, h, t) + ch * 8;
+      next[0] = *reinterpret_cast<const uint4 *>(dout + off);
+      next[1] = *reinterpret_cast<const uint4 *>(out_lt + off);
+      next[2] = *reinterpret_cast<const uint4 *>(out_st + off);
+    }
+  };
+  load(qb * rows + lr);
+#pragma unroll 1
+  for (int t0 = qb * rows; t0 < t_end; t0 += RPB) {
     const int t = t0 + lr;
     const bool in_rec = t < t_end, row = in_rec && t < s.L, valid = row && t >= pad0;
     const int64_t off = row ? row_offset(s, n, h, t) + ch * 8 : 0;
     float g[8], ol[8], os[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) g[e] = ol[e] = os[e] = 0.f;
-    if (valid) {
-      unpack8(*reinterpret_cast<const uint4 *>(dout + off), g);
-      unpack8(*reinterpret_cast<const uint4 *>(out_lt + off), ol);
-      unpack8(*reinterpret_cast<const uint4 *>(out_st + off), os);
-    }
+    unpack8(next[0], g);
+    unpack8(next[1], ol);
+    unpack8(next[2], os);
+    load(t + RPB);
     float aL = 0.f, aS = 0.f, woL = 0.f, woS = 0.f;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -199,7 +212,7 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
     }
   }
   // The warp's rows: lanes that share columns exchange halves, each ends with 16 LPR / 32 sums (all of every
-  // row's in shared memory and added there took 33 KB a CTA and 27 us for B 16, H 4, L 900, D 64: now 23 us).
+  // row's in shared memory and added there: 33 KB a CTA).
   int at = ch * 8;
 #pragma unroll
   for (int o = LPR, m = 8; o < 32; o <<= 1, m >>= 1) {
@@ -249,10 +262,11 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
   const int Lpad = (s.L + 63) / 64 * 64;
   {
     LaunchScope ls(K_BWD_PREP, st);
-    const unsigned grid = (unsigned)(s.B * s.H) * (unsigned)s.M;
+    const int prows = gate_prep_rows(s), parts = (s.L + prows - 1) / prows;
+    const unsigned grid = (unsigned)(s.B * s.H) * (unsigned)parts;
     launch_chained(s.D == 32 ? gate_prep_kernel<32> : gate_prep_kernel<64>, dim3(grid), dim3(256), 0, st, s, gate, seq_lens,
                    (const bf *)out_lt, (const bf *)out_st, lse, (const bf *)dout, (bf *)ws.gate_glt, (bf *)ws.gate_gst,
-                   ws.qstats, ws.qstats2, ws.dgate_part, Lpad, ws.status_bwd);
+                   ws.qstats, ws.qstats2, ws.dgate_part, Lpad, prows, parts, ws.status_bwd);
     if (cudaGetLastError() != cudaSuccess) return BLOSSOM_ERR_CUDA;
   }
   // The lists of both passes in one launch; the second pass adds to the first one's gradients as it writes them
