@@ -148,9 +148,25 @@ __device__ __noinline__ Columns exact_columns(const T *q, int64_t sh, int64_t sl
   return out;
 }
 
+// A head's share of a row's scores: pr (+)= e inv over the candidates, four loads of each ahead of the stores (the compiler
+// does not move a load before a store to a table that might be the same).
+__device__ __forceinline__ void add_head(int hg, int n, const float *e, float inv, float *pr) {
+  for (int c = 0; c < n; c += 4) {
+    float x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x[i] = c + i < n ? e[c + i] : 0.f;
+      y[i] = hg && c + i < n ? pr[c + i] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (c + i < n) pr[c + i] = hg ? fmaf(x[i], inv, y[i]) : x[i] * inv;
+  }
+}
+
 // PQ: one selection per query position.
 template <typename T, int D, bool PQ>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_kernel(
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) score_rows_kernel(
     Shape sh, SelGeom g, RowsGeom rg, const T *__restrict__ q, const float *__restrict__ mean32,
     const float *__restrict__ norm, const double *__restrict__ mean, const int32_t *__restrict__ seq_lens,
     int32_t *__restrict__ idx, int32_t *__restrict__ worklist, int32_t *__restrict__ work_count) {
@@ -262,6 +278,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
         else cs[3] += a;
       }
     };
+    uint32_t qnext[kMma && PQ ? D / 16 : 1][4];  // (PQ) the next 16 rows' queries, a product loop ahead: few warps a scheduler
+    if constexpr (kMma && PQ)
+      sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G, 0), sh.sl, row0 + warp * 32, pad0, sh.L, lane, qnext);
 #pragma unroll 1
     for (int hg = 0; hg < sh.G; ++hg) {  // the heads of the group in ascending order (Eq. 12)
       if constexpr (kMma) {
@@ -271,7 +290,17 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
         for (int mt = 0; mt < 2; ++mt) {  // 16 rows at a time
           const int tm = row0 + warp * 32 + 16 * mt;
           uint32_t qa[D / 16][4];
-          sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg, 0), sh.sl, tm, pad0, sh.L, lane, qa);
+          if constexpr (PQ) {
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) qa[k][e] = qnext[k][e];
+            if (mt == 0 || hg + 1 < sh.G)
+              sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg + mt, 0), sh.sl, row0 + warp * 32 + 16 * (1 - mt), pad0,
+                                 sh.L, lane, qnext);
+          } else {
+            sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg, 0), sh.sl, tm, pad0, sh.L, lane, qa);
+          }
           float ref[2] = {0.f, 0.f}, den[2] = {0.f, 0.f}, qh[2];
 #pragma unroll
           for (int k = 0; k < D / 16; ++k)
@@ -334,7 +363,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
         if (PQ && sh.G > 1) {
           float *pr = pt + lane * rg.pitch;
           const float inv = inv_s[warp][lane];
-          for (int c = 0; c < nc_warp; ++c) pr[c] = hg == 0 ? er[c] * inv : fmaf(er[c], inv, pr[c]);
+          add_head(hg, nc_warp, er, inv, pr);
           __syncwarp();
         }
       } else {
@@ -381,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
       if (PQ) {
         if (sh.G > 1) {
           float *pr = pt + lane * rg.pitch;
-          for (int c = 0; c < nc_warp; ++c) pr[c] = hg == 0 ? er[c] * inv : fmaf(er[c], inv, pr[c]);
+          add_head(hg, nc_warp, er, inv, pr);
         }
       } else {
         inv_s[warp][lane] = inv;
@@ -427,26 +456,34 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
         float *S = sh.G > 1 ? pt + lane * rg.pitch : et + lane * rg.pitch;
         if (!g.plain) {
           float *o = sh.G > 1 ? et + lane * rg.pitch : pt + lane * rg.pitch;  // the table that is free
-          for (int j = jmin; j < b; ++j) {
-            float a = 0.f;
+          for (int j = jmin; j < b; j += 4) {  // (four at a time, as in add_head)
+            float a[4] = {0.f, 0.f, 0.f, 0.f};
             for (int m = 0; m < g.rs; ++m)
-              for (int e = 0; e < g.rl; ++e) {
-                const int i = g.rs * j - m - e - cmin;
-                if (i >= 0 && i < nc) a += S[i];
-              }
-            o[j - jmin] = a;
+              for (int e = 0; e < g.rl; ++e)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                  const int i = g.rs * (j + y) - m - e - cmin;
+                  if (i >= 0 && i < nc) a[y] += S[i];
+                }
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+              if (j + y < b) o[j + y - jmin] = a[y];
           }
           S = o;
         }
         const int ns = b - jmin;
         float kept = 0.f, dropped = 0.f;
-        for (int k = 0; k <= want; ++k) {  // the want best, then the best that is left out
+        // The want best, then the best that is left out.  A chain of loads per lane and few warps a scheduler: what is
+        // taken is overwritten.  (A test of its bit per score and one load after the other: with add_head's and Eq. 11's
+        // loads one by one too 36.6 us at B 8, 8 heads on 2, L 1500, D 64, 72.7 at B 64; now 30.9 and 64.6, and 28.1 and
+        // 58.0 with the queries loaded ahead.)
+        for (int k = 0; k <= want; ++k) {
           float best = -1.f;
           int bi = 0;
+#pragma unroll 8
           for (int j = 0; j < ns; ++j) {
-            const uint32_t tk = j < 64 ? (j < 32 ? taken[0] : taken[1]) : (j < 96 ? taken[2] : taken[3]);
             const float x = S[j];
-            if (x > best && !((tk >> (j & 31)) & 1u)) {
+            if (x > best) {
               best = x;
               bi = j;
             }
@@ -455,6 +492,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 5 : 4) score_rows_k
             dropped = best;
           } else {
             kept = best;
+            S[bi] = -1.f;
             const uint32_t bit = 1u << (bi & 31);
             if (bi < 32) taken[0] |= bit;
             else if (bi < 64) taken[1] |= bit;
