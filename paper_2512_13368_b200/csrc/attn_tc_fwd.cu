@@ -33,9 +33,9 @@
 // never exchange anything inside the loop; the two partial results are merged, exactly as two
 // halves of an online softmax, when a phase ends.  Sixteen softmax warps per SM instead of eight
 // hide the latency of a thread's dependent chain (load, maximum, exponentials, store).
-// Warps 8, 9, 10 stay converged and one elected lane of each loads K/V tiles (TMA), issues
-// S = Q K^T, and issues the two O += P V products with P read from tensor memory.  Warp 11 stores the
-// finished rows and fetches the next tile's lists and queries.
+// Warps 8 and 9 stay converged; one elected lane of the first loads K/V tiles (TMA), one of the second issues
+// S = Q K^T and the two O += P V products with P read from tensor memory.  Warp 11 stores the
+// finished rows and fetches the next tile's lists and queries (warp 10 is spare).
 //
 // Tensor memory (256 columns): two logits / probability buffers [0,64) [64,128), O_A [128,128+D),
 // O_B [192,192+D).  Item i uses buffer i % 2: S(i) lands there as fp32, a softmax thread reads its
