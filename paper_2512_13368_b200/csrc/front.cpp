@@ -53,24 +53,29 @@ Tensor fresh(at::IntArrayRef sizes, at::ScalarType type, const at::Device &dev) 
   return at::detail::empty_cuda(sizes, type, dev, std::nullopt);
 }
 
-// src's values in `dst` (same sizes, another layout).  Rows in 16-byte pieces go through the library's copy, every
-// other form (types, strides of the last dimension, views that have to be resolved, empty tensors) through PyTorch's.
-Tensor copied(const Tensor &src, Tensor dst) {
-  if (src.is_cuda() && src.dim() == 4 && src.scalar_type() == dst.scalar_type() && src.device() == dst.device() &&
-      src.sizes() == dst.sizes() && src.numel() > 0 && src.stride(3) == 1 && dst.stride(3) == 1 && !src.is_neg() &&
-      !src._is_zerotensor() && src.size(0) <= INT32_MAX && src.size(1) <= INT32_MAX && src.size(2) <= INT32_MAX &&
-      src.size(3) <= 1024) {
-    const int64_t e = src.element_size();
-    const int64_t ss[3] = {src.stride(0) * e, src.stride(1) * e, src.stride(2) * e},
-                  ds[3] = {dst.stride(0) * e, dst.stride(1) * e, dst.stride(2) * e};
-    if (blossom_copy_rows((int32_t)src.size(0), (int32_t)src.size(1), (int32_t)src.size(2), (int32_t)(src.size(3) * e),
-                          src.data_ptr(), ss, dst.data_ptr(), ds,
-                          (blossom_stream_t)c10::cuda::getCurrentCUDAStream(dst.device().index()).stream()) == BLOSSOM_OK)
-      return dst;
-  }
-  return dst.copy_(src);
+// src's values in `dst` (same sizes, another layout) by the library's copy of rows in 16-byte pieces.  False, and
+// nothing done, for every other form: types, strides of the last dimension, views that have to be resolved, tensors
+// without memory of their own, empty ones.
+bool copy_rows(const Tensor &src, const Tensor &dst) {
+  if (!src.is_cuda() || !src.has_storage() || src.unsafeGetTensorImpl()->is_python_dispatch() || src.dim() != 4 ||
+      src.scalar_type() != dst.scalar_type() || src.device() != dst.device() || src.sizes() != dst.sizes() ||
+      src.numel() == 0 || src.stride(3) != 1 || dst.stride(3) != 1 || src.is_neg() || src._is_zerotensor() ||
+      src.size(0) > INT32_MAX || src.size(1) > INT32_MAX || src.size(2) > INT32_MAX || src.size(3) > 1024)
+    return false;
+  const int64_t e = src.element_size();
+  const int64_t ss[3] = {src.stride(0) * e, src.stride(1) * e, src.stride(2) * e},
+                ds[3] = {dst.stride(0) * e, dst.stride(1) * e, dst.stride(2) * e};
+  return blossom_copy_rows((int32_t)src.size(0), (int32_t)src.size(1), (int32_t)src.size(2), (int32_t)(src.size(3) * e),
+                           src.data_ptr(), ss, dst.data_ptr(), ds,
+                           (blossom_stream_t)c10::cuda::getCurrentCUDAStream(dst.device().index()).stream()) == BLOSSOM_OK;
 }
-Tensor packed(const Tensor &t) { return t.is_contiguous() ? t : copied(t, at::empty(t.sizes(), t.options())); }
+Tensor copied(const Tensor &src, const Tensor &dst) { return copy_rows(src, dst) ? dst : dst.copy_(src); }
+Tensor packed(const Tensor &t) {
+  if (t.is_contiguous() || !t.is_cuda() || !t.has_storage() || t.unsafeGetTensorImpl()->is_python_dispatch())
+    return t.contiguous();
+  const Tensor dst = at::empty(t.sizes(), t.options());
+  return copy_rows(t, dst) ? dst : t.contiguous();
+}
 
 std::string failure(const char *where, int rc) {
   return std::string(where) + ": " + blossom_status_string(rc) + " (status " + std::to_string(rc) + ")";

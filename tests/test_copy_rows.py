@@ -50,3 +50,28 @@ def test_every_order_of_the_dimensions(B, H, L, D):
     dst = torch.empty_like(x)
     assert copy_rows(x[:1, :, :1].expand(B, H, L, D), dst) == 0         # strides of zero repeat
     assert torch.equal(dst, x[:1, :, :1].expand(B, H, L, D))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,D", [("bf16", 32), ("fp32", 64)])
+def test_gradients_that_are_not_plain_memory(dtype, D):
+    """Negated views, zero tensors, misaligned and repeated rows: what their plain copies give."""
+    import torch
+    from paper_2512_13368_b200.autograd import blossom_attention
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(D)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda").to(dt)  # noqa: E731
+    B, H, L = 2, 2, 40
+    q, k, v = (mk(B, H, L, D).requires_grad_(True) for _ in range(3))
+    gate = torch.randn((H, 2), generator=g, device="cuda").requires_grad_(True)
+    out = blossom_attention(q, k, v, gate, 16, 2, 9)
+    grads = lambda d: torch.autograd.grad(out, (q, k, v, gate), d, retain_graph=True)  # noqa: E731
+    x = mk(B, L, H, D).transpose(1, 2)
+    flat = torch.zeros(B * L * H * D + 1, dtype=dt, device="cuda")
+    odd = flat[1:].view(B, L, H, D).transpose(1, 2)      # rows that start off a 16-byte boundary
+    odd.copy_(x)
+    for d in (torch._neg_view(x), torch._efficientzerotensor((B, L, H, D), dtype=dt, device="cuda").transpose(1, 2),
+              odd, x[:, :, :1].expand(B, H, L, D)):
+        plain = torch.empty(B, H, L, D, dtype=dt, device="cuda").copy_(d)
+        for a, b in zip(grads(plain), grads(d)):
+            assert torch.equal(a, b)
