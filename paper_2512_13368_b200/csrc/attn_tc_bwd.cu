@@ -1015,10 +1015,15 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     LaunchScope ls(K_BWD_DKDV_TC, st);
     // Grouped heads: a CTA walks its tile list once per head, so with few CTAs the one with the first keys
     // is the kernel's time (170 us at B 8, 8 heads on 2, L 1500, 192 CTAs): the heads are split over clusters
-    // while two waves of CTAs are not full.
+    // of 2 and 4 while SMs are idle or a CTA's walk (key tiles times heads) is long against what a CTA costs
+    // outside it.  The line from 100 shapes (two and four heads a group, L 450 - 1400, 150 - 580 CTAs), us with / without
+    // the next split at D 64: four heads, L 450, 312 CTAs 47 / 51, 400 63 / 52; L 700 396 CTAs 57 / 66, 576 84 / 72; two
+    // heads left, L 450, 192 CTAs 25 / 26, 304 39 / 32; L 900 320 CTAs 46 / 46, 512 65 / 48; L 1400 484 CTAs 51 / 57.
     const unsigned ctas = (unsigned)nST * (unsigned)(s.B * s.Hkv);
     unsigned hs = 1;
-    while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < 592) hs *= 2;
+    while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < 592 &&
+           (ctas * hs < 148 || ctas * hs <= (D == 64 ? 20u : 24u) * (unsigned)nST * ((unsigned)s.G / hs)))
+      hs *= 2;
     const dim3 grid_k((ctas + (dgate_here ? 1 : 0)) * hs);
     if (hs > 1)
       launch_chained_cluster(kern_kv, grid_k, dim3(kKvThreads), smem_kv, hs, st, q64, k128, v128, g64, s, seq_lens,
