@@ -58,6 +58,8 @@
 // (tc_common.cuh); the softmax warps, which meet at named barriers, agree on every tile they start.
 #include "tc_common.cuh"
 
+#include <cfloat>
+
 namespace blossom {
 namespace tc {
 namespace {
@@ -357,7 +359,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     const int r = quarter * 32 + lane, g = r / s.Bk;
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const uint32_t acc_own = (grp ? tmem_ob : tmem_oa) + lane_off;
-    const float sc2 = s.scale * kLog2e;
+    // (not zero, which a scale among the denormals is flushed to: a hidden logit, -infinity, times it has to stay so)
+    const float sc2 = fmaxf(s.scale * kLog2e, FLT_MIN);
     int it = 0;  // items of the tiles before
     for (int k = 0;; ++k) {
       if (warp == 0) {  // one warp decides for all: the named barriers below need every one of them
