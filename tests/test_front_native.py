@@ -197,3 +197,43 @@ def test_every_layout_gives_what_the_dense_tensors_give():
     k1, d1 = mk(1, 1, L, D).expand(B, H, L, D), mk(1, 1, 1, D).expand(B, H, L, D)   # (strides of zero)
     for y, z in zip(step(q, k1.contiguous(), v, d1.contiguous()), step(q, k1, v, d1)):
         assert torch.equal(y, z)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,L,D", [("bf16", 70, 32), ("bf16", 450, 64), ("fp32", 70, 64)])
+def test_negated_views_and_zero_tensors_in_a_layout_that_needs_no_copy(dtype, L, D):
+    """Inputs and gradients that are dense, in q's own layout, but not plain memory: what plain copies give."""
+    import torch
+    from paper_2512_13368_b200.autograd import blossom_attention
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda *s: torch.randn(s, generator=g, device="cuda")  # noqa: E731
+    B, H = 2, 3
+    layouts = (lambda x: x, lambda x: x.transpose(1, 2).contiguous().transpose(1, 2))
+    for layout in layouts:
+        t = {n: layout(mk(B, H, L, D).to(dt)) for n in ("q", "k", "v", "dout")}
+        t["gate"], t["phi"] = mk(H, 2), mk(16)
+        t["lens"] = torch.tensor([L, L // 3], dtype=torch.int32, device="cuda")
+
+        def step(a):
+            leaves = [a[n].detach().requires_grad_(True) for n in ("q", "k", "v", "gate")]
+            out, idx = blossom_attention(*leaves, 16, 3, 9, seq_lens=a["lens"], phi_logits=a["phi"], return_indices=True)
+            with torch.no_grad():
+                alone = blossom_attention(*(a[n] for n in ("q", "k", "v", "gate")), 16, 3, 9, seq_lens=a["lens"],
+                                          phi_logits=a["phi"])
+            return [out.detach(), idx, alone] + list(torch.autograd.grad(out, leaves, a["dout"]))
+
+        want = step(t)
+        for n, x in t.items():
+            neg = torch._neg_view(-x)
+            assert neg.is_neg() and torch.equal(neg, x) and neg.stride() == x.stride()
+            for a, b in zip(want, step(dict(t, **{n: neg}))):
+                assert torch.equal(a, b), n
+            if n in ("lens", "phi"):
+                continue
+            zero = torch._efficientzerotensor(x.shape, dtype=x.dtype, device="cuda")
+            if n != "gate" and layout is not layouts[0]:
+                zero = torch._efficientzerotensor((B, L, H, D), dtype=dt, device="cuda").transpose(1, 2)
+            assert zero._is_zerotensor()
+            for a, b in zip(step(dict(t, **{n: torch.zeros_like(x)})), step(dict(t, **{n: zero}))):
+                assert torch.equal(a, b), n
