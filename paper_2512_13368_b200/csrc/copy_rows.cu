@@ -64,8 +64,8 @@ extern "C" int blossom_copy_rows(int32_t B, int32_t H, int32_t L, int32_t row_by
   if ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) return BLOSSOM_ERR_UNSUPPORTED;
   for (int i = 0; i < 3; ++i)
     if (src_strides[i] < 0 || dst_strides[i] < 0 || ((src_strides[i] | dst_strides[i]) & 15)) return BLOSSOM_ERR_UNSUPPORTED;
-  const int64_t rows = (int64_t)B * H * L;
-  if (rows > (int64_t)1 << 30) return BLOSSOM_ERR_UNSUPPORTED;  // (row numbers in 32 bits, the last CTA's too)
+  const int64_t most = (int64_t)1 << 30, units = (int64_t)B * H, rows = units * L;  // (row numbers in 32 bits, the last CTA's too)
+  if (units > most || rows > most) return BLOSSOM_ERR_UNSUPPORTED;  // (units first: their product with L may not fit 64 bits)
   int bits = 0;
   while (1 << bits < chunks) ++bits;
   const int64_t per_cta = (int64_t)(kCopyThreads >> bits) * kCopyRows;

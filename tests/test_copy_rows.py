@@ -28,6 +28,16 @@ def test_what_is_not_in_whole_pieces_is_refused():
         assert call(**kw) == 2, kw
 
 
+@pytest.mark.parametrize("B,H,L", [(1 << 22, 1 << 22, 1 << 20),             # 2^64 rows: 0 in 64 bits
+                                   (1 << 22, 1 << 21, (1 << 21) + 1),       # 2^64 + 2^43
+                                   ((1 << 31) - 1, (1 << 31) - 1, (1 << 31) - 1),
+                                   (1 << 15, 1 << 15, 2)])                  # 2^31
+def test_more_rows_than_64_bits_count_are_refused(B, H, L):
+    build.build()
+    s = (ctypes.c_int64 * 3)(1024, 512, 64)
+    assert binding.load().blossom_copy_rows(B, H, L, 64, ctypes.c_void_p(4096), s, ctypes.c_void_p(8192), s, None) == 2
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("B,H,L,D", [(1, 1, 1, 8), (2, 3, 5, 32), (1, 1, 255, 32), (1, 2, 129, 64), (3, 300, 1, 32),
                                      (70, 7, 3, 64), (2, 2, 33, 2048), (5, 2, 1024, 32)])
