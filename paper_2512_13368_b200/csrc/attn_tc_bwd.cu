@@ -314,7 +314,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   __syncthreads();
   tc_fence_after();
   mbar_wait(b_meta, 0, &abort_flag, 223);
-  const int nvis = uniform(*reinterpret_cast<const int *>(meta + ml.counts));
+  const int listed = *reinterpret_cast<const int *>(meta + ml.counts);
+  const int nvis = uniform(*(volatile int *)&abort_flag ? 0 : listed);  // (the lists may not be there)
   const uint32_t tmem_base = (uint32_t)uniform((int)tmem_slot);
   // buffers at tmem_base + 64 * (half tile % 2); Q and dO as first operands (bf16 pairs, D / 2
   // columns each) at 128 and 160; the dQ accumulator at 192
@@ -325,13 +326,14 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     setmaxnreg_dec<kProducerRegs>();
     if (warp == kComputeWarps && nvis > 0) {
       // ---- loader: Q, dO once; K/V tiles up to STAGES ahead of their consumers ----
+      bool go = true;
       for (int j = 0; j < nvis; ++j) {
         const int sj = j % STAGES;
-        if (j >= STAGES) mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 205);
+        if (j >= STAGES) go = mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 205) && go;
         const uint32_t bar = b_full + 8 * sj;
         const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
         const int row = (int)list[j] * 64;
-        if (elect_one()) {
+        if (elect_one() && go) {
           mbar_expect_tx(bar, 2 * C::kSmallBytes);
           tma_load_4d(kt, &tmk, bar, 0, row, h / s.G, n);  // the key/value head of this query head
           tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, h / s.G, n);
@@ -717,7 +719,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   mbar_wait(b_meta, 0, &abort_flag, 224);
   // The tile list is the same for every query head of the group (one selection per group): the
   // kernel walks it once per head, item x = (head x / nlist, tile list[x % nlist]).
-  const int nlist = uniform(*reinterpret_cast<const int *>(meta + ml.counts));
+  const int listed = *reinterpret_cast<const int *>(meta + ml.counts);
+  const int nlist = uniform(*(volatile int *)&abort_flag ? 0 : listed);  // (the lists may not be there)
   const int nvis = nlist * Gs;
   const uint32_t tmem_base = (uint32_t)uniform((int)tmem_slot);
   // the half tile of group hh uses the buffer at column 64 hh: S^T in its first 32 columns, dP^T behind
@@ -729,14 +732,15 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     if (warp == kComputeWarps && nvis > 0) {
       // ---- loader: K, V once; Q, dO tiles and their row records up to STAGES ahead ----
       int lj = 0, h = h_first;
+      bool go = true;
       for (int j = 0; j < nvis; ++j) {
         const int sj = j % STAGES;
-        if (j >= STAGES) mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 214);
+        if (j >= STAGES) go = mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 214) && go;
         const uint32_t bar = b_full + 8 * sj;
         const uint32_t qt_ = smem_u32(qg_tiles + sj * kStageBytes);
         if (lj == nlist) { lj = 0; ++h; }  // the next query head of the group walks the same list
         const int row = (int)list[lj++] * 64;
-        if (elect_one()) {
+        if (elect_one() && go) {
           mbar_expect_tx(bar, kStageBytes);
           tma_load_4d(qt_, &tmq, bar, 0, row, h, n);
           tma_load_4d(qt_ + C::kSmallBytes, &tmg, bar, 0, row, h, n);

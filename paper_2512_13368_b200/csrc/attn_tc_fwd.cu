@@ -285,12 +285,13 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         if (warp == kSoftmaxWarps) {
           // ---- loader: K/V tiles, up to STAGES ahead of their consumers ----
           const int u = tile_unit(x), n = unit_batch(u), hk = unit_head(u) / s.G;
+          bool go = true;
           for (int j = 0; j < nI; ++j, ++it, step()) {
             const int row = (int)items[j] * 64;
-            if (it >= STAGES) mbar_wait(b_empty + 8 * sj, sph ^ 1, &abort_flag, 105);
+            if (it >= STAGES) go = mbar_wait(b_empty + 8 * sj, sph ^ 1, &abort_flag, 105) && go;
             const uint32_t bar = b_full + 8 * sj;
             const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
-            if (elect_one()) {
+            if (elect_one() && go) {
               mbar_expect_tx(bar, 2 * C::kSmallBytes);
               tma_load_4d(kt, &tmk, bar, 0, row, hk, n);  // the key/value head of this query head
               tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, hk, n);

@@ -54,18 +54,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // `site` (non-zero) names the wait in the kernel's source; the first wait of a CTA that runs out
 // leaves it in the abort flag, from where it reaches word 1 of the workspace status.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+// False: this wait or an earlier one of the CTA has run out.  From then on every wait returns at once, whatever it waited
+// for: what loads behind it must not (the barrier's loads may still be on their way); products, their reports and
+// arithmetic on whatever lies in the tiles end by themselves (see finish).
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                           int site = 1) {
-  if (mbar_try_wait(bar, parity)) return;
-  if (*abort_flag) return;
+  if (mbar_try_wait(bar, parity)) return true;
+  if (*abort_flag) return false;
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
-    if (*abort_flag) return;
+    if (*abort_flag) return false;
     if (clock64() - t0 > kTimeoutCycles) {
       *abort_flag = site;
-      return;
+      return false;
     }
   }
+  return true;
 }
 
 // Move registers between the warpgroups of a CTA (every thread of a warpgroup executes it).
@@ -503,10 +507,15 @@ __device__ __forceinline__ void finish(int warp, uint32_t tmem_base, uint32_t nc
                                        int32_t *status) {
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem_base, ncols);
+  if (warp == 0) {
+    if (*abort_flag) {  // what is in flight that nobody has waited for, copies and products, ends before its memory is given back
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000LL) {}
+      __syncwarp();
+    }
+    tmem_dealloc(tmem_base, ncols);
+  }
   if (threadIdx.x == 0 && *abort_flag) {
-    const long long t0 = clock64();
-    while (clock64() - t0 < 2000000LL) {}  // grace period for copies still in flight
     if (atomicCAS(status, 0, (int32_t)BLOSSOM_ERR_TIMEOUT) == 0) {  // first reporter: where it happened
       status[1] = *abort_flag;
       status[2] = (int32_t)blockIdx.x;
