@@ -269,6 +269,12 @@ int blossom_selftest_wait_timeout(void *workspace, size_t workspace_bytes, bloss
  * library was loaded (unset or "0" = off).  Returns BLOSSOM_ERR_INVALID_ARG for other arguments. */
 int blossom_debug_switch(int which, int value);
 
+/* Diagnostic (no counterpart in the paper), host only: how the backward of these params (with seq_lens if `lengths` is
+ * not 0) would be launched.  which = 0: thread blocks that share the heads of a key tile in the short-history kernel;
+ * 1: the same in the tensor-core dK/dV kernel; 2: rows of a thread block of the tensor-core path's pre-pass for the
+ * input-dependent gate.  0 where that kernel does not run, -1 for invalid arguments. */
+int blossom_launch_plan(const blossom_params *params /* host */, int which, int lengths);
+
 /* Human-readable name of a blossom_status (host string, static storage). */
 const char *blossom_status_string(int status);
 

@@ -29,7 +29,7 @@ EXPORTS = (
     "blossom_device_status", "blossom_status_string", "blossom_version", "blossom_launch_count",
     "blossom_profile_start", "blossom_profile_every", "blossom_profile_stop", "blossom_kernel_name",
     "blossom_debug_switch",
-    "blossom_selftest_wait_timeout", "blossom_copy_rows",
+    "blossom_selftest_wait_timeout", "blossom_copy_rows", "blossom_launch_plan",
 )
 
 
@@ -96,6 +96,8 @@ def load():
     lib.blossom_kernel_name.argtypes = [ctypes.c_int]
     lib.blossom_selftest_wait_timeout.restype = ctypes.c_int
     lib.blossom_selftest_wait_timeout.argtypes = [vp, sz, vp]
+    lib.blossom_launch_plan.restype = ctypes.c_int
+    lib.blossom_launch_plan.argtypes = [pp, ctypes.c_int, ctypes.c_int]
     lib.blossom_debug_switch.restype = ctypes.c_int
     lib.blossom_debug_switch.argtypes = [ctypes.c_int, ctypes.c_int]
     _lib = lib
@@ -252,6 +254,19 @@ def blossom_debug_switch(which: int, value: int) -> None:
     rc = load().blossom_debug_switch(int(which), int(value))
     if rc:
         raise BlossomError(rc, "blossom_debug_switch")
+
+
+PLAN_SHORT_SPLIT = 0
+PLAN_DKDV_SPLIT = 1
+PLAN_GATE_ROWS = 2
+
+
+def blossom_launch_plan(params, which: int, lengths: bool) -> int:
+    """How the backward of these params is launched (a ``PLAN_`` constant says what of it); 0 where that kernel does not run."""
+    n = int(load().blossom_launch_plan(ctypes.byref(params), int(which), int(bool(lengths))))
+    if n < 0:
+        raise BlossomError(BLOSSOM_ERR_INVALID_ARG, "blossom_launch_plan")
+    return n
 
 
 def blossom_selftest_wait_timeout(workspace, stream=None) -> None:

@@ -386,6 +386,16 @@ int blossom_selftest_wait_timeout(void *workspace, size_t workspace_bytes, bloss
   return tc::launch_wait_selftest(static_cast<int32_t *>(workspace), (cudaStream_t)stream);
 }
 
+int blossom_launch_plan(const blossom_params *params, int which, int lengths) {
+  Shape s;
+  if (make_shape(params, &s) || which < 0 || which > 2) return -1;
+  const bool bwd_short = !force_simt() && sh::bwd_short_supported(s, params->dtype);
+  const bool bwd_tc = !bwd_short && !force_simt() && tc::fwd_tc_supported(s, params->dtype);
+  if (which == 0) return bwd_short ? sh::head_split(s) : 0;
+  if (which == 1) return bwd_tc ? tc::dkdv_split(s, lengths != 0) : 0;
+  return bwd_tc && s.gate_mode ? gate_prep_rows(s) : 0;
+}
+
 int blossom_debug_switch(int which, int value) {
   if (value < -1 || value > 1) return BLOSSOM_ERR_INVALID_ARG;
   if (which == 0) g_force_simt_override = value;

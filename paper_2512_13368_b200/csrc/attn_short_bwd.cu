@@ -430,7 +430,7 @@ bool bwd_short_supported(const Shape &s, int dtype) {
 // The chip full, the copies of the fixed part (selection, K and V rows, the sums over the cluster) cost 3 - 17 %: B 128
 // 141 -> 146 with two CTAs and 163 with four.  The lines, from 178 shapes (two to eight heads a group, L 50 - 300,
 // B 2 - 256): as many CTAs as divide the heads while (batch, key/value head) pairs x CTAs stay below them.
-static int head_split(const Shape &s) {
+int head_split(const Shape &s) {
   const int64_t units = (int64_t)s.B * s.Hkv;
   for (int split = 8; split > 1; split /= 2) {
     const int line = split == s.G ? (s.D == 32 ? 256 : 192) : (s.D == 32 ? 384 : 256);

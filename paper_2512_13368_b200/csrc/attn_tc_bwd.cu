@@ -961,6 +961,22 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
 
 }  // namespace
 
+// Grouped heads: a CTA walks its tile list once per head, so with few CTAs the one with the first keys is the kernel's
+// time (170 us at B 8, 8 heads on 2, L 1500, 192 CTAs): the heads are split over clusters of 2 and 4 while the CTAs fit the
+// chip's places or a CTA's walk (key tiles times heads) is long against what it costs outside it.  With lengths, CTAs that
+// hold padding alone end at once, so more of them are split.  The lines, from whole backward passes of 3834 shapes (two to eight
+// heads a group, L 330 - 4000, 100 - 590 CTAs, every mask and option; 1514 of them with lengths down to 1, L / 10, L / 4 and
+// L / 2): 0.4 % off the best split on average, at worst 14 (lengths: 19) %; one line for both was 1.9 % off, at worst 49 %.
+// us with 1 / 2 / 4 CTAs, D 64, four heads a group: L 700, 108 CTAs 63 / 47 / 56, 360 111 / 125 / 156; L 2048, 160 147 / 103 /
+// 113; two heads: L 1400, 352 CTAs 82 / 94; L 4000, 512 182 / 197 with links, L 1280, 420 with lengths from 320 82 / 74.
+int dkdv_split(const Shape &s, bool lengths) {
+  const int64_t nST = (s.L + 127) / 128, ctas = nST * s.B * s.Hkv;
+  const int64_t walk = lengths ? 16 : 6, fixed = lengths ? 100 : 120, most = lengths ? 1000 : 592;
+  int hs = 1;
+  while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < most && ctas * hs <= walk * nST * (s.G / hs) + fixed) hs *= 2;
+  return hs;
+}
+
 template <int D>
 int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                     const int32_t *seq_lens, const int32_t *idx, const void *out_lt,
@@ -1017,17 +1033,8 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   float *dgate_here = branches == 3 ? dgate : nullptr;
   {
     LaunchScope ls(K_BWD_DKDV_TC, st);
-    // Grouped heads: a CTA walks its tile list once per head, so with few CTAs the one with the first keys
-    // is the kernel's time (170 us at B 8, 8 heads on 2, L 1500, 192 CTAs): the heads are split over clusters
-    // of 2 and 4 while SMs are idle or a CTA's walk (key tiles times heads) is long against what a CTA costs
-    // outside it.  The line from 100 shapes (two and four heads a group, L 450 - 1400, 150 - 580 CTAs), us with / without
-    // the next split at D 64: four heads, L 450, 312 CTAs 47 / 51, 400 63 / 52; L 700 396 CTAs 57 / 66, 576 84 / 72; two
-    // heads left, L 450, 192 CTAs 25 / 26, 304 39 / 32; L 900 320 CTAs 46 / 46, 512 65 / 48; L 1400 484 CTAs 51 / 57.
     const unsigned ctas = (unsigned)nST * (unsigned)(s.B * s.Hkv);
-    unsigned hs = 1;
-    while (hs < 4 && s.G % (2 * hs) == 0 && ctas * hs < 592 &&
-           (ctas * hs < 148 || ctas * hs <= (D == 64 ? 20u : 24u) * (unsigned)nST * ((unsigned)s.G / hs)))
-      hs *= 2;
+    const unsigned hs = (unsigned)dkdv_split(s, seq_lens != nullptr);
     const dim3 grid_k((ctas + (dgate_here ? 1 : 0)) * hs);
     if (hs > 1)
       launch_chained_cluster(kern_kv, grid_k, dim3(kKvThreads), smem_kv, hs, st, q64, k128, v128, g64, s, seq_lens,

@@ -281,6 +281,7 @@ int launch_rope(const Shape &s, int dtype, int dir, const void *qs, void *qd, co
 namespace tc {
 int launch_wait_selftest(int32_t *status, cudaStream_t st);
 bool fwd_tc_supported(const Shape &s, int dtype);
+int dkdv_split(const Shape &s, bool lengths);  // CTAs of a cluster that share a key tile's heads in the backward
 size_t tc_meta_bytes(const Shape &s);  // bytes of one of the two tile-list areas of the workspace
 size_t tc_inv_bits_bytes(const Shape &s);  // (selection per position) bytes of the bit table behind the second
 // branches: bit 0 long-term, bit 1 short-term branch: the tile lists hold only the tiles those
@@ -309,6 +310,7 @@ namespace sh {
 // forward saves for a backward) alone, so a backward knows what the forward before it ran.
 bool fwd_short_supported(const Shape &s, int dtype, bool training);
 bool bwd_short_supported(const Shape &s, int dtype);
+int head_split(const Shape &s);  // the same in the short backward
 int launch_fwd_short(const Shape &s, const void *q, const void *k, const void *v, const float *gate,
                      const int32_t *seq_lens, int32_t *idx, int idx_is_input, void *out, void *out_lt, void *out_st,
                      float *lse, const Workspace &ws, cudaStream_t st);
