@@ -19,7 +19,7 @@
 //
 // What the products of a half tile wait for is one thing, its second operand in tensor memory: the warp that
 // issues them puts the first stage of the next half tile behind the second stage of this one, into the same
-// buffer, without waiting in between (products of one thread run in the order of their issue).  With eight
+// buffer, without waiting in between (the order assumed in tc_common.cuh).  With eight
 // warps on every half tile (16 columns each, twice the hand-offs and their instructions), a warp for each
 // stage and without the uniform registers of tc_common.cuh the kernels took 197 and 232 us at B 128, H 4,
 // L 1024, D 64 (now 181 and 223), 384 and 479 at B 16, H 8, L 4096 (353 and 453), 64 and 80 with a selection
@@ -343,8 +343,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     } else if (warp == kComputeWarps + 1 && nvis > 0) {
       // ---- S = Q K^T and dP = dO V^T of a half tile (32 keys) into buffer x % 2, then, once its dS is in
       // tensor memory, dQ += dS K (K MN-major) and behind it the first stage of half tile x + 2 into the same
-      // buffer: products of one thread run in the order of their issue, so nothing has to wait in between for
-      // the second stage to have read the buffer.  Q and dO are read from tensor memory (the compute warps
+      // buffer, without a wait for the second stage to have read it (the order assumed in tc_common.cuh).  Q and dO are read from tensor memory (the compute warps
       // copied the resident tiles there), so a product fetches only its 32 keys from shared memory instead
       // of 128 rows of Q or dO as well ----
       constexpr uint32_t idesc_s = instr_desc(128, 32, 0, 0), idesc_dq = instr_desc(128, D, 0, 1);

@@ -17,8 +17,8 @@
 // tensor pipe 24 %, 0.56 instructions a cycle and scheduler, four softmax warps each.
 //
 // One warp issues both products of an item.  With a warp for each, S(i + 2) waited for the products of item
-// i to be reported complete; products of one thread run in the order of their issue, so it can follow them
-// at once.  That, and roles, loop bounds and addresses in uniform registers (tc_common.cuh), took the kernel
+// i to be reported complete; in the order that products of one thread are taken to run in (tc_common.cuh) it follows
+// them at once.  That, and roles, loop bounds and addresses in uniform registers (tc_common.cuh), took the kernel
 // from 199 to 179 us at B 128, H 4, L 1024, D 64 and from 360 to 332 at B 16, H 8, L 4096.
 // One code serves all items, masked or not, and both phases' ends: the logits that a row does not see become
 // -infinity before the maximum is taken.  With variants for masked items, a vote which to take and the merge inlined three
@@ -301,8 +301,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         } else {
           // ---- S(i) = Q K^T into buffer i % 2; once a group's probabilities of item i are in tensor memory,
           // O_A += P(i)[:, 0:32] V[0:32], O_B += P(i)[:, 32:64] V[32:64], and behind them S(i + 2) into the same
-          // buffer: products of one thread run in the order of their issue, so nothing has to wait in between
-          // for the probabilities to have been read ----
+          // buffer, without a wait for the probabilities to have been read (the order assumed in tc_common.cuh) ----
           constexpr uint32_t idesc_s = instr_desc(128, 64, 0, 0), idesc_pv = instr_desc(128, D, 0, 1);
           const uint64_t dq = smem_desc(smem_u32(q_tiles) + (k & 1) * C::kBigBytes, 16, C::kAtomBytes, C::kSwizzle);
           auto logits = [&](int b, int stage, int phase) {
@@ -443,8 +442,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         l = 0.f;
       };
       // the products of the item before `it` (of either phase) have completed
-      // (A parity only tells a barrier's last two phases apart.  The one before, item it - 3's, has passed: this
-      // warp has seen the logits of item it - 1, which were issued behind those products, and reported behind them.)
+      // (A parity only tells a barrier's last two phases apart.  The one before, item it - 3's, has passed: this warp has
+      // seen the logits of item it - 1, which were issued behind those products and are taken to be reported behind them.)
       auto products_done = [&](int site) {
         mbar_wait(b_done + 8 * ((it - 1) & 1), ((it - 1) >> 1) & 1, &abort_flag, site);
         __syncwarp();

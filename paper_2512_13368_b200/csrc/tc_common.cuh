@@ -161,6 +161,19 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
+// An assumption about the hardware.  The products of one thread (tcgen05.mma) are taken to read and write in the order of
+// their issue, and their reports (tcgen05.commit) to arrive in it.  PTX promises the first for products with the same
+// accumulator and shape only.  Two things here rest on more than that:
+// - the products that overwrite a logits buffer (M 128, N 64 in the forward, N 32 in the backward) are issued, without a wait,
+//   behind those that read their first operand from it (M 128, N = D into another accumulator, 32 keys each);
+// - the forward's products_done() looks at a barrier whose phase before it knows from a later report only.
+// What speaks for it: the outputs of 60 random shapes of the three kernels (D 32 and 64, L 320 - 4096, all masks and
+// options, three passes each) were the same bits with a wait for the report between the two.  What that wait costs: forward
+// 0.7 % (B 128, H 4, L 1024, D 64 264.7 -> 266.6 us), 2.6 % at B 4, H 8, L 4096; dQ and dK/dV 4 % (413 -> 430 us; L 4096 3 %),
+// where it is part of the chain of a half tile.  Where the order does not hold, the issuers have to commit the readers to a barrier
+// per buffer and wait for it before they overwrite; in the forward that settles products_done() too.  (Other ways to settle
+// that one alone: the issuer waits for the report of item i - 1 before it issues item i's products, 272 us; the softmax warps
+// see every report, 268.6 us.)
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by ONE thread.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                           uint32_t idesc, uint32_t accumulate) {
