@@ -452,67 +452,67 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       int i = 0;
 #pragma unroll 1
       for (int phase = 0; phase < 2; ++phase) {  // the long-term items, the short-term items
-      const int phase_end = phase ? nI : nL;
-      const bool isL = phase == 0;
+        const int phase_end = phase ? nI : nL;
+        const bool isL = phase == 0;
 #pragma unroll 1
-      for (; i < phase_end; ++i, ++it) {
-        const int jt = jt_n, cls = (cls_n >> (2 * grp)) & 3, p0 = jt * 64;
-        if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
-          jt_n = items[i + 1];
-          cls_n = icls[(i + 1) * 4 + quarter];
-        }
-        const int b = it & 1, ph = (it >> 1) & 1;
-        uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
-        bool doB = cls == 1;
-        if (cls == 2) {
-          const int c0 = p0 + 32 * grp;
-          hm = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
-          if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, 32 * grp);
-          else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> (32 * grp)) : st_window32(s, t, c0, causal);
-          doB = __any_sync(0xffffffffu, hm != 0u);
-        }
-        const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
-
-        mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 107);
-        __syncwarp();
-        tc_fence_after();
-        uint32_t pk[16];
-        if (doB) {
-          float sv[32];
-          tmem_ld32(t_b, sv);
-          tmem_wait_ld();
-          float fac = 1.f;
-          if (cls == 2)  // (one code behind it for all items: the instructions have to be fetched, and that is felt)
-#pragma unroll
-            for (int c = 0; c < 32; ++c) sv[c] = (hm >> c) & 1u ? sv[c] : -INFINITY;
-          const float mt = half_row_max(sv) * sc2;
-          const bool need = mt > m + kRescaleThreshold;  // also true on the row's first keys, before which
-          const bool scale_acc = need && l > 0.f;        // the accumulator holds sums of zero probabilities
-          if (need) {
-            fac = exp2f(m - mt);
-            l *= fac;
-            m = mt;
+        for (; i < phase_end; ++i, ++it) {
+          const int jt = jt_n, cls = (cls_n >> (2 * grp)) & 3, p0 = jt * 64;
+          if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
+            jt_n = items[i + 1];
+            cls_n = icls[(i + 1) * 4 + quarter];
           }
-          half_row_probs(sv, sc2, m == -INFINITY ? 0.f : -m, l, pk);  // (no key yet: all logits are -infinity)
-          if (__any_sync(0xffffffffu, scale_acc)) {  // rescaling needs the products of item i-1
-            products_done(108);
-            rescale_acc<D>(acc_own, fac);
+          const int b = it & 1, ph = (it >> 1) & 1;
+          uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
+          bool doB = cls == 1;
+          if (cls == 2) {
+            const int c0 = p0 + 32 * grp;
+            hm = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
+            if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, 32 * grp);
+            else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> (32 * grp)) : st_window32(s, t, c0, causal);
+            doB = __any_sync(0xffffffffu, hm != 0u);
           }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) pk[c] = 0u;
-        }
-        tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
-        tmem_wait_st();
-        tc_fence_before();
-        warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
-      }
+          const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
 
-      if (phase_end > (phase ? nL : 0)) products_done(110 + phase);
-      if (phase && nI == 0) mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 112);  // (nothing else waited for the queries)
-      // sl: the tile before has been stored (at once for the first); the long-term rows have been stored
-      mbar_wait(b_stored, phase ^ 1, &abort_flag, 118 + phase);
-      merge(phase == 1);
+          mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 107);
+          __syncwarp();
+          tc_fence_after();
+          uint32_t pk[16];
+          if (doB) {
+            float sv[32];
+            tmem_ld32(t_b, sv);
+            tmem_wait_ld();
+            float fac = 1.f;
+            if (cls == 2)  // (one code behind it for all items: the instructions have to be fetched, and that is felt)
+#pragma unroll
+              for (int c = 0; c < 32; ++c) sv[c] = (hm >> c) & 1u ? sv[c] : -INFINITY;
+            const float mt = half_row_max(sv) * sc2;
+            const bool need = mt > m + kRescaleThreshold;  // also true on the row's first keys, before which
+            const bool scale_acc = need && l > 0.f;        // the accumulator holds sums of zero probabilities
+            if (need) {
+              fac = exp2f(m - mt);
+              l *= fac;
+              m = mt;
+            }
+            half_row_probs(sv, sc2, m == -INFINITY ? 0.f : -m, l, pk);  // (no key yet: all logits are -infinity)
+            if (__any_sync(0xffffffffu, scale_acc)) {  // rescaling needs the products of item i-1
+              products_done(108);
+              rescale_acc<D>(acc_own, fac);
+            }
+          } else {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) pk[c] = 0u;
+          }
+          tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
+          tmem_wait_st();
+          tc_fence_before();
+          warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
+        }
+
+        if (phase_end > (phase ? nL : 0)) products_done(110 + phase);
+        if (phase && nI == 0) mbar_wait(b_res + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 112);  // (nothing else waited for the queries)
+        // sl: the tile before has been stored (at once for the first); the long-term rows have been stored
+        mbar_wait(b_stored, phase ^ 1, &abort_flag, 118 + phase);
+        merge(phase == 1);
       }
     }
   }

@@ -345,18 +345,6 @@ __device__ __forceinline__ uint64_t cols_ge(int lo) {  // columns c >= lo
 __device__ __forceinline__ uint64_t cols_le(int hi) {  // columns c <= hi
   return hi < 0 ? 0ull : (hi >= 63 ? ~0ull : ((2ull << hi) - 1ull));
 }
-// bit i of `bits` covers columns [i*bk, (i+1)*bk) of a 64-column tile
-__device__ __forceinline__ uint64_t expand_block_bits(uint32_t bits, int bk) {
-  if (bk == 64) return (bits & 1u) ? ~0ull : 0ull;
-  if (bk == 32)
-    return ((bits & 1u) ? 0x00000000FFFFFFFFull : 0ull) | ((bits & 2u) ? 0xFFFFFFFF00000000ull : 0ull);
-  uint64_t m = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    if (bits & (1u << i)) m |= 0xFFFFull << (16 * i);
-  return m;
-}
-
 // the smallest power of two >= x (1 for x <= 1)
 __device__ __forceinline__ int pow2_at_least(int x) { return x <= 1 ? 1 : 1 << (32 - __clz(x - 1)); }
 
@@ -367,8 +355,8 @@ __device__ __forceinline__ uint32_t cols32_ge(int lo) {  // columns c >= lo
   return m;
 }
 __device__ __forceinline__ uint32_t cols32_le(int hi) { return ~cols32_ge(hi + 1); }  // columns c <= hi
-// expand_block_bits for the 32 columns from column c0 (a multiple of 16) of the tile: bits past the tile's
-// 64 columns are not asked for
+// bit i of `bits` covers columns [i*bk, (i+1)*bk) of a 64-column tile: the 32 columns from column c0 (a multiple of 16);
+// bits past the tile's 64 columns are not asked for
 __device__ __forceinline__ uint32_t expand_block_bits32(uint32_t bits, int bk, int c0) {
   // (16 columns from 16: the low ones count; no division by bk)
   if (bk >= 32) return ((bk == 64 ? bits : bits >> (c0 >> 5)) & 1u) ? 0xffffffffu : 0u;
