@@ -77,9 +77,11 @@ Tensor packed(const Tensor &t) {
   return copy_rows(t, dst) ? dst : t.contiguous();
 }
 
-// `t`, whose layout is already the one wanted, as plain memory: the library reads addresses, which know nothing of a view
+// Makes `t`, whose layout is already the one wanted, plain memory: the library reads addresses, which know nothing of a view
 // that negates (wrong signs) and of a zero tensor (no memory).
-Tensor plain(const Tensor &t) { return t.is_neg() || t._is_zerotensor() ? like(t).copy_(t) : t; }
+void make_plain(Tensor &t) {
+  if (t.defined() && (t.is_neg() || t._is_zerotensor())) t = like(t).copy_(t);
+}
 
 std::string failure(const char *where, int rc) {
   return std::string(where) + ": " + blossom_status_string(rc) + " (status " + std::to_string(rc) + ")";
@@ -129,7 +131,7 @@ struct BlossomAttentionBackward : public Node {
     Tensor dout = grads[0];
     if (dout.strides() != q.strides() || dout.scalar_type() != q.scalar_type())  // the library wants q's layout
       dout = copied(dout, like(q));
-    dout = plain(dout);
+    make_plain(dout);
     Tensor dq = like(q), dk = like(k), dv = like(k);
     Tensor dgate = fresh(gate.sizes(), at::kFloat, q.device());
     // The workspace is this call's own and its last user was the training forward (or an earlier
@@ -248,12 +250,7 @@ PyObject *attention(PyObject *, PyObject *const *a, Py_ssize_t n) {
         v = copied(v, like(q));
       }
       if (gate.scalar_type() != at::kFloat || !gate.is_contiguous()) gate = gate.to(at::kFloat).contiguous();
-      q = plain(q);
-      k = plain(k);
-      v = plain(v);
-      gate = plain(gate);
-      if (lens.defined()) lens = plain(lens);
-      if (phi.defined()) phi = plain(phi);
+      for (Tensor *t : {&q, &k, &v, &gate, &lens, &phi}) make_plain(*t);
     }
     p.batch = (int32_t)B;
     p.heads = (int32_t)H;
