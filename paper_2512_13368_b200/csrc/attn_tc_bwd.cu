@@ -22,12 +22,13 @@
 // buffer, without waiting in between (the order assumed in tc_common.cuh).  With eight
 // warps on every half tile (16 columns each, twice the hand-offs and their instructions), a warp for each
 // stage and without the uniform registers of tc_common.cuh the kernels took 197 and 232 us at B 128, H 4,
-// L 1024, D 64 (now 181 and 223), 384 and 479 at B 16, H 8, L 4096 (353 and 453), 64 and 80 with a selection
-// per position at B 8, L 1500 (50 and 73).  Then the code: half tiles of one branch without masks are one code for
+// L 1024, D 64 (without: 181 and 223), 384 and 479 at B 16, H 8, L 4096 (353 and 453), 64 and 80 with a selection
+// per position at B 8, L 1500 (50 and 73).  After that the code: half tiles of one branch without masks are one code for
 // either branch, everything else goes through one masked code; with a code for each branch, both, and masked tiles the
 // instructions did not come fast enough (173 and 221 -> 166 and 212 us; 341 and 450 -> 331 and 435; D 32 82 and 98 -> 78
 // and 93).  What is left is the chain of a half tile: arithmetic 1300 cycles, from there to the next logits 700, while
-// the issue slots are 42 % and the tensor pipe 30 % busy; and the 8000 cycles that a CTA spends outside its loop.
+// the issue slots are 49 % (dQ) and 41 % (dK/dV) and the tensor pipe 39 % busy (B 4, H 8, L 4096); and the 8000 cycles that a
+// CTA spends outside its loop.
 //
 //  dQ     resident Q, dO (128 queries: 128 positions of a head, or with grouped heads 64 positions
 //         of two heads of a group, as in the forward); streams K, V 64-key tiles (same walk as the forward) and

@@ -13,8 +13,8 @@
 // a CTA per tile: with four items a tile 146 us for 4096 tiles of D 64, 98 - 104 us so; 11.5 items
 // 228 -> 204 us, 27 items (L 4096) 388 -> 365 us, D 32 97 -> 91 us.  The roles therefore run on from
 // tile to tile (item counters, stages and barrier phases continue), each as far ahead as its own inputs
-// allow, while the softmax warps merge.  What is left is bound by the softmax warps' instructions:
-// tensor pipe 24 %, 0.56 instructions a cycle and scheduler, four softmax warps each.
+// allow, while the softmax warps merge.  What is left is bound by the softmax warps' instructions, four warps a
+// scheduler: issue slots 57 %, tensor pipe 34 % busy (B 4, H 8, L 4096, D 64).
 //
 // One warp issues both products of an item.  With a warp for each, S(i + 2) waited for the products of item
 // i to be reported complete; in the order that products of one thread are taken to run in (tc_common.cuh) it follows

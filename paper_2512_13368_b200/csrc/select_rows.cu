@@ -164,7 +164,10 @@ __device__ __forceinline__ void add_head(int hg, int n, const float *e, float in
   }
 }
 
-// PQ: one selection per query position.
+// PQ: one selection per query position.  Four CTAs an SM then: in the registers of five (96 a thread) the queries loaded ahead
+// do not fit.  The selection alone, us with four | five: 8 heads on 2 L 50, B 256, D 32 20.2 | 20.4; L 200, B 128, D 32
+// 32.5 | 34.6, D 64 37.1 | 41.9; L 1500, B 16, D 32 50.4 | 50.3, D 64 62.5 | 64.3; ungrouped L 200, B 256, D 32 26.9 | 27.3.  Five are
+// better by 1 - 2 % with many candidates at D 32: L 300, B 128 48.4 | 47.7, four heads L 1500, B 16 34.6 | 33.8.
 template <typename T, int D, bool PQ>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) score_rows_kernel(
     Shape sh, SelGeom g, RowsGeom rg, const T *__restrict__ q, const float *__restrict__ mean32,

@@ -383,7 +383,7 @@ __device__ __forceinline__ uint64_t pow2_queries(int e0) {  // columns c with e0
 // The links part of the masks below, out of line: the kernels' own instructions have to be fetched by every CTA and
 // warp, which is felt (inline, windows alone: forward 175 -> 172 us at B 128, H 4, L 1024, D 64, dK/dV 100 -> 98 at D 32;
 // with links and a selection per position at B 8, L 1500 dK/dV 70 -> 72).  For mask blocks of one position in closed
-// form: a walk over the powers of two took forward, dQ and dK/dV 55, 47 and 74 us there, now 50, 43 and 70.
+// form: a walk over the powers of two took forward, dQ and dK/dV 55, 47 and 74 us there, this 50, 43 and 70.
 static __device__ __noinline__ uint64_t link_key_cols(int L, int blk, int t, int p0, bool causal) {
   uint64_t m = cols_ge(L - blk - p0);
   if (blk == 1) {

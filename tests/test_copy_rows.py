@@ -65,7 +65,8 @@ def test_every_order_of_the_dimensions(B, H, L, D):
 @pytest.mark.gpu
 @pytest.mark.parametrize("dtype,D", [("bf16", 32), ("fp32", 64)])
 def test_gradients_that_are_not_plain_memory(dtype, D):
-    """Negated views, zero tensors, misaligned and repeated rows: what their plain copies give."""
+    """Transposed negated views and zero tensors (those in the output's own layout are in test_front_native.py), misaligned
+    and repeated rows: what their plain copies give."""
     import torch
     from paper_2512_13368_b200.autograd import blossom_attention
     dt = torch.bfloat16 if dtype == "bf16" else torch.float32
