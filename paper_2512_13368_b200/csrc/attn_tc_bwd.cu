@@ -10,10 +10,10 @@
 //
 // Main kernels: CTA = 384 threads.  Warps 0..7 compute; warps 8, 9 stay converged and one elected lane
 // of each issues the TMA loads and the MMAs (10 and 11 are spare); registers move from those warps to the
-// compute warps (setmaxnreg).  A CTA owns a resident 128-row tile (rows = TMEM lanes) and streams 64-row
-// tiles past it in two half tiles of 32 columns, each with a buffer in tensor memory and four compute warps of
-// its own: warps w and w + 4 both address TMEM lane quarter w % 4; the first takes columns 0..31 of every
-// tile, the second columns 32..63, so the two halves never wait for each other.  The tile arithmetic runs in
+// compute warps (setmaxnreg).  A CTA owns a resident 128-row tile (rows = TMEM lanes) and streams pairs of
+// half tiles of 32 rows past it (any two: tc_meta_kernel lists only those that are needed), each half with a buffer in tensor memory and four compute warps of
+// its own: warps w and w + 4 both address TMEM lane quarter w % 4; the first takes the first half of every
+// pair, the second the other, so the two halves never wait for each other.  The tile arithmetic runs in
 // 16-column passes, two columns per FMA / ADD / MUL (packed f32x2); outputs are staged in shared
 // memory and written with whole-line TMA stores.
 //
@@ -31,8 +31,7 @@
 // CTA spends outside its loop.
 //
 //  dQ     resident Q, dO (128 queries: 128 positions of a head, or with grouped heads 64 positions
-//         of two heads of a group, as in the forward); streams K, V 64-key tiles (same walk as the forward) and
-//         works through them in half tiles of 32 keys.  Tensor memory: a buffer of 64 columns
+//         of two heads of a group, as in the forward); streams pairs of half tiles of K, V (same walk as the forward), 32 keys each.  Tensor memory: a buffer of 64 columns
 //         for each half (S in its first 32 columns, dP in the other 32),
 //         Q and dO as first operands of the first-stage products [128,128+D/2), [160,160+D/2)
 //         (read from shared memory they cost 4 KB per product, more than the data pipe delivers
@@ -41,9 +40,8 @@
 //         branches, they share K).  A thread writes the dS (bf16 pairs) of a pass's 16 columns over the first 8
 //         of them in S, from where dQ += dS K reads it: the compute warps wait for one
 //         thing per half tile (its S and dP).  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities, subtracted pair by pair.
-//  dK/dV  transposed: resident K, V of 128 keys, streams Q, dO 64-query tiles (and their row
-//         records, by bulk copy) that selected one of its key blocks or whose window reaches them.
-//         It works through them in half tiles of 32 queries.  Tensor memory: a buffer of 64
+//  dK/dV  transposed: resident K, V of 128 keys, streams pairs of half tiles of Q, dO, 32 queries each (and their row
+//         records, by bulk copy), that selected one of its key blocks or whose window reaches them.  Tensor memory: a buffer of 64
 //         columns for each half (S^T in its first 32 columns, dP^T in the other
 //         32), dV [128,128+D), dK [192,192+D).  S^T = K Q^T, dP^T = V dO^T; thread = key row and
 //         32 query columns; it writes W^T = P'_lt + P'_st and dS^T (bf16 pairs) of a pass's 16 columns over
@@ -217,6 +215,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
     const float *__restrict__ gate, const int32_t *__restrict__ seq_lens, const float *__restrict__ lse,
     const uint8_t *__restrict__ qmeta, const __grid_constant__ CUtensorMap tmdq,
+    const __grid_constant__ CUtensorMap tmk32, const __grid_constant__ CUtensorMap tmv32,
     const float4 *__restrict__ qstats, double *__restrict__ dalpha_part, int32_t *__restrict__ status,
     int nT, const __nv_bfloat16 *add_dq) {
   constexpr bool PLAIN = MODE == kPlain, ADDS = MODE == kPass;
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
   const uint16_t *list = reinterpret_cast<const uint16_t *>(meta + ml.list);
   const uint8_t *lflags = meta + ml.flags;
-  const uint8_t *jcls = meta + ml.jcls;  // [tile][half tile][compute warp]
+  const uint8_t *jcls = meta + ml.jcls;  // [pair][half][compute warp]
 
   const uint32_t b_full = smem_u32(&bars[0]), b_empty = smem_u32(&bars[STAGES]);
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 1]);
@@ -333,11 +332,12 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
         if (j >= STAGES) go = mbar_wait(b_empty + 8 * sj, ((j - STAGES) / STAGES) & 1, &abort_flag, 205) && go;
         const uint32_t bar = b_full + 8 * sj;
         const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
-        const int row = (int)list[j] * 64;
+        const uint32_t pair = reinterpret_cast<const uint32_t *>(list)[j];
+        const int row0 = (int)(pair & 0xffffu) * 32, row1 = (int)(pair >> 16) * 32, hk = h / s.G;  // the key/value head of this query head
         if (elect_one() && go) {
           mbar_expect_tx(bar, 2 * C::kSmallBytes);
-          tma_load_4d(kt, &tmk, bar, 0, row, h / s.G, n);  // the key/value head of this query head
-          tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, h / s.G, n);
+          tma_load_halves(kt, C::kSmallBytes / 2, &tmk, &tmk32, bar, row0, row1, hk, n);
+          tma_load_halves(kt + C::kSmallBytes, C::kSmallBytes / 2, &tmv, &tmv32, bar, row0, row1, hk, n);
         }
         __syncwarp();
       }
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
       warp_arrive(b_aready, lane);
     }
 
-    // Keys 32 half ... of every tile belong to the four warps of group `half`, which have a buffer of their own:
+    // Half `half` of every pair belongs to the four warps of group `half`, which have a buffer of their own:
     // a thread takes all 32 columns, in two passes of 16.
     const uint32_t tb = tmem_base + 64 * half + lane_off;  // S; dP 32 columns further
     const uint8_t *jc = jcls + 8 * half + quarter;  // classes of the half tile's two column halves: [0], [4]
@@ -440,10 +440,10 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
       uint32_t hL = 0u, hS = 0u;  // this thread's 32 keys
       const bool masked = ((cls0 | cls1) & 8) || (cls0 & 3) == 3 || (cls1 & 3) == 3;
       if ((cls0 | cls1) & 8) {  // mixed: per-lane column masks
-        const int jt = list[i], f = lflags[i], p0 = jt * 64, col = 32 * half, c0 = p0 + col;
+        const int hx = list[2 * i + half], f = lflags[2 * i + half], jt = hx >> 1, col = 32 * (hx & 1), c0 = 32 * hx;
         const uint32_t mc = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
         if (f & 1) hL = mc & expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, col);
-        if (f & 2) hS = mc & (s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> col) : st_window32(s, t, c0, causal));
+        if (f & 2) hS = mc & (s.stis_mode ? (uint32_t)(st_key_cols(s, t, jt * 64, causal) >> col) : st_window32(s, t, c0, causal));
       } else if (masked) {
         hL = (cls0 & 1 ? 0xffffu : 0u) | (cls1 & 1 ? 0xffff0000u : 0u);
         hS = (cls0 & 2 ? 0xffffu : 0u) | (cls1 & 2 ? 0xffff0000u : 0u);
@@ -626,7 +626,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmg, Shape s,
     const int32_t *__restrict__ seq_lens, const uint8_t *__restrict__ kmeta,
     const float4 *__restrict__ qstats, const __grid_constant__ CUtensorMap tmdk,
-    const __grid_constant__ CUtensorMap tmdv, int32_t *__restrict__ status, int nT, int hs,
+    const __grid_constant__ CUtensorMap tmdv, const __grid_constant__ CUtensorMap tmq32,
+    const __grid_constant__ CUtensorMap tmg32, int32_t *__restrict__ status, int nT, int hs,
     __nv_bfloat16 *dk, __nv_bfloat16 *dv, const float *__restrict__ gate,
     const double *__restrict__ dalpha_part, float *__restrict__ dgate, int accumulate) {
   constexpr bool PLAIN = MODE == kPlain, ADDS = MODE == kPass;
@@ -676,7 +677,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   const uint8_t *invb = meta;                           // [8][nT] bytes: per key block, per query tile
   const uint16_t *list = reinterpret_cast<const uint16_t *>(meta + ml.list);
   const uint8_t *lflags = meta + ml.flags;
-  const uint8_t *kcls = meta + ml.jcls;                 // [listed tile][compute warp]
+  const uint8_t *kcls = meta + ml.jcls;                 // [listed pair][half][compute warp]
 
   const uint32_t b_full = smem_u32(&bars[0]), b_empty = smem_u32(&bars[STAGES]);
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 1]);
@@ -718,7 +719,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   tc_fence_after();
   mbar_wait(b_meta, 0, &abort_flag, 224);
   // The tile list is the same for every query head of the group (one selection per group): the
-  // kernel walks it once per head, item x = (head x / nlist, tile list[x % nlist]).
+  // kernel walks it once per head, item x = (head x / nlist, pair x % nlist).
   const int listed = *reinterpret_cast<const int *>(meta + ml.counts);
   const int nlist = uniform(*(volatile int *)&abort_flag ? 0 : listed);  // (the lists may not be there)
   const int nvis = nlist * Gs;
@@ -739,12 +740,20 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
         const uint32_t bar = b_full + 8 * sj;
         const uint32_t qt_ = smem_u32(qg_tiles + sj * kStageBytes);
         if (lj == nlist) { lj = 0; ++h; }  // the next query head of the group walks the same list
-        const int row = (int)list[lj++] * 64;
+        const uint32_t pair = reinterpret_cast<const uint32_t *>(list)[lj++];
+        const int row0 = (int)(pair & 0xffffu) * 32, row1 = (int)(pair >> 16) * 32;
+        const float4 *rec = qstats + ((int64_t)n * s.H + h) * Lpad;
         if (elect_one() && go) {
           mbar_expect_tx(bar, kStageBytes);
-          tma_load_4d(qt_, &tmq, bar, 0, row, h, n);
-          tma_load_4d(qt_ + C::kSmallBytes, &tmg, bar, 0, row, h, n);
-          bulk_load(qt_ + 2 * C::kSmallBytes, qstats + ((int64_t)n * s.H + h) * Lpad + row, kStatBytes, bar);
+          tma_load_halves(qt_, C::kSmallBytes / 2, &tmq, &tmq32, bar, row0, row1, h, n);
+          tma_load_halves(qt_ + C::kSmallBytes, C::kSmallBytes / 2, &tmg, &tmg32, bar, row0, row1, h, n);
+          const int rec1 = row1 < Lpad ? row1 : row0;  // (the half behind the last has no records)
+          if (rec1 == row0 + 32) {
+            bulk_load(qt_ + 2 * C::kSmallBytes, rec + row0, kStatBytes, bar);
+          } else {
+            bulk_load(qt_ + 2 * C::kSmallBytes, rec + row0, kStatBytes / 2, bar);
+            bulk_load(qt_ + 2 * C::kSmallBytes + kStatBytes / 2, rec + rec1, kStatBytes / 2, bar);
+          }
         }
         __syncwarp();
       }
@@ -810,14 +819,14 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const float sc2 = s.scale * kLog2e;
 
-    // Half tile hh of every tile (32 queries) belongs to the four warps of group hh = half, which have a buffer of
+    // Half hh of every pair (32 queries) belongs to the four warps of group hh = half, which have a buffer of
     // their own: a thread takes all 32 columns, in two passes of 16.
     const uint32_t tb = tmem_base + 64 * half + lane_off;
     const int q0 = 32 * half;
     int li = 0;
     for (int i = 0; i < nvis; ++i) {
       if (li == nlist) li = 0;
-      const int qt = list[li], f = lflags[li], t0 = qt * 64 + q0;
+      const int hx = list[2 * li + half], f = lflags[2 * li + half], qt = hx >> 1, col = 32 * (hx & 1), t0 = 32 * hx;
       const uint8_t *cls2 = kcls + li * 16 + 8 * half + quarter;  // classes of the half tile's two column halves
       const int cls0 = cls2[0], cls1 = cls2[4];
       ++li;
@@ -826,8 +835,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
       if ((cls0 | cls1) & 8) {  // a mixed half: per-lane column masks
         if (row_valid) {
           const uint32_t mc = cols32_ge((causal ? p : pad0) - t0) & cols32_le(s.L - 1 - t0);
-          if (f & 1) hL = mc & (pq ? (uint32_t)(inv64[g * nT + qt] >> q0) : expand_block_bits32(invb[g * nT + qt], s.Bk, q0));
-          if (f & 2) hS = mc & (uint32_t)(st_query_cols(s, p, qt * 64, causal) >> q0);
+          if (f & 1) hL = mc & (pq ? (uint32_t)(inv64[g * nT + qt] >> col) : expand_block_bits32(invb[g * nT + qt], s.Bk, col));
+          if (f & 2) hS = mc & (uint32_t)(st_query_cols(s, p, qt * 64, causal) >> col);
         }
       } else if (masked) {
         hL = (cls0 & 1 ? 0xffffu : 0u) | (cls1 & 1 ? 0xffff0000u : 0u);
@@ -984,7 +993,7 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
                     void *dv, float *dgate, const Workspace &ws, cudaStream_t st, int branches, const float4 *records) {
   typedef __nv_bfloat16 bf;
   using C = Cfg<D>;
-  CUtensorMap q128, k64, v64, g128, q64, k128, v128, g64, tdq, tdk, tdv;
+  CUtensorMap q128, k64, v64, g128, q64, k128, v128, g64, tdq, tdk, tdv, k32, v32, q32, g32;
   // (head-packed dQ kernel: a query-side box is 64 positions of two heads)
   const int qrows = s.pack ? 64 : 128, qheads = s.pack ? 2 : 1;
   if (make_tensor_map(&q128, q, s, qrows, false, qheads) || make_tensor_map(&k64, k, s, 64, true) ||
@@ -992,7 +1001,8 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
       make_tensor_map(&q64, q, s, 64) || make_tensor_map(&k128, k, s, 128, true) ||
       make_tensor_map(&v128, v, s, 128, true) || make_tensor_map(&g64, dout, s, 64) ||
       make_tensor_map(&tdq, dq, s, qrows, false, qheads) || make_tensor_map(&tdk, dk, s, 128, true) ||
-      make_tensor_map(&tdv, dv, s, 128, true))
+      make_tensor_map(&tdv, dv, s, 128, true) || make_tensor_map(&k32, k, s, 32, true) ||
+      make_tensor_map(&v32, v, s, 32, true) || make_tensor_map(&q32, q, s, 32) || make_tensor_map(&g32, dout, s, 32))
     return BLOSSOM_ERR_CUDA;
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const unsigned grid = (unsigned)nST * (unsigned)(s.B * s.H);
@@ -1025,7 +1035,7 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     LaunchScope ls(K_BWD_DQ_TC, st);
     const unsigned grid_q = s.pack ? (unsigned)nT * (unsigned)(s.B * (s.H / 2)) : grid;
     launch_chained(kern_dq, dim3(grid_q), dim3(kKvThreads), smem_dq, st, q128, k64, v64, g128, s, gate, seq_lens, lse,
-                   (const uint8_t *)ws.qmeta, tdq, rec, ws.dalpha, ws.status_bwd, nT,
+                   (const uint8_t *)ws.qmeta, tdq, k32, v32, rec, ws.dalpha, ws.status_bwd, nT,
                    branches == 2 ? (const bf *)dq : nullptr);
   }
   if (dgate && branches != 3)  // between the two: it depends on neither, and its latency disappears
@@ -1038,11 +1048,11 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     const dim3 grid_k((ctas + (dgate_here ? 1 : 0)) * hs);
     if (hs > 1)
       launch_chained_cluster(kern_kv, grid_k, dim3(kKvThreads), smem_kv, hs, st, q64, k128, v128, g64, s, seq_lens,
-                             (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, (int)hs, (bf *)dk, (bf *)dv, gate,
+                             (const uint8_t *)ws.kmeta, rec, tdk, tdv, q32, g32, ws.status_bwd, nT, (int)hs, (bf *)dk, (bf *)dv, gate,
                              (const double *)ws.dalpha, dgate_here, branches == 2);
     else
       launch_chained(kern_kv, grid_k, dim3(kKvThreads), smem_kv, st, q64, k128, v128, g64, s, seq_lens,
-                     (const uint8_t *)ws.kmeta, rec, tdk, tdv, ws.status_bwd, nT, 1, (bf *)dk, (bf *)dv, gate,
+                     (const uint8_t *)ws.kmeta, rec, tdk, tdv, q32, g32, ws.status_bwd, nT, 1, (bf *)dk, (bf *)dv, gate,
                      (const double *)ws.dalpha, dgate_here, branches == 2);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;

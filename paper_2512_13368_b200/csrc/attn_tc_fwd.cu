@@ -1,8 +1,8 @@
 // Tensor-core forward of the fused two-branch attention (bf16 storage, fp32 accumulate).
 //
-// A CTA owns 128 query rows (128 / Bk query blocks) and walks a list of items, one 64-key tile of
-// one branch each: first the tiles any of its query blocks selected (Eq. 14, 16), then the tiles
-// its rows reach through the window (Eq. 15, 17).  A tile that belongs to both branches is visited
+// A CTA owns 128 query rows (128 / Bk query blocks) and walks a list of items, two half tiles of 32 keys of
+// one branch each (any two: tc_meta_kernel lists only those that some row needs): first what any of its query blocks
+// selected (Eq. 14, 16), then what its rows reach through the window (Eq. 15, 17).  Keys that belong to both branches are visited
 // once per phase.  With grouped heads (an even number per key/value head) the 128 rows are instead
 // the same 64 positions of two heads of a group, which share their selection (Eq. 12), their window
 // tiles and their K/V: every tile on the list then has work for every row (template flag PACK).
@@ -27,8 +27,8 @@
 // blocks of 32 was selected).
 //
 // CTA = 384 threads.  Warps 0..7 are softmax warps: a query row (= TMEM lane) is shared by two
-// threads, warp w and warp w + 4, which split the KEYS of every tile: group 0 (warps 0..3) takes
-// keys 0..31, group 1 keys 32..63.  Each group keeps its own running maximum and sum and its own
+// threads, warp w and warp w + 4, which split the KEYS of every item: group 0 (warps 0..3) takes
+// the first half, group 1 the second.  Each group keeps its own running maximum and sum and its own
 // accumulator (O_A += P[:, 0:32] V[0:32], O_B += P[:, 32:64] V[32:64]), so the two threads of a row
 // never exchange anything inside the loop; the two partial results are merged, exactly as two
 // halves of an online softmax, when a phase ends.  Sixteen softmax warps per SM instead of eight
@@ -136,7 +136,8 @@ template <int D, bool PLAIN, bool PACK>
 __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
     const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmo,
-    const __grid_constant__ CUtensorMap tmol, const __grid_constant__ CUtensorMap tmos, Shape s,
+    const __grid_constant__ CUtensorMap tmol, const __grid_constant__ CUtensorMap tmos,
+    const __grid_constant__ CUtensorMap tmk32, const __grid_constant__ CUtensorMap tmv32, Shape s,
     const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
     const uint8_t *__restrict__ qmeta, int training, float *__restrict__ lse,
     int32_t *__restrict__ status, int32_t *__restrict__ tickets, int nT, int n_tiles, int n_meta) {
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         const int x = uniform(*(volatile int *)&abort_flag ? -1 : *(volatile int *)&tile_id[k & 1]);
         if (x < 0) break;
         const uint8_t *meta = metas + (k & 1) * meta_step;
-        const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
+        const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT][2]
         const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
         const int nL = uniform(counts[1]), nI = nL + uniform(counts[2]);
         if (warp == kSoftmaxWarps) {
@@ -287,14 +288,15 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           const int u = tile_unit(x), n = unit_batch(u), hk = unit_head(u) / s.G;
           bool go = true;
           for (int j = 0; j < nI; ++j, ++it, step()) {
-            const int row = (int)items[j] * 64;
+            const uint32_t pair = reinterpret_cast<const uint32_t *>(items)[j];
+            const int row0 = (int)(pair & 0xffffu) * 32, row1 = (int)(pair >> 16) * 32;
             if (it >= STAGES) go = mbar_wait(b_empty + 8 * sj, sph ^ 1, &abort_flag, 105) && go;
             const uint32_t bar = b_full + 8 * sj;
             const uint32_t kt = smem_u32(kv_tiles + sj * 2 * C::kSmallBytes);
             if (elect_one() && go) {
               mbar_expect_tx(bar, 2 * C::kSmallBytes);
-              tma_load_4d(kt, &tmk, bar, 0, row, hk, n);  // the key/value head of this query head
-              tma_load_4d(kt + C::kSmallBytes, &tmv, bar, 0, row, hk, n);
+              tma_load_halves(kt, C::kSmallBytes / 2, &tmk, &tmk32, bar, row0, row1, hk, n);  // (the key/value head of this query head)
+              tma_load_halves(kt + C::kSmallBytes, C::kSmallBytes / 2, &tmv, &tmv32, bar, row0, row1, hk, n);
             }
             __syncwarp();
           }
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       const uint8_t *meta = metas + (k & 1) * meta_step;
       const uint8_t *selb = meta;
       const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
-      const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT]
+      const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT][2]
       const uint8_t *icls = meta + ml.icls;                                         // [2 nT][4]
       const int *counts = reinterpret_cast<const int *>(meta + ml.counts);
       const int nL = uniform(counts[1]), nI = nL + uniform(counts[2]);
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       const int t_last = row_ok && (causal || t >= pad0) ? (causal ? t : s.L - 1) : -1;
       float m = -INFINITY, l = 0.f;  // this group's running maximum (log2 units) and sum of the row
       const float alpha = gate_alpha(gate, hr), beta = 1.f - alpha;
-      int jt_n = nI > 0 ? items[0] : 0, cls_n = nI > 0 ? icls[quarter] : 0;
+      int hx_n = nI > 0 ? items[grp] : 0, cls_n = nI > 0 ? icls[quarter] : 0;
       uint8_t *so = q_tiles + (k & 1) * C::kBigBytes;  // the gate mix is staged over the queries, free by then
 
       // End of a phase: the two groups' halves of every row are merged (maxima, sums, accumulators),
@@ -456,19 +458,19 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         const bool isL = phase == 0;
 #pragma unroll 1
         for (; i < phase_end; ++i, ++it) {
-          const int jt = jt_n, cls = (cls_n >> (2 * grp)) & 3, p0 = jt * 64;
-          if (i + 1 < nI) {  // the next item's tile and class, ahead of their use
-            jt_n = items[i + 1];
+          const int hx = hx_n, cls = (cls_n >> (2 * grp)) & 3;  // this group's half, 32 keys from 32 hx
+          if (i + 1 < nI) {  // the next item's half and class, ahead of their use
+            hx_n = items[2 * (i + 1) + grp];
             cls_n = icls[(i + 1) * 4 + quarter];
           }
           const int b = it & 1, ph = (it >> 1) & 1;
           uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
           bool doB = cls == 1;
           if (cls == 2) {
-            const int c0 = p0 + 32 * grp;
+            const int c0 = 32 * hx, jt = hx >> 1, col = 32 * (hx & 1);
             hm = cols32_le(t_last - c0) & cols32_ge(pad0 - c0);
-            if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, 32 * grp);
-            else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, p0, causal) >> (32 * grp)) : st_window32(s, t, c0, causal);
+            if (isL) hm &= expand_block_bits32(pq ? rowb[r * nT + jt] : selb[g * nT + jt], s.Bk, col);
+            else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, jt * 64, causal) >> col) : st_window32(s, t, c0, causal);
             doB = __any_sync(0xffffffffu, hm != 0u);
           }
           const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
@@ -526,12 +528,12 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
                     const int32_t *seq_lens, const int32_t *idx, void *out, void *out_lt,
                     void *out_st, float *lse, const Workspace &ws, cudaStream_t st) {
   using C = Cfg<D>;
-  CUtensorMap tq, tk, tv, to, tol, tos;
+  CUtensorMap tq, tk, tv, to, tol, tos, tk32, tv32;
   const int training = out_lt != nullptr;
   // (head-packed: a query-side box is 64 positions of two heads)
   const int qrows = s.pack ? 64 : 128, qheads = s.pack ? 2 : 1;
   if (make_tensor_map(&tq, q, s, qrows, false, qheads) || make_tensor_map(&tk, k, s, 64, true) ||
-      make_tensor_map(&tv, v, s, 64, true) || make_tensor_map(&to, out, s, qrows, false, qheads) ||
+      make_tensor_map(&tv, v, s, 64, true) || make_tensor_map(&tk32, k, s, 32, true) || make_tensor_map(&tv32, v, s, 32, true) || make_tensor_map(&to, out, s, qrows, false, qheads) ||
       make_tensor_map(&tol, training ? out_lt : out, s, qrows, false, qheads) ||
       make_tensor_map(&tos, training ? out_st : out, s, qrows, false, qheads))
     return BLOSSOM_ERR_CUDA;
@@ -554,7 +556,7 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training ? ws.kmeta : nullptr, st, ws.status + kTicketWord, 3, 1)) return rc;
   {
     LaunchScope ls(K_FWD_TC, st);
-    launch_chained(kern, dim3(grid), dim3(kFwdThreads), smem, st, tq, tk, tv, to, tol, tos, s, gate, seq_lens,
+    launch_chained(kern, dim3(grid), dim3(kFwdThreads), smem, st, tq, tk, tv, to, tol, tos, tk32, tv32, s, gate, seq_lens,
                    (const uint8_t *)ws.qmeta, training, lse, ws.status, ws.status + kTicketWord, nT, n_tiles, n_meta);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;

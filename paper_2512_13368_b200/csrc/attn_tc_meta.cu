@@ -1,8 +1,8 @@
 // Tile bookkeeping of the tensor-core attention kernels, built once per call.
 //
-// Which 64-key tiles a 128-row query tile has to visit (the blocks its query blocks selected,
-// Eq. 13, and the tiles its window reaches, Eq. 15), in which order, and which of its warps a tile
-// concerns, depends only on the block indices and the sequence lengths.  Building that inside the
+// Which half tiles of 32 keys a 128-row query tile has to visit (the blocks its query blocks selected,
+// Eq. 13, and what its window reaches, Eq. 15), in which order, two at a time, and which of its warps they
+// concern, depends only on the block indices and the sequence lengths.  Building that inside the
 // attention kernels cost every CTA several thousand cycles before its first product; here a warp
 // (or four, see the kernel) per attention CTA builds the image of the bookkeeping the attention kernel wants in shared
 // memory, and the attention kernel fetches it with one bulk copy while its first tiles load.
@@ -10,12 +10,17 @@
 // Query-major image (forward and dQ kernel), see meta_layout():
 //   [8][nT] selection bytes   bit c of byte (g, jt): query block g of the CTA selected key block
 //                             jt * (64 / Bk) + c
-//   list[nT], flags[nT]       the tiles any row of the CTA needs, ascending; bit 0: some selected
-//                             block lies in the tile, bit 1: the window of some row reaches it
-//   items[2 nT], icls[2 nT][4] (forward) the long-term tiles, then the short-term tiles, and the
-//                             classes of every (item, row quarter), two bits per half of the keys
-//   jcls[nT][2][8]            (dQ) class of every (listed tile, half tile, compute warp)
-//   counts                    {tiles on the list, long-term items, short-term items}
+//   list[2 nT], flags[2 nT]   the halves any row of the CTA needs; bit 0: some selected
+//                             block lies in the half, bit 1: the window of some row reaches it
+//   items[2 nT][2], icls[2 nT][4] (forward) the long-term halves, then the short-term halves, two an item, and the
+//                             classes of every (item, row quarter), two bits per half
+//   jcls[nT][2][8]            (dQ) class of every (listed pair, half of it, compute warp)
+//   counts                    {pairs on the list, long-term items, short-term items}
+// The attention kernels work on 64 columns at a time, 32 for each group of their compute warps: any two halves
+// make such a pair (an odd one out is paired with the half behind the last, which reads as zeros and has class 0).
+// With tiles of 64 adjacent rows, halves of 32 that no row needs were worked through as well: with blocks of 32 and 128 rows
+// a CTA 8 % of the items at L 1024 with 8 blocks each, 22 % at L 777 without the causal mask with 6.  us, forward + backward:
+// B 128, H 4, L 1024, D 64 726 -> 695; H 2, D 32 296 -> 284; without the mask, B 16, H 4, L 777 114 -> 108.
 // Head-packed variant (Shape::pack): the CTA's rows 0..63 and 64..127 are the same 64 positions of
 // two query heads with a common key/value head, so both halves have the same selection bytes and
 // every listed tile concerns both.
@@ -24,10 +29,12 @@
 // one bit per (key block, position) in a table in global memory (launch 1), and the key-major
 // images copy the words of their key blocks from it (launch 2).
 // Key-major image (dK/dV kernel): [8][nT] bytes: bit c of byte (g, qt): query block
-// qt * (64 / Bk) + c selected key block g of the CTA; list / flags of the 64-query tiles that
-// visit the CTA's keys; jcls[nT][2][8] class of every (listed tile, half tile, compute warp);
-// counts {tiles on the list}.
+// qt * (64 / Bk) + c selected key block g of the CTA; list / flags of the halves of 32 queries that
+// visit the CTA's keys; jcls[nT][2][8] class of every (listed pair, half of it, compute warp);
+// counts {pairs on the list}.
 #include "tc_common.cuh"
+
+#include <type_traits>
 
 namespace blossom {
 namespace tc {
@@ -73,7 +80,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     if (branches == 2) image -= image_end / 2, qmeta = qmeta2, kmeta = kmeta2;
   }
   const int Lw = (s.L + 31) >> 5;  // words per key block of the bit table
-  const int slice = ml.bytes + ((3 * nT + 15) / 16) * 16;  // the image and a scratch list behind it
+  const int slice = ml.bytes + ((6 * nT + 15) / 16) * 16;  // the image and a scratch list behind it
   uint8_t *meta = meta_all + (size_t)sub * slice;
   const int nST = (s.L + 127) >> 7;
   const bool key_major = image >= n_query_ctas;
@@ -108,6 +115,100 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   };
   const int row_0 = tid / s.topk, slot_0 = tid % s.topk;
 
+  // place of the k-th of n entries of one kind among those of both kinds: two of the first, two of the second, and so
+  // on while there are pairs of both, then what is left
+  auto alternate = [](int k, int second, int n, int other) {
+    const int m = min(n, other) & ~1;
+    if (k < m) return 2 * (k & ~1) + (k & 1) + 2 * second;
+    return second ? k + other : k + m;
+  };
+  // one warp: the list of n halves becomes one of pairs
+  auto pad_list = [&](int n) {
+    if (lane == 0) {
+      if (n & 1) {
+        list[n] = (uint16_t)(2 * nT);
+        lflags[n] = 0;
+      }
+      counts[0] = (n + 1) / 2;
+    }
+  };
+  // One warp: the halves hx_min ... hx_max that the CTA's rows (or keys) lo ... hi need, ascending, a lane per tile of two.
+  // selected(jt, first, second): bits of tile jt's selections by the first and by the other 64 rows.  In a query-major
+  // image the flags also hold which of the two 64-row halves need it, through the long-term branch (bits 2, 3) and at all
+  // (bits 4, 5); n_long, n_all count them by that class.
+  auto half_row0 = [&](int row0, int hf) { return pack ? row0 : row0 + 64 * hf; };
+  int n_long[4] = {0, 0, 0, 0}, n_all[4] = {0, 0, 0, 0};
+  auto list_halves = [&](int hx_min, int hx_max, bool live, int lo, int hi, auto by_key, auto selected) {
+    constexpr bool KEYS = decltype(by_key)::value;
+    int nv = 0;
+    uint32_t one_long = 0u, both_long = 0u, one_all = 0u;  // this lane's counts of classes 1 and 2 (low, high half), of class 3
+    for (int base = hx_min >> 1; live && base <= hx_max >> 1; base += 32) {
+      const int jt = base + lane;
+      uint32_t first[2] = {0u, 0u}, second[2] = {0u, 0u};
+      if (jt <= hx_max >> 1) selected(jt, first, second);
+      int f[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int hx = 2 * jt + x, p0 = hx * 32, p1 = p0 + 31;
+        f[x] = 0;
+        if (hx >= hx_min && hx <= hx_max && p1 >= pad0) {
+          if (KEYS ? touch(p0, min(p1, s.L - 1), lo, hi) : touch(lo, hi, p0, p1)) f[x] = 2;
+          int c = (first[x] ? 1 : 0) | (second[x] ? 2 : 0);
+          f[x] = (f[x] | (c ? 1 : 0)) & branches;
+          if (!KEYS) {
+            if (!(f[x] & 1)) c = 0;
+            f[x] |= c << 2;
+            if (f[x] & 2)
+              for (int hf = 0; hf < 2; ++hf)
+                if ((p0 <= half_row0(lo, hf) + 63 || !causal) && touch(half_row0(lo, hf), half_row0(lo, hf) + 63, p0, p1)) c |= 1 << hf;
+            if (f[x]) f[x] |= (c ? c : 3) << 4;
+          }
+        }
+        if (!KEYS) {
+          const int cl = (f[x] >> 2) & 3, ca = f[x] >> 4;
+          one_long += cl == 1 ? 1u : cl == 2 ? 0x10000u : 0u;
+          both_long += cl == 3 ? 1u : 0u;
+          one_all += ca == 1 ? 1u : ca == 2 ? 0x10000u : 0u;
+        }
+      }
+      const unsigned b0 = __ballot_sync(0xffffffffu, f[0] != 0), b1 = __ballot_sync(0xffffffffu, f[1] != 0);
+      int pos = nv + __popc(b0 & lt) + __popc(b1 & lt);
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        if (f[x]) {
+          list[pos] = (uint16_t)(2 * jt + x);
+          lflags[pos++] = (uint8_t)f[x];
+        }
+      nv += __popc(b0) + __popc(b1);
+    }
+    if (!KEYS) {
+      one_long = __reduce_add_sync(0xffffffffu, one_long);
+      n_long[1] = (int)(one_long & 0xffffu);
+      n_long[2] = (int)(one_long >> 16);
+      n_long[3] = (int)__reduce_add_sync(0xffffffffu, both_long);
+      one_all = __reduce_add_sync(0xffffffffu, one_all);
+      n_all[1] = (int)(one_all & 0xffffu);
+      n_all[2] = (int)(one_all >> 16);
+      n_all[3] = nv - n_all[1] - n_all[2];
+    }
+    return nv;
+  };
+  // One warp: the list's entries in the order both 64-row halves, then alternately two of the first and two of the second,
+  // by the class in the flags from bit `shift`; place(entry, position) takes them down.
+  auto order = [&](int nv, int shift, const int (&n)[4], auto place) {
+    int c1 = 0, c2 = 0, c3 = 0;
+    for (int base = 0; base < nv; base += 32) {
+      const int j = base + lane, c = j < nv ? (lflags[j] >> shift) & 3 : 0;
+      const unsigned b1 = __ballot_sync(0xffffffffu, c == 1), b2 = __ballot_sync(0xffffffffu, c == 2), b3 = __ballot_sync(0xffffffffu, c == 3);
+      if (c)
+        place(j, c == 3 ? c3 + __popc(b3 & lt)
+                        : n[3] + (c == 1 ? alternate(c1 + __popc(b1 & lt), 0, n[1], n[2]) : alternate(c2 + __popc(b2 & lt), 1, n[2], n[1])));
+      c1 += __popc(b1);
+      c2 += __popc(b2);
+      c3 += __popc(b3);
+    }
+  };
+
   for (int i = tid; i < ml.bytes / 4; i += NT) selw[i] = 0u;  // the whole image
   sync();
 
@@ -116,7 +217,6 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     const int row0 = pack ? st * 64 : st * 128, row_last = min(s.L - 1, row0 + (pack ? 63 : 127));
     // first position of the 32 rows of TMEM lane quarter w, and of the 64-row half hf
     auto quarter_row0 = [&](int w) { return row0 + 32 * (pack ? (w & 1) : w); };
-    auto half_row0 = [&](int hf) { return pack ? row0 : row0 + 64 * hf; };
     if (pq) {
       // a selection per query position: every row's own bytes, and their union per query block
       // (which is what the tile list and the item order below are built from)
@@ -149,76 +249,30 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
     }
     sync();
-    if (scans) {  // the tiles any row of the CTA needs, ascending
-      int nv = 0;
-      const int jt_max = (causal ? row_last : s.L - 1) >> 6;
-      for (int base = 0; base <= jt_max; base += 32) {
-        const int jt = base + lane;
-        int f = 0;
-        if (jt <= jt_max && row_last >= pad0 && jt * 64 + 63 >= pad0) {
-          for (int g = 0; g < G; ++g) f |= selb[g * nT + jt] ? 1 : 0;
-          if (touch(row0, row_last, jt * 64, jt * 64 + 63)) f |= 2;
-          f &= branches;
+    if (scans) {  // the halves any row of the CTA needs, ascending
+      const int nv = list_halves(0, (causal ? row_last : s.L - 1) >> 5, row_last >= pad0, row0, row_last, std::false_type(),
+                                 [&](int jt, uint32_t (&first)[2], uint32_t (&second)[2]) {
+        for (int g = 0; g < G / 2; ++g) {
+          first[0] |= selb[g * nT + jt];
+          second[0] |= selb[(g + G / 2) * nT + jt];
         }
-        const unsigned bal = __ballot_sync(0xffffffffu, f != 0);
-        if (f) {
-          const int pos = nv + __popc(bal & lt);
-          list[pos] = (uint16_t)jt;
-          lflags[pos] = (uint8_t)f;
-        }
-        nv += __popc(bal);
-      }
+        first[1] = first[0] & half_bits(1, bk_shift);
+        first[0] &= half_bits(0, bk_shift);
+        second[1] = second[0] & half_bits(1, bk_shift);
+        second[0] &= half_bits(0, bk_shift);
+      });
       if (lane == 0) counts[0] = nv;
     }
     sync();
     const int nv = counts[0];
-    const int gh = G / 2;
     if (with_fwd) {
     if (scans) {  // ---- the forward's items and their classes ----
-    // Long-term items: the tiles both 64-row halves of the CTA need, then alternately a tile only
-    // rows 0..63 need and a tile only rows 64..127 need.  A softmax warp may run ahead of the
+    // Long-term items: the halves that rows of both 64-row halves of the CTA need, then alternately two that only
+    // rows 0..63 need and two that only rows 64..127 need.  A softmax warp may run ahead of the
     // slowest one, so with alternating items both pairs of warps have work at once.
-    int nA = 0, nB = 0, nC = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-      int cA = 0, cB = 0, cC = 0;
-      for (int base = 0; base < nv; base += 32) {
-        const int j = base + lane;
-        int c = 0;
-        if (j < nv) {
-          if (pass == 0) {
-            if (lflags[j] & 1) {
-              const int jt = list[j];
-              for (int g = 0; g < G; ++g)
-                if (selb[g * nT + jt]) c |= g < gh ? 1 : 2;
-            }
-            icls[j] = (uint8_t)c;  // (for the second pass; the classes come later)
-          } else {
-            c = icls[j];
-          }
-        }
-        const unsigned bA = __ballot_sync(0xffffffffu, c == 1), bB = __ballot_sync(0xffffffffu, c == 2),
-                       bC = __ballot_sync(0xffffffffu, c == 3);
-        if (pass == 1 && c) {
-          int pos;
-          if (c == 3) pos = cC + __popc(bC & lt);
-          else if (c == 1) {
-            const int k = cA + __popc(bA & lt);
-            pos = nC + (k < nB ? 2 * k : nB + k);
-          } else {
-            const int k = cB + __popc(bB & lt);
-            pos = nC + (k < nA ? 2 * k + 1 : nA + k);
-          }
-          items[pos] = list[j];
-        }
-        cA += __popc(bA);
-        cB += __popc(bB);
-        cC += __popc(bC);
-      }
-      nA = cA;
-      nB = cB;
-      nC = cC;
-    }
-    const int nl = nA + nB + nC;
+    order(nv, 2, n_long, [&](int j, int pos) { items[pos] = list[j]; });
+    const int n_lt = n_long[1] + n_long[2] + n_long[3], nl = (n_lt + 1) & ~1;
+    if (lane == 0 && nl > n_lt) items[nl - 1] = (uint16_t)(2 * nT);
     int count = nl;
     for (int base = 0; base < nv; base += 32) {  // short-term items in ascending order
       const int j = base + lane;
@@ -228,8 +282,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       count += __popc(bal);
     }
     if (lane == 0) {
-      counts[1] = nl;
-      counts[2] = count - nl;
+      if (count & 1) items[count++] = (uint16_t)(2 * nT);
+      counts[1] = nl / 2;
+      counts[2] = (count - nl) / 2;
     }
     }
     sync();
@@ -239,20 +294,19 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     const bool uni = s.Bk >= 32;  // a quarter's 32 rows share one query block
     for (int e = tid; e < count * 4; e += NT) {
       const int it = e >> 2, w = e & 3;
-      const int jt = items[it], t_lo = quarter_row0(w), t_hi = t_lo + 31;
+      const int t_lo = quarter_row0(w), t_hi = t_lo + 31;
       const bool rows = t_hi >= pad0 && t_lo < s.L, rows_in = t_lo >= pad0 && t_hi < s.L;
-      const uint32_t bits = it < nl && uni ? selb[((w * 32) >> bk_shift) * nT + jt] : 0u;
       int cls = 0;
 #pragma unroll 1
       for (int hf = 0; hf < 2; ++hf) {
-        const int k_lo = jt * 64 + 32 * hf, k_hi = k_lo + 31;
+        const int hx = items[2 * it + hf], k_lo = hx * 32, k_hi = k_lo + 31;
         int c = 0;
         if (rows && (k_lo <= t_hi || !causal) && k_hi >= pad0 && k_lo < s.L) {
           // every row of the quarter may see every key of the half as far as validity and causality go
           const bool inner = rows_in && k_lo >= pad0 && (causal ? k_hi <= t_lo : k_hi < s.L);
           if (it < nl) {
             if (!uni) c = 2;
-            else if ((bits >> ((32 * hf) >> bk_shift)) & 1u) c = !pq && inner ? 1 : 2;  // (per position: the rows differ)
+            else if (selb[((w * 32) >> bk_shift) * nT + (hx >> 1)] & half_bits(hx, bk_shift)) c = !pq && inner ? 1 : 2;  // (per position: the rows differ)
           } else if (touch(t_lo, t_hi, k_lo, k_hi)) {
             c = (inner && k_lo >= t_hi - s.window + 1 && (causal || k_hi <= t_lo + s.window - 1)) ? 1 : 2;  // 1: inside every row's window
           }
@@ -263,79 +317,40 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
     }  // the forward's part
     sync();
-    // The dQ kernel walks `list` itself (a tile serves both branches there).  Same idea as above:
-    // tiles both 64-row halves need first, then alternately a tile only rows 0..63 need and one
-    // only rows 64..127 need, so that the two halves' warps work on neighbouring tiles at once.
+    // The dQ kernel walks `list` itself (a half serves both branches there).  Same idea as above:
+    // what both 64-row halves need first, then alternately two that only rows 0..63 need and two
+    // only rows 64..127 need, so that the two halves' warps work on neighbouring pairs at once.
     // (Backward call only; the forward reads `items`.)
     if (kmeta && scans) {
       uint16_t *tlist = reinterpret_cast<uint16_t *>(meta + ml.bytes);
-      uint8_t *tflags = meta + ml.bytes + 2 * nT;
-      int nA = 0, nB = 0, nC = 0;
-      for (int pass = 0; pass < 2; ++pass) {
-        int cA = 0, cB = 0, cC = 0;
-        for (int base = 0; base < nv; base += 32) {
-          const int j = base + lane;
-          int c = 0;
-          if (j < nv && pass == 1) {
-            c = jcls[j];
-          } else if (j < nv) {
-            const int jt = list[j], p0 = jt * 64;
-            if (lflags[j] & 1)
-              for (int g = 0; g < G; ++g)
-                if (selb[g * nT + jt]) c |= g < gh ? 1 : 2;
-            if (lflags[j] & 2)
-              for (int hf = 0; hf < 2; ++hf)
-                if ((p0 <= half_row0(hf) + 63 || !causal) &&
-                    touch(half_row0(hf), half_row0(hf) + 63, p0, p0 + 63))
-                  c |= 1 << hf;
-            if (c == 0) c = 3;
-            jcls[j] = (uint8_t)c;  // (for the second pass)
-          }
-          const unsigned bA = __ballot_sync(0xffffffffu, c == 1), bB = __ballot_sync(0xffffffffu, c == 2),
-                         bC = __ballot_sync(0xffffffffu, c == 3);
-          if (pass == 1 && c) {
-            int pos;
-            if (c == 3) pos = cC + __popc(bC & lt);
-            else if (c == 1) {
-              const int k = cA + __popc(bA & lt);
-              pos = nC + (k < nB ? 2 * k : nB + k);
-            } else {
-              const int k = cB + __popc(bB & lt);
-              pos = nC + (k < nA ? 2 * k + 1 : nA + k);
-            }
-            tlist[pos] = list[j];
-            tflags[pos] = lflags[j];
-          }
-          cA += __popc(bA);
-          cB += __popc(bB);
-          cC += __popc(bC);
-        }
-        nA = cA;
-        nB = cB;
-        nC = cC;
-      }
+      uint8_t *tflags = meta + ml.bytes + 4 * nT;
+      order(nv, 4, n_all, [&](int j, int pos) {
+        tlist[pos] = list[j];
+        tflags[pos] = lflags[j];
+      });
       __syncwarp();
       for (int j = lane; j < nv; j += 32) {
         list[j] = tlist[j];
         lflags[j] = tflags[j];
       }
     }
+    if (scans) pad_list(nv);
     sync();
-    // dQ kernel: class of every (listed tile, half tile of 32 keys, compute warp).  Warp w works
-    // on rows 32 (w % 4) ... and keys 16 (w / 4) ... of the half tile.  Bit 0 / bit 1: every row of
+    // dQ kernel: class of every (listed pair, half of 32 keys, compute warp).  Warp w works
+    // on rows 32 (w % 4) ... and keys 16 (w / 4) ... of the half.  Bit 0 / bit 1: every row of
     // the warp sees all 16 keys through the long-term / short-term branch and no row sees only a
     // part of them; 8: mixed, the warp builds per-lane column masks.  (A forward-only call has no
     // use for them.)
-    for (int e = tid; e < (kmeta ? nv * 16 : 0); e += NT) {
-      const int it = e >> 4, hh = (e >> 3) & 1, w = e & 7, qtr = w & 3, c = w >> 2;
-      const int jt = list[it], f = lflags[it];
-      const int k_lo = jt * 64 + 32 * hh + 16 * c, k_hi = k_lo + 15, t_lo = quarter_row0(qtr), t_hi = t_lo + 31;
+    for (int e = tid; e < (kmeta ? (nv + 1) / 2 * 16 : 0); e += NT) {
+      const int j = e >> 3, w = e & 7, qtr = w & 3, c = w >> 2;
+      const int hx = list[j], f = lflags[j], jt = hx >> 1;
+      const int k_lo = hx * 32 + 16 * c, k_hi = k_lo + 15, t_lo = quarter_row0(qtr), t_hi = t_lo + 31;
       const bool rows_in = t_lo >= pad0 && t_hi < s.L, rows_none = t_hi < pad0 || t_lo >= s.L;
       const bool past = rows_in && k_lo >= pad0 && (causal ? k_hi <= t_lo : k_hi < s.L);  // every key visible to every row (validity, causality)
       const bool reach = !rows_none && (k_lo <= t_hi || !causal) && k_hi >= pad0 && k_lo < s.L;  // some key may be visible to some row
       int cL = 0, cS = 0;  // 0 none, 1 all, 2 mixed
       if ((f & 1) && reach) {
-        const int kb = (32 * hh + 16 * c) >> bk_shift;  // key block within the tile
+        const int kb = (32 * (hx & 1) + 16 * c) >> bk_shift;  // key block within the tile
         bool any_sel = false, all_sel = true;
         for (int gq = (qtr * 32) >> bk_shift; gq <= (qtr * 32 + 31) >> bk_shift; ++gq) {
           const bool sel = (selb[gq * nT + jt] >> kb) & 1u;
@@ -396,36 +411,34 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       }
     }
     sync();
-    const int qt_min = causal ? key0 >> 6 : 0, qt_max = (s.L - 1) >> 6;
     if (scans) {
-    int count = 0;
-    for (int base = qt_min; base <= qt_max; base += 32) {
-      const int qt = base + lane;
-      int f = 0;
-      if (qt <= qt_max && key_last >= pad0) {
-        for (int g = 0; g < G; ++g) f |= selb[g * nT + qt] ? 1 : 0;
-        if (touch(qt * 64, min(qt * 64 + 63, s.L - 1), key0, key_last)) f |= 2;
-        f &= branches;
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, f != 0);
-      if (f) {
-        const int pos = count + __popc(bal & lt);
-        list[pos] = (uint16_t)qt;
-        lflags[pos] = (uint8_t)f;
-      }
-      count += __popc(bal);
-    }
-    if (lane == 0) counts[0] = count;
+      const int count = list_halves(causal ? key0 >> 5 : 0, (s.L - 1) >> 5, key_last >= pad0, key0, key_last, std::true_type(),
+                                    [&](int qt, uint32_t (&sel)[2], uint32_t (&)[2]) {
+        for (int g = 0; g < G; ++g) {
+          if (pq) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(meta + ml.rows) + 2 * (g * nT + qt);
+            sel[0] |= w[0];
+            sel[1] |= w[1];
+          } else {
+            sel[0] |= selb[g * nT + qt];
+          }
+        }
+        if (!pq) {
+          sel[1] = sel[0] & half_bits(1, bk_shift);
+          sel[0] &= half_bits(0, bk_shift);
+        }
+      });
+      __syncwarp();
+      pad_list(count);
     }
     sync();
-    const int count = counts[0];
-    // dK/dV kernel: class of every (listed tile, half tile of 32 queries, compute warp).  Warp w
-    // works on key rows 32 (w % 4) ... of the CTA and on query columns 16 (w / 4) ... of the half
-    // tile.  Same code as for the dQ kernel: bit 0 / bit 1 = every key row of the warp is seen in
+    const int count = 2 * counts[0];
+    // dK/dV kernel: class of every (listed pair, half of 32 queries, compute warp).  Warp w
+    // works on key rows 32 (w % 4) ... of the CTA and on query columns 16 (w / 4) ... of the half.  Same code as for the dQ kernel: bit 0 / bit 1 = every key row of the warp is seen in
     // full by all 16 queries through the long-term / short-term branch and none in part; 8 = mixed.
-    for (int e = tid; e < count * 16; e += NT) {
-      const int it = e >> 4, hh = (e >> 3) & 1, w = e & 7, qtr = w & 3, hf = w >> 2;
-      const int qt = list[it], f = lflags[it], c_lo = 32 * hh + 16 * hf;
+    for (int e = tid; e < count * 8; e += NT) {
+      const int j = e >> 3, w = e & 7, qtr = w & 3, hf = w >> 2;
+      const int hx = list[j], qt = hx >> 1, f = lflags[j], c_lo = 32 * (hx & 1) + 16 * hf;
       const int p_lo = key0 + 32 * qtr, p_hi = p_lo + 31, t_lo = qt * 64 + c_lo, t_hi = t_lo + 15;
       const bool rows_in = p_lo >= pad0 && p_hi < s.L, rows_none = p_hi < pad0 || p_lo >= s.L;
       const bool past = rows_in && t_hi < s.L && (causal ? t_lo >= p_hi : t_lo >= pad0);  // every query sees every key (validity, causality)
@@ -471,7 +484,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   // four warps took 26 us and one 17.
   const bool wide = n_images * (qmeta2 ? 2 : 1) <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;
-  const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((3 * nT + 15) / 16) * 16);
+  const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((6 * nT + 15) / 16) * 16);
   const bool plain = s.causal && !s.pq && s.stis_mode == 0;
   auto kern = wide ? (plain ? tc_meta_kernel<kMetaWarps, true> : tc_meta_kernel<kMetaWarps, false>)
                    : (plain ? tc_meta_kernel<1, true> : tc_meta_kernel<1, false>);

@@ -109,6 +109,16 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
+// Two half tiles of 32 rows, one behind the other: one copy where the rows follow one another, else two.
+__device__ __forceinline__ void tma_load_halves(uint32_t dst, uint32_t half_bytes, const CUtensorMap *map64, const CUtensorMap *map32,
+                                                uint32_t bar, int row0, int row1, int h, int n) {
+  if (row1 == row0 + 32) {
+    tma_load_4d(dst, map64, bar, 0, row0, h, n);
+  } else {
+    tma_load_4d(dst, map32, bar, 0, row0, h, n);
+    tma_load_4d(dst + half_bytes, map32, bar, 0, row1, h, n);
+  }
+}
 // 4-D tiled store shared -> global (rows past the tensor's extent are not written); the caller
 // commits and waits for the bulk group before the shared memory is reused or the CTA exits.
 __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, uint32_t src, int c0, int c1, int c2,
@@ -471,10 +481,10 @@ struct Cfg {
 };
 
 // Per-CTA tile bookkeeping, built once per call by tc_meta_kernel and brought into shared memory
-// by one bulk copy: [8][nT] selection bytes, nT list entries, nT flags, (forward) 2 nT per-phase
-// items with 4 class bytes each, (dQ kernel) 16 class bytes per listed tile, and the counts {tiles
-// on the list, long-term items, short-term items}.  Offsets in bytes; every part starts on a
-// 16-byte boundary where a copy needs it.
+// by one bulk copy: [8][nT] selection bytes, 2 nT list entries and flags (half tiles of 32 rows), (forward) up to
+// 4 nT halves as per-phase items of two with 4 class bytes each, (dQ, dK/dV) 16 class bytes per two listed halves, and the
+// counts {pairs of halves on the list, long-term items, short-term items}.  Offsets in bytes; every part starts on a
+// 16-byte boundary where a copy needs it, and the two halves of a pair or an item share an aligned word.
 // With a selection per query position (pq) an area of 128 nT bytes follows: in a query-major
 // image [128 rows][nT] bytes, bit c of byte (r, jt): row r of the CTA selected key block
 // jt * (64 / Bk) + c (the [8][nT] bytes at the start are then the union over a query block's
@@ -486,9 +496,9 @@ struct MetaLayout {
 __host__ __device__ inline MetaLayout meta_layout(int nT, int pq = 0) {
   MetaLayout m;
   m.list = ((8 * nT + 15) / 16) * 16;
-  m.flags = m.list + 2 * nT;
-  m.items = ((m.flags + nT + 15) / 16) * 16;
-  m.icls = m.items + 4 * nT;
+  m.flags = m.list + 4 * nT;
+  m.items = ((m.flags + 2 * nT + 15) / 16) * 16;
+  m.icls = m.items + 8 * nT;
   m.jcls = ((m.icls + 8 * nT + 15) / 16) * 16;
   m.counts = m.jcls + 16 * nT;
   m.rows = m.counts + 16;
@@ -496,6 +506,10 @@ __host__ __device__ inline MetaLayout meta_layout(int nT, int pq = 0) {
   return m;
 }
 __host__ __device__ inline int meta_bytes(int nT, int pq = 0) { return meta_layout(nT, pq).bytes; }
+// selection bits of half tile hx (32 rows) in the byte of its 64-row tile
+__device__ __forceinline__ uint32_t half_bits(int hx, int bk_shift) {
+  return bk_shift == 6 ? 1u : bk_shift == 5 ? 1u << (hx & 1) : 3u << (2 * (hx & 1));
+}
 
 // one arrival per warp, after all its lanes are done
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
