@@ -552,8 +552,9 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   const int resident = 148 * (smem <= kPair ? 2 : 1);
   const unsigned grid = (unsigned)(n_tiles < resident ? n_tiles : resident);
   // A training call also builds the backward's tile lists (the same launch: one warp per image):
-  // a backward call told to reuse them (blossom_params::reuse_tile_lists) then builds none.
-  if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training ? ws.kmeta : nullptr, st, ws.status + kTicketWord, 3, 1)) return rc;
+  // a backward call told to reuse them (blossom_params::reuse_tile_lists) then builds none.  (The backward of an
+  // input-dependent gate takes lists of one branch at a time: it builds its own.)
+  if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training && !s.gate_mode ? ws.kmeta : nullptr, st, ws.status + kTicketWord, 3, 1)) return rc;
   {
     LaunchScope ls(K_FWD_TC, st);
     launch_chained(kern, dim3(grid), dim3(kFwdThreads), smem, st, tq, tk, tv, to, tol, tos, tk32, tv32, s, gate, seq_lens,

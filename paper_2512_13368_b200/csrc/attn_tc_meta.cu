@@ -57,8 +57,10 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                                                                   int branches, int with_fwd,
                                                                   uint32_t *__restrict__ inv_bits,
                                                                   int32_t *__restrict__ tickets,
-                                                                  uint8_t *qmeta2, uint8_t *kmeta2) {
-  grid_chain_enter();
+                                                                  uint8_t *qmeta2, uint8_t *kmeta2, int release_late) {
+  if (!release_late) grid_release();
+  grid_wait();
+  if (release_late) grid_release();
   if (blockIdx.x == 0 && threadIdx.x == 0) *tickets = 0;  // of the persistent kernel behind
   constexpr int NT = 32 * NW;  // threads per image
   const bool causal = PLAIN || s.causal;
@@ -471,11 +473,11 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
 
 int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, uint8_t *qmeta,
                    uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches, int with_fwd, uint8_t *qmeta2,
-                   uint8_t *kmeta2) {
+                   uint8_t *kmeta2, bool release_late) {
   if (with_fwd < 0) with_fwd = kmeta == nullptr;
   if (qmeta2 && s.pq) {  // (a selection per position takes two launches for each set)
     if (int rc = launch_tc_meta(s, seq_lens, idx, qmeta, kmeta, st, tickets, 1, with_fwd)) return rc;
-    return launch_tc_meta(s, seq_lens, idx, qmeta2, kmeta2, st, tickets, 2, with_fwd);
+    return launch_tc_meta(s, seq_lens, idx, qmeta2, kmeta2, st, tickets, 2, with_fwd, nullptr, nullptr, release_late);
   }
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
@@ -493,7 +495,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
     LaunchScope ls(K_TC_META, st);
     launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,
                    seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits, tickets, qmeta2,
-                   kmeta2);
+                   kmeta2, (int)release_late);
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it

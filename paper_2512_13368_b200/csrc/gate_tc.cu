@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
                                                         float4 *__restrict__ rec_lt, float4 *__restrict__ rec_st,
                                                         double *__restrict__ dgate_part, int Lpad, int rows, int parts,
                                                         int32_t *__restrict__ status) {
-  grid_chain_enter();
+  grid_release();  // (no wait here: the tile lists' kernel before it, of which it needs nothing, waits first and lets it start then)
   if (blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;  // the backward's status words
   constexpr int LPR = D / 8, RPB = 256 / LPR, GW = 2 * D + 1;
   __shared__ double red[8][GW];
@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(256) gate_prep_kernel(Shape s, const float *__
     for (int r = 0; r < 8; ++r) a += red[r][d];  // fixed order
     dgate_part[((int64_t)u * s.M + qb) * GW + d] = a;
   }
+  if (threadIdx.x == 0) grid_wait();  // who waits for this kernel has then waited for the lists too
 }
 
 }  // namespace
@@ -260,6 +261,12 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
                        const float *lse, const void *dout, void *dq, void *dk, void *dv, float *dgate,
                        const Workspace &ws, cudaStream_t st) {
   const int Lpad = (s.L + 63) / 64 * 64;
+  // The lists of both passes in one launch; the second pass adds to the first one's gradients as it writes them
+  // (three scratch tensors, an addition kernel and a launch of lists less: 234 -> 204 us for a step of B 16,
+  // H 4, L 900, D 64 with rotary positions), and beside the pre-pass, which needs none of it: one behind the other, and key-major
+  // lists of both branches from the forward that nobody read, 165.5 us, now 160.1.
+  int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, ws.kmeta, st, ws.status + kTicketWord, 3, 0, ws.qmeta2, ws.kmeta2, true);
+  if (rc) return rc;
   {
     LaunchScope ls(K_BWD_PREP, st);
     const int prows = gate_prep_rows(s), parts = (s.L + prows - 1) / prows;
@@ -269,11 +276,6 @@ int launch_bwd_tc_gate(const Shape &s, const void *q, const void *k, const void 
                    ws.qstats, ws.qstats2, ws.dgate_part, Lpad, prows, parts, ws.status_bwd);
     if (cudaGetLastError() != cudaSuccess) return BLOSSOM_ERR_CUDA;
   }
-  // The lists of both passes in one launch; the second pass adds to the first one's gradients as it writes them
-  // (three scratch tensors, an addition kernel and a launch of lists less: 234 -> 204 us for a step of B 16,
-  // H 4, L 900, D 64 with rotary positions).
-  int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, ws.kmeta, st, ws.status + kTicketWord, 3, 0, ws.qmeta2, ws.kmeta2);
-  if (rc) return rc;
   rc = launch_bwd_tc(s, q, k, v, gate, seq_lens, idx, out_lt, out_st, lse, ws.gate_glt, dq, dk, dv, dgate, ws, st, 1,
                      ws.qstats);
   if (rc) return rc;

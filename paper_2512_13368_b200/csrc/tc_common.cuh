@@ -562,10 +562,11 @@ int make_tensor_map(CUtensorMap *map, const void *base, const Shape &s, int box_
 // rest; a training forward may build everything at once for a backward that reuses it).
 // qmeta2, kmeta2: the images of the long-term branch go to qmeta, kmeta and those of the short-term branch
 // there, in one launch (but for a selection per position).
+// release_late: the kernel behind does not wait for this one at its start (grid_wait, grid_release).
 constexpr int kTicketWord = 20;  // word of the status area: tiles the CTAs of a persistent kernel have taken
 int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, uint8_t *qmeta,
                    uint8_t *kmeta, cudaStream_t st, int32_t *tickets, int branches = 3, int with_fwd = -1,
-                   uint8_t *qmeta2 = nullptr, uint8_t *kmeta2 = nullptr);
+                   uint8_t *qmeta2 = nullptr, uint8_t *kmeta2 = nullptr, bool release_late = false);
 
 // per-file launchers behind launch_fwd_tc / launch_bwd_tc
 template <int D>
