@@ -185,9 +185,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
   float *ms = fsm, *tab = fsm + rg.means;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float *et = tab + warp * kTab * rg.pitch;  // [kTab][pitch] this warp's exponentials / scores
-  float *pt = et + kWarps * 32 * rg.pitch;   // (PQ with grouped heads) [32][pitch] probabilities summed over heads
   const int M = sh.M, Bk = sh.Bk;
-  const int ntiles = (sh.L + kRows - 1) / kRows, nU = sh.B * sh.Hkv;
+  // (PQ) hs warps share 32 rows: a head each, then a share of the rows' choices.  A tile is 128 / hs rows.
+  const int lg = PQ && kMma ? rg.lg_heads : 0, hs = 1 << lg, rw = warp >> lg, hw = warp & (hs - 1), rows = kRows >> lg;
+  const int ntiles = (sh.L + rows - 1) / rows, nU = sh.B * sh.Hkv;
   // late tiles have the most candidates: they go first (tile-major)
   const int tile = ntiles - 1 - (int)(blockIdx.x / nU), u = (int)(blockIdx.x % nU), n = u / sh.Hkv, hk = u % sh.Hkv;
   int len = seq_lens ? seq_lens[n] : sh.L;
@@ -195,8 +196,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
   const int pad0 = sh.L - len;
   const bool causal = sh.causal;
   const int own = causal ? 0 : 1;
-  const int row0 = tile * kRows, t = row0 + tid;  // this lane's query position
-  const int qb0 = row0 / Bk, nqb = min(kRows / Bk, M - qb0);
+  const int row0 = tile * rows, wrow0 = row0 + 32 * rw;  // first row of the CTA, of the warp
+  // this lane's query position: of its warp's rows; where warps share rows, hs lanes make the choice of one
+  const int lrow = hw * (32 >> lg) + (lane >> lg), sub = lane & (hs - 1), t = wrow0 + lrow;
+  float *pt = tab + (kWarps * kTab + rw * 32) * rg.pitch;  // (PQ with grouped heads or Eq. 11) [32][pitch] probabilities summed over heads
+  const int qb0 = row0 / Bk, nqb = min((row0 + rows - 1) / Bk + 1, M) - qb0;
   const int cmin = first_live_scored(g, pad0), jmin = pad0 / Bk;
   const int c_hi = causal ? n_candidates(sh, g, min(M - 1, qb0 + nqb - 1)) : g.n;
   const bool ok = t >= pad0 && t < sh.L;
@@ -259,7 +263,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
     kn = fmaxf(fmaxf(kn_w[0], kn_w[1]), fmaxf(kn_w[2], kn_w[3]));
     // this lane's candidates: columns < nc of the table (the own block's column left out without the mask)
     const int nc = ok ? max(0, (causal ? n_candidates(sh, g, b) : g.n) - cmin) : 0;
-    const int nc_warp = __reduce_max_sync(0xffffffffu, (unsigned)nc);
+    int nc_warp = __reduce_max_sync(0xffffffffu, (unsigned)nc);
+    if (hs > 1) {  // of all 32 rows: under the causal mask (a selection per position has it) the last one's
+      const int tl = min(wrow0 + 31, sh.L - 1);
+      nc_warp = tl >= pad0 && wrow0 < sh.L ? max(0, n_candidates(sh, g, tl / Bk) - cmin) : 0;
+    }
     const float sc2 = sh.scale * 1.4426950408889634f;
     float *er = et + lane * rg.pitch;
     const bool up = lane >= 16;
@@ -283,23 +291,23 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
     };
     uint32_t qnext[kMma && PQ ? D / 16 : 1][4];  // (PQ) the next 16 rows' queries, a product loop ahead: few warps a scheduler
     if constexpr (kMma && PQ)
-      sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G, 0), sh.sl, row0 + warp * 32, pad0, sh.L, lane, qnext);
+      sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hw, 0), sh.sl, wrow0, pad0, sh.L, lane, qnext);
 #pragma unroll 1
-    for (int hg = 0; hg < sh.G; ++hg) {  // the heads of the group in ascending order (Eq. 12)
+    for (int hg = hw; hg < sh.G; hg += hs) {  // the heads of the group in ascending order (Eq. 12)
       if constexpr (kMma) {
         const int gid = lane >> 2, tig = lane & 3;
         const uint32_t tiles = sh::smem_addr(ms) + sh::lane_off_nt<D>(lane), part_bytes = (uint32_t)rg.cols * D * 2;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {  // 16 rows at a time
-          const int tm = row0 + warp * 32 + 16 * mt;
+          const int tm = wrow0 + 16 * mt;
           uint32_t qa[D / 16][4];
           if constexpr (PQ) {
 #pragma unroll
             for (int k = 0; k < D / 16; ++k)
 #pragma unroll
               for (int e = 0; e < 4; ++e) qa[k][e] = qnext[k][e];
-            if (mt == 0 || hg + 1 < sh.G)
-              sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg + mt, 0), sh.sl, row0 + warp * 32 + 16 * (1 - mt), pad0,
+            if (mt == 0 || hg + hs < sh.G)
+              sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg + mt * hs, 0), sh.sl, wrow0 + 16 * (1 - mt), pad0,
                                  sh.L, lane, qnext);
           } else {
             sh::load_a_rows<D>(q + row_offset(sh, n, hk * sh.G + hg, 0), sh.sl, tm, pad0, sh.L, lane, qa);
@@ -364,10 +372,21 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
           }
         }
         if (PQ && sh.G > 1) {
-          float *pr = pt + lane * rg.pitch;
-          const float inv = inv_s[warp][lane];
-          add_head(hg, nc_warp, er, inv, pr);
-          __syncwarp();
+          if (hs == 1) {
+            add_head(hg, nc_warp, er, inv_s[warp][lane], pt + lane * rg.pitch);
+            __syncwarp();
+          } else {  // the hs heads in ascending order too: a lane takes every hs-th candidate of its row
+            __syncthreads();
+            const float *eh = tab + (rw * hs * 32 + lrow) * rg.pitch;
+            float *pr = pt + lrow * rg.pitch;
+#pragma unroll 4
+            for (int c = sub; c < nc_warp; c += hs) {
+              float a = hg >= hs ? pr[c] : 0.f;
+              for (int h = 0; h < hs; ++h) a = fmaf(eh[h * 32 * rg.pitch + c], inv_s[rw * hs + h][lrow], a);
+              pr[c] = a;
+            }
+            __syncthreads();
+          }
         }
       } else {
       // The products are shared by two lanes: lanes l and l + 16 hold the lower and the upper half of the
@@ -425,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
       }
     }
     if constexpr (kMma) {
-      qn = rowq_s[warp][lane];
+      for (int h = 0; h < hs; ++h) qn = fmaxf(qn, rowq_s[rw * hs + h][lrow]);
       loose = qn == INFINITY;
     }
   }
@@ -441,72 +460,78 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? (PQ ? 4 : 5) : 4) s
   auto lost = [&](int rows) { return (float)(rows * sh.G * g.rs * g.rl) * kLost; };
 
   if (PQ) {
-    // ---- Eq. 11, Eq. 13 and the certificate for this lane's own row ----
-    if (t < sh.L) {
+    // ---- Eq. 11, Eq. 13 and the certificate for this lane's row, or its share of it ----
+    int want = 0;
+    const bool scored = ok && choice(b, &want) && n_candidates(sh, g, b) > cmin;
+    const int nc = max(0, n_candidates(sh, g, b) - cmin), ns = scored ? b - jmin : 0;
+    float *S = (sh.G > 1 ? pt : et) + lrow * rg.pitch;
+    if (!g.plain) {
+      // the other table (with hs warps on a row its first one's: nobody reads the exponentials any more)
+      float *o = sh.G > 1 ? tab + (rw * hs * 32 + lrow) * rg.pitch : pt + lrow * rg.pitch;
+      for (int j = jmin + 4 * sub; j < jmin + ns; j += 4 * hs) {  // (four at a time, as in add_head)
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int m = 0; m < g.rs; ++m)
+          for (int e = 0; e < g.rl; ++e)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+              const int i = g.rs * (j + y) - m - e - cmin;
+              if (i >= 0 && i < nc) a[y] += S[i];
+            }
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (j + y < b) o[j + y - jmin] = a[y];
+      }
+      S = o;
+      __syncwarp();
+    }
+    uint32_t taken[4] = {0u, 0u, 0u, 0u};  // bit j - jmin (at most 128 blocks)
+    float kept = 0.f, dropped = 0.f;
+    // The want best, then the best that is left out.  A chain of loads per lane and few warps a scheduler: what is
+    // taken is overwritten.  (A test of its bit per score and one load after the other: with add_head's and Eq. 11's
+    // loads one by one too 36.6 us at B 8, 8 heads on 2, L 1500, D 64, 72.7 at B 64; now 30.9 and 64.6, and 28.1 and
+    // 58.0 with the queries loaded ahead.)
+    const int most = __reduce_max_sync(0xffffffffu, (unsigned)(scored ? want + 1 : 0));
+    for (int k = 0; k < most; ++k) {
+      float best = -1.f;
+      int bi = 0;
+      if (k <= want) {
+#pragma unroll 8
+        for (int j = sub; j < ns; j += hs) {
+          const float x = S[j];
+          if (x > best) {
+            best = x;
+            bi = j;
+          }
+        }
+      }
+      for (int o = 1; o < hs; o <<= 1) {  // the best of the row's lanes, ties to the lower index
+        const float x = __shfl_xor_sync(0xffffffffu, best, o);
+        const int xi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (x > best || (x == best && xi < bi)) {
+          best = x;
+          bi = xi;
+        }
+      }
+      if (scored && k == want) dropped = best;
+      if (scored && k < want) {
+        kept = best;
+        if ((bi & (hs - 1)) == sub) S[bi] = -1.f;
+        const uint32_t bit = 1u << (bi & 31);
+        if (bi < 32) taken[0] |= bit;
+        else if (bi < 64) taken[1] |= bit;
+        else if (bi < 96) taken[2] |= bit;
+        else taken[3] |= bit;
+      }
+    }
+    if (t < sh.L && sub == 0) {
       int32_t *row = idx + ((int64_t)u * sh.L + t) * sh.topk;
       if (!ok) {
         for (int i = 0; i < sh.topk; ++i) row[i] = -1;
         return;
       }
-      int want;
-      const bool ch = choice(b, &want);
-      const int nc = max(0, n_candidates(sh, g, b) - cmin);
-      uint32_t taken[4] = {0u, 0u, 0u, 0u};  // bit j - jmin (at most 128 blocks)
-      bool certain = true;
-      if (!ch || nc == 0) {  // everything, or (no candidate yet: every score is zero) the lowest blocks
+      if (!scored)  // everything, or (no candidate yet: every score is zero) the lowest blocks
         for (int i = 0; i < want; ++i) taken[i >> 5] |= 1u << (i & 31);
-      } else {
-        float *S = sh.G > 1 ? pt + lane * rg.pitch : et + lane * rg.pitch;
-        if (!g.plain) {
-          float *o = sh.G > 1 ? et + lane * rg.pitch : pt + lane * rg.pitch;  // the table that is free
-          for (int j = jmin; j < b; j += 4) {  // (four at a time, as in add_head)
-            float a[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int m = 0; m < g.rs; ++m)
-              for (int e = 0; e < g.rl; ++e)
-#pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                  const int i = g.rs * (j + y) - m - e - cmin;
-                  if (i >= 0 && i < nc) a[y] += S[i];
-                }
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-              if (j + y < b) o[j + y - jmin] = a[y];
-          }
-          S = o;
-        }
-        const int ns = b - jmin;
-        float kept = 0.f, dropped = 0.f;
-        // The want best, then the best that is left out.  A chain of loads per lane and few warps a scheduler: what is
-        // taken is overwritten.  (A test of its bit per score and one load after the other: with add_head's and Eq. 11's
-        // loads one by one too 36.6 us at B 8, 8 heads on 2, L 1500, D 64, 72.7 at B 64; now 30.9 and 64.6, and 28.1 and
-        // 58.0 with the queries loaded ahead.)
-        for (int k = 0; k <= want; ++k) {
-          float best = -1.f;
-          int bi = 0;
-#pragma unroll 8
-          for (int j = 0; j < ns; ++j) {
-            const float x = S[j];
-            if (x > best) {
-              best = x;
-              bi = j;
-            }
-          }
-          if (k == want) {
-            dropped = best;
-          } else {
-            kept = best;
-            S[bi] = -1.f;
-            const uint32_t bit = 1u << (bi & 31);
-            if (bi < 32) taken[0] |= bit;
-            else if (bi < 64) taken[1] |= bit;
-            else if (bi < 96) taken[2] |= bit;
-            else taken[3] |= bit;
-          }
-        }
-        certain = !loose &&
-                  (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f + lost(1);
-      }
-      if (certain) {
+      if (!scored || (!loose && (kept - dropped) > error(qn, (float)den_adds(nc)) * (kept + dropped) * 1.001f + lost(1))) {
         int pos = 0;
 #pragma unroll
         for (int x = 0; x < 4; ++x)
@@ -702,8 +727,18 @@ bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_
   rg->means = mma ? 3 * rg->cols * sh.D / 2 : rg->cols * (sh.D + 4);  // (a multiple of four)
   const int wide = sh.M > rg->cols ? sh.M : rg->cols;  // (per position the table also holds the scores of the selection blocks)
   rg->pitch = (sh.pq ? wide : rg->cols) | 1;
+  // (Per position) warps that share rows, a head each, while tiles of 128 rows are fewer than the CTAs that fit: a warp with all
+  // heads of its rows is a chain of some 3000 instructions, and its scheduler had one or two such.  With more tiles the
+  // copies of the means in each CTA cost more.  us of a forward, 8 heads, with 1 | 2 | 4 heads at once:
+  //   2 key/value heads, L 1500, D 64: 48 tiles 84 | 81 | 76, 192 115 | 109 | 98, 384 150 | 152 | 145, 768 209 | 211 | 213;
+  //     L 600, D 32: 160 71 | 66 | 62, 640 118 | 114 | 116; L 200, D 32: 64 47 | 45 | 42, 512 88 | 87 | 87
+  //   4 key/value heads, 1 | 2: L 1500, D 64: 384 79 | 75, 768 132 | 136; L 600, D 32: 320 66 | 62; L 200: 512 60 | 60
+  const int64_t tiles = (int64_t)((sh.L + kRows - 1) / kRows) * sh.B * sh.Hkv;
+  rg->lg_heads = 0;
+  if (sh.pq && mma && tiles <= 448)
+    while (rg->lg_heads < 2 && sh.G % (2 << rg->lg_heads) == 0) ++rg->lg_heads;
   const bool two = sh.pq && (sh.G > 1 || !g.plain);
-  const size_t tables = (size_t)(two ? 2 : 1) * kWarps * (mma && !sh.pq ? 16 : 32) * rg->pitch * 4;
+  const size_t tables = (size_t)(kWarps + (two ? kWarps >> rg->lg_heads : 0)) * (mma && !sh.pq ? 16 : 32) * rg->pitch * 4;
   const size_t tail = (size_t)(8 * 128 + 2 * kWarps * 132) * 4 + kWarps * 128;
   *smem = (size_t)rg->means * 4 + (tables > tail ? tables : tail) + 16;
   // What single precision cannot certify (some percent of the blocks) the kernel decides itself while that
@@ -714,8 +749,8 @@ bool rows_geom(const Shape &sh, const SelGeom &g, int dtype, RowsGeom *rg, size_
   //     x up to              16384   24576   32768   45056   65536  131072
   //     fewer than 1480 CTAs  1.07    1.05    0.95    0.99    0.85    0.73
   //     1480 CTAs and more    1.13    1.08    1.04    1.01    1.01    0.94
-  const int64_t x = (int64_t)sh.G * sh.Bk * g.n * sh.D, ctas = (int64_t)((sh.L + kRows - 1) / kRows) * sh.B * sh.Hkv;
-  rg->list = sh.pq || sh.G * sh.Bk > 128 || x > (ctas >= 1480 ? 65536 : 24576);
+  const int64_t x = (int64_t)sh.G * sh.Bk * g.n * sh.D;
+  rg->list = sh.pq || sh.G * sh.Bk > 128 || x > (tiles >= 1480 ? 65536 : 24576);
   const size_t own = ((size_t)16 * ((g.n + 1) | 1) + kWarps * 128 + 128 + 128) * 8 + 128;
   if (!rg->list && *smem < own) *smem = own;
   return *smem <= 200 * 1024;
@@ -727,7 +762,8 @@ static int launch_t(const Shape &sh, const SelGeom &g, const RowsGeom &rg, size_
                     int32_t *list, int32_t *count, cudaStream_t st) {
   auto kern = sh.pq ? score_rows_kernel<T, D, true> : score_rows_kernel<T, D, false>;
   if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
-  const unsigned grid = (unsigned)((sh.L + kRows - 1) / kRows) * (unsigned)(sh.B * sh.Hkv);
+  const int rows = kRows >> rg.lg_heads;
+  const unsigned grid = (unsigned)((sh.L + rows - 1) / rows) * (unsigned)(sh.B * sh.Hkv);
   LaunchScope ls(K_SCORE_FAST, st);
   return launch_chained(kern, dim3(grid), dim3(kThreads), smem, st, sh, g, rg, q, mean32, norm, mean, seq_lens, idx,
                         list, count) == cudaSuccess

@@ -7,6 +7,7 @@ namespace blossom {
 struct RowsGeom {
   int cols, pitch;  // candidates in the table of means; pitch of a row's table of exponentials (floats)
   int means;        // floats of the table of means
+  int lg_heads;     // (per position) log2 of the heads of the group that as many warps take at once
   int list;         // what is not certain goes to the list (else the kernel decides it itself)
 };
 // Whether the kernel takes the problem (up to 128 scored and selection blocks), its plan and its shared memory.
