@@ -74,6 +74,17 @@ constexpr int kProducerRegs = 40, kSoftmaxRegs = 96;
 static_assert(256 * kSoftmaxRegs + 128 * kProducerRegs <= kFwdThreads * 80, "register pool of a CTA");
 constexpr uint32_t kFwdTmemCols = 256;
 __host__ __device__ constexpr int fwd_stages(int D) { return D == 64 ? 3 : 4; }
+constexpr int NB = 2;  // logits / probability buffers (a third, for which D 32 leaves room: B 128, H 2, L 1024 282 -> 286 us)
+// The buffer of the next item and its phase, and those of the item before.  The issuer and the softmax warps count for
+// themselves (with the loader's counter for the issuer too: L 4096, B 1, H 8 70.4 -> 71.4 us; D 32, L 1024 286 -> 284).
+struct Turn {
+  int x = 0;
+  __device__ __forceinline__ int buffer() const { return x & 1; }
+  __device__ __forceinline__ int phase() const { return (x >> 1) & 1; }
+  __device__ __forceinline__ int last_buffer() const { return (x - 1) & 1; }
+  __device__ __forceinline__ int last_phase() const { return ((x - 1) >> 1) & 1; }
+  __device__ __forceinline__ void step() { ++x; }
+};
 
 // maximum of 32 logits
 __device__ __forceinline__ float half_row_max(const float (&v)[32]) {
@@ -146,9 +157,9 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   constexpr int STAGES = fwd_stages(D);
   constexpr int DC = D / 2;  // output columns a softmax thread merges and stages
   extern __shared__ uint8_t smem_raw[];
-  // barriers: full[STAGES], empty[STAGES], then by tile res[2], meta[2], per buffer s_full[2],
-  // t_full[group][2], done[2], then staged, stored and by tile roles[2]
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 16];
+  // barriers: full[STAGES], empty[STAGES], then by tile res[2], meta[2], roles[2], then staged, stored, then per buffer
+  // s_full[NB], t_full[group][NB], done[NB]
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 8 + 4 * NB];
   __shared__ int softmax_tile, tile_id[2];  // the tile whose lists lie (or are about to) behind meta[.]; -1: no more
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -177,10 +188,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   auto unit_head = [&](int u) { return PACK ? 2 * (u % (s.H / 2)) : u % s.H; };
   const uint32_t b_full = smem_u32(&bars[0]), b_empty = smem_u32(&bars[STAGES]);
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 2]);
-  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 4]), b_tfull = smem_u32(&bars[2 * STAGES + 6]);  // [group][buffer]
-  const uint32_t b_done = smem_u32(&bars[2 * STAGES + 10]);
-  const uint32_t b_staged = smem_u32(&bars[2 * STAGES + 12]), b_stored = smem_u32(&bars[2 * STAGES + 13]);
-  const uint32_t b_roles = smem_u32(&bars[2 * STAGES + 14]);
+  const uint32_t b_roles = smem_u32(&bars[2 * STAGES + 4]);
+  const uint32_t b_staged = smem_u32(&bars[2 * STAGES + 6]), b_stored = smem_u32(&bars[2 * STAGES + 7]);
+  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 8]), b_tfull = b_sfull + 8 * NB;  // [group][buffer]
+  const uint32_t b_done = b_tfull + 16 * NB;
   // one thread: the lists (and which tile's they are) and the queries of this CTA's k-th tile, number x
   auto fetch_meta = [&](int k, int x) {
     tile_id[k & 1] = x;
@@ -213,9 +224,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       mbar_init(b_res + 8 * i, 1);
       mbar_init(b_meta + 8 * i, 1);
       mbar_init(b_roles + 8 * i, 2);
+    }
+    for (int i = 0; i < NB; ++i) {
       mbar_init(b_sfull + 8 * i, 1);
-      mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);        // group 0
-      mbar_init(b_tfull + 8 * (2 + i), kSoftmaxWarps / 2);  // group 1
+      mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);         // group 0
+      mbar_init(b_tfull + 8 * (NB + i), kSoftmaxWarps / 2);  // group 1
       mbar_init(b_done + 8 * i, 1);
     }
     mbar_init(b_staged, kSoftmaxWarps);
@@ -274,6 +287,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     } else if (warp < kSoftmaxWarps + 2) {
       int it = 0;              // items of the tiles before
       int sj = 0, sph = 0;     // their stage and its phase
+      Turn turn;               // (the issuer's)
       auto step = [&] { if (++sj == STAGES) { sj = 0; sph ^= 1; } };
       for (int k = 0;; ++k) {
         mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 113);
@@ -320,9 +334,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           tc_fence_after();
           int ss = sj, sp = sph;  // stage and phase of the next logits
           auto step_s = [&] { if (++ss == STAGES) { ss = 0; sp ^= 1; } };
-          for (int i = 0; i < 2 && i < nI; ++i, step_s()) logits((it + i) & 1, ss, sp);
-          for (int i = 0; i < nI; ++i, ++it, step()) {
-            const int b = it & 1, ph = (it >> 1) & 1;
+          Turn ahead = turn;
+          for (int i = 0; i < NB && i < nI; ++i, step_s(), ahead.step()) logits(ahead.buffer(), ss, sp);
+          for (int i = 0; i < nI; ++i, step()) {
+            const int b = turn.buffer(), ph = turn.phase();
+            turn.step();
             const uint64_t dv = smem_desc(smem_u32(kv_tiles + sj * 2 * C::kSmallBytes + C::kSmallBytes),
                                           C::kSmallBytes, C::kAtomBytes, C::kSwizzle);
             const uint32_t tp = tmem_base + 64 * b;
@@ -335,7 +351,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
                 umma_bf16_ts(tmem_oa, tp + 8 * c, dv + c * C::kKStep, idesc_pv, (first | (uint32_t)c) != 0u);
             }
             __syncwarp();
-            mbar_wait(b_tfull + 8 * (2 + b), ph, &abort_flag, 109);
+            mbar_wait(b_tfull + 8 * (NB + b), ph, &abort_flag, 109);
             tc_fence_after();
             if (elect_one()) {
 #pragma unroll
@@ -345,7 +361,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
               umma_commit(b_empty + 8 * sj);  // S(i) completed before the softmax warps read it
             }
             __syncwarp();
-            if (i + 2 < nI) {
+            if (i + NB < nI) {
               logits(b, ss, sp);
               step_s();
             }
@@ -363,7 +379,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     const uint32_t acc_own = (grp ? tmem_ob : tmem_oa) + lane_off;
     // (not zero, which a scale among the denormals is flushed to: a hidden logit, -infinity, times it has to stay so)
     const float sc2 = fmaxf(s.scale * kLog2e, FLT_MIN);
-    int it = 0;  // items of the tiles before
+    Turn turn;
     for (int k = 0;; ++k) {
       if (warp == 0) {  // one warp decides for all: the named barriers below need every one of them
         mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 117);
@@ -443,11 +459,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         m = -INFINITY;
         l = 0.f;
       };
-      // the products of the item before `it` (of either phase) have completed
-      // (A parity only tells a barrier's last two phases apart.  The one before, item it - 3's, has passed: this warp has
-      // seen the logits of item it - 1, which were issued behind those products and are taken to be reported behind them.)
+      // the products of the item before (of either phase) have completed
+      // (A parity only tells a barrier's last two phases apart.  The one before, of the item NB earlier, has passed: this warp
+      // has seen the logits of the item before, which were issued behind those products and are taken to be reported behind them.)
       auto products_done = [&](int site) {
-        mbar_wait(b_done + 8 * ((it - 1) & 1), ((it - 1) >> 1) & 1, &abort_flag, site);
+        mbar_wait(b_done + 8 * turn.last_buffer(), turn.last_phase(), &abort_flag, site);
         __syncwarp();
         tc_fence_after();
       };
@@ -457,13 +473,12 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         const int phase_end = phase ? nI : nL;
         const bool isL = phase == 0;
 #pragma unroll 1
-        for (; i < phase_end; ++i, ++it) {
+        for (; i < phase_end; ++i) {
           const int hx = hx_n, cls = (cls_n >> (2 * grp)) & 3;  // this group's half, 32 keys from 32 hx
           if (i + 1 < nI) {  // the next item's half and class, ahead of their use
             hx_n = items[2 * (i + 1) + grp];
             cls_n = icls[(i + 1) * 4 + quarter];
           }
-          const int b = it & 1, ph = (it >> 1) & 1;
           uint32_t hm = 0u;  // this thread's 32 keys of the tile that the row sees
           bool doB = cls == 1;
           if (cls == 2) {
@@ -473,9 +488,10 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
             else hm &= s.stis_mode ? (uint32_t)(st_key_cols(s, t, jt * 64, causal) >> col) : st_window32(s, t, c0, causal);
             doB = __any_sync(0xffffffffu, hm != 0u);
           }
+          const int b = turn.buffer();
           const uint32_t t_b = tmem_base + 64 * b + lane_off + 32 * grp;
 
-          mbar_wait(b_sfull + 8 * b, ph, &abort_flag, 107);
+          mbar_wait(b_sfull + 8 * b, turn.phase(), &abort_flag, 107);
           __syncwarp();
           tc_fence_after();
           uint32_t pk[16];
@@ -507,7 +523,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
           tmem_wait_st();
           tc_fence_before();
-          warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
+          warp_arrive(b_tfull + 8 * (NB * grp + b), lane);  // the stores have completed (wait::st)
+          turn.step();
         }
 
         if (phase_end > (phase ? nL : 0)) products_done(110 + phase);

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   // One warp: the halves hx_min ... hx_max that the CTA's rows (or keys) lo ... hi need, ascending, a lane per tile of two.
   // selected(jt, first, second): bits of tile jt's selections by the first and by the other 64 rows.  In a query-major
   // image the flags also hold which of the two 64-row halves need it, through the long-term branch (bits 2, 3) and at all
-  // (bits 4, 5); n_long, n_all count them by that class.
+  // (bits 4, 5, of a backward's image); n_long, n_all count them by that class.
   auto half_row0 = [&](int row0, int hf) { return pack ? row0 : row0 + 64 * hf; };
   int n_long[4] = {0, 0, 0, 0}, n_all[4] = {0, 0, 0, 0};
   auto list_halves = [&](int hx_min, int hx_max, bool live, int lo, int hi, auto by_key, auto selected) {
@@ -160,10 +160,10 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
           if (!KEYS) {
             if (!(f[x] & 1)) c = 0;
             f[x] |= c << 2;
-            if (f[x] & 2)
+            if ((f[x] & 2) && kmeta)
               for (int hf = 0; hf < 2; ++hf)
                 if ((p0 <= half_row0(lo, hf) + 63 || !causal) && touch(half_row0(lo, hf), half_row0(lo, hf) + 63, p0, p1)) c |= 1 << hf;
-            if (f[x]) f[x] |= (c ? c : 3) << 4;
+            if (f[x] && kmeta) f[x] |= (c ? c : 3) << 4;
           }
         }
         if (!KEYS) {
