@@ -48,7 +48,10 @@ constexpr int kMetaWarps = 4;  // warps per CTA
 // so a launch of few images is shorter with the loops split.  The compactions stay with the first warp.
 // PLAIN: the causal mask, one selection per query block, a window: the other modes' tests fold away, and their code out of
 // the instruction cache (22.7 -> 20.5 us for the 8192 images of B 128, H 4, L 1024, 16.4 -> 14.4 at H 2, 38 -> 35 at B 16, H 8, L 4096).
-template <int NW, bool PLAIN>
+// WHOLE (blocks of 64): a block is needed whole, so the lists' unit is a tile, i.e. its two halves in one word: half as much to
+// list, class and order, and both halves of every pair adjacent.  us with lists of halves -> of tiles, H 8, D 64, 16 blocks:
+// forward at B 1, L 4096 70.2 -> 69.1; forward + backward at B 16, L 4096 1254 -> 1248, at B 1, L 10240 461 -> 457.
+template <int NW, bool PLAIN, bool WHOLE>
 __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const int32_t *__restrict__ seq_lens,
                                                                   const int32_t *__restrict__ idx,
                                                                   uint8_t *__restrict__ qmeta,
@@ -99,14 +102,19 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   const int pad0 = s.L - len;
   uint32_t *selw = reinterpret_cast<uint32_t *>(meta);
   uint8_t *selb = meta;
-  uint16_t *list = reinterpret_cast<uint16_t *>(meta + ml.list);
-  uint8_t *lflags = meta + ml.flags;
-  uint16_t *items = reinterpret_cast<uint16_t *>(meta + ml.items);
+  constexpr int PER = WHOLE ? 1 : 2;  // entries of a list, or of the items, in a pair of halves
+  using Entry = std::conditional_t<WHOLE, uint32_t, uint16_t>;
+  using Flag = std::conditional_t<WHOLE, uint16_t, uint8_t>;
+  auto entry = [](int hx) { return (Entry)(WHOLE ? hx | (hx + 1) << 16 : hx); };
+  Entry *list = reinterpret_cast<Entry *>(meta + ml.list), *items = reinterpret_cast<Entry *>(meta + ml.items);
+  Flag *lflags = reinterpret_cast<Flag *>(meta + ml.flags);
+  const uint16_t *list_half = reinterpret_cast<const uint16_t *>(list), *item_half = reinterpret_cast<const uint16_t *>(items);
+  const uint8_t *flags_half = meta + ml.flags;
   uint8_t *icls = meta + ml.icls;
   uint8_t *jcls = meta + ml.jcls;
   int *counts = reinterpret_cast<int *>(meta + ml.counts);
   const unsigned lt = (1u << lane) - 1u;
-  const int bk_shift = __ffs(s.Bk) - 1, nb_shift = 6 - bk_shift;  // Bk is a power of two
+  const int bk_shift = WHOLE ? 6 : __ffs(s.Bk) - 1, nb_shift = 6 - bk_shift;  // Bk is a power of two
   const int G = 128 >> bk_shift, nb = 1 << nb_shift;  // query blocks of a CTA, blocks of a tile
   // index rows: entry i of a run is slot i % topk of row i / topk; a thread's next entry lies NT further
   const int step_row = NT / s.topk, step_slot = NT % s.topk;
@@ -117,24 +125,25 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   };
   const int row_0 = tid / s.topk, slot_0 = tid % s.topk;
 
-  // place of the k-th of n entries of one kind among those of both kinds: two of the first, two of the second, and so
+  // place of the k-th of n entries of one kind among those of both kinds: a pair of the first, a pair of the second, and so
   // on while there are pairs of both, then what is left
   auto alternate = [](int k, int second, int n, int other) {
-    const int m = min(n, other) & ~1;
-    if (k < m) return 2 * (k & ~1) + (k & 1) + 2 * second;
+    const int m = min(n, other) / PER * PER;
+    if (k < m) return 2 * (k / PER * PER) + k % PER + PER * second;
     return second ? k + other : k + m;
   };
-  // one warp: the list of n halves becomes one of pairs
+  // one warp: the list of n entries becomes one of pairs
   auto pad_list = [&](int n) {
     if (lane == 0) {
-      if (n & 1) {
-        list[n] = (uint16_t)(2 * nT);
+      if (n % PER) {
+        list[n] = (Entry)(2 * nT);
         lflags[n] = 0;
       }
-      counts[0] = (n + 1) / 2;
+      counts[0] = (n + PER - 1) / PER;
     }
   };
-  // One warp: the halves hx_min ... hx_max that the CTA's rows (or keys) lo ... hi need, ascending, a lane per tile of two.
+  // One warp: the halves hx_min ... hx_max (or their tiles) that the CTA's rows (or keys) lo ... hi need, ascending, a lane
+  // per tile of two.
   // selected(jt, first, second): bits of tile jt's selections by the first and by the other 64 rows.  In a query-major
   // image the flags also hold which of the two 64-row halves need it, through the long-term branch (bits 2, 3) and at all
   // (bits 4, 5, of a backward's image); n_long, n_all count them by that class.
@@ -148,14 +157,13 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       const int jt = base + lane;
       uint32_t first[2] = {0u, 0u}, second[2] = {0u, 0u};
       if (jt <= hx_max >> 1) selected(jt, first, second);
-      int f[2];
+      int f[2] = {0, 0};
 #pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const int hx = 2 * jt + x, p0 = hx * 32, p1 = p0 + 31;
-        f[x] = 0;
+      for (int x = 0; x < PER; ++x) {
+        const int hx = 2 * jt + x, p0 = hx * 32, p1 = p0 + 64 / PER - 1;
         if (hx >= hx_min && hx <= hx_max && p1 >= pad0) {
           if (KEYS ? touch(p0, min(p1, s.L - 1), lo, hi) : touch(lo, hi, p0, p1)) f[x] = 2;
-          int c = (first[x] ? 1 : 0) | (second[x] ? 2 : 0);
+          int c = ((WHOLE ? first[0] | first[1] : first[x]) ? 1 : 0) | ((WHOLE ? second[0] | second[1] : second[x]) ? 2 : 0);
           f[x] = (f[x] | (c ? 1 : 0)) & branches;
           if (!KEYS) {
             if (!(f[x] & 1)) c = 0;
@@ -173,13 +181,13 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
           one_all += ca == 1 ? 1u : ca == 2 ? 0x10000u : 0u;
         }
       }
-      const unsigned b0 = __ballot_sync(0xffffffffu, f[0] != 0), b1 = __ballot_sync(0xffffffffu, f[1] != 0);
+      const unsigned b0 = __ballot_sync(0xffffffffu, f[0] != 0), b1 = WHOLE ? 0u : __ballot_sync(0xffffffffu, f[1] != 0);
       int pos = nv + __popc(b0 & lt) + __popc(b1 & lt);
 #pragma unroll
       for (int x = 0; x < 2; ++x)
         if (f[x]) {
-          list[pos] = (uint16_t)(2 * jt + x);
-          lflags[pos++] = (uint8_t)f[x];
+          list[pos] = entry(2 * jt + x);
+          lflags[pos++] = (Flag)(WHOLE ? f[x] * 0x101 : f[x]);
         }
       nv += __popc(b0) + __popc(b1);
     }
@@ -195,7 +203,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
     return nv;
   };
-  // One warp: the list's entries in the order both 64-row halves, then alternately two of the first and two of the second,
+  // One warp: the list's entries in the order both 64-row halves, then alternately a pair of the first and one of the second,
   // by the class in the flags from bit `shift`; place(entry, position) takes them down.
   auto order = [&](int nv, int shift, const int (&n)[4], auto place) {
     int c1 = 0, c2 = 0, c3 = 0;
@@ -269,12 +277,12 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     const int nv = counts[0];
     if (with_fwd) {
     if (scans) {  // ---- the forward's items and their classes ----
-    // Long-term items: the halves that rows of both 64-row halves of the CTA need, then alternately two that only
-    // rows 0..63 need and two that only rows 64..127 need.  A softmax warp may run ahead of the
+    // Long-term items: the halves that rows of both 64-row halves of the CTA need, then alternately a pair that only
+    // rows 0..63 need and a pair that only rows 64..127 need.  A softmax warp may run ahead of the
     // slowest one, so with alternating items both pairs of warps have work at once.
     order(nv, 2, n_long, [&](int j, int pos) { items[pos] = list[j]; });
-    const int n_lt = n_long[1] + n_long[2] + n_long[3], nl = (n_lt + 1) & ~1;
-    if (lane == 0 && nl > n_lt) items[nl - 1] = (uint16_t)(2 * nT);
+    const int n_lt = n_long[1] + n_long[2] + n_long[3], nl = (n_lt + PER - 1) / PER * PER;
+    if (lane == 0 && nl > n_lt) items[nl - 1] = (Entry)(2 * nT);
     int count = nl;
     for (int base = 0; base < nv; base += 32) {  // short-term items in ascending order
       const int j = base + lane;
@@ -284,9 +292,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       count += __popc(bal);
     }
     if (lane == 0) {
-      if (count & 1) items[count++] = (uint16_t)(2 * nT);
-      counts[1] = nl / 2;
-      counts[2] = (count - nl) / 2;
+      if (count % PER) items[count++] = (Entry)(2 * nT);
+      counts[1] = nl / PER;
+      counts[2] = (count - nl) / PER;
     }
     }
     sync();
@@ -301,7 +309,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
       int cls = 0;
 #pragma unroll 1
       for (int hf = 0; hf < 2; ++hf) {
-        const int hx = items[2 * it + hf], k_lo = hx * 32, k_hi = k_lo + 31;
+        const int hx = item_half[2 * it + hf], k_lo = hx * 32, k_hi = k_lo + 31;
         int c = 0;
         if (rows && (k_lo <= t_hi || !causal) && k_hi >= pad0 && k_lo < s.L) {
           // every row of the quarter may see every key of the half as far as validity and causality go
@@ -320,12 +328,12 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }  // the forward's part
     sync();
     // The dQ kernel walks `list` itself (a half serves both branches there).  Same idea as above:
-    // what both 64-row halves need first, then alternately two that only rows 0..63 need and two
+    // what both 64-row halves need first, then alternately a pair that only rows 0..63 need and one
     // only rows 64..127 need, so that the two halves' warps work on neighbouring pairs at once.
     // (Backward call only; the forward reads `items`.)
     if (kmeta && scans) {
-      uint16_t *tlist = reinterpret_cast<uint16_t *>(meta + ml.bytes);
-      uint8_t *tflags = meta + ml.bytes + 4 * nT;
+      Entry *tlist = reinterpret_cast<Entry *>(meta + ml.bytes);
+      Flag *tflags = reinterpret_cast<Flag *>(meta + ml.bytes + 4 * nT);
       order(nv, 4, n_all, [&](int j, int pos) {
         tlist[pos] = list[j];
         tflags[pos] = lflags[j];
@@ -343,9 +351,9 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     // the warp sees all 16 keys through the long-term / short-term branch and no row sees only a
     // part of them; 8: mixed, the warp builds per-lane column masks.  (A forward-only call has no
     // use for them.)
-    for (int e = tid; e < (kmeta ? (nv + 1) / 2 * 16 : 0); e += NT) {
+    for (int e = tid; e < (kmeta ? (nv + PER - 1) / PER * 16 : 0); e += NT) {
       const int j = e >> 3, w = e & 7, qtr = w & 3, c = w >> 2;
-      const int hx = list[j], f = lflags[j], jt = hx >> 1;
+      const int hx = list_half[j], f = flags_half[j], jt = hx >> 1;
       const int k_lo = hx * 32 + 16 * c, k_hi = k_lo + 15, t_lo = quarter_row0(qtr), t_hi = t_lo + 31;
       const bool rows_in = t_lo >= pad0 && t_hi < s.L, rows_none = t_hi < pad0 || t_lo >= s.L;
       const bool past = rows_in && k_lo >= pad0 && (causal ? k_hi <= t_lo : k_hi < s.L);  // every key visible to every row (validity, causality)
@@ -440,7 +448,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     // full by all 16 queries through the long-term / short-term branch and none in part; 8 = mixed.
     for (int e = tid; e < count * 8; e += NT) {
       const int j = e >> 3, w = e & 7, qtr = w & 3, hf = w >> 2;
-      const int hx = list[j], qt = hx >> 1, f = lflags[j], c_lo = 32 * (hx & 1) + 16 * hf;
+      const int hx = list_half[j], qt = hx >> 1, f = flags_half[j], c_lo = 32 * (hx & 1) + 16 * hf;
       const int p_lo = key0 + 32 * qtr, p_hi = p_lo + 31, t_lo = qt * 64 + c_lo, t_hi = t_lo + 15;
       const bool rows_in = p_lo >= pad0 && p_hi < s.L, rows_none = p_hi < pad0 || p_lo >= s.L;
       const bool past = rows_in && t_hi < s.L && (causal ? t_lo >= p_hi : t_lo >= pad0);  // every query sees every key (validity, causality)
@@ -488,8 +496,12 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   const int per_cta = wide ? 1 : kMetaWarps;
   const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((6 * nT + 15) / 16) * 16);
   const bool plain = s.causal && !s.pq && s.stis_mode == 0;
-  auto kern = wide ? (plain ? tc_meta_kernel<kMetaWarps, true> : tc_meta_kernel<kMetaWarps, false>)
-                   : (plain ? tc_meta_kernel<1, true> : tc_meta_kernel<1, false>);
+  auto of = [&](auto whole) {
+    constexpr bool W = decltype(whole)::value;
+    return wide ? (plain ? tc_meta_kernel<kMetaWarps, true, W> : tc_meta_kernel<kMetaWarps, false, W>)
+                : (plain ? tc_meta_kernel<1, true, W> : tc_meta_kernel<1, false, W>);
+  };
+  auto kern = s.Bk == 64 ? of(std::true_type()) : of(std::false_type());
   if (!allow_smem(kern, smem)) return BLOSSOM_ERR_CUDA;
   auto launch = [&](int image0, int image_end, uint32_t *inv_bits) {
     LaunchScope ls(K_TC_META, st);
