@@ -117,10 +117,10 @@ Workspace carve_workspace(const Shape &s, void *base) {
     w.gate_ost = take(on ? qspan * 2 : 0);
     w.qstats2 = reinterpret_cast<float4 *>(take(on ? units * (size_t)((s.L + 63) / 64 * 64) * sizeof(float4) : 0));
     w.qmeta2 = reinterpret_cast<uint8_t *>(take(on ? tc::tc_meta_bytes(s) : 0));
-    w.kmeta2 = reinterpret_cast<uint8_t *>(take(on ? tc::tc_meta_bytes(s) + tc::tc_inv_bits_bytes(s) : 0));
+    w.kmeta2 = reinterpret_cast<uint8_t *>(take(on ? tc::tc_key_meta_bytes(s) + tc::tc_inv_bits_bytes(s) : 0));
   }
   w.qmeta = reinterpret_cast<uint8_t *>(take(tc::tc_meta_bytes(s)));
-  w.kmeta = reinterpret_cast<uint8_t *>(take(tc::tc_meta_bytes(s) + tc::tc_inv_bits_bytes(s)));
+  w.kmeta = reinterpret_cast<uint8_t *>(take(tc::tc_key_meta_bytes(s) + tc::tc_inv_bits_bytes(s)));
   w.bytes = off;
   return w;
 }

@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
   const bool causal = PLAIN || s.causal;
   const int pq = PLAIN ? 0 : s.pq;
   const MetaLayout ml = meta_layout(nT, pq);
-  const uint8_t *selb = meta;
+  const uint8_t *selb = meta + ml.sel;
   const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
   const uint16_t *list = reinterpret_cast<const uint16_t *>(meta + ml.list);
   const uint8_t *lflags = meta + ml.flags;
@@ -297,8 +297,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dq_tc_kernel(
     mbar_init(b_all, 1);
     mbar_fence_init();
     // the CTA's tile lists (the streamed tiles wait for them) and its resident tiles
-    mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
-    bulk_load(smem_u32(meta), qmeta + ((size_t)u * nQT + (nQT - 1 - st)) * ml.bytes, (uint32_t)ml.bytes, b_meta);
+    mbar_expect_tx(b_meta, (uint32_t)ml.bwd);
+    bulk_load(smem_u32(meta), qmeta + ((size_t)u * nQT + (nQT - 1 - st)) * ml.bytes, (uint32_t)ml.bwd, b_meta);
     mbar_expect_tx(b_res, 2 * C::kBigBytes);
     tma_load_4d(smem_u32(q_tile), &tmq, b_res, 0, row0, h, n);
     tma_load_4d(smem_u32(g_tile), &tmg, b_res, 0, row0, h, n);
@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
   const int pq = PLAIN ? 0 : s.pq;
   const MetaLayout ml = meta_layout(nT, pq);
   const uint64_t *inv64 = reinterpret_cast<const uint64_t *>(meta + ml.rows);  // (selection per query position) [8][nT]
-  const uint8_t *invb = meta;                           // [8][nT] bytes: per key block, per query tile
+  const uint8_t *invb = meta + ml.sel;                  // [8][nT] bytes: per key block, per query tile
   const uint16_t *list = reinterpret_cast<const uint16_t *>(meta + ml.list);
   const uint8_t *lflags = meta + ml.flags;
   const uint8_t *kcls = meta + ml.jcls;                 // [listed pair][half][compute warp]
@@ -703,8 +703,8 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     mbar_init(b_all, 1);
     mbar_fence_init();
     // the CTA's tile lists and its resident tiles
-    mbar_expect_tx(b_meta, (uint32_t)ml.bytes);
-    bulk_load(smem_u32(meta), kmeta + ((size_t)uk * nKT + kt) * ml.bytes, (uint32_t)ml.bytes, b_meta);
+    mbar_expect_tx(b_meta, (uint32_t)ml.bwd);
+    bulk_load(smem_u32(meta), kmeta + ((size_t)uk * nKT + kt) * ml.bwd, (uint32_t)ml.bwd, b_meta);
     mbar_expect_tx(b_res, 2 * C::kBigBytes);
     tma_load_4d(smem_u32(k_tile), &tmk, b_res, 0, key0, hk, n);
     tma_load_4d(smem_u32(v_tile), &tmv, b_res, 0, key0, hk, n);
@@ -1006,9 +1006,9 @@ int launch_bwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
     return BLOSSOM_ERR_CUDA;
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const unsigned grid = (unsigned)nST * (unsigned)(s.B * s.H);
-  const size_t smem_dq = 1024 + 2 * C::kBigBytes + kDqStages * 2 * C::kSmallBytes + meta_bytes(nT, s.pq);
-  const size_t smem_kv =
-      1024 + 2 * C::kBigBytes + kKvStages * (2 * C::kSmallBytes + kStatBytes) + meta_bytes(nT, s.pq);
+  const size_t lists = meta_layout(nT, s.pq).bwd;
+  const size_t smem_dq = 1024 + 2 * C::kBigBytes + kDqStages * 2 * C::kSmallBytes + lists;
+  const size_t smem_kv = 1024 + 2 * C::kBigBytes + kKvStages * (2 * C::kSmallBytes + kStatBytes) + lists;
   auto kern_dq = bwd_dq_tc_kernel<D, kGeneral, false>;
   auto kern_kv = bwd_dkdv_tc_kernel<D, kGeneral>;
   if (branches != 3) {

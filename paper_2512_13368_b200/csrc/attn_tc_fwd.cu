@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     const __grid_constant__ CUtensorMap tmk32, const __grid_constant__ CUtensorMap tmv32, Shape s,
     const float *__restrict__ gate, const int32_t *__restrict__ seq_lens,
     const uint8_t *__restrict__ qmeta, int training, float *__restrict__ lse,
-    int32_t *__restrict__ status, int32_t *__restrict__ tickets, int nT, int n_tiles, int n_meta) {
+    int32_t *__restrict__ status, int32_t *__restrict__ tickets, int nT, int n_tiles, int n_meta, int image_bytes, MetaLayout ml) {
   grid_chain_enter();
   using C = Cfg<D>;
   constexpr int STAGES = fwd_stages(D);
@@ -175,10 +175,9 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   uint8_t *q_tiles = tiles;                                  // [2]: the tile's queries, then its staged rows of out
   uint8_t *kv_tiles = q_tiles + 2 * C::kBigBytes;            // [stage][K, V]
   uint8_t *sl = kv_tiles + STAGES * 2 * C::kSmallBytes;      // staged rows: the long-term branch, then the short-term one
-  uint8_t *metas = sl + C::kBigBytes;                        // [n_meta] images built by tc_meta_kernel
+  uint8_t *metas = sl + C::kBigBytes;                        // [n_meta] the forward's part of an image built by tc_meta_kernel
   const bool causal = PLAIN || s.causal;
   const int pq = PLAIN ? 0 : s.pq;
-  const MetaLayout ml = meta_layout(nT, pq);
   const int meta_step = n_meta == 2 ? ml.bytes : 0;
   // tile x of this grid: its rows (tile st of unit u; long rows first, every unit's last tile, then every
   // unit's last but one, ...) and heads
@@ -201,7 +200,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
     } else {
       mbar_expect_tx(bar, (uint32_t)ml.bytes);
       bulk_load(smem_u32(metas) + (k & 1) * meta_step,
-                qmeta + ((size_t)tile_unit(x) * nQT + x / nU) * ml.bytes, (uint32_t)ml.bytes, bar);
+                qmeta + ((size_t)tile_unit(x) * nQT + x / nU) * image_bytes, (uint32_t)ml.bytes, bar);
     }
   };
   auto fetch_queries = [&](int k, int x) {
@@ -390,7 +389,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       if (x < 0) break;
       mbar_wait(b_meta + 8 * (k & 1), (k >> 1) & 1, &abort_flag, 120);  // (complete: makes the lists visible to this warp)
       const uint8_t *meta = metas + (k & 1) * meta_step;
-      const uint8_t *selb = meta;
+      const uint8_t *selb = meta + ml.sel;
       const uint8_t *rowb = meta + ml.rows;  // (selection per query position) [128 rows][nT]
       const uint16_t *items = reinterpret_cast<const uint16_t *>(meta + ml.items);  // [2 nT][2]
       const uint8_t *icls = meta + ml.icls;                                         // [2 nT][4]
@@ -557,7 +556,11 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   // Two CTAs share an SM (228 KB with 1 KB for each and its static part): a second buffer for the lists as long
   // as that stays so.
-  const size_t tiles = 1024 + 3 * C::kBigBytes + fwd_stages(D) * 2 * C::kSmallBytes, list = meta_bytes(nT, s.pq);
+  // (The offsets go to the kernel as an argument: computed there they take registers of the softmax loop: 317 us instead of
+  // 308 at B 16, H 8, L 4096, D 64.)
+  const MetaLayout ml = meta_layout(nT, s.pq, false);
+  const size_t tiles = 1024 + 3 * C::kBigBytes + fwd_stages(D) * 2 * C::kSmallBytes, list = ml.bytes,
+               image = meta_layout(nT, s.pq).bytes;  // (of which the kernel reads the end)
   const size_t kPair = 110 * 1024;
   const int n_meta = tiles + 2 * list <= kPair ? 2 : 1;
   const size_t smem = tiles + n_meta * list;
@@ -575,7 +578,8 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   {
     LaunchScope ls(K_FWD_TC, st);
     launch_chained(kern, dim3(grid), dim3(kFwdThreads), smem, st, tq, tk, tv, to, tol, tos, tk32, tv32, s, gate, seq_lens,
-                   (const uint8_t *)ws.qmeta, training, lse, ws.status, ws.status + kTicketWord, nT, n_tiles, n_meta);
+                   (const uint8_t *)ws.qmeta + (image - list), training, lse, ws.status, ws.status + kTicketWord, nT, n_tiles, n_meta,
+                   (int)image, ml);
   }
   return cudaGetLastError() == cudaSuccess ? BLOSSOM_OK : BLOSSOM_ERR_CUDA;
 }

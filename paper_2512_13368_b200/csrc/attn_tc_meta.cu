@@ -8,14 +8,14 @@
 // memory, and the attention kernel fetches it with one bulk copy while its first tiles load.
 //
 // Query-major image (forward and dQ kernel), see meta_layout():
+//   list[2 nT], flags[2 nT]   (dQ) the halves any row of the CTA needs; bit 0: some selected
+//                             block lies in the half, bit 1: the window of some row reaches it
+//   jcls[nT][2][8]            (dQ) class of every (listed pair, half of it, compute warp)
 //   [8][nT] selection bytes   bit c of byte (g, jt): query block g of the CTA selected key block
 //                             jt * (64 / Bk) + c
-//   list[2 nT], flags[2 nT]   the halves any row of the CTA needs; bit 0: some selected
-//                             block lies in the half, bit 1: the window of some row reaches it
+//   counts                    {pairs on the list, long-term items, short-term items}
 //   items[2 nT][2], icls[2 nT][4] (forward) the long-term halves, then the short-term halves, two an item, and the
 //                             classes of every (item, row quarter), two bits per half
-//   jcls[nT][2][8]            (dQ) class of every (listed pair, half of it, compute warp)
-//   counts                    {pairs on the list, long-term items, short-term items}
 // The attention kernels work on 64 columns at a time, 32 for each group of their compute warps: any two halves
 // make such a pair (an odd one out is paired with the half behind the last, which reads as zeros and has class 0).
 // With tiles of 64 adjacent rows, halves of 32 that no row needs were worked through as well: with blocks of 32 and 128 rows
@@ -85,8 +85,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     if (branches == 2) image -= image_end / 2, qmeta = qmeta2, kmeta = kmeta2;
   }
   const int Lw = (s.L + 31) >> 5;  // words per key block of the bit table
-  const int slice = ml.bytes + ((6 * nT + 15) / 16) * 16;  // the image and a scratch list behind it
-  uint8_t *meta = meta_all + (size_t)sub * slice;
+  uint8_t *meta = meta_all + (size_t)sub * ml.bytes;
   const int nST = (s.L + 127) >> 7;
   const bool key_major = image >= n_query_ctas;
   const int cta = key_major ? image - n_query_ctas : image;
@@ -100,8 +99,8 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   int len = seq_lens ? seq_lens[n] : s.L;
   len = min(max(len, 0), s.L);
   const int pad0 = s.L - len;
-  uint32_t *selw = reinterpret_cast<uint32_t *>(meta);
-  uint8_t *selb = meta;
+  uint32_t *selw = reinterpret_cast<uint32_t *>(meta + ml.sel);
+  uint8_t *selb = meta + ml.sel;
   constexpr int PER = WHOLE ? 1 : 2;  // entries of a list, or of the items, in a pair of halves
   using Entry = std::conditional_t<WHOLE, uint32_t, uint16_t>;
   using Flag = std::conditional_t<WHOLE, uint16_t, uint8_t>;
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
   };
 
-  for (int i = tid; i < ml.bytes / 4; i += NT) selw[i] = 0u;  // the whole image
+  for (int i = ml.rows / 4 + tid; i < ml.bwd / 4; i += NT) reinterpret_cast<uint32_t *>(meta)[i] = 0u;  // what is not written throughout
   sync();
 
   if (!key_major) {
@@ -332,8 +331,8 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     // only rows 64..127 need, so that the two halves' warps work on neighbouring pairs at once.
     // (Backward call only; the forward reads `items`.)
     if (kmeta && scans) {
-      Entry *tlist = reinterpret_cast<Entry *>(meta + ml.bytes);
-      Flag *tflags = reinterpret_cast<Flag *>(meta + ml.bytes + 4 * nT);
+      Entry *tlist = reinterpret_cast<Entry *>(jcls);  // (the classes come later)
+      Flag *tflags = reinterpret_cast<Flag *>(jcls + 4 * nT);
       order(nv, 4, n_all, [&](int j, int pos) {
         tlist[pos] = list[j];
         tflags[pos] = lflags[j];
@@ -472,9 +471,11 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
   }
   sync();
-  uint4 *dst = reinterpret_cast<uint4 *>((key_major ? kmeta : qmeta) + (size_t)cta * ml.bytes);
+  // the parts that this call's kernels read (see MetaLayout)
+  uint4 *dst = reinterpret_cast<uint4 *>(key_major ? kmeta + (size_t)cta * ml.bwd : qmeta + (size_t)cta * ml.bytes);
   const uint4 *src = reinterpret_cast<const uint4 *>(meta);
-  for (int i = tid; i < ml.bytes / 16; i += NT) dst[i] = src[i];
+  const int begin = kmeta ? 0 : ml.rows, end = key_major || !with_fwd ? ml.bwd : ml.bytes;
+  for (int i = begin / 16 + tid; i < end / 16; i += NT) dst[i] = src[i];
 }
 
 }  // namespace
@@ -494,7 +495,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   // four warps took 26 us and one 17.
   const bool wide = n_images * (qmeta2 ? 2 : 1) <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;
-  const size_t smem = (size_t)per_cta * (meta_bytes(nT, s.pq) + ((6 * nT + 15) / 16) * 16);
+  const size_t smem = (size_t)per_cta * meta_layout(nT, s.pq).bytes;
   const bool plain = s.causal && !s.pq && s.stis_mode == 0;
   auto of = [&](auto whole) {
     constexpr bool W = decltype(whole)::value;
@@ -511,7 +512,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it
-    uint32_t *inv_bits = reinterpret_cast<uint32_t *>(kmeta + tc_meta_bytes(s));
+    uint32_t *inv_bits = reinterpret_cast<uint32_t *>(kmeta + tc_key_meta_bytes(s));
     if (cudaMemsetAsync(inv_bits, 0, tc_inv_bits_bytes(s), st) != cudaSuccess) return BLOSSOM_ERR_CUDA;
     launch(0, nq, inv_bits);
     launch(nq, n_images, inv_bits);

@@ -282,7 +282,8 @@ namespace tc {
 int launch_wait_selftest(int32_t *status, cudaStream_t st);
 bool fwd_tc_supported(const Shape &s, int dtype);
 int dkdv_split(const Shape &s, bool lengths);  // CTAs of a cluster that share a key tile's heads in the backward
-size_t tc_meta_bytes(const Shape &s);  // bytes of one of the two tile-list areas of the workspace
+size_t tc_meta_bytes(const Shape &s);  // bytes of the query-major tile lists in the workspace
+size_t tc_key_meta_bytes(const Shape &s);  // of the key-major ones
 size_t tc_inv_bits_bytes(const Shape &s);  // (selection per position) bytes of the bit table behind the second
 // branches: bit 0 long-term, bit 1 short-term branch: the tile lists hold only the tiles those
 // branches need.  records: null = computed from out_lt, out_st, lse, dout and the per-head gate by

@@ -480,32 +480,40 @@ struct Cfg {
   static constexpr int kKStep = (16 * kRowBytes) >> 4;       // descriptor advance of 16 rows
 };
 
-// Per-CTA tile bookkeeping, built once per call by tc_meta_kernel and brought into shared memory
-// by one bulk copy: [8][nT] selection bytes, 2 nT list entries and flags (half tiles of 32 rows), (forward) up to
-// 4 nT halves as per-phase items of two with 4 class bytes each, (dQ, dK/dV) 16 class bytes per two listed halves, and the
-// counts {pairs of halves on the list, long-term items, short-term items}.  Offsets in bytes; every part starts on a
-// 16-byte boundary where a copy needs it, and the two halves of a pair or an item share an aligned word.
-// With a selection per query position (pq) an area of 128 nT bytes follows: in a query-major
+// Per-CTA tile bookkeeping, an image built once per call by tc_meta_kernel and brought into shared memory by one bulk copy
+// of the parts that a kernel reads:
+//   dQ, dK/dV  list[2 nT], flags[2 nT] half tiles of 32 rows; jcls: 16 class bytes per two listed halves
+//   all        rows (below); sel[8][nT] selection bytes; counts {pairs of halves on the list, long-term items, short-term items}
+//   forward    items: up to 4 nT halves as per-phase items of two, icls: 4 class bytes for each
+// dQ and dK/dV copy the first `bwd` bytes, which is all that a key-major image has, the forward the rest from `rows` on
+// (its layout: without `back`).
+// (At D 64 dK/dV keep their second CTA on an SM up to L 25.6k so, dQ up to 34k, the forward up to 35k and its second list buffer
+// up to 17.7k; with whole images, 46 bytes a tile, everywhere it was 16.5k, 22k, 18k and 9k.
+// us, B 1, H 8, D 64, blocks of 64: forward at L 20480 183 -> 127, dK/dV 304 -> 190; dK/dV at L 17408 256 -> 162.)
+// Offsets in bytes; every part starts on a 16-byte boundary where a copy needs it, and the two halves of a pair or an item
+// share an aligned word.
+// With a selection per query position (pq) `rows` has 128 nT bytes: in a query-major
 // image [128 rows][nT] bytes, bit c of byte (r, jt): row r of the CTA selected key block
-// jt * (64 / Bk) + c (the [8][nT] bytes at the start are then the union over a query block's
+// jt * (64 / Bk) + c (the selection bytes are then the union over a query block's
 // rows); in a key-major image [8][nT] 64-bit words, bit i of word (g, qt): query position
 // 64 qt + i selected key block g of the CTA.
 struct MetaLayout {
-  int list, flags, items, icls, jcls, counts, rows, bytes;
+  int list, flags, jcls, sel, rows, counts, bwd, items, icls, bytes;
 };
-__host__ __device__ inline MetaLayout meta_layout(int nT, int pq = 0) {
+__host__ __device__ inline MetaLayout meta_layout(int nT, int pq = 0, bool back = true) {
   MetaLayout m;
-  m.list = ((8 * nT + 15) / 16) * 16;
+  m.list = 0;
   m.flags = m.list + 4 * nT;
-  m.items = ((m.flags + 2 * nT + 15) / 16) * 16;
+  m.jcls = ((m.flags + 2 * nT + 15) / 16) * 16;
+  m.rows = back ? m.jcls + 16 * nT : 0;
+  m.sel = m.rows + (pq ? 128 * nT : 0);
+  m.counts = m.sel + ((8 * nT + 15) / 16) * 16;
+  m.bwd = m.counts + 16;
+  m.items = m.bwd;
   m.icls = m.items + 8 * nT;
-  m.jcls = ((m.icls + 8 * nT + 15) / 16) * 16;
-  m.counts = m.jcls + 16 * nT;
-  m.rows = m.counts + 16;
-  m.bytes = m.rows + (pq ? 128 * nT : 0);
+  m.bytes = m.icls + 8 * nT;
   return m;
 }
-__host__ __device__ inline int meta_bytes(int nT, int pq = 0) { return meta_layout(nT, pq).bytes; }
 // selection bits of half tile hx (32 rows) in the byte of its 64-row tile
 __device__ __forceinline__ uint32_t half_bits(int hx, int bk_shift) {
   return bk_shift == 6 ? 1u : bk_shift == 5 ? 1u << (hx & 1) : 3u << (2 * (hx & 1));
@@ -555,7 +563,7 @@ int make_tensor_map(CUtensorMap *map, const void *base, const Shape &s, int box_
                     int box_heads = 1);
 
 // Builds the bookkeeping of every query-major CTA (forward, dQ) into qmeta and, if kmeta is not
-// null, of every key-major CTA (dK/dV) into kmeta: meta_bytes(nT) bytes per CTA, CTA-major.
+// null, of every key-major CTA (dK/dV) into kmeta: CTA-major, an image (key-major: its first `bwd` bytes) per CTA.
 // branches: bit 0 long-term, bit 1 short-term: tiles that only the other branch needs are left out.
 // with_fwd: 1 = the query-major images carry the forward's items, 0 = not, -1 = only when no
 // key-major images are asked for (a forward call builds the forward's part, a backward call the
