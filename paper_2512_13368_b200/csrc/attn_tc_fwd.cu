@@ -74,9 +74,9 @@ constexpr int kProducerRegs = 40, kSoftmaxRegs = 96;
 static_assert(256 * kSoftmaxRegs + 128 * kProducerRegs <= kFwdThreads * 80, "register pool of a CTA");
 constexpr uint32_t kFwdTmemCols = 256;
 __host__ __device__ constexpr int fwd_stages(int D) { return D == 64 ? 3 : 4; }
-constexpr int NB = 2;  // logits / probability buffers (a third, for which D 32 leaves room: B 128, H 2, L 1024 282 -> 286 us)
-// The buffer of the next item and its phase, and those of the item before.  The issuer and the softmax warps count for
-// themselves (with the loader's counter for the issuer too: L 4096, B 1, H 8 70.4 -> 71.4 us; D 32, L 1024 286 -> 284).
+// Two logits / probability buffers take turns: the next item's and its phase, and those of the item before.  The issuer
+// and the softmax warps count for themselves (with the loader's counter for the issuer too: L 4096, B 1, H 8 70.4 -> 71.4 us;
+// D 32, L 1024 286 -> 284).
 struct Turn {
   int x = 0;
   __device__ __forceinline__ int buffer() const { return x & 1; }
@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   constexpr int DC = D / 2;  // output columns a softmax thread merges and stages
   extern __shared__ uint8_t smem_raw[];
   // barriers: full[STAGES], empty[STAGES], then by tile res[2], meta[2], roles[2], then staged, stored, then per buffer
-  // s_full[NB], t_full[group][NB], done[NB]
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 8 + 4 * NB];
+  // s_full[2], t_full[group][2], done[2]
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 16];
   __shared__ int softmax_tile, tile_id[2];  // the tile whose lists lie (or are about to) behind meta[.]; -1: no more
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
   const uint32_t b_res = smem_u32(&bars[2 * STAGES]), b_meta = smem_u32(&bars[2 * STAGES + 2]);
   const uint32_t b_roles = smem_u32(&bars[2 * STAGES + 4]);
   const uint32_t b_staged = smem_u32(&bars[2 * STAGES + 6]), b_stored = smem_u32(&bars[2 * STAGES + 7]);
-  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 8]), b_tfull = b_sfull + 8 * NB;  // [group][buffer]
-  const uint32_t b_done = b_tfull + 16 * NB;
+  const uint32_t b_sfull = smem_u32(&bars[2 * STAGES + 8]), b_tfull = b_sfull + 16;  // [group][buffer]
+  const uint32_t b_done = b_tfull + 32;
   // one thread: the lists (and which tile's they are) and the queries of this CTA's k-th tile, number x
   auto fetch_meta = [&](int k, int x) {
     tile_id[k & 1] = x;
@@ -223,11 +223,9 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
       mbar_init(b_res + 8 * i, 1);
       mbar_init(b_meta + 8 * i, 1);
       mbar_init(b_roles + 8 * i, 2);
-    }
-    for (int i = 0; i < NB; ++i) {
       mbar_init(b_sfull + 8 * i, 1);
-      mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);         // group 0
-      mbar_init(b_tfull + 8 * (NB + i), kSoftmaxWarps / 2);  // group 1
+      mbar_init(b_tfull + 8 * i, kSoftmaxWarps / 2);        // group 0
+      mbar_init(b_tfull + 8 * (2 + i), kSoftmaxWarps / 2);  // group 1
       mbar_init(b_done + 8 * i, 1);
     }
     mbar_init(b_staged, kSoftmaxWarps);
@@ -334,7 +332,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           int ss = sj, sp = sph;  // stage and phase of the next logits
           auto step_s = [&] { if (++ss == STAGES) { ss = 0; sp ^= 1; } };
           Turn ahead = turn;
-          for (int i = 0; i < NB && i < nI; ++i, step_s(), ahead.step()) logits(ahead.buffer(), ss, sp);
+          for (int i = 0; i < 2 && i < nI; ++i, step_s(), ahead.step()) logits(ahead.buffer(), ss, sp);
           for (int i = 0; i < nI; ++i, step()) {
             const int b = turn.buffer(), ph = turn.phase();
             turn.step();
@@ -350,7 +348,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
                 umma_bf16_ts(tmem_oa, tp + 8 * c, dv + c * C::kKStep, idesc_pv, (first | (uint32_t)c) != 0u);
             }
             __syncwarp();
-            mbar_wait(b_tfull + 8 * (NB + b), ph, &abort_flag, 109);
+            mbar_wait(b_tfull + 8 * (2 + b), ph, &abort_flag, 109);
             tc_fence_after();
             if (elect_one()) {
 #pragma unroll
@@ -360,7 +358,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
               umma_commit(b_empty + 8 * sj);  // S(i) completed before the softmax warps read it
             }
             __syncwarp();
-            if (i + NB < nI) {
+            if (i + 2 < nI) {
               logits(b, ss, sp);
               step_s();
             }
@@ -459,7 +457,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
         l = 0.f;
       };
       // the products of the item before (of either phase) have completed
-      // (A parity only tells a barrier's last two phases apart.  The one before, of the item NB earlier, has passed: this warp
+      // (A parity only tells a barrier's last two phases apart.  The one before, of the item two earlier, has passed: this warp
       // has seen the logits of the item before, which were issued behind those products and are taken to be reported behind them.)
       auto products_done = [&](int site) {
         mbar_wait(b_done + 8 * turn.last_buffer(), turn.last_phase(), &abort_flag, site);
@@ -522,7 +520,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) fwd_tc_kernel(
           tmem_st16u(t_b, pk);  // the probabilities replace this thread's logits
           tmem_wait_st();
           tc_fence_before();
-          warp_arrive(b_tfull + 8 * (NB * grp + b), lane);  // the stores have completed (wait::st)
+          warp_arrive(b_tfull + 8 * (2 * grp + b), lane);  // the stores have completed (wait::st)
           turn.step();
         }
 
