@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
                                                                   int branches, int with_fwd,
                                                                   uint32_t *__restrict__ inv_bits,
                                                                   int32_t *__restrict__ tickets,
-                                                                  uint8_t *qmeta2, uint8_t *kmeta2, int release_late) {
+                                                                  uint8_t *qmeta2, uint8_t *kmeta2, int release_late,
+                                                                  const MetaLayout ml) {
   if (!release_late) grid_release();
   grid_wait();
   if (release_late) grid_release();
@@ -75,7 +76,6 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     else __syncthreads();
   };
   extern __shared__ __align__(16) uint8_t meta_all[];
-  const MetaLayout ml = meta_layout(nT, pq);
   const int lane = threadIdx.x & 31, tid = threadIdx.x % NT, sub = threadIdx.x / NT;
   const bool scans = tid < 32;  // the warp that compacts
   int image = image0 + (int)blockIdx.x * (kMetaWarps / NW) + sub;  // this launch builds [image0, image_end)
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
     }
   };
 
-  for (int i = ml.rows / 4 + tid; i < ml.bwd / 4; i += NT) reinterpret_cast<uint32_t *>(meta)[i] = 0u;  // what is not written throughout
+  for (int i = ml.sel / 4 + tid; i < ml.bwd / 4; i += NT) reinterpret_cast<uint32_t *>(meta)[i] = 0u;  // what is not written throughout
   sync();
 
   if (!key_major) {
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kMetaWarps * 32) tc_meta_kernel(Shape s, const
   // the parts that this call's kernels read (see MetaLayout)
   uint4 *dst = reinterpret_cast<uint4 *>(key_major ? kmeta + (size_t)cta * ml.bwd : qmeta + (size_t)cta * ml.bytes);
   const uint4 *src = reinterpret_cast<const uint4 *>(meta);
-  const int begin = kmeta ? 0 : ml.rows, end = key_major || !with_fwd ? ml.bwd : ml.bytes;
+  const int begin = kmeta ? 0 : ml.sel, end = key_major || !with_fwd ? ml.bwd : ml.bytes;
   for (int i = begin / 16 + tid; i < end / 16; i += NT) dst[i] = src[i];
 }
 
@@ -495,7 +495,9 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   // four warps took 26 us and one 17.
   const bool wide = n_images * (qmeta2 ? 2 : 1) <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;
-  const size_t smem = (size_t)per_cta * meta_layout(nT, s.pq).bytes;
+  // (an argument of the kernel: computed there the offsets cost launches of few images 0.5 to 1.5 of their 9 to 12 us)
+  const MetaLayout ml = meta_layout(nT, s.pq);
+  const size_t smem = (size_t)per_cta * ml.bytes;
   const bool plain = s.causal && !s.pq && s.stis_mode == 0;
   auto of = [&](auto whole) {
     constexpr bool W = decltype(whole)::value;
@@ -508,7 +510,7 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
     LaunchScope ls(K_TC_META, st);
     launch_chained(kern, dim3((unsigned)((image_end - image0 + per_cta - 1) / per_cta)), dim3(kMetaWarps * 32), smem, st, s,
                    seq_lens, idx, qmeta, kmeta, nT, nq, image0, image_end, branches, with_fwd, inv_bits, tickets, qmeta2,
-                   kmeta2, (int)release_late);
+                   kmeta2, (int)release_late, ml);
   };
   if (s.pq && kmeta) {
     // selection per position: the query-major images fill the bit table, then the key-major ones read it

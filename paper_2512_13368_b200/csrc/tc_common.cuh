@@ -483,9 +483,9 @@ struct Cfg {
 // Per-CTA tile bookkeeping, an image built once per call by tc_meta_kernel and brought into shared memory by one bulk copy
 // of the parts that a kernel reads:
 //   dQ, dK/dV  list[2 nT], flags[2 nT] half tiles of 32 rows; jcls: 16 class bytes per two listed halves
-//   all        rows (below); sel[8][nT] selection bytes; counts {pairs of halves on the list, long-term items, short-term items}
+//   all        sel[8][nT] selection bytes; counts {pairs of halves on the list, long-term items, short-term items}; rows
 //   forward    items: up to 4 nT halves as per-phase items of two, icls: 4 class bytes for each
-// dQ and dK/dV copy the first `bwd` bytes, which is all that a key-major image has, the forward the rest from `rows` on
+// dQ and dK/dV copy the first `bwd` bytes, which is all that a key-major image has, the forward the rest from `sel` on
 // (its layout: without `back`).
 // (At D 64 dK/dV keep their second CTA on an SM up to L 25.6k so, dQ up to 34k, the forward up to 35k and its second list buffer
 // up to 17.7k; with whole images, 46 bytes a tile, everywhere it was 16.5k, 22k, 18k and 9k.
@@ -505,10 +505,10 @@ __host__ __device__ inline MetaLayout meta_layout(int nT, int pq = 0, bool back 
   m.list = 0;
   m.flags = m.list + 4 * nT;
   m.jcls = ((m.flags + 2 * nT + 15) / 16) * 16;
-  m.rows = back ? m.jcls + 16 * nT : 0;
-  m.sel = m.rows + (pq ? 128 * nT : 0);
+  m.sel = back ? m.jcls + 16 * nT : 0;
   m.counts = m.sel + ((8 * nT + 15) / 16) * 16;
-  m.bwd = m.counts + 16;
+  m.rows = m.counts + 16;
+  m.bwd = m.rows + (pq ? 128 * nT : 0);
   m.items = m.bwd;
   m.icls = m.items + 8 * nT;
   m.bytes = m.icls + 8 * nT;
