@@ -11,9 +11,9 @@
 // Main kernels: CTA = 384 threads.  Warps 0..7 compute; warps 8, 9 stay converged and one elected lane
 // of each issues the TMA loads and the MMAs (10 and 11 are spare); registers move from those warps to the
 // compute warps (setmaxnreg).  A CTA owns a resident 128-row tile (rows = TMEM lanes) and streams pairs of
-// half tiles of 32 rows past it (any two: tc_meta_kernel lists only those that are needed), each half with a buffer in tensor memory and four compute warps of
-// its own: warps w and w + 4 both address TMEM lane quarter w % 4; the first takes the first half of every
-// pair, the second the other, so the two halves never wait for each other.  The tile arithmetic runs in
+// half tiles of 32 rows past it (any two: tc_meta_kernel lists only those that are needed), each half with a buffer in
+// tensor memory and four compute warps of its own: warps w and w + 4 both address TMEM lane quarter w % 4; the first
+// takes the first half of every pair, the second the other, so the two halves never wait for each other.  The tile arithmetic runs in
 // 16-column passes, two columns per FMA / ADD / MUL (packed f32x2); outputs are staged in shared
 // memory and written with whole-line TMA stores.
 //
@@ -31,8 +31,8 @@
 // CTA spends outside its loop.
 //
 //  dQ     resident Q, dO (128 queries: 128 positions of a head, or with grouped heads 64 positions
-//         of two heads of a group, as in the forward); streams pairs of half tiles of K, V (same walk as the forward), 32 keys each.  Tensor memory: a buffer of 64 columns
-//         for each half (S in its first 32 columns, dP in the other 32),
+//         of two heads of a group, as in the forward); streams pairs of half tiles of K, V (same walk as the
+//         forward), 32 keys each.  Tensor memory: a buffer of 64 columns for each half (S in its first 32 columns, dP in the other 32),
 //         Q and dO as first operands of the first-stage products [128,128+D/2), [160,160+D/2)
 //         (read from shared memory they cost 4 KB per product, more than the data pipe delivers
 //         in the product's run time), and dQ [192,192+D).  S = Q K^T, dP = dO V^T; P_x = exp(S - lse_x);
@@ -40,9 +40,9 @@
 //         branches, they share K).  A thread writes the dS (bf16 pairs) of a pass's 16 columns over the first 8
 //         of them in S, from where dQ += dS K reads it: the compute warps wait for one
 //         thing per half tile (its S and dP).  d alpha = sum (P_lt - P_st) dP from the fp32 probabilities, subtracted pair by pair.
-//  dK/dV  transposed: resident K, V of 128 keys, streams pairs of half tiles of Q, dO, 32 queries each (and their row
-//         records, by bulk copy), that selected one of its key blocks or whose window reaches them.  Tensor memory: a buffer of 64
-//         columns for each half (S^T in its first 32 columns, dP^T in the other
+//  dK/dV  transposed: resident K, V of 128 keys, streams pairs of half tiles of Q, dO, 32 queries each (and
+//         their row records, by bulk copy), that selected one of its key blocks or whose window reaches them.
+//         Tensor memory: a buffer of 64 columns for each half (S^T in its first 32 columns, dP^T in the other
 //         32), dV [128,128+D), dK [192,192+D).  S^T = K Q^T, dP^T = V dO^T; thread = key row and
 //         32 query columns; it writes W^T = P'_lt + P'_st and dS^T (bf16 pairs) of a pass's 16 columns over
 //         the first 8 of them in S^T / dP^T, from where dV += W^T dO and dK += dS^T Q read
@@ -67,7 +67,7 @@ constexpr int kComputeWarps = 8;
 constexpr int kDqStages = 4;
 constexpr int kKvStages = 4;
 constexpr uint32_t kBwdTmemCols = 256;
-constexpr int kStatBytes = 64 * 16;  // one 64-query tile of row records
+constexpr int kStatBytes = 64 * 16;  // row records of a pair of half tiles of queries
 
 __device__ __forceinline__ bool bit(uint32_t w, int c) { return (w >> c) & 1u; }
 

@@ -569,7 +569,7 @@ int launch_fwd_tc_t(const Shape &s, const void *q, const void *k, const void *v,
   const int n_tiles = s.pack ? nT * (s.B * (s.H / 2)) : nST * (s.B * s.H);
   const int resident = 148 * (smem <= kPair ? 2 : 1);
   const unsigned grid = (unsigned)(n_tiles < resident ? n_tiles : resident);
-  // A training call also builds the backward's tile lists (the same launch: one warp per image):
+  // A training call also builds the backward's tile lists (the same launch):
   // a backward call told to reuse them (blossom_params::reuse_tile_lists) then builds none.  (The backward of an
   // input-dependent gate takes lists of one branch at a time: it builds its own.)
   if (int rc = launch_tc_meta(s, seq_lens, idx, ws.qmeta, training && !s.gate_mode ? ws.kmeta : nullptr, st, ws.status + kTicketWord, 3, 1)) return rc;

@@ -20,7 +20,7 @@
 // make such a pair (an odd one out is paired with the half behind the last, which reads as zeros and has class 0).
 // With tiles of 64 adjacent rows, halves of 32 that no row needs were worked through as well: with blocks of 32 and 128 rows
 // a CTA 8 % of the items at L 1024 with 8 blocks each, 22 % at L 777 without the causal mask with 6.  us, forward + backward:
-// B 128, H 4, L 1024, D 64 726 -> 695; H 2, D 32 296 -> 284; without the mask, B 16, H 4, L 777 114 -> 108.
+// B 128, H 4, L 1024, D 64 677 -> 654; H 2, D 32 293 -> 287; without the mask, B 16, H 4, L 777 117 -> 112.
 // Head-packed variant (Shape::pack): the CTA's rows 0..63 and 64..127 are the same 64 positions of
 // two query heads with a common key/value head, so both halves have the same selection bytes and
 // every listed tile concerns both.
@@ -44,10 +44,10 @@ constexpr int kMetaWarps = 4;  // warps per CTA
 
 // NW warps build one image.  One: no block-wide barrier anywhere, so the images of a large launch are in
 // flight at once and the issue slots are what counts.  Four: an image's loops are a chain of loads and
-// atomics that one warp takes 8 - 40 us for (the selection per position has 128 index rows to go through),
+// atomics that one warp takes 8 - 25 us for (the selection per position has 128 index rows to go through),
 // so a launch of few images is shorter with the loops split.  The compactions stay with the first warp.
 // PLAIN: the causal mask, one selection per query block, a window: the other modes' tests fold away, and their code out of
-// the instruction cache (22.7 -> 20.5 us for the 8192 images of B 128, H 4, L 1024, 16.4 -> 14.4 at H 2, 38 -> 35 at B 16, H 8, L 4096).
+// the instruction cache (22.7 -> 20.7 us for the 8192 images of B 128, H 4, L 1024, 17.0 -> 14.6 at H 2, 33.2 -> 29.5 at B 16, H 8, L 4096).
 // WHOLE (blocks of 64): a block is needed whole, so the lists' unit is a tile, i.e. its two halves in one word: half as much to
 // list, class and order, and both halves of every pair adjacent.  us with lists of halves -> of tiles, H 8, D 64, 16 blocks:
 // forward at B 1, L 4096 70.2 -> 69.1; forward + backward at B 16, L 4096 1254 -> 1248, at B 1, L 10240 461 -> 457.
@@ -490,9 +490,10 @@ int launch_tc_meta(const Shape &s, const int32_t *seq_lens, const int32_t *idx, 
   }
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
   const int nq = s.pack ? nT * s.B * (s.H / 2) : nST * s.B * s.H, n_images = kmeta ? nq + nST * s.B * s.Hkv : nq;
-  // Four warps per image while its loops are long (a selection per position: 46 -> 28 us for 960 images at
-  // L 1500) or the images do not fill the SMs (11 -> 10 us for 256 images at L 4096); at 4096 images of L 1024
-  // four warps took 26 us and one 17.
+  // Four warps per image while its loops are long (a selection per position) or the images do not fill the SMs.  us with
+  // one | four, by the number of images: L 1024, blocks of 32, 1024 12.0 | 10.6, 2048 12.5 | 14.1, 8192 20.7 | 32.5; L 4096,
+  // blocks of 64, 1024 14.8 | 11.7, 2048 16.5 | 14.4, 4096 20.0 | 21.6; a selection per position, both launches, L 1500 960
+  // 46.6 | 31.4, 3840 54.2 | 54.3, 7680 79 | 86, L 400 1152 31.6 | 25.5, 4608 39.9 | 45.1.
   const bool wide = n_images * (qmeta2 ? 2 : 1) <= 148 * (s.pq ? 48 : 8);
   const int per_cta = wide ? 1 : kMetaWarps;
   // (an argument of the kernel: computed there the offsets cost launches of few images 0.5 to 1.5 of their 9 to 12 us)
