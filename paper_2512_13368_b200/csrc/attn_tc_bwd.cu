@@ -826,14 +826,13 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
     int li = 0;
     for (int i = 0; i < nvis; ++i) {
       if (li == nlist) li = 0;
-      const int hx = list[2 * li + half], f = lflags[2 * li + half], qt = hx >> 1, col = 32 * (hx & 1), t0 = 32 * hx;
       const uint8_t *cls2 = kcls + li * 16 + 8 * half + quarter;  // classes of the half tile's two column halves
       const int cls0 = cls2[0], cls1 = cls2[4];
-      ++li;
       uint32_t hL = 0u, hS = 0u;
       const bool masked = ((cls0 | cls1) & 8) || (cls0 & 3) == 3 || (cls1 & 3) == 3;
       if ((cls0 | cls1) & 8) {  // a mixed half: per-lane column masks
         if (row_valid) {
+          const int hx = list[2 * li + half], f = lflags[2 * li + half], qt = hx >> 1, col = 32 * (hx & 1), t0 = 32 * hx;
           const uint32_t mc = cols32_ge((causal ? p : pad0) - t0) & cols32_le(s.L - 1 - t0);
           if (f & 1) hL = mc & (pq ? (uint32_t)(inv64[g * nT + qt] >> col) : expand_block_bits32(invb[g * nT + qt], s.Bk, col));
           if (f & 2) hS = mc & (uint32_t)(st_query_cols(s, p, qt * 64, causal) >> col);
@@ -842,6 +841,7 @@ __global__ void __launch_bounds__(kKvThreads, 2) bwd_dkdv_tc_kernel(
         hL = (cls0 & 1 ? 0xffffu : 0u) | (cls1 & 1 ? 0xffff0000u : 0u);
         hS = (cls0 & 2 ? 0xffffu : 0u) | (cls1 & 2 ? 0xffff0000u : 0u);
       }
+      ++li;
       mbar_wait(b_full + 8 * (i % STAGES), (i / STAGES) & 1, &abort_flag, 216);  // the row records have landed
       const float4 *stt = reinterpret_cast<const float4 *>(qg_tiles + (i % STAGES) * kStageBytes + 2 * C::kSmallBytes);
       mbar_wait(b_sfull + 8 * half, i & 1, &abort_flag, 217);
