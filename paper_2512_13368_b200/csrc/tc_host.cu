@@ -93,9 +93,10 @@ size_t tc_meta_bytes(const Shape &s) {
   return ((size_t)s.B * s.H * nST * (size_t)meta_layout(nT, s.pq).bytes + 255) / 256 * 256;
 }
 
+// (room for as many images as there are query heads: the workspace does not depend on the key/value heads)
 size_t tc_key_meta_bytes(const Shape &s) {
   const int nT = (s.L + 63) / 64, nST = (s.L + 127) / 128;
-  return ((size_t)s.B * s.Hkv * nST * (size_t)meta_layout(nT, s.pq).bwd + 255) / 256 * 256;
+  return ((size_t)s.B * s.H * nST * (size_t)meta_layout(nT, s.pq).bwd + 255) / 256 * 256;
 }
 
 // Selection per query position: one bit per (batch, key/value head, key block, position) = that
